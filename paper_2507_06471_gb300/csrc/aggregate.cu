@@ -16,6 +16,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "rowwalk.cuh"
 
 namespace cd {
 namespace {
@@ -104,15 +105,27 @@ __global__ void k_iota(int32_t* a, int64_t n) {
 
 // ------------------------------------------------------------------ modularity
 
+// A label outside [0, n) sets acc[3] (the other kernels use labels only to
+// compare them), so checking a caller's labels costs no pass of its own.
 __global__ void k_mod_vol(const int32_t* __restrict__ labels, const int64_t* __restrict__ degw,
-                          int64_t n, unsigned long long* volc) {
+                          int64_t n, unsigned long long* volc, unsigned long long* acc) {
+  __shared__ CtaSums vol;
+  vol.clear();
+  __syncthreads();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride)
-    atomicAdd(&volc[labels[v]], (unsigned long long)degw[v]);
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+    const int32_t c = labels[v];
+    if (c < 0 || c >= n)
+      acc[3] = 1;
+    else
+      vol.add(volc, c, (unsigned long long)degw[v]);
+  }
+  __syncthreads();
+  vol.flush(volc);
 }
 
 // acc[0..1]: 128-bit unsigned accumulator (low, high) for sum vol(c)^2;
-// acc[2]: I, the weight of arcs inside communities.
+// acc[2]: I, the weight of arcs inside communities; acc[3]: 1 = a bad label.
 __device__ __forceinline__ void atomic_add_u128(unsigned long long* acc, unsigned __int128 x) {
   const unsigned long long lo = (unsigned long long)x, hi = (unsigned long long)(x >> 64);
   const unsigned long long old = atomicAdd(&acc[0], lo);
@@ -138,19 +151,37 @@ __global__ void __launch_bounds__(NT) k_mod_sq(const unsigned long long* __restr
   if (threadIdx.x == 0 && part[0]) atomic_add_u128(acc, part[0]);
 }
 
+// I: the arcs split evenly over the warps (see rowwalk.cuh). The columns are
+// the library's own arrays, which start on a 16-byte boundary and carry
+// COL_PAD spare entries, so a 16-byte load that starts before m is inside.
 template <class W>
 __global__ void __launch_bounds__(NT) k_mod_internal(const int64_t* __restrict__ off,
                                                      const int32_t* __restrict__ cols, const void* w,
-                                                     int64_t n, const int32_t* __restrict__ labels,
+                                                     int64_t n, int64_t m, int64_t piece,
+                                                     const int32_t* __restrict__ labels,
                                                      unsigned long long* acc) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * NT) >> 5;
+  __shared__ __align__(16) int32_t mark[NT / 32][WALK_TILE];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t step = (((int64_t)gridDim.x * NT) >> 5) * piece;
   int64_t s = 0;
-  for (int64_t v = warp; v < n; v += nwarps) {
-    const int32_t a = labels[v];
-    for (int64_t e = off[v] + lane; e < off[v + 1]; e += 32)
-      if (labels[cols[e]] == a) s += W::get(w, e);
+  for (int64_t e0 = (((int64_t)blockIdx.x * NT + threadIdx.x) >> 5) * piece; e0 < m; e0 += step) {  // uniform in the warp
+    const int64_t e1 = e0 + piece < m ? e0 + piece : m;
+    int64_t cur = warp_row_of(off, n, e0);
+    for (int64_t ts = e0; ts < e1; ts += WALK_TILE) {
+      const int64_t e = ts + 4 * lane;
+      const int4 c4 = e < e1 ? __ldg(reinterpret_cast<const int4*>(cols + e)) : make_int4(0, 0, 0, 0);
+      const int32_t cs[4] = {c4.x, c4.y, c4.z, c4.w};
+      int32_t lc[4], lr[4];
+      int64_t row[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) lc[j] = e + j < e1 ? labels[cs[j]] : -1;
+      warp_tile_rows(off, n, ts, cur, mark[wid], row);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) lr[j] = e + j < e1 ? labels[row[j]] : -2;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (lc[j] == lr[j]) s += W::get(w, e + j);
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
@@ -292,12 +323,13 @@ int modularity(cd_graph* g, const int32_t* labels_dev, double* q_out) {
   cudaStream_t s = g->stream;
   const int64_t n = g->n;
   if (g->vol == 0) {
-    *q_out = 0.0;
-    return CD_OK;
+    const int rc = check_labels(g, labels_dev);
+    if (!rc) *q_out = 0.0;
+    return rc;
   }
   unsigned long long *volc = nullptr, *acc = nullptr;
   int rc = dev_alloc_t(&volc, n, s);
-  if (!rc) rc = dev_alloc_t(&acc, 3, s);
+  if (!rc) rc = dev_alloc_t(&acc, 4, s);
   if (rc) {
     dev_free(volc, s);
     return rc;
@@ -306,23 +338,26 @@ int modularity(cd_graph* g, const int32_t* labels_dev, double* q_out) {
     const int wbytes = g->wkind == W_UNIT ? 0 : g->wkind == W_I32 ? 4 : 8;
     KTimer t(g, K_MODULARITY, (double)n * (8 + 4 + 4 + 8 + 8 + 8) + (double)g->nnz * (4 + 4 + wbytes));
     cudaMemsetAsync(volc, 0, n * 8, s);
-    cudaMemsetAsync(acc, 0, 3 * 8, s);
-    CD_LAUNCH(k_mod_vol<<<grid_cap((n + NT - 1) / NT), NT, 0, s>>>(labels_dev, g->degw, n, volc));
+    cudaMemsetAsync(acc, 0, 4 * 8, s);
+    CD_LAUNCH(k_mod_vol<<<grid_cap((n + NT - 1) / NT, 152 * 8), NT, 0, s>>>(labels_dev, g->degw, n, volc, acc));
     CD_LAUNCH(k_mod_sq<<<grid_cap((n + NT - 1) / NT, 152 * 4), NT, 0, s>>>(volc, n, acc));
-    const unsigned gr = grid_cap(n * 32 / NT + 1);
+    const int64_t m = g->nnz;
+    const unsigned gr = grid_cap((m + 8 * WALK_TILE - 1) / (8 * WALK_TILE), 152 * 8);
+    const int64_t piece = walk_piece(m, (int64_t)gr * (NT / 32));
     if (g->wkind == W_UNIT)
-      CD_LAUNCH(k_mod_internal<WUnit><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, labels_dev, acc));
+      CD_LAUNCH(k_mod_internal<WUnit><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, m, piece, labels_dev, acc));
     else if (g->wkind == W_I32)
-      CD_LAUNCH(k_mod_internal<WI32><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, labels_dev, acc));
+      CD_LAUNCH(k_mod_internal<WI32><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, m, piece, labels_dev, acc));
     else
-      CD_LAUNCH(k_mod_internal<WI64><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, labels_dev, acc));
+      CD_LAUNCH(k_mod_internal<WI64><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, m, piece, labels_dev, acc));
   }
-  unsigned long long h[3] = {0, 0, 0};
+  unsigned long long h[4] = {0, 0, 0, 0};
   CD_CHECK(cudaGetLastError());
   CD_CHECK(cudaMemcpyAsync(h, acc, sizeof(h), cudaMemcpyDeviceToHost, s));
   CD_CHECK(cudaStreamSynchronize(s));
   dev_free(volc, s);
   dev_free(acc, s);
+  if (h[3]) return CD_EINVAL;
   const unsigned __int128 S = ((unsigned __int128)h[1] << 64) | h[0];
   const i128 num = (i128)(int64_t)h[2] * g->vol - (i128)S;
   const i128 den = (i128)g->vol * g->vol;
@@ -368,7 +403,6 @@ int cd_modularity(cd_graph* g, const int32_t* labels, int on_device, double* q_o
   int32_t* d = nullptr;
   bool owned = false;
   int rc = stage_labels(g, labels, on_device, &d, &owned);
-  if (!rc) rc = check_labels(g, d);
   if (!rc) rc = modularity(g, d, q_out);
   if (owned) dev_free(d, g->stream);
   if (!rc) rc = profile_flush(g);

@@ -11,6 +11,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "rowwalk.cuh"
 
 namespace cd {
 namespace {
@@ -119,24 +120,57 @@ __global__ void k_bmod_sq(const unsigned long long* __restrict__ volc, const int
   }
 }
 
+// The arcs split evenly over the warps (see rowwalk.cuh). A lane sums arcs of
+// one graph and adds the sum to I when its next arc is another graph's.
 template <class W>
 __global__ void __launch_bounds__(NT) k_bmod_internal(const int64_t* __restrict__ off,
                                                       const int32_t* __restrict__ cols, const void* w,
-                                                      int64_t n, const int32_t* __restrict__ lab,
+                                                      int64_t n, int64_t m, int64_t piece,
+                                                      const int32_t* __restrict__ lab,
                                                       const int32_t* __restrict__ gid,
                                                       unsigned long long* I) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * NT) >> 5;
-  for (int64_t v = warp; v < n; v += nwarps) {
-    const int32_t a = lab[v];
-    int64_t s = 0;
-    for (int64_t e = off[v] + lane; e < off[v + 1]; e += 32)
-      if (lab[cols[e]] == a) s += W::get(w, e);
+  __shared__ __align__(16) int32_t mark[NT / 32][WALK_TILE];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t step = (((int64_t)gridDim.x * NT) >> 5) * piece;
+  int64_t s = 0;
+  int32_t b = -1;
+  for (int64_t e0 = (((int64_t)blockIdx.x * NT + threadIdx.x) >> 5) * piece; e0 < m; e0 += step) {  // uniform in the warp
+    const int64_t e1 = e0 + piece < m ? e0 + piece : m;
+    int64_t cur = warp_row_of(off, n, e0);
+    for (int64_t ts = e0; ts < e1; ts += WALK_TILE) {
+      const int64_t e = ts + 4 * lane;
+      const int4 c4 = e < e1 ? __ldg(reinterpret_cast<const int4*>(cols + e)) : make_int4(0, 0, 0, 0);
+      const int32_t cs[4] = {c4.x, c4.y, c4.z, c4.w};
+      int32_t lc[4], lr[4], br[4];
+      int64_t row[4];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
-    if (lane == 0 && s) atomicAdd(&I[gid[v]], (unsigned long long)s);
+      for (int j = 0; j < 4; ++j) lc[j] = e + j < e1 ? lab[cs[j]] : -1;
+      warp_tile_rows(off, n, ts, cur, mark[wid], row);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        lr[j] = e + j < e1 ? lab[row[j]] : -2;
+        br[j] = e + j < e1 ? gid[row[j]] : b;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (lc[j] != lr[j]) continue;
+        if (br[j] != b) {
+          if (s) atomicAdd(&I[b], (unsigned long long)s);
+          s = 0;
+          b = br[j];
+        }
+        s += W::get(w, e + j);
+      }
+    }
   }
+  // one addition per graph that the warp ends in
+  const unsigned peers = __match_any_sync(FULL, b);
+  int64_t sum = 0;
+  for (int l = 0; l < 32; ++l) {
+    const int64_t x = __shfl_sync(FULL, s, l);
+    if ((peers >> l) & 1u) sum += x;
+  }
+  if (b >= 0 && sum && (__ffs(peers) - 1) == lane) atomicAdd(&I[b], (unsigned long long)sum);
 }
 
 void free_batches(cd_graph* g) {
@@ -217,13 +251,15 @@ int batch_modularity(cd_graph* g, const int32_t* lab, std::vector<double>& q) {
     if (n > 0) {
       CD_LAUNCH(k_bmod_vol<<<grid_cap((n + NT - 1) / NT), NT, 0, s>>>(lab, g->degw, g->gid, n, volc, cgid));
       CD_LAUNCH(k_bmod_sq<<<grid_cap((n + NT - 1) / NT), NT, 0, s>>>(volc, cgid, n, S));
-      const unsigned gr = grid_cap(n * 32 / NT + 1);
+      const int64_t m = g->nnz;
+      const unsigned gr = grid_cap((m + 8 * WALK_TILE - 1) / (8 * WALK_TILE), 152 * 8);
+      const int64_t piece = walk_piece(m, (int64_t)gr * (NT / 32));
       if (g->wkind == W_UNIT)
-        CD_LAUNCH(k_bmod_internal<WUnit><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, lab, g->gid, I));
+        CD_LAUNCH(k_bmod_internal<WUnit><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, m, piece, lab, g->gid, I));
       else if (g->wkind == W_I32)
-        CD_LAUNCH(k_bmod_internal<WI32><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, lab, g->gid, I));
+        CD_LAUNCH(k_bmod_internal<WI32><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, m, piece, lab, g->gid, I));
       else
-        CD_LAUNCH(k_bmod_internal<WI64><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, lab, g->gid, I));
+        CD_LAUNCH(k_bmod_internal<WI64><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, m, piece, lab, g->gid, I));
     }
   }
   std::vector<unsigned long long> hS(2 * nb), hI(nb);

@@ -255,7 +255,7 @@ int aggregate(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_dev, 
 // Aggregation by hash-combining per community (no sort of the arcs).
 int aggregate_hash(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_dev, int64_t k,
                    cd_graph** coarse_out);
-int modularity(cd_graph* g, const int32_t* labels_dev, double* q_out);
+int modularity(cd_graph* g, const int32_t* labels_dev, double* q_out);  // CD_EINVAL if a label is out of [0, n)
 
 // prims.cu: device-wide primitives on the graph's stream
 int exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* total_dev,

@@ -21,14 +21,16 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "rowwalk.cuh"
 
 namespace {
 
 constexpr int64_t kNoallocMaxN = 1 << 21;  // vertices (and community ids) at most
-constexpr int kCtlWords = 8;               // S low, S high, I, vol(V), status
+// S low, S high, I, vol(V), status of the offsets and labels, status of the arcs
+constexpr int kCtlWords = 8;
 constexpr int NT = 256;
 
-static __device__ __align__(256) unsigned long long g_noalloc_scratch[kNoallocMaxN + kCtlWords];
+static __device__ __align__(256) unsigned long long g_noalloc_scratch[kCtlWords + kNoallocMaxN];  // control words first: one clear covers a call
 
 constexpr int kMaxDevices = 64;
 unsigned long long* g_scratch_dev[kMaxDevices] = {};
@@ -56,70 +58,98 @@ int scratch_on_current_device(unsigned long long** out) {
   return CD_OK;
 }
 
-__device__ __forceinline__ void na_fail(unsigned long long* ctl, int code) {
-  atomicCAS(&ctl[4], 0ull, (unsigned long long)(unsigned)(-code));
+__device__ __forceinline__ void na_fail(unsigned long long* word, int code) {
+  atomicCAS(word, 0ull, (unsigned long long)(unsigned)(-code));
 }
 
-// Warp per vertex: deg_w(v) (a loop counted twice) into the volume of v's
-// community, the weight of arcs inside communities (a loop arc counts 2L) and
-// vol(V). Every index is checked before use; a bad one sets the status word.
+// deg_w(v) (a loop counted twice) into the volume of v's community, the weight
+// of arcs inside communities (a loop arc counts 2L) and vol(V). The arcs are
+// split evenly over the warps (rowwalk.cuh), so a long row is no serial chain;
+// columns and weights are read 4 bytes at a time, since the caller's arrays may
+// start anywhere. Every index is checked before use; a bad one sets a status
+// word: offsets and labels are checked by vertex, and their word is reported
+// before that of the arcs, whose rows mean nothing if the offsets are bad.
 template <bool UNIT>
 __global__ void __launch_bounds__(NT) k_noalloc_pass(const int64_t* __restrict__ off,
                                                      const int32_t* __restrict__ cols,
                                                      const int32_t* __restrict__ w,
                                                      const int32_t* __restrict__ labels, int64_t n,
                                                      int64_t nnz, unsigned long long* scratch) {
-  unsigned long long* volc = scratch;
-  unsigned long long* ctl = scratch + kNoallocMaxN;
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * NT) >> 5;
-  unsigned long long my_in = 0, my_vol = 0;
-  for (int64_t v = warp; v < n; v += nwarps) {
+  __shared__ __align__(16) int32_t mark[NT / 32][cd::WALK_TILE];
+  __shared__ cd::CtaSums vol;
+  vol.clear();
+  __syncthreads();
+  unsigned long long* ctl = scratch;
+  unsigned long long* volc = scratch + kCtlWords;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t tid = (int64_t)blockIdx.x * NT + threadIdx.x;
+  const int64_t threads = (int64_t)gridDim.x * NT;
+  for (int64_t v = tid; v < n; v += threads) {
     const int32_t a = labels[v];
     const int64_t beg = off[v], end = off[v + 1];
-    if (a < 0 || a >= n) {
-      if (lane == 0) na_fail(ctl, CD_EINVAL);
-      continue;
-    }
-    if (beg < 0 || end < beg || end > nnz) {
-      if (lane == 0) na_fail(ctl, CD_ENOTSYM);
-      continue;
-    }
-    long long s = 0, in = 0;
-    for (int64_t e = beg + lane; e < end; e += 32) {
-      const int32_t u = cols[e];
-      const long long x = UNIT ? 1 : (long long)w[e];
-      if (u < 0 || u >= n) {
-        na_fail(ctl, CD_EBOUNDS);
-        continue;
-      }
-      if (x < 1) na_fail(ctl, CD_EINVAL);
-      s += u == v ? 2 * x : x;
-      if (labels[u] == a) in += u == v ? 2 * x : x;
-    }
+    if (a < 0 || a >= n) na_fail(&ctl[4], CD_EINVAL);
+    else if (beg < 0 || end < beg || end > nnz) na_fail(&ctl[4], CD_ENOTSYM);
+  }
+  int64_t m0 = off[0], m1 = off[n];  // the rows' arcs
+  if (m0 < 0) m0 = 0;
+  if (m1 > nnz) m1 = nnz;
+  const int64_t piece = cd::walk_piece(m1 - m0, threads >> 5);
+  unsigned long long my_in = 0, my_vol = 0;
+  for (int64_t e0 = m0 + (tid >> 5) * piece; e0 < m1; e0 += (threads >> 5) * piece) {  // uniform in the warp
+    const int64_t e1 = e0 + piece < m1 ? e0 + piece : m1;
+    int64_t cur = cd::warp_row_of(off, n, e0);
+    for (int64_t ts = e0; ts < e1; ts += cd::WALK_TILE) {
+      const int64_t e = ts + 4 * lane;
+      int32_t u[4];
+      long long x[4];
+      int64_t row[4];
+      unsigned long long val[4];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s += __shfl_xor_sync(cd::FULL, s, o);
-      in += __shfl_xor_sync(cd::FULL, in, o);
+      for (int j = 0; j < 4; ++j) {
+        u[j] = e + j < e1 ? cols[e + j] : -1;
+        x[j] = UNIT || e + j >= e1 ? 1 : (long long)w[e + j];
+      }
+      cd::warp_tile_rows(off, n, ts, cur, mark[wid], row);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        val[j] = 0;
+        if (e + j >= e1) {
+          row[j] = -1;
+          continue;
+        }
+        if (x[j] < 1) na_fail(&ctl[5], CD_EINVAL);
+        if (u[j] < 0 || u[j] >= n) {
+          na_fail(&ctl[5], CD_EBOUNDS);
+          continue;
+        }
+        val[j] = (unsigned long long)(u[j] == row[j] ? 2 * x[j] : x[j]);
+        my_vol += val[j];
+        if (labels[u[j]] == labels[row[j]]) my_in += val[j];
+      }
+      cd::warp_rows_sum(row, val, [&](int64_t r, unsigned long long sum) {
+        const int32_t a = labels[r];
+        if (a >= 0 && a < n) vol.add(volc, a, sum);
+      });
     }
-    if (lane == 0) {
-      atomicAdd(&volc[a], (unsigned long long)s);
-      my_in += (unsigned long long)in;
-      my_vol += (unsigned long long)s;
-    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    my_in += __shfl_xor_sync(cd::FULL, my_in, o);
+    my_vol += __shfl_xor_sync(cd::FULL, my_vol, o);
   }
   if (lane == 0) {
     if (my_in) atomicAdd(&ctl[2], my_in);
     if (my_vol) atomicAdd(&ctl[3], my_vol);
   }
+  __syncthreads();
+  vol.flush(volc);
 }
 
 // Sum of squared community volumes, exact in 128 bits (ctl[0] low, ctl[1] high).
 __global__ void __launch_bounds__(NT) k_noalloc_square(int64_t n, unsigned long long* scratch) {
   __shared__ unsigned __int128 part[NT];
-  const unsigned long long* volc = scratch;
-  unsigned long long* ctl = scratch + kNoallocMaxN;
+  const unsigned long long* volc = scratch + kCtlWords;
+  unsigned long long* ctl = scratch;
   unsigned __int128 s = 0;
   const int64_t stride = (int64_t)gridDim.x * NT;
   for (int64_t c = (int64_t)blockIdx.x * NT + threadIdx.x; c < n; c += stride)
@@ -158,12 +188,14 @@ extern "C" int cd_modularity_noalloc(const int64_t* off, const int32_t* cols, co
   unsigned long long* scratch = nullptr;
   int rc = scratch_on_current_device(&scratch);
   if (rc) return rc;
-  unsigned long long* ctl = scratch + kNoallocMaxN;
-  CD_CHECK(cudaMemsetAsync(scratch, 0, (size_t)n * sizeof(unsigned long long), s));
-  CD_CHECK(cudaMemsetAsync(ctl, 0, kCtlWords * sizeof(unsigned long long), s));
+  CD_CHECK(cudaMemsetAsync(scratch, 0, (size_t)(kCtlWords + n) * sizeof(unsigned long long), s));
   if (n > 0) {
-    int64_t blocks = (n * 32 + NT - 1) / NT;
-    const unsigned grid = (unsigned)(blocks < 152 * 16 ? blocks : 152 * 16);
+    // from 1,024 arcs or vertices a CTA up to one CTA per SM (latency), then 8,192 (each popular community
+    // costs a CTA one atomic), 8 CTAs per SM at most
+    const int64_t work = nnz > n ? nnz : n;
+    int64_t blocks = (work + 1023) / 1024;
+    if (blocks > 152) blocks = work / 8192 < 152 ? 152 : work / 8192 < 152 * 8 ? work / 8192 : 152 * 8;
+    const unsigned grid = (unsigned)blocks;
     if (w)
       CD_LAUNCH(k_noalloc_pass<false><<<grid, NT, 0, s>>>(off, cols, w, labels, n, nnz, scratch));
     else
@@ -173,9 +205,10 @@ extern "C" int cd_modularity_noalloc(const int64_t* off, const int32_t* cols, co
     CD_CHECK(cudaGetLastError());
   }
   unsigned long long h[kCtlWords] = {};
-  CD_CHECK(cudaMemcpyAsync(h, ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
+  CD_CHECK(cudaMemcpyAsync(h, scratch, sizeof(h), cudaMemcpyDeviceToHost, s));
   CD_CHECK(cudaStreamSynchronize(s));
   if (h[4]) return -(int)h[4];
+  if (h[5]) return -(int)h[5];
   const int64_t vol = (int64_t)h[3];
   if (vol == 0) {
     *q_out = 0.0;

@@ -1,0 +1,67 @@
+"""Sums over arcs split evenly over the warps (modularity and its batched and allocation-free forms) on rows that end,
+start or repeat where a tile of 128 arcs does: empty rows in runs, one long row, rows of 1 to 4 arcs, offsets of the
+caller's arrays that are not 16-byte aligned. Integer sums and one division, so results equal the oracle's to 1e-12."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _star_mix(n, hub, arcs_hub, seed, wmax, loops):
+    """A hub joined to `arcs_hub` vertices, pairs elsewhere, runs of isolated vertices between them."""
+    rng = np.random.default_rng(seed)
+    edges = {(min(hub, int(v)), max(hub, int(v))) for v in rng.choice(n, arcs_hub, replace=False) if v != hub}
+    for u in range(0, n - 5, 97):
+        edges.add((u, u + 1 + int(rng.integers(0, 4))))
+    edges = sorted(edges)
+    ws = rng.integers(1, wmax + 1, len(edges)).tolist()
+    lo = {int(v): int(rng.integers(1, 4)) for v in rng.choice(n, loops, replace=False)} if loops else None
+    return synth.from_edge_list(n, edges, ws if wmax > 1 else None, lo)
+
+
+GRAPHS = [(2, 0, 1, 1, 0), (300, 299, 127, 1, 0), (300, 0, 128, 1, 5), (5000, 2500, 129, 7, 0), (20000, 19999, 9000, 5, 30)]
+
+
+@pytest.mark.parametrize("n,hub,arcs,wmax,loops", GRAPHS)
+def test_modularity_forms(n, hub, arcs, wmax, loops):
+    import paper_2507_06471_gb300 as cd
+    g = _star_mix(n, hub, arcs, 3 + n, wmax, loops)
+    off, cols, w = g.numpy()
+    rng = np.random.default_rng(1)
+    G = cd.Graph(g.off.cuda(), g.cols.cuda(), None if g.w is None else g.w.cuda())
+    # the allocation-free call on arrays that start 4 bytes past a 16-byte boundary
+    dcols = torch.cat([torch.zeros(1, dtype=torch.int32), g.cols]).cuda()[1:]
+    dw = None if g.w is None else torch.cat([torch.zeros(1, dtype=torch.int32), g.w]).cuda()[1:]
+    for lab in (np.arange(n), rng.integers(0, 3, n), np.full(n, n - 1)):
+        lab = lab.astype(np.int32)
+        q = oracle.modularity(off, cols, w, lab)[0]
+        tol = 1e-12 * max(1.0, abs(q))
+        dl = torch.from_numpy(lab).cuda()
+        assert abs(G.modularity(dl) - q) <= tol
+        assert abs(cd.cd_modularity_noalloc(g.off.cuda(), dcols, dw, dl) - q) <= tol
+    bad = torch.full((n,), n, dtype=torch.int32, device="cuda")
+    for call in (lambda: G.modularity(bad), lambda: cd.cd_modularity_noalloc(g.off.cuda(), dcols, dw, bad)):
+        with pytest.raises(cd.CDError) as e:
+            call()
+        assert e.value.status == cd.CD_EINVAL
+    G.close()
+
+
+def test_batched_modularity_of_many_graphs_per_tile():
+    import paper_2507_06471_gb300 as cd
+    graphs = [synth.from_edge_list(n, [(i, i + 1) for i in range(n - 1)]) for n in (2, 3, 5, 400, 1, 2, 7, 130)] * 3
+    packed, vstart = synth.pack_batch(graphs)
+    G = cd.Graph(packed.off.cuda(), packed.cols.cuda())
+    G.set_batches(vstart)
+    lab, levels, q = G.batch_louvain()
+    lab = lab.cpu().numpy()
+    for b, g in enumerate(graphs):
+        off, cols, w = g.numpy()
+        olab, olv, oq, _ = oracle.louvain(off, cols, w)
+        assert np.array_equal(lab[vstart[b]:vstart[b + 1]], olab) and levels[b] == olv
+        assert abs(q[b] - oq) <= 1e-12
+    G.close()
