@@ -152,8 +152,8 @@ struct cd_graph {
   int32_t* csize = nullptr;
   uint32_t* flag[2] = {nullptr, nullptr};  // needCheck / tmpNeedCheck bitmaps (n bits each)
 
-  int32_t* mv_v = nullptr;  // committed moves: vertex, new label, old label
-  int32_t* mv_c = nullptr;
+  int32_t* mv_v = nullptr;  // committed moves: vertex, new label, old label (three parts of one
+  int32_t* mv_c = nullptr;  // array, each n rounded up to whole flag words)
   int32_t* mv_a = nullptr;
   int64_t* ctr = nullptr;      // device counters
   int64_t* h_ctr = nullptr;    // pinned host copy
@@ -232,7 +232,8 @@ struct RunOpts {
   int32_t level;
   int async_mode = 0;  // committed moves take effect at once (the coin still defers half of them)
   bool singleton_start = false;  // the run starts from C[v] = v (Sigma_tot = deg_w, sizes 1)
-  bool device_loop = false;      // rounds after the first run as one captured graph (batched runs)
+  bool device_loop = false;      // the round loop runs on the device where that is possible and pays
+  bool graph_loop = false;       // graphs with hubs: rounds after the first run as one captured graph (batched runs)
   bool device_loop_all = false;  // ... in every run
 };
 // Algorithm 1 / Algorithm 2 round loops on g->C (device). Louvain: g->C holds
@@ -246,6 +247,15 @@ void release_batches(cd_graph* g);
 int run_local_move(cd_graph* g, const RunOpts& o, int init_given, int64_t* moves_out,
                    int32_t* rounds_out);
 RunOpts opts_from(const cd_params* p, int32_t level);
+// cd_params.device_loop of the server's workers when the caller left the
+// default: resident loops, but no captured graphs (several workers
+// instantiating graphs at once cost more than the read-backs they save).
+constexpr int32_t LOOP_NO_GRAPH = 0x10000;
+
+// rounds.cu: the whole round loop as one resident kernel (graphs without hubs).
+bool resident_rounds_apply(const cd_graph* g, const RunOpts& o, bool per_graph_stop);
+int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, int64_t* moves_out, int32_t* rounds_out,
+                    std::vector<int32_t>* graph_rounds);
 int begin_run(cd_graph* g, const cd_params* p);  // validates params, resets trace/profile
 
 // aggregate.cu

@@ -436,7 +436,7 @@ void free_arrays(cd_graph* g) {
                 g->hub_blist,    g->hub_mlist,     g->hub_lcnt,     g->C,            g->sigma,        g->csize,
                 g->hub_log,
                 g->sigma32,
-                g->flag[0],      g->flag[1],       g->mv_v,         g->mv_c,         g->mv_a,
+                g->flag[0],      g->flag[1],       g->mv_v,
                 g->ctr,          g->status,        g->gid,          g->gbase,        g->gvol,
                 g->gfrozen,      g->gcnt};
   for (void* p : ps) dev_free(p, s);
@@ -722,11 +722,11 @@ int ensure_run_state(cd_graph* g) {
   if ((rc = dev_alloc_t(&g->csize, g->n, s))) return rc;
   if ((rc = dev_alloc_t(&g->flag[0], (g->n + 31) / 32 + 1, s))) return rc;
   if ((rc = dev_alloc_t(&g->flag[1], (g->n + 31) / 32 + 1, s))) return rc;
-  if ((rc = dev_alloc_t(&g->mv_v, g->n, s))) return rc;
-  if ((rc = dev_alloc_t(&g->mv_c, g->n, s))) return rc;
-  if ((rc = dev_alloc_t(&g->mv_a, g->n, s))) return rc;
+  const int64_t n32 = (g->n + 31) / 32 * 32;
+  if ((rc = dev_alloc_t(&g->mv_v, 3 * n32, s))) return rc;
+  g->mv_c = g->mv_v + n32;
+  g->mv_a = g->mv_v + 2 * n32;
   if ((rc = dev_alloc_t(&g->ctr, C_COUNT, s))) return rc;
-  if (!g->h_ctr) CD_CHECK(cudaMallocHost(&g->h_ctr, C_COUNT * sizeof(int64_t)));
   return CD_OK;
 }
 

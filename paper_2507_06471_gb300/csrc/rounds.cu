@@ -1,0 +1,742 @@
+// The round loop of a run or Louvain level as one resident kernel, for graphs
+// without hubs: every round of Label Propagation (Algorithm 1) or local moving
+// (Algorithm 2), synchronous, with the decisions, coins, counters and stop
+// tests of the per-round kernels in scan.cu (the results are the same).
+//
+// Why: a round of a small graph, or a late round of a large one, examines few
+// vertices, and its time is latency: a dozen launches of 3 to 8 us each, a
+// compaction over all n list entries, a read-back and a synchronisation. The
+// 10,000-vertex planted partition took 49 us a round that way (43 rounds, 2.1
+// ms), the 1M-vertex LFR-style graph 165 us (233 rounds, 38.5 ms).
+//
+// How: one cooperative launch of at most one wave of 256-thread CTAs. The
+// vertices are dealt out in units of 1 to 32 consecutive ids round robin, so
+// that every CTA gets an even share of whatever is active. In a round a CTA
+//   1. takes its vertices' flags (clearing them: the map is the next round's
+//      for the other parity), sorts the flagged ones by degree bin into a list in
+//      shared memory and scans them: a half CTA per vertex of degree t_warp+1
+//      to 1,024, warps for degree 33..t_warp and 4/8/16/32-lane tiles below
+//      (tasks taken from a counter in shared memory, longest first); it marks
+//      the neighbours of its moves in the next map and keeps its moves;
+//   2. meets the others at a barrier whose one atomic per CTA also sums moved +
+//      deferred (the stop test);
+//   3. applies its moves (labels, Sigma_tot, sizes) and meets the others again.
+// The grid has at most as many CTAs as are resident at once (cooperative
+// launch), so the barrier's waits end; they are bounded all the same.
+//
+// Sigma_tot is kept in 32 bits when vol(V) < 2^31 (integers: exact), in 64
+// otherwise.
+#include <algorithm>
+#include <atomic>
+
+#include "scan.cuh"
+
+namespace cd {
+namespace {
+
+constexpr int PNT = 256, PNW = PNT / 32;  // threads and warps of a CTA
+constexpr int PCAP = WARP_CAP_SLOTS;      // table slots per warp; four warps' tables make a half CTA's
+static_assert(4 * PCAP == BLK1_CAP_SLOTS, "a half CTA's table is its four warps' tables");
+constexpr int CH_VERTS = 2048;            // vertices a CTA takes per step
+constexpr int CH_PER_WARP = CH_VERTS / PNT;
+// Arcs per CTA at least: a small graph gets fewer CTAs, which meet faster.
+constexpr int64_t ARCS_PER_CTA = 512;
+constexpr int PBINS = 6;                  // task order: half CTA, warp, 32, 16, 8, 4 lanes
+constexpr int TRACE_COLS = 8;             // examined, arcs, moved, deferred, candidates, arcs of moved, -, -
+constexpr int HEAD = 8;                   // int64 words before the trace: rounds, moves, status
+constexpr int64_t WAIT_LIMIT = (int64_t)1 << 24;  // polls of one barrier (seconds), then CD_ETIMEOUT
+
+struct LoopCtx {
+  int64_t n, nwords, n32;  // vertices, flag words, vertices rounded up to whole words
+  int64_t nunits;          // units of 1 << lgu consecutive vertices; unit q belongs to CTA q mod gridDim.x
+  int32_t lgu;
+  uint32_t* flag0;  // read in even rounds, written in odd ones
+  uint32_t* flag1;
+  int32_t max_iter, first_rows, t_warp, per_graph;
+  int64_t threshold;
+  int32_t* last_change;       // per_graph: 1 + the last round in which a vertex of the graph wanted to move
+  unsigned long long* bar;    // two words per round, zero
+  unsigned long long* head;   // HEAD words, then TRACE_COLS per round, zero
+  uint32_t* sigma32;          // NK: Sigma_tot
+};
+
+// Every CTA arrives once; `add` is summed over the CTAs. False: a wait ran out.
+__device__ __forceinline__ bool grid_meet(unsigned long long* word, unsigned add, unsigned long long& sum,
+                                          int32_t* status) {
+  __shared__ unsigned long long got;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(word, (1ull << 40) | add);
+    unsigned long long x;
+    int64_t polls = 0;
+    do {
+      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(word) : "memory");
+    } while ((x >> 40) < gridDim.x && ++polls < WAIT_LIMIT);
+    if ((x >> 40) < gridDim.x) {
+      atomicCAS(status, 0, CD_ETIMEOUT);
+      x = ~0ull;
+    }
+    __threadfence();
+    got = x;
+  }
+  __syncthreads();
+  const unsigned long long x = got;
+  sum = x & ((1ull << 40) - 1);
+  return x != ~0ull;
+}
+
+// Barrier of a half CTA (fixed numbers: a number in a register would reserve all sixteen).
+__device__ __forceinline__ void half_sync(int half) {
+  if (half) asm volatile("bar.sync 2, 128;" ::: "memory");
+  else asm volatile("bar.sync 1, 128;" ::: "memory");
+}
+
+// One CTA's part of a round.
+struct Tally {
+  uint32_t act = 0, arcs = 0, cand = 0, def = 0, marcs = 0;
+};
+
+__device__ __forceinline__ void set_flag(uint32_t* nxt, int32_t u) { atomicOr(&nxt[u >> 5], 1u << (u & 31)); }
+
+template <bool LOUV, class W, class V, bool NK>
+struct Scan {
+  typedef typename KeyOf<LOUV, NK>::T K;
+  const ScanCtx& s;
+  const LoopCtx& L;
+  int round;
+  bool first;        // every label is the vertex's own id and no row repeats a column
+  uint32_t* nxt;     // null: no frontier
+  int32_t* mv;       // this CTA's moves: vertex, new, old label in three arrays of mv_stride
+  int64_t mv_stride;
+  int* n_mv;         // in shared memory
+
+  // The lanes with `want` hold a vertex v whose decision `target` differs from
+  // its label: coin, move list, flag. Returns whether the lane's move commits.
+  __device__ __forceinline__ bool act(bool want, int32_t v, int32_t cur, int32_t target) const {
+    const int lane = threadIdx.x & 31;
+    const bool commit = want && commit_coin(s.seed, s.level, round, local_id(s, v));
+    const unsigned cm = __ballot_sync(FULL, commit);
+    if (cm) {
+      const int lead = __ffs(cm) - 1;
+      int p0 = 0;
+      if (lane == lead) p0 = atomicAdd(n_mv, __popc(cm));
+      p0 = __shfl_sync(FULL, p0, lead);
+      if (commit) {
+        const int64_t p = p0 + __popc(cm & ((1u << lane) - 1u));
+        mv[p] = v;
+        mv[mv_stride + p] = target;
+        mv[2 * mv_stride + p] = cur;
+      }
+    }
+    if (want) {
+      if (nxt) set_flag(nxt, v);
+      if (L.per_graph) L.last_change[s.gid[v]] = round + 1;
+    }
+    return commit;
+  }
+
+  // 2^lgt lanes per vertex, one arc per lane; the warp takes 32 >> lgt vertices
+  // of list[0, count) from `base` on.
+  __device__ __forceinline__ void tile(const int32_t* list, int base, int count, int lgt, int64_t* stage,
+                                       Tally& t) const {
+    const int lane = threadIdx.x & 31;
+    const int tw = 1 << lgt, sub = lane & (tw - 1), tbase = lane - sub;
+    const unsigned tmask = (tw == 32 ? FULL : ((1u << tw) - 1u)) << tbase;
+    const int i = base + (lane >> lgt);
+    const bool on = i < count;
+    const int32_t v = on ? list[i] : 0;
+    int64_t beg = 0;
+    int d = 0;
+    if (on) {
+      beg = __ldg(s.off + v);
+      d = (int)(__ldg(s.off + v + 1) - beg);
+    }
+    const int32_t cur = on ? s.C[v] : 0;
+    const bool has = on && sub < d;
+    const int32_t u = has ? __ldg(s.cols + beg + sub) : v;
+    const int64_t wt = has ? W::get(s.w, beg + sub) : 0;
+    const int64_t dv = (LOUV && on) ? __ldg(s.degw + v) : 0;
+    const int64_t volv = (LOUV && on) ? vol_of(s, v) : 0;
+    const bool cand = has && u != v;
+    const int32_t lbl = cand ? (first ? u : s.C[u]) : (int32_t)(0x80000000u | (unsigned)lane);
+    const unsigned peers = __match_any_sync(FULL, lbl) & tmask;
+    const int64_t gsum = group_sum<W>(peers, wt, stage);
+    const bool leader = cand && (__ffs(peers) - 1) == lane;
+    const unsigned cm = __ballot_sync(FULL, cand && lbl == cur) & tmask;
+    int64_t kcur = __shfl_sync(FULL, gsum, cm ? __ffs(cm) - 1 : lane);
+    if (!cm) kcur = 0;
+    const bool ok = leader && (!LOUV || lbl != cur);
+    K bk = ok ? cand_key<LOUV, NK>(s, lbl, gsum, dv, volv) : K(0);
+    int32_t bc = ok ? lbl : NOCAND;
+    reduce_best(bk, bc, tw);
+    int32_t target = cur;
+    if (on) target = decide<LOUV, NK>(s, v, cur, bk, bc, cm != 0, kcur, volv);
+    const bool want = on && target != cur;
+    const bool mine = act(want && sub == 0, v, cur, target);
+    const bool commit = __shfl_sync(FULL, (int)mine, tbase) != 0;
+    if (nxt && commit && has) set_flag(nxt, u);  // the neighbours of a moved vertex
+    if (sub == 0 && on) {
+      ++t.act;
+      t.arcs += d;
+      if (want && !mine) ++t.def;
+      if (mine) t.marcs += d;
+    }
+    if (leader) ++t.cand;
+  }
+
+  // A warp takes the vertices list[base, base + vb): lane j loads vertex j's
+  // header, the warp scans the rows one after another, and the decisions run
+  // one lane per vertex.
+  __device__ __forceinline__ void warp_batch(const int32_t* list, int base, int count, int vb, int32_t* keys, V* vals,
+                                             uint16_t* occ, int* occ_n, int64_t* stage, Tally& t) const {
+    const int lane = threadIdx.x & 31;
+    const bool on = lane < vb && base + lane < count;
+    const int32_t my_v = on ? list[base + lane] : 0;
+    int64_t my_beg = 0, my_end = 0, my_dv = 0, my_vol = 0;
+    int32_t my_cur = 0;
+    if (on) {
+      my_beg = __ldg(s.off + my_v);
+      my_end = __ldg(s.off + my_v + 1);
+      my_cur = s.C[my_v];
+      if (LOUV) {
+        my_dv = __ldg(s.degw + my_v);
+        my_vol = vol_of(s, my_v);
+      }
+    }
+    K my_bk = K(0);
+    int32_t my_bc = NOCAND;
+    bool my_hc = false;
+    int64_t my_kc = 0, ncand = 0;
+    for (unsigned am = __ballot_sync(FULL, on); am; am &= am - 1) {
+      const int j = __ffs(am) - 1;
+      const int32_t v = __shfl_sync(FULL, my_v, j), cur = __shfl_sync(FULL, my_cur, j);
+      const int64_t beg = __shfl_sync(FULL, my_beg, j), end = __shfl_sync(FULL, my_end, j);
+      const int64_t dv = LOUV ? __shfl_sync(FULL, my_dv, j) : 0;
+      const int64_t volv = LOUV ? __shfl_sync(FULL, my_vol, j) : 0;
+      K bk = K(0);
+      int32_t bc = NOCAND;
+      bool hc = false;
+      int64_t kc = 0;
+      if (first) {  // distinct labels along the row: no table
+        for (int64_t e = beg + lane; e < end; e += 32) {
+          const int32_t u = __ldg(s.cols + e);
+          if (u == v) continue;
+          const K key = cand_key<LOUV, NK>(s, u, W::get(s.w, e), dv, volv);
+          ++ncand;
+          if (better(key, u, bk, bc)) {
+            bk = key;
+            bc = u;
+          }
+        }
+        reduce_best(bk, bc, 32);
+      } else {
+        const unsigned lg = 64 - __clzll((unsigned long long)(2 * (end - beg) - 1));  // 2^lg >= 2 deg
+        group_insert<W, V, 32>(s, v, beg, end, lane, keys, vals, occ, occ_n, lg, stage);
+        __syncwarp();
+        group_eval<LOUV, V, 32, NK>(s, cur, dv, volv, lane, keys, vals, occ, *occ_n, bk, bc, hc, kc, ncand);
+        reduce_best(bk, bc, 32);
+        const unsigned hm = __ballot_sync(FULL, hc);
+        hc = hm != 0;
+        if (hm) kc = __shfl_sync(FULL, kc, __ffs(hm) - 1);
+        __syncwarp();
+        if (lane == 0) *occ_n = 0;
+        __syncwarp();
+      }
+      if (lane == j) {
+        my_bk = bk;
+        my_bc = bc;
+        my_hc = hc;
+        my_kc = kc;
+      }
+    }
+    int32_t target = my_cur;
+    if (on) target = decide<LOUV, NK>(s, my_v, my_cur, my_bk, my_bc, my_hc, my_kc, my_vol);
+    const bool want = on && target != my_cur;
+    const bool commit = act(want, my_v, my_cur, target);
+    if (on) {
+      const uint32_t d = (uint32_t)(my_end - my_beg);
+      ++t.act;
+      t.arcs += d;
+      if (want && !commit) ++t.def;
+      if (commit) t.marcs += d;
+    }
+    t.cand += (uint32_t)ncand;
+    if (nxt)
+      for (unsigned m = __ballot_sync(FULL, commit); m; m &= m - 1) {
+        const int j = __ffs(m) - 1;
+        const int64_t beg = __shfl_sync(FULL, my_beg, j), end = __shfl_sync(FULL, my_end, j);
+        for (int64_t e = beg + lane; e < end; e += 32) set_flag(nxt, __ldg(s.cols + e));
+      }
+  }
+
+  // A half CTA (128 threads, named barrier `half` + 1) scans vertex v with the
+  // four warps' tables as one.
+  struct HalfRed {
+    K k[4];
+    int64_t kc[4];
+    int32_t c[4], hc[4];
+    int32_t moved;
+  };
+  __device__ __forceinline__ void half_cta(int32_t v, int half, int32_t* keys, V* vals, uint16_t* occ, int* occ_n,
+                                           int64_t* stage, HalfRed* red, Tally& t) const {
+    const int lane = threadIdx.x & 31, gl = threadIdx.x & 127, wig = gl >> 5;
+    const int64_t beg = __ldg(s.off + v), end = __ldg(s.off + v + 1);
+    const int32_t cur = s.C[v];
+    const int64_t dv = LOUV ? __ldg(s.degw + v) : 0;
+    const int64_t volv = LOUV ? vol_of(s, v) : 0;
+    const unsigned lg = 64 - __clzll((unsigned long long)(2 * (end - beg) - 1));
+    group_insert<W, V, 128>(s, v, beg, end, gl, keys, vals, occ, occ_n, lg, stage);
+    half_sync(half);
+    K bk = K(0);
+    int32_t bc = NOCAND;
+    bool hc = false;
+    int64_t kc = 0, ncand = 0;
+    group_eval<LOUV, V, 128, NK>(s, cur, dv, volv, gl, keys, vals, occ, *occ_n, bk, bc, hc, kc, ncand);
+    t.cand += (uint32_t)ncand;
+    reduce_best(bk, bc, 32);
+    unsigned hm = __ballot_sync(FULL, hc);
+    if (hm) kc = __shfl_sync(FULL, kc, __ffs(hm) - 1);
+    if (lane == 0) {
+      red->k[wig] = bk;
+      red->c[wig] = bc;
+      red->hc[wig] = hm != 0;
+      red->kc[wig] = kc;
+    }
+    half_sync(half);
+    if (wig == 0) {
+      bk = lane < 4 ? red->k[lane] : K(0);
+      bc = lane < 4 ? red->c[lane] : NOCAND;
+      reduce_best(bk, bc, 32);
+      hm = __ballot_sync(FULL, lane < 4 && red->hc[lane & 3]);
+      kc = hm ? red->kc[__ffs(hm) - 1] : 0;
+      int32_t target = cur;
+      if (lane == 0) target = decide<LOUV, NK>(s, v, cur, bk, bc, hm != 0, kc, volv);
+      const bool want = lane == 0 && target != cur;
+      const bool commit = act(want, v, cur, target);
+      if (lane == 0) {
+        ++t.act;
+        t.arcs += (uint32_t)(end - beg);
+        if (want && !commit) ++t.def;
+        if (commit) t.marcs += (uint32_t)(end - beg);
+        *occ_n = 0;
+        red->moved = commit;
+      }
+    }
+    half_sync(half);
+    if (red->moved && nxt)
+      for (int64_t e = beg + gl; e < end; e += 128) set_flag(nxt, __ldg(s.cols + e));
+    half_sync(half);  // red is written again for the next vertex
+  }
+};
+
+template <class V> constexpr size_t loop_smem() {
+  return (size_t)PNW * PCAP * (sizeof(V) + 4 + 2) + (size_t)PNW * 32 * 8 + (size_t)CH_VERTS * 4;
+}
+
+template <bool LOUV, class W, class V, bool NK>
+__global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __grid_constant__ ScanCtx s,
+                                                                       const __grid_constant__ LoopCtx L) {
+  typedef Scan<LOUV, W, V, NK> S;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ typename S::HalfRed red[2];
+  __shared__ int occ_n[PNW];
+  __shared__ int bincnt[2][8];  // by parity of the step: vertices per bin, then [7]: next task
+  __shared__ int n_mv;
+  __shared__ unsigned long long sums[5];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, half = tid >> 7;
+  V* vals0 = (V*)smem;
+  int32_t* keys0 = (int32_t*)(smem + (size_t)PNW * PCAP * sizeof(V));
+  int64_t* stage = (int64_t*)(smem + (size_t)PNW * PCAP * (sizeof(V) + 4)) + wid * 32;
+  int32_t* list = (int32_t*)(smem + (size_t)PNW * PCAP * (sizeof(V) + 4) + (size_t)PNW * 32 * 8);
+  uint16_t* occ0 = (uint16_t*)(list + CH_VERTS);
+  for (int j = tid; j < PNW * PCAP; j += PNT) {
+    keys0[j] = EMPTY;
+    vals0[j] = 0;
+  }
+  if (tid < PNW) occ_n[tid] = 0;
+  if (tid < 16) bincnt[tid >> 3][tid & 7] = 0;
+  __syncthreads();
+  // this CTA's units: blockIdx.x + i gridDim.x; its moves have room for all their vertices
+  const int64_t G = gridDim.x, b = blockIdx.x;
+  const int U = 1 << L.lgu;
+  const int64_t my_verts = (L.nunits / G + (b < L.nunits % G ? 1 : 0)) << L.lgu;
+  const int64_t mv_at = (b * (L.nunits / G) + (b < L.nunits % G ? b : L.nunits % G)) << L.lgu;
+  int32_t* mv = s.mv_v + mv_at;
+  const int64_t mv_stride = L.n32;
+  int step = 0;
+  int32_t round = 0;
+  for (; round < L.max_iter;) {
+    uint32_t* cur_map = round & 1 ? L.flag1 : L.flag0;
+    uint32_t* nxt_map = round & 1 ? L.flag0 : L.flag1;
+    const bool frontier = s.mark != 0;
+    if (tid == 0) n_mv = 0;
+    if (tid < 5) sums[tid] = 0;
+    const S sc{s, L, round, round == 0 && L.first_rows, frontier ? nxt_map : nullptr, mv, mv_stride, &n_mv};
+    Tally t;
+    for (int64_t c0 = 0; c0 < my_verts; c0 += CH_VERTS) {
+      // the lane's vertices of this step, c0 + (wid CH_PER_WARP + k) 32 + lane of the CTA's, and their flags
+      int32_t vk[CH_PER_WARP];  // -1: not flagged
+      uint32_t fw[CH_PER_WARP];
+#pragma unroll
+      for (int k = 0; k < CH_PER_WARP; ++k) {
+        const int64_t i = c0 + (wid * CH_PER_WARP + k) * 32 + lane;
+        const int64_t v = ((b + (i >> L.lgu) * G) << L.lgu) + (i & (U - 1));
+        vk[k] = i < my_verts && v < L.n ? (int32_t)v : -1;
+        fw[k] = FULL;
+        if (frontier && vk[k] >= 0) fw[k] = __ldcg(cur_map + (v >> 5));
+      }
+      bool any = false;
+#pragma unroll
+      for (int k = 0; k < CH_PER_WARP; ++k) {
+        if (vk[k] < 0) continue;
+        const int32_t v = vk[k];
+        if (frontier && (v & (U - 1)) == 0) {  // the unit's flags are taken
+          const uint32_t mask = (U == 32 ? FULL : ((1u << U) - 1u)) << (v & 31);
+          if (fw[k] & mask) {
+            if (U == 32) cur_map[v >> 5] = 0;
+            else atomicAnd(&cur_map[v >> 5], ~mask);
+          }
+        }
+        if ((fw[k] >> (v & 31)) & 1u) any = true;
+        else vk[k] = -1;
+      }
+      int* cnt = bincnt[step & 1];
+      if (!__syncthreads_or(any)) continue;
+      // degree bins; the vertex's rank inside its bin of the warp
+      int deg[CH_PER_WARP];
+      int8_t bin[CH_PER_WARP];
+      int16_t rank[CH_PER_WARP];
+      int wcnt[PBINS] = {0, 0, 0, 0, 0, 0};
+#pragma unroll
+      for (int k = 0; k < CH_PER_WARP; ++k) {
+        deg[k] = 0;
+        if (vk[k] >= 0) {
+          const int32_t v = vk[k];
+          deg[k] = (int)(__ldg(s.off + v + 1) - __ldg(s.off + v));
+          if (s.gfrozen && s.gfrozen[s.gid[v]]) deg[k] = 0;
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < CH_PER_WARP; ++k) {
+        const int d = deg[k];
+        bin[k] = d == 0 ? -1 : d <= 4 ? 5 : d <= 8 ? 4 : d <= 16 ? 3 : d <= 32 ? 2 : d <= L.t_warp ? 1 : 0;
+        rank[k] = 0;
+        if (!__any_sync(FULL, d != 0)) continue;
+#pragma unroll
+        for (int q = 0; q < PBINS; ++q) {
+          const unsigned m = __ballot_sync(FULL, bin[k] == q);
+          if (bin[k] == q) rank[k] = (int16_t)(wcnt[q] + __popc(m & ((1u << lane) - 1u)));
+          wcnt[q] += __popc(m);
+        }
+      }
+      int mine = 0;
+#pragma unroll
+      for (int q = 0; q < PBINS; ++q)
+        if (lane == q) mine = wcnt[q];
+      int at = 0;
+      if (lane < PBINS && mine) at = atomicAdd(&cnt[lane], mine);
+      __syncthreads();
+      int first_of[PBINS + 1];  // where each bin starts in the list
+      first_of[0] = 0;
+#pragma unroll
+      for (int q = 0; q < PBINS; ++q) first_of[q + 1] = first_of[q] + cnt[q];
+#pragma unroll
+      for (int q = 0; q < PBINS; ++q)
+        if (lane == q) at += first_of[q];
+#pragma unroll
+      for (int k = 0; k < CH_PER_WARP; ++k) {
+        const int p = __shfl_sync(FULL, at, bin[k] < 0 ? 0 : bin[k]) + rank[k];
+        if (bin[k] >= 0) list[p] = vk[k];
+      }
+      if (tid < 8) bincnt[(step + 1) & 1][tid] = 0;  // the next step's
+      __syncthreads();
+      // half CTAs
+      int n_half = first_of[1];
+      if (!sc.first) {
+        for (int i = half; i < n_half; i += 2)
+          sc.half_cta(list[i], half, keys0 + half * 4 * PCAP, vals0 + half * 4 * PCAP, occ0 + half * 4 * PCAP,
+                      &occ_n[half * 4], stage, &red[half], t);
+      } else {
+        n_half = 0;  // rows without tables: the warps take them
+      }
+      // warps: batches of wb vertices of the warp bin, then tiles
+      const int nw = first_of[2] - n_half;
+      int wb = (nw + PNW - 1) / PNW;
+      wb = wb < 1 ? 1 : wb > 32 ? 32 : wb;
+      const int t_wb = (nw + wb - 1) / wb;
+      const int t_32 = t_wb + cnt[2], t_16 = t_32 + (cnt[3] + 1) / 2, t_8 = t_16 + (cnt[4] + 3) / 4,
+                t_4 = t_8 + (cnt[5] + 7) / 8;
+      for (;;) {
+        int task = 0;
+        if (lane == 0) task = atomicAdd(&cnt[7], 1);
+        task = __shfl_sync(FULL, task, 0);
+        if (task >= t_4) break;
+        if (task < t_wb) {
+          sc.warp_batch(list, n_half + task * wb, first_of[2], wb, keys0 + wid * PCAP, vals0 + wid * PCAP,
+                        occ0 + wid * PCAP, &occ_n[wid], stage, t);
+        } else {
+          const int q = task < t_32 ? 2 : task < t_16 ? 3 : task < t_8 ? 4 : 5;
+          const int t0 = q == 2 ? t_wb : q == 3 ? t_32 : q == 4 ? t_16 : t_8;
+          const int f = q == 2 ? first_of[2] : q == 3 ? first_of[3] : q == 4 ? first_of[4] : first_of[5];
+          const int e = q == 2 ? first_of[3] : q == 3 ? first_of[4] : q == 4 ? first_of[5] : first_of[6];
+          sc.tile(list, f + ((task - t0) << (q - 2)), e, 7 - q, stage, t);
+        }
+      }
+      ++step;
+    }
+    // the CTA's counters
+    unsigned long long c[5] = {t.act, t.arcs, t.cand, t.def, t.marcs};
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) c[q] += __shfl_xor_sync(FULL, c[q], o);
+      if (lane == 0 && c[q]) atomicAdd(&sums[q], c[q]);
+    }
+    __syncthreads();
+    const int nm = n_mv;
+    const unsigned changed = (unsigned)nm + (unsigned)sums[3];
+    if (tid < 6) {
+      const unsigned long long x = tid == 0 ? sums[0] : tid == 1 ? sums[1] : tid == 2 ? (unsigned long long)nm
+                                 : tid == 3 ? sums[3] : tid == 4 ? sums[2] : sums[4];
+      if (x) atomicAdd(&L.head[HEAD + (int64_t)round * TRACE_COLS + tid], x);
+    }
+    unsigned long long total, none;
+    if (!grid_meet(L.bar + 2 * (int64_t)round, changed, total, s.status)) return;
+    // the moves
+    for (int base = wid * 32; base < nm; base += PNT) {
+      const int i = base + lane;
+      const bool ok = i < nm;
+      int32_t v = 0, to = -1, from = -1;
+      if (ok) {
+        v = mv[i];
+        to = mv[mv_stride + i];
+        s.C_w[v] = to;
+      }
+      if constexpr (LOUV) {
+        int64_t d = 0;
+        if (ok) {
+          from = mv[2 * mv_stride + i];
+          d = __ldg(s.degw + v);
+        }
+        // one atomic per distinct community of the warp: popular targets would serialise
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+          const int32_t key = side ? from : to;
+          const unsigned peers = __match_any_sync(FULL, key);
+          stage[lane] = side ? -d : d;
+          __syncwarp();
+          if (key >= 0 && (__ffs(peers) - 1) == lane) {
+            int64_t sum = 0;
+            for (unsigned m = peers; m; m &= m - 1) sum += stage[__ffs(m) - 1];
+            if constexpr (NK) atomicAdd(&L.sigma32[key], (uint32_t)sum);
+            else atomicAdd((unsigned long long*)&s.sigma_w[key], (unsigned long long)sum);
+            atomicAdd(&s.csize_w[key], side ? -__popc(peers) : __popc(peers));
+          }
+          __syncwarp();
+        }
+      }
+    }
+    ++round;
+    if (LOUV ? total == 0 : (int64_t)total <= L.threshold) break;
+    if (round < L.max_iter && !grid_meet(L.bar + 2 * (int64_t)round - 1, 0, none, s.status)) return;
+  }
+  if (b == 0 && tid == 0) L.head[0] = (unsigned long long)round;
+}
+
+// The state a run starts from: labels v, Sigma_tot = deg_w and sizes 1 (singletons) or Sigma_tot's copy of a given
+// start; every vertex flagged; the barrier words, header and trace zero.
+__global__ void __launch_bounds__(PNT) k_rounds_init(LoopCtx L, int32_t* C, int64_t* sigma, int32_t* csize,
+                                                     const int64_t* __restrict__ degw, int louv, int singletons,
+                                                     int64_t zero_words) {
+  const int64_t stride = (int64_t)gridDim.x * PNT, tid = (int64_t)blockIdx.x * PNT + threadIdx.x;
+  for (int64_t v = tid; v < L.n; v += stride) {
+    int64_t sg = 0;
+    if (singletons) {
+      C[v] = (int32_t)v;
+      if (louv) {
+        sg = degw[v];
+        if (!L.sigma32) sigma[v] = sg;
+        csize[v] = 1;
+      }
+    } else if (louv) {
+      sg = sigma[v];
+    }
+    if (louv && L.sigma32) L.sigma32[v] = (uint32_t)sg;
+  }
+  for (int64_t w = tid; w < L.nwords; w += stride) {
+    L.flag0[w] = FULL;
+    L.flag1[w] = 0;
+  }
+  for (int64_t i = tid; i < zero_words; i += stride) L.bar[i] = 0;  // the header and the trace follow the barrier words
+  if (L.per_graph)
+    for (int64_t i = tid; i < L.per_graph; i += stride) L.last_change[i] = 0;
+}
+
+int loop_sms() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
+template <bool LOUV, class W, class V, bool NK>
+int launch_loop(cd_graph* g, const ScanCtx& s, LoopCtx L) {
+  static std::atomic<int> resident{0};  // CTAs at once; the same for every thread that gets here
+  auto kern = k_rounds<LOUV, W, V, NK>;
+  constexpr size_t sm = loop_smem<V>();
+  int r = resident.load();
+  if (r == 0) {
+    CD_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    int per = 0;
+    CD_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, PNT, sm));
+    r = std::max(1, per) * loop_sms();
+    resident.store(r);
+  }
+  const int64_t grid = std::max<int64_t>(1, std::min(std::min<int64_t>(r, L.n), g->nnz / ARCS_PER_CTA));
+  // the largest units that still give every CTA four
+  L.lgu = 5;
+  while (L.lgu > 0 && (L.n >> L.lgu) < 4 * grid) --L.lgu;
+  L.nunits = (L.n + ((int64_t)1 << L.lgu) - 1) >> L.lgu;
+  void* args[] = {(void*)&s, (void*)&L};
+  note_launch();
+  CD_CHECK(cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)grid), dim3(PNT), args, sm, g->stream));
+  return CD_OK;
+}
+
+template <bool LOUV, bool NK>
+int dispatch_loop(cd_graph* g, const ScanCtx& s, const LoopCtx& L) {
+  const bool v32 = g->max_degw < ((int64_t)1 << 32);
+  if (g->wkind == W_UNIT)
+    return v32 ? launch_loop<LOUV, WUnit, uint32_t, NK>(g, s, L) : launch_loop<LOUV, WUnit, unsigned long long, NK>(g, s, L);
+  if (g->wkind == W_I32)
+    return v32 ? launch_loop<LOUV, WI32, uint32_t, NK>(g, s, L) : launch_loop<LOUV, WI32, unsigned long long, NK>(g, s, L);
+  return v32 ? launch_loop<LOUV, WI64, uint32_t, NK>(g, s, L) : launch_loop<LOUV, WI64, unsigned long long, NK>(g, s, L);
+}
+
+// The parts of the context the resident kernel uses (no hubs, no counters).
+ScanCtx loop_ctx(cd_graph* g, const RunOpts& o, bool louv, bool nk) {
+  ScanCtx s{};
+  s.off = g->off;
+  s.cols = g->cols;
+  s.w = g->w;
+  s.degw = g->degw;
+  s.vol = g->vol;
+  s.C = g->C;
+  s.C_w = g->C;
+  s.sigma = g->sigma;
+  s.sigma_w = louv ? g->sigma : nullptr;
+  s.sigma32 = nk ? g->sigma32 : nullptr;
+  s.csize = g->csize;
+  s.csize_w = g->csize;
+  s.mark = o.use_frontier ? 1 : 0;
+  s.mv_v = g->mv_v;
+  s.status = g->status;
+  s.seed = o.sched_seed;
+  s.level = o.level;
+  s.tie_keep = o.tie_keep_current;
+  s.singleton_rule = o.singleton_rule;
+  s.gid = o.batched ? g->gid : nullptr;
+  s.gbase = o.batched ? g->gbase : nullptr;
+  s.gvol = o.batched ? g->gvol : nullptr;
+  s.gfrozen = o.batched ? g->gfrozen : nullptr;
+  return s;
+}
+
+}  // namespace
+
+bool resident_rounds_apply(const cd_graph* g, const RunOpts& o, bool per_graph_stop) {
+  return o.device_loop && !g->timing && !o.async_mode && o.max_iter > 0 && g->n > 0 && g->nhubs == 0 &&
+         g->bin_start[B_BLK4 + 1] == g->bin_start[B_BLK4] && (!per_graph_stop || (o.threshold == 0 && o.use_frontier));
+}
+
+// All rounds of a run or level (see the head of this file). The labels (and,
+// for a given start, sigma and csize) are set here or by the caller.
+int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, int64_t* moves_out, int32_t* rounds_out,
+                    std::vector<int32_t>* graph_rounds) {
+  const cudaStream_t st = g->stream;
+  const bool per_graph = graph_rounds != nullptr;
+  const bool nk = louv && g->vol < ((int64_t)1 << 31);
+  int rc;
+  if (nk && !g->sigma32 && (rc = dev_alloc_t(&g->sigma32, g->n, st))) return rc;
+  LoopCtx L{};
+  L.n = g->n;
+  L.nwords = (g->n + 31) / 32;
+  L.n32 = L.nwords * 32;
+  L.flag0 = g->flag[0];
+  L.flag1 = g->flag[1];
+  L.max_iter = o.max_iter;
+  L.first_rows = singletons && g->cols_distinct;
+  L.t_warp = g->t_warp;
+  L.threshold = o.threshold;
+  L.per_graph = per_graph ? (int32_t)g->nb : 0;
+  L.sigma32 = nk ? g->sigma32 : nullptr;
+  const int64_t words = 2 * (int64_t)o.max_iter + HEAD + (int64_t)TRACE_COLS * o.max_iter;
+  unsigned long long* work = nullptr;
+  if ((rc = dev_alloc_t(&work, words, st))) return rc;
+  if (per_graph && (rc = dev_alloc_t(&L.last_change, g->nb, st))) {
+    dev_free(work, st);
+    return rc;
+  }
+  L.bar = work;
+  L.head = work + 2 * (int64_t)o.max_iter;
+  std::vector<unsigned long long> h;
+  std::vector<int32_t> hl;
+  int32_t status = 0;
+  auto run = [&]() -> int {
+    if (per_graph) CD_CHECK(cudaMemsetAsync(g->gfrozen, 0, g->nb, st));
+    const unsigned gi = (unsigned)std::max<int64_t>(1, std::min<int64_t>((g->n + PNT - 1) / PNT, 152 * 8));
+    CD_LAUNCH(k_rounds_init<<<gi, PNT, 0, st>>>(L, g->C, g->sigma, g->csize, g->degw, louv ? 1 : 0, singletons ? 1 : 0,
+                                                words));
+    const ScanCtx s = loop_ctx(g, o, louv, nk);
+    int r = !louv ? dispatch_loop<false, false>(g, s, L) : nk ? dispatch_loop<true, true>(g, s, L)
+                                                              : dispatch_loop<true, false>(g, s, L);
+    if (r) return r;
+    CD_CHECK(cudaGetLastError());
+    // the header and the rounds of a usual run in one copy
+    const int64_t some = std::min<int64_t>(o.max_iter, 128);
+    h.resize(HEAD + TRACE_COLS * some);
+    CD_CHECK(cudaMemcpyAsync(h.data(), L.head, h.size() * 8, cudaMemcpyDeviceToHost, st));
+    CD_CHECK(cudaMemcpyAsync(&status, g->status, 4, cudaMemcpyDeviceToHost, st));
+    if (per_graph) {
+      hl.resize(g->nb);
+      CD_CHECK(cudaMemcpyAsync(hl.data(), L.last_change, g->nb * 4, cudaMemcpyDeviceToHost, st));
+    }
+    CD_CHECK(cudaStreamSynchronize(st));
+    if (!status && (int64_t)h[0] > some) {
+      const int64_t all = (int64_t)h[0];
+      h.resize(HEAD + TRACE_COLS * all);
+      CD_CHECK(cudaMemcpyAsync(h.data(), L.head, h.size() * 8, cudaMemcpyDeviceToHost, st));
+      CD_CHECK(cudaStreamSynchronize(st));
+    }
+    return status;
+  };
+  rc = run();
+  dev_free(work, st);
+  dev_free(L.last_change, st);
+  if (rc) return rc;
+  const int32_t rounds = (int32_t)h[0];
+  int64_t moves = 0;
+  for (int32_t r = 0; r < rounds; ++r) {
+    const unsigned long long* t = h.data() + HEAD + (int64_t)TRACE_COLS * r;
+    cd_round_trace tr;
+    tr.level = o.level;
+    tr.round = r;
+    tr.active = (int64_t)t[0] + ((r == 0 || !o.use_frontier) ? g->n_isolated : 0);
+    tr.arcs = (int64_t)t[1];
+    tr.moved = (int64_t)t[2];
+    tr.deferred = (int64_t)t[3];
+    tr.cands = (int64_t)t[4];
+    tr.moved_arcs = (int64_t)t[5];
+    tr.scan_ms = tr.round_ms = 0.f;
+    g->trace.push_back(tr);
+    moves += tr.moved;
+  }
+  if (per_graph)  // a graph stops after its first round without a change
+    for (int64_t b = 0; b < g->nb; ++b) (*graph_rounds)[b] = std::min(o.max_iter, hl[b] + 1);
+  if (moves_out) *moves_out = moves;
+  if (rounds_out) *rounds_out = rounds;
+  return CD_OK;
+}
+
+}  // namespace cd

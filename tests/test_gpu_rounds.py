@@ -1,0 +1,80 @@
+"""The resident round loop against the host round loop and the oracle at the sizes where it can go wrong: degrees at the
+edges of the tiles, the warp and the half-CTA classes, vertex counts around a flag word and around what a CTA takes at
+a time, every weight kind and key width, each parameter that changes a round. Integers: everything must be equal."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+EDGES = [1, 4, 5, 8, 9, 16, 17, 32, 33, 127, 128, 129, 255, 256, 257, 511, 512, 1023, 1024]
+
+
+def degrees_graph(n, degs, seed, wmax, loops=0):
+    """Vertices of the given degrees (and one arc more or fewer where they meet) in a sparse random graph on n."""
+    rng = np.random.default_rng(seed)
+    edges = set()
+    for i, d in enumerate(degs):
+        if d >= n:
+            continue
+        others = rng.choice(np.setdiff1d(np.arange(n), [i]), d, replace=False)
+        edges |= {(min(i, int(x)), max(i, int(x))) for x in others}
+    edges |= {(int(a), int(b)) for a, b in np.sort(rng.integers(0, n, (n, 2)), axis=1) if a != b}
+    edges = sorted(edges)
+    ws = rng.integers(1, wmax + 1, len(edges)).tolist() if wmax > 1 else None
+    lo = {int(v): int(rng.integers(1, wmax + 1)) for v in rng.choice(n, loops, replace=False)} if loops else None
+    return synth.from_edge_list(n, edges, ws, lo)
+
+
+def check(g, params):
+    import paper_2507_06471_gb300 as cd
+    G = cd.Graph(g.off.cuda(), g.cols.cuda(), None if g.w is None else g.w.cuda())
+    out = []
+    for loop in (1, 0):
+        lab, rounds = G.lpa(device_loop=loop, **params)
+        tr = [(t["active"], t["arcs"], t["moved"], t["deferred"], t["cands"], t["moved_arcs"]) for t in G.trace()]
+        lab2, moves, rounds2 = G.local_move(device_loop=loop, **params)
+        tr2 = [(t["active"], t["arcs"], t["moved"], t["deferred"], t["cands"], t["moved_arcs"]) for t in G.trace()]
+        lab3, moves3, rounds3 = G.local_move(labels=lab, device_loop=loop, **params)
+        lv = G.louvain(device_loop=loop, **params)
+        out.append((lab.cpu().numpy(), rounds, tr, lab2.cpu().numpy(), moves, rounds2, tr2, lab3.cpu().numpy(), moves3,
+                    rounds3, lv[0].cpu().numpy(), lv[1], lv[2]))
+    G.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b) if isinstance(a, np.ndarray) else a == b
+    return out[0]
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 613, 1131, 2048, 2049, 5000])
+@pytest.mark.parametrize("wmax,loops", [(1, 0), (9, 0), (7, 11), (300_000, 1), (2_000_000_000, 0)])
+def test_equals_host_loop_and_oracle(n, wmax, loops):
+    g = degrees_graph(n, [d for d in EDGES if d < n // 2], n + wmax % 97, wmax, min(loops, n))
+    got = check(g, {})
+    off, cols, w = g.numpy()
+    lab, tr = oracle.lpa(off, cols, w)
+    assert np.array_equal(got[0], lab) and got[1] == tr.rounds
+    lab, lv, q, _ = oracle.louvain(off, cols, w)
+    assert np.array_equal(got[10], lab) and got[11] == lv and abs(got[12] - q) <= 1e-12 * max(1.0, abs(q))
+
+
+@pytest.mark.parametrize("params", [{"use_frontier": 0}, {"threshold": 40}, {"tie_keep_current": 0}, {"max_iter": 1},
+                                    {"max_iter": 300, "sched_seed": 77}, {"singleton_rule": 0}])
+def test_parameters(params):
+    check(degrees_graph(3000, EDGES, 5, 3), params)
+
+
+def test_batched_equals_host_loop():
+    import paper_2507_06471_gb300 as cd
+    graphs = [degrees_graph(n, [d for d in EDGES if d < n // 2], n, 4) for n in (1, 2, 40, 700, 33, 1500, 64, 3)]
+    packed, vstart = synth.pack_batch(graphs)
+    G = cd.Graph(packed.off.cuda(), packed.cols.cuda(), packed.w.cuda())
+    G.set_batches(vstart)
+    for params in ({}, {"threshold": 5}, {"max_iter": 3}, {"use_frontier": 0}):
+        a, b = (G.batch_lpa(device_loop=loop, **params) for loop in (1, 0))
+        assert np.array_equal(a[0].cpu().numpy(), b[0].cpu().numpy()) and np.array_equal(a[1], b[1])
+        a, b = (G.batch_louvain(device_loop=loop, **params) for loop in (1, 0))
+        assert np.array_equal(a[0].cpu().numpy(), b[0].cpu().numpy()) and np.array_equal(a[1], b[1])
+        assert np.array_equal(a[2], b[2])
+    G.close()
