@@ -161,13 +161,13 @@ struct Scan {
     const bool cand = has && u != v;
     const int32_t lbl = cand ? (first ? u : s.C[u]) : (int32_t)(0x80000000u | (unsigned)lane);
     const unsigned peers = __match_any_sync(FULL, lbl) & tmask;
-    const int64_t gsum = group_sum<W>(peers, wt, stage);
+    const int64_t gsum = group_sum<W>(peers, wt, stage, sizeof(V) == 4);
     const bool leader = cand && (__ffs(peers) - 1) == lane;
     const unsigned cm = __ballot_sync(FULL, cand && lbl == cur) & tmask;
     int64_t kcur = __shfl_sync(FULL, gsum, cm ? __ffs(cm) - 1 : lane);
     if (!cm) kcur = 0;
     const bool ok = leader && (!LOUV || lbl != cur);
-    K bk = ok ? cand_key<LOUV, NK>(s, lbl, gsum, dv, volv) : K(0);
+    K bk = ok ? cand_key<LOUV, NK>(s, lbl, gsum, dv, volv) : no_key<K>();
     int32_t bc = ok ? lbl : NOCAND;
     reduce_best(bk, bc, tw);
     int32_t target = cur;
@@ -189,7 +189,7 @@ struct Scan {
   // header, the warp scans the rows one after another, and the decisions run
   // one lane per vertex.
   __device__ __forceinline__ void warp_batch(const int32_t* list, int base, int count, int vb, int32_t* keys, V* vals,
-                                             uint16_t* occ, int* occ_n, int64_t* stage, Tally& t) const {
+                                             uint16_t* occ, int* occ_n, Tally& t) const {
     const int lane = threadIdx.x & 31;
     const bool on = lane < vb && base + lane < count;
     const int32_t my_v = on ? list[base + lane] : 0;
@@ -204,7 +204,7 @@ struct Scan {
         my_vol = vol_of(s, my_v);
       }
     }
-    K my_bk = K(0);
+    K my_bk = no_key<K>();
     int32_t my_bc = NOCAND;
     bool my_hc = false;
     int64_t my_kc = 0, ncand = 0;
@@ -214,7 +214,7 @@ struct Scan {
       const int64_t beg = __shfl_sync(FULL, my_beg, j), end = __shfl_sync(FULL, my_end, j);
       const int64_t dv = LOUV ? __shfl_sync(FULL, my_dv, j) : 0;
       const int64_t volv = LOUV ? __shfl_sync(FULL, my_vol, j) : 0;
-      K bk = K(0);
+      K bk = no_key<K>();
       int32_t bc = NOCAND;
       bool hc = false;
       int64_t kc = 0;
@@ -232,7 +232,7 @@ struct Scan {
         reduce_best(bk, bc, 32);
       } else {
         const unsigned lg = 64 - __clzll((unsigned long long)(2 * (end - beg) - 1));  // 2^lg >= 2 deg
-        group_insert<W, V, 32>(s, v, beg, end, lane, keys, vals, occ, occ_n, lg, stage);
+        group_insert<W, V, 32>(s, v, beg, end, lane, keys, vals, occ, occ_n, lg);
         __syncwarp();
         group_eval<LOUV, V, 32, NK>(s, cur, dv, volv, lane, keys, vals, occ, *occ_n, bk, bc, hc, kc, ncand);
         reduce_best(bk, bc, 32);
@@ -279,16 +279,16 @@ struct Scan {
     int32_t moved;
   };
   __device__ __forceinline__ void half_cta(int32_t v, int half, int32_t* keys, V* vals, uint16_t* occ, int* occ_n,
-                                           int64_t* stage, HalfRed* red, Tally& t) const {
+                                           HalfRed* red, Tally& t) const {
     const int lane = threadIdx.x & 31, gl = threadIdx.x & 127, wig = gl >> 5;
     const int64_t beg = __ldg(s.off + v), end = __ldg(s.off + v + 1);
     const int32_t cur = s.C[v];
     const int64_t dv = LOUV ? __ldg(s.degw + v) : 0;
     const int64_t volv = LOUV ? vol_of(s, v) : 0;
     const unsigned lg = 64 - __clzll((unsigned long long)(2 * (end - beg) - 1));
-    group_insert<W, V, 128>(s, v, beg, end, gl, keys, vals, occ, occ_n, lg, stage);
+    group_insert<W, V, 128>(s, v, beg, end, gl, keys, vals, occ, occ_n, lg);
     half_sync(half);
-    K bk = K(0);
+    K bk = no_key<K>();
     int32_t bc = NOCAND;
     bool hc = false;
     int64_t kc = 0, ncand = 0;
@@ -305,7 +305,7 @@ struct Scan {
     }
     half_sync(half);
     if (wig == 0) {
-      bk = lane < 4 ? red->k[lane] : K(0);
+      bk = lane < 4 ? red->k[lane] : no_key<K>();
       bc = lane < 4 ? red->c[lane] : NOCAND;
       reduce_best(bk, bc, 32);
       hm = __ballot_sync(FULL, lane < 4 && red->hc[lane & 3]);
@@ -454,9 +454,10 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
       // half CTAs
       int n_half = first_of[1];
       if (!sc.first) {
-        for (int i = half; i < n_half; i += 2)
+        // a few: one half takes them while the other starts on the warps' tasks
+        for (int i = n_half < 4 ? (half ? n_half : 0) : half; i < n_half; i += n_half < 4 ? 1 : 2)
           sc.half_cta(list[i], half, keys0 + half * 4 * PCAP, vals0 + half * 4 * PCAP, occ0 + half * 4 * PCAP,
-                      &occ_n[half * 4], stage, &red[half], t);
+                      &occ_n[half * 4], &red[half], t);
       } else {
         n_half = 0;  // rows without tables: the warps take them
       }
@@ -474,7 +475,7 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
         if (task >= t_4) break;
         if (task < t_wb) {
           sc.warp_batch(list, n_half + task * wb, first_of[2], wb, keys0 + wid * PCAP, vals0 + wid * PCAP,
-                        occ0 + wid * PCAP, &occ_n[wid], stage, t);
+                        occ0 + wid * PCAP, &occ_n[wid], t);
         } else {
           const int q = task < t_32 ? 2 : task < t_16 ? 3 : task < t_8 ? 4 : 5;
           const int t0 = q == 2 ? t_wb : q == 3 ? t_32 : q == 4 ? t_16 : t_8;

@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(NT) k_hub_apply_log(ScanCtx s) {
 // TILE lanes per vertex, one arc per lane (degree <= TILE).
 template <int TILE, bool LOUV, class W, bool NK>
 __global__ void __launch_bounds__(NT, 6) k_scan_tile(ScanCtx s, const int32_t* __restrict__ list,
-                                                  const unsigned long long* __restrict__ count_p, int bin) {
+                                                  const unsigned long long* __restrict__ count_p, int bin, bool v32) {
   typedef typename KeyOf<LOUV, NK>::T K;
   const int64_t count = (int64_t)*count_p;
   __shared__ int64_t stage[NW][32];
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(NT, 6) k_scan_tile(ScanCtx s, const int32_t* _
     const bool cand = has && u != v;
     const int32_t lbl = cand ? s.C[u] : (int32_t)(0x80000000u | (unsigned)lane);
     const unsigned peers = __match_any_sync(FULL, lbl) & tmask;
-    const int64_t gsum = group_sum<W>(peers, wt, stage[wid]);
+    const int64_t gsum = group_sum<W>(peers, wt, stage[wid], v32);
     const bool leader = cand && (__ffs(peers) - 1) == lane;
     const int32_t cur = act ? s.C[v] : 0;
     const unsigned cm = __ballot_sync(FULL, cand && lbl == cur) & tmask;
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(NT, 6) k_scan_tile(ScanCtx s, const int32_t* _
     const int64_t dv = (LOUV && act) ? s.degw[v] : 0;
     const int64_t volv = (LOUV && act) ? vol_of(s, v) : 0;
     const bool ok = leader && (!LOUV || lbl != cur);
-    K bk = ok ? cand_key<LOUV, NK>(s, lbl, gsum, dv, volv) : K(0);
+    K bk = ok ? cand_key<LOUV, NK>(s, lbl, gsum, dv, volv) : no_key<K>();
     int32_t bc = ok ? lbl : NOCAND;
     reduce_best(bk, bc, TILE);
     int32_t target = cur;
@@ -147,9 +147,7 @@ __global__ void __launch_bounds__(NTB, GROUP == 32 ? ((LOUV || !W::unit) ? 4 : 5
   const int gid = threadIdx.x / GROUP, gl = threadIdx.x % GROUP, wig = gl >> 5;
   V* vals = (V*)smem + (size_t)gid * CAP;
   int32_t* keys = (int32_t*)(smem + (size_t)GPB * CAP * sizeof(V)) + (size_t)gid * CAP;
-  int64_t* stage = (int64_t*)(smem + (size_t)GPB * CAP * (sizeof(V) + 4)) + wid * 32;
-  uint16_t* occ = (uint16_t*)(smem + (size_t)GPB * CAP * (sizeof(V) + 4) + (size_t)(NTB / 32) * 32 * 8) +
-                  (size_t)gid * CAP;
+  uint16_t* occ = (uint16_t*)(smem + (size_t)GPB * CAP * (sizeof(V) + 4)) + (size_t)gid * CAP;
   for (int j = gl; j < CAP; j += GROUP) {
     keys[j] = EMPTY;
     vals[j] = 0;
@@ -187,12 +185,12 @@ __global__ void __launch_bounds__(NTB, GROUP == 32 ? ((LOUV || !W::unit) ? 4 : 5
     const int64_t d = end - beg;
     const unsigned lg = ceil_log2(2 * d);
     const int32_t cur = h.cur;
-    group_insert<W, V, GROUP>(s, v, beg, end, gl, keys, vals, occ, &occ_n[gid], lg, stage);
+    group_insert<W, V, GROUP>(s, v, beg, end, gl, keys, vals, occ, &occ_n[gid], lg);
     group_sync<GROUP, NTB>(gid);
     const int64_t dv = h.dv;
     const int64_t volv = h.vol;
     const int nocc = occ_n[gid];
-    K bk = K(0);
+    K bk = no_key<K>();
     int32_t bc = NOCAND;
     bool hc = false;
     int64_t kc = 0;
@@ -209,7 +207,7 @@ __global__ void __launch_bounds__(NTB, GROUP == 32 ? ((LOUV || !W::unit) ? 4 : 5
       }
       group_sync<GROUP, NTB>(gid);
       if (wig == 0) {
-        bk = lane < WPG ? red_k[gid][lane] : K(0);
+        bk = lane < WPG ? red_k[gid][lane] : no_key<K>();
         bc = lane < WPG ? red_c[gid][lane] : NOCAND;
         reduce_best(bk, bc, 32);
         hm = __ballot_sync(FULL, lane < WPG && red_hc[gid][lane]);
@@ -259,8 +257,7 @@ __global__ void __launch_bounds__(256, (LOUV || !W::unit) ? 4 : 5)
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   V* vals = (V*)smem + (size_t)wid * CAP;
   int32_t* keys = (int32_t*)(smem + (size_t)WPB * CAP * sizeof(V)) + (size_t)wid * CAP;
-  int64_t* stage = (int64_t*)(smem + (size_t)WPB * CAP * (sizeof(V) + 4)) + wid * 32;
-  uint16_t* occ = (uint16_t*)(smem + (size_t)WPB * CAP * (sizeof(V) + 4) + (size_t)WPB * 32 * 8) + (size_t)wid * CAP;
+  uint16_t* occ = (uint16_t*)(smem + (size_t)WPB * CAP * (sizeof(V) + 4)) + (size_t)wid * CAP;
   for (int j = lane; j < CAP; j += 32) {
     keys[j] = EMPTY;
     vals[j] = 0;
@@ -276,7 +273,7 @@ __global__ void __launch_bounds__(256, (LOUV || !W::unit) ? 4 : 5)
     const bool in = lane < vb && i < count;
     const int32_t my_v = in ? list[i] : 0;
     const VHdr h = load_hdr<LOUV>(s, my_v, in);
-    K my_bk = K(0);
+    K my_bk = no_key<K>();
     int32_t my_bc = NOCAND;
     bool my_hc = false;
     int64_t my_kc = 0;
@@ -288,9 +285,9 @@ __global__ void __launch_bounds__(256, (LOUV || !W::unit) ? 4 : 5)
       const int64_t dv = LOUV ? __shfl_sync(FULL, h.dv, j) : 0;
       const int64_t volv = LOUV ? __shfl_sync(FULL, h.vol, j) : 0;
       const unsigned lg = 64 - __clzll((unsigned long long)(2 * (end - beg) - 1));  // 2^lg >= 2 deg
-      group_insert<W, V, 32>(s, v, beg, end, lane, keys, vals, occ, &occ_n[wid], lg, stage);
+      group_insert<W, V, 32>(s, v, beg, end, lane, keys, vals, occ, &occ_n[wid], lg);
       __syncwarp();
-      K bk = K(0);
+      K bk = no_key<K>();
       int32_t bc = NOCAND;
       bool hc = false;
       int64_t kc = 0;
@@ -624,8 +621,7 @@ __global__ void __launch_bounds__(HUB_NT) k_hub_build(ScanCtx s) {
   __shared__ int occ_n;
   V* vals = (V*)smem;
   int32_t* keys = (int32_t*)(smem + (size_t)HUB_CAP * sizeof(V));
-  int64_t* stage = (int64_t*)(smem + (size_t)HUB_CAP * (sizeof(V) + 4)) + (threadIdx.x >> 5) * 32;
-  uint16_t* occ = (uint16_t*)(smem + (size_t)HUB_CAP * (sizeof(V) + 4) + (size_t)(HUB_NT / 32) * 32 * 8);
+  uint16_t* occ = (uint16_t*)(smem + (size_t)HUB_CAP * (sizeof(V) + 4));
   for (int j = threadIdx.x; j < HUB_CAP; j += HUB_NT) {
     keys[j] = EMPTY;
     vals[j] = 0;
@@ -640,7 +636,7 @@ __global__ void __launch_bounds__(HUB_NT) k_hub_build(ScanCtx s) {
     const int64_t a0 = s.hub_item_arc[it];
     const int64_t rowend = s.off[v + 1];
     const int64_t end = a0 + HUB_CHUNK < rowend ? a0 + HUB_CHUNK : rowend;
-    group_insert<W, V, HUB_NT>(s, v, a0, end, threadIdx.x, keys, vals, occ, &occ_n, 13, stage);
+    group_insert<W, V, HUB_NT>(s, v, a0, end, threadIdx.x, keys, vals, occ, &occ_n, 13);
     __syncthreads();
     const int nocc = occ_n;
     for (int j = threadIdx.x; j < nocc; j += HUB_NT) {
@@ -705,7 +701,7 @@ __global__ void __launch_bounds__(NT) k_hub_eval_small(ScanCtx s) {
     const int64_t volv = LOUV ? vol_of(s, v) : 0;
     const int64_t base = s.hub_tab[h];
     const int64_t cap = s.hub_cc[h];
-    K bk = K(0);
+    K bk = no_key<K>();
     int32_t bc = NOCAND;
     bool hc = false;
     int64_t kc = 0;
@@ -788,7 +784,7 @@ __global__ void __launch_bounds__(NT) k_hub_eval(ScanCtx s) {
     const int64_t cap = s.hub_cc[h];
     const int64_t e0 = s.hub_ev_slot[it];
     const int64_t e1 = e0 + HUB_SLICE < cap ? e0 + HUB_SLICE : cap;
-    K bk = K(0);
+    K bk = no_key<K>();
     int32_t bc = NOCAND;
     unsigned nl = 0;
     constexpr int HB = 6;  // slots per thread per batch: all loads, then all gathers, in flight together
@@ -848,7 +844,7 @@ __global__ void __launch_bounds__(NT) k_hub_eval(ScanCtx s) {
     if (s_last && threadIdx.x == 0) {
       __threadfence();
       const volatile int64_t* part = s.hub_part;
-      K fk = K(0);
+      K fk = no_key<K>();
       int32_t fc = NOCAND;
       const int64_t p0 = s.hub_ev_first[h], p1 = p0 + (cap + HUB_SLICE - 1) / HUB_SLICE;
       for (int64_t p = p0; p < p1; ++p) {
@@ -918,7 +914,7 @@ __global__ void __launch_bounds__(NT) k_first_round(ScanCtx s, const int32_t* __
         volv = vol_of(s, v);
       }
     }
-    K bk = K(0);
+    K bk = no_key<K>();
     int32_t bc = NOCAND;
     for (int64_t e = beg + gl; e < end; e += PER) {
       const int32_t u = s.cols[e];
@@ -1286,13 +1282,11 @@ int warp_batch(KERN kernel, size_t smem, int64_t cnt) {
 }
 
 // Group-kernel configurations: (GROUP threads per vertex, CTA size, table slots).
-template <class V> constexpr size_t group_smem(int gpb, int cap, int ntb) {
-  return (size_t)gpb * cap * (sizeof(V) + 4) + (size_t)(ntb / 32) * 32 * 8 + (size_t)gpb * cap * 2;
-}
-template <class V> constexpr size_t warp_smem() { return group_smem<V>(8, WARP_CAP_SLOTS, 256); }
-template <class V> constexpr size_t blk1_smem() { return group_smem<V>(4, BLK1_CAP_SLOTS, 512); }
-template <class V> constexpr size_t blk4_smem() { return group_smem<V>(1, BLK4_CAP_SLOTS, 512); }
-template <class V> constexpr size_t hub_smem() { return group_smem<V>(1, HUB_CAP, HUB_NT); }
+template <class V> constexpr size_t group_smem(int gpb, int cap) { return (size_t)gpb * cap * (sizeof(V) + 4 + 2); }
+template <class V> constexpr size_t warp_smem() { return group_smem<V>(8, WARP_CAP_SLOTS); }
+template <class V> constexpr size_t blk1_smem() { return group_smem<V>(4, BLK1_CAP_SLOTS); }
+template <class V> constexpr size_t blk4_smem() { return group_smem<V>(1, BLK4_CAP_SLOTS); }
+template <class V> constexpr size_t hub_smem() { return group_smem<V>(1, HUB_CAP); }
 
 template <bool LOUV, class W, class V, bool NK>
 int set_smem_attrs() {
@@ -1502,7 +1496,7 @@ int launch_round(cd_graph* g, ScanCtx& s, const int32_t* lists, const unsigned l
       KTimer t(g, K_SCAN_T32);
       auto kern = k_scan_tile<32, LOUV, W, NK>;
       CD_LAUNCH(kern<<<wave_grid(kern, NT, 0, (cnt(B_T32) + NW - 1) / (NW)), NT, 0, st>>>(
-          s, lst(B_T32), dcnt(B_T32), B_T32));
+          s, lst(B_T32), dcnt(B_T32), B_T32, sizeof(V) == 4));
     }
     if (g->ktiming) mark(B_T32);
   }
@@ -1511,7 +1505,7 @@ int launch_round(cd_graph* g, ScanCtx& s, const int32_t* lists, const unsigned l
       KTimer t(g, K_SCAN_T16);
       auto kern = k_scan_tile<16, LOUV, W, NK>;
       CD_LAUNCH(kern<<<wave_grid(kern, NT, 0, (cnt(B_T16) + 2 * NW - 1) / (2 * NW)), NT, 0, st>>>(
-          s, lst(B_T16), dcnt(B_T16), B_T16));
+          s, lst(B_T16), dcnt(B_T16), B_T16, sizeof(V) == 4));
     }
     if (g->ktiming) mark(B_T16);
   }
@@ -1520,7 +1514,7 @@ int launch_round(cd_graph* g, ScanCtx& s, const int32_t* lists, const unsigned l
       KTimer t(g, K_SCAN_T8);
       auto kern = k_scan_tile<8, LOUV, W, NK>;
       CD_LAUNCH(kern<<<wave_grid(kern, NT, 0, (cnt(B_T8) + 4 * NW - 1) / (4 * NW)), NT, 0, st>>>(
-          s, lst(B_T8), dcnt(B_T8), B_T8));
+          s, lst(B_T8), dcnt(B_T8), B_T8, sizeof(V) == 4));
     }
     if (g->ktiming) mark(B_T8);
   }
@@ -1529,7 +1523,7 @@ int launch_round(cd_graph* g, ScanCtx& s, const int32_t* lists, const unsigned l
       KTimer t(g, K_SCAN_T4);
       auto kern = k_scan_tile<4, LOUV, W, NK>;
       CD_LAUNCH(kern<<<wave_grid(kern, NT, 0, (cnt(B_T4) + 8 * NW - 1) / (8 * NW)), NT, 0, st>>>(
-          s, lst(B_T4), dcnt(B_T4), B_T4));
+          s, lst(B_T4), dcnt(B_T4), B_T4, sizeof(V) == 4));
     }
     if (g->ktiming) mark(B_T4);
   }

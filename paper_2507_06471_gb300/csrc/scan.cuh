@@ -45,16 +45,32 @@ __device__ __forceinline__ i128 shfl_xor_key(i128 x, int o) {
   return (i128)(((unsigned __int128)hi << 64) | lo);
 }
 
+// The key of "no candidate" (with the id NOCAND): below every candidate's key,
+// so that comparing needs no case of its own.
+template <class K> __device__ __forceinline__ K no_key();
+template <> __device__ __forceinline__ int64_t no_key<int64_t>() { return INT64_MIN; }
+template <> __device__ __forceinline__ i128 no_key<i128>() { return (i128)INT64_MIN << 64; }
+
 // Is candidate (k1, c1) preferred over (k0, c0)? Larger key, then smaller id.
 template <class K>
 __device__ __forceinline__ bool better(K k1, int32_t c1, K k0, int32_t c0) {
-  if (c1 == NOCAND) return false;
-  if (c0 == NOCAND) return true;
   return k1 > k0 || (k1 == k0 && c1 < c0);
 }
 
+// The best of each group of `width` consecutive lanes, in every lane of it.
 template <class K>
 __device__ __forceinline__ void reduce_best(K& k, int32_t& c, int width) {
+  if constexpr (sizeof(K) == 8) {
+    if (width == 32) {  // whole warps: three hardware reductions instead of five exchanges of three words
+      const int32_t hi = (int32_t)(k >> 32);
+      const int32_t mh = __reduce_max_sync(FULL, hi);
+      const uint32_t ml = __reduce_max_sync(FULL, hi == mh ? (uint32_t)k : 0u);
+      const K best = (K)(((uint64_t)(uint32_t)mh << 32) | ml);
+      c = __reduce_min_sync(FULL, k == best ? c : NOCAND);
+      k = best;
+      return;
+    }
+  }
   for (int o = width / 2; o > 0; o >>= 1) {
     K ok = shfl_xor_key(k, o);
     int32_t oc = __shfl_xor_sync(FULL, c, o);
@@ -179,24 +195,23 @@ __device__ __forceinline__ int64_t sig_of(const ScanCtx& s, int32_t c) {
   return s.sigma[c];
 }
 
+// vol(V) k - deg_w(v) Sigma_tot[c], or k for LPA. When vol(V) < 2^31 all four
+// factors fit in 32 bits, so each product is one 32 x 32 -> 64 multiplication.
 template <bool LOUV, bool NK>
-__device__ __forceinline__ typename KeyOf<LOUV, NK>::T cand_key(const ScanCtx& s, int32_t c, int64_t k,
-                                                            int64_t d, int64_t vol) {
+__device__ __forceinline__ typename KeyOf<LOUV, NK>::T cand_key_sg(int64_t sig, int64_t k, int64_t d, int64_t vol) {
   if constexpr (LOUV && NK)
-    return vol * k - d * sig_of<NK>(s, c);  // each product < 2^62 when vol(V) < 2^31
+    return (int64_t)((uint64_t)(uint32_t)vol * (uint32_t)k) - (int64_t)((uint64_t)(uint32_t)d * (uint32_t)sig);
   else if constexpr (LOUV)
-    return (i128)vol * k - (i128)d * s.sigma[c];
+    return (i128)vol * k - (i128)d * sig;
   else
     return k;
 }
 
-// The same key with Sigma_tot[c] already loaded.
 template <bool LOUV, bool NK>
-__device__ __forceinline__ typename KeyOf<LOUV, NK>::T cand_key_sg(int64_t sig, int64_t k, int64_t d, int64_t vol) {
-  if constexpr (LOUV && NK)
-    return vol * k - d * sig;
-  else if constexpr (LOUV)
-    return (i128)vol * k - (i128)d * sig;
+__device__ __forceinline__ typename KeyOf<LOUV, NK>::T cand_key(const ScanCtx& s, int32_t c, int64_t k,
+                                                            int64_t d, int64_t vol) {
+  if constexpr (LOUV)
+    return cand_key_sg<LOUV, NK>(sig_of<NK>(s, c), k, d, vol);
   else
     return k;
 }
@@ -212,9 +227,19 @@ __device__ __forceinline__ int32_t decide(const ScanCtx& s, int32_t v, int32_t c
     return bc;
   } else {
     int64_t d = s.degw[v];
-    i128 G = (i128)bk - (i128)vol * kcur + (i128)d * (sig_of<NK>(s, cur) - d);
-    if (G <= 0) return cur;  // only strictly positive gains
-    if (s.singleton_rule && s.csize[cur] == 1 && s.csize[bc] == 1 && bc > cur) return cur;
+    bool gain;
+    if constexpr (NK) {
+      // vol(V) < 2^31: vol k, d Sigma < 2^62 and Sigma[cur] >= d, so the sum stays inside (-2^63, 2^63)
+      gain = bk - (int64_t)((uint64_t)(uint32_t)vol * (uint32_t)kcur) +
+                 (int64_t)((uint64_t)(uint32_t)d * (uint32_t)(sig_of<NK>(s, cur) - d)) > 0;
+    } else {
+      gain = (i128)bk - (i128)vol * kcur + (i128)d * (s.sigma[cur] - d) > 0;
+    }
+    if (!gain) return cur;  // only strictly positive gains
+    if (s.singleton_rule && bc > cur) {
+      const int32_t na = s.csize[cur], nb = s.csize[bc];  // two loads in flight, not one after the other
+      if (na == 1 && nb == 1) return cur;
+    }
     return bc;
   }
 }
@@ -272,14 +297,27 @@ __device__ __forceinline__ bool is_active(const ScanCtx& s, int32_t v) {
   return s.all_active || ((s.flag_cur[v >> 5] >> (v & 31)) & 1u);
 }
 
-// Group weight of the lanes in `peers` (equal labels): popcount for unit
-// weights, else a sum over the warp's staging row.
+// Group weight of the lanes in `peers` (equal labels; every lane takes part):
+// popcount for unit weights, else sums over the warp's staging row. When every
+// deg_w < 2^32 (v32) the lanes add into their group's first word, one shared
+// atomic each; walking the peers instead takes as many dependent loads as the
+// largest group has lanes, which is the whole row once labels have settled.
 template <class W>
-__device__ __forceinline__ int64_t group_sum(unsigned peers, int64_t wt, int64_t* stage) {
+__device__ __forceinline__ int64_t group_sum(unsigned peers, int64_t wt, int64_t* stage, bool v32) {
   if constexpr (W::unit) {
     return (int64_t)__popc(peers);
   } else {
     const int lane = threadIdx.x & 31;
+    if (v32) {  // uniform
+      uint32_t* row = (uint32_t*)stage;
+      row[lane] = 0;
+      __syncwarp();
+      atomicAdd(&row[__ffs(peers) - 1], (uint32_t)wt);
+      __syncwarp();
+      const uint32_t sum = row[__ffs(peers) - 1];
+      __syncwarp();
+      return (int64_t)sum;
+    }
     stage[lane] = wt;
     __syncwarp();
     int64_t s = 0;
@@ -427,19 +465,26 @@ __device__ __forceinline__ void hub_neighbour_moved(const ScanCtx& s, int32_t u,
 // ------------------------------------------------------------------ shared-memory tables
 
 // Open addressing with linear probing; capacity 2^lg >= 2 x the arcs inserted,
-// so a free slot is always found within `cap` probes. A newly claimed slot is
-// appended to the table's occupied list, so that reading the table costs the
-// number of distinct labels rather than its capacity.
+// so a free slot is always found within `cap` probes. A probe is a plain load;
+// only an empty slot is claimed with a compare-and-swap. A newly claimed slot
+// is appended to the table's occupied list, so that reading the table costs
+// the number of distinct labels rather than its capacity.
 template <class V>
 __device__ __forceinline__ void smem_insert(int32_t* keys, V* vals, uint16_t* occ, int* occ_n,
                                             unsigned lg, int32_t key, V w, int32_t* status) {
   const unsigned mask = (1u << lg) - 1u;
   unsigned h = ((uint32_t)key * 2654435761u) >> (32 - lg);
   for (unsigned probe = 0; probe <= mask; ++probe) {
-    const int32_t prev = atomicCAS(&keys[h], EMPTY, key);
-    if (prev == EMPTY || prev == key) {
+    int32_t k = *(volatile int32_t*)&keys[h];
+    if (k == EMPTY) {
+      k = atomicCAS(&keys[h], EMPTY, key);
+      if (k == EMPTY) {
+        occ[atomicAdd(occ_n, 1)] = (uint16_t)h;
+        k = key;
+      }
+    }
+    if (k == key) {
       atomicAdd(vals + h, w);
-      if (prev == EMPTY) occ[atomicAdd(occ_n, 1)] = (uint16_t)h;
       return;
     }
     h = (h + 1) & mask;
@@ -466,14 +511,16 @@ __device__ __forceinline__ void group_sync(int gid) {
 }
 
 // Insert the arcs [beg, end) of vertex v into a group's table. Columns are
-// read 16 bytes at a time (4 arcs per lane, 4 label gathers in flight); equal
-// labels inside a warp are combined with __match_any_sync before the atomics.
+// read 16 bytes at a time (4 arcs per lane, 4 label gathers in flight), and
+// every arc goes into the table by itself: combining the equal labels of a
+// warp first (a match, then a walk over the peers) took several times the
+// instructions of the shared atomics it saved.
 // Column arrays carry COL_PAD spare entries, so a 16-byte load that starts
 // before `end` stays inside the allocation.
 template <class W, class V, int GROUP>
 __device__ __forceinline__ void group_insert(const ScanCtx& s, int32_t v, int64_t beg, int64_t end,
                                              int gl, int32_t* keys, V* vals, uint16_t* occ, int* occ_n,
-                                             unsigned lg, int64_t* stage) {
+                                             unsigned lg) {
   const int lane = threadIdx.x & 31;
   const int wig = gl >> 5;
   const int64_t a0 = beg & ~(int64_t)3;
@@ -482,22 +529,17 @@ __device__ __forceinline__ void group_insert(const ScanCtx& s, int32_t v, int64_
     const int4 c4 = base < end ? __ldg(reinterpret_cast<const int4*>(s.cols + base)) : make_int4(0, 0, 0, 0);
     const int32_t cs[4] = {c4.x, c4.y, c4.z, c4.w};
     int32_t lbl[4];
-    int64_t wt[4];
+    V wt[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int64_t e = base + j;
       const bool has = e >= beg && e < end;
-      const bool cand = has && cs[j] != v;
-      lbl[j] = cand ? s.C[cs[j]] : (int32_t)(0x80000000u | (unsigned)(lane * 4 + j));
-      wt[j] = (has && !W::unit) ? W::get(s.w, e) : 1;
+      lbl[j] = has && cs[j] != v ? s.C[cs[j]] : -1;
+      wt[j] = (has && !W::unit) ? (V)W::get(s.w, e) : (V)1;
     }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const unsigned peers = __match_any_sync(FULL, lbl[j]);
-      const int64_t gsum = group_sum<W>(peers, wt[j], stage);
-      if (lbl[j] >= 0 && (__ffs(peers) - 1) == lane)
-        smem_insert(keys, vals, occ, occ_n, lg, lbl[j], (V)gsum, s.status);
-    }
+    for (int j = 0; j < 4; ++j)
+      if (lbl[j] >= 0) smem_insert(keys, vals, occ, occ_n, lg, lbl[j], wt[j], s.status);
   }
 }
 
