@@ -122,7 +122,7 @@ struct cd_graph {
   int32_t* hub_ev_hub = nullptr;           // per evaluate item (HUB_SLICE entries): hub
   int64_t* hub_ev_slot = nullptr;          // per evaluate item: first slot
   int64_t* hub_ev_first = nullptr;         // nhubs+1: first evaluate item of each hub
-  int64_t* hub_part = nullptr;             // per evaluate item: (key hi, key lo, community)
+  int64_t* hub_part = nullptr;             // per evaluate item (first round: build/mark item): (key hi, key lo, community)
   int64_t* hub_cur = nullptr;              // nhubs: weight into the hub's own label
   int32_t* hub_hascur = nullptr;           // nhubs
   int32_t* hub_done = nullptr;             // nhubs: finished evaluate items this round
@@ -213,6 +213,7 @@ void profile_reset(cd_graph* g);
 int profile_flush(cd_graph* g);  // syncs, accumulates pending events
 
 // graph.cu
+constexpr int INGEST_STATS = 5 + NBINS;  // words of the ingest statistics: [0] vol, [2] isolated, [3] largest deg_w, ...
 // Takes ownership of device arrays in the internal convention (loop arcs 2L).
 int graph_adopt(cudaStream_t s, int64_t n, int64_t nnz, int64_t* off, int32_t* cols, void* w,
                 int wkind, cd_graph** out, int64_t* degw_pre = nullptr,

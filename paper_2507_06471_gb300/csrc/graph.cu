@@ -105,7 +105,7 @@ int profile_flush(cd_graph* g) {
 namespace {
 
 constexpr int NT = 256;
-constexpr int NSTATS = 5 + NBINS;
+constexpr int NSTATS = INGEST_STATS;
 
 __device__ __forceinline__ void fail(int32_t* status, int code) { atomicCAS(status, 0, code); }
 
@@ -598,7 +598,7 @@ int build_bins(cd_graph* g) {
     if ((rc = dev_alloc_t(&g->hub_ev_hub, g->hub_eval_items, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_ev_slot, g->hub_eval_items, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_ev_first, nh + 1, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_part, 3 * g->hub_eval_items, s))) return rc;
+    if ((rc = dev_alloc_t(&g->hub_part, 3 * std::max(g->hub_eval_items, g->hub_items), s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_cur, nh, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_hascur, nh, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_done, nh, s))) return rc;

@@ -64,6 +64,20 @@ __device__ __forceinline__ void warp_tile_rows(const int64_t* __restrict__ off, 
     more = __all_sync(FULL, in);
   }
   for (int64_t nr = cur + 33; more; nr += 128) {  // short rows: 4 independent loads a lane
+    if (nr > cur + 33 + 512) {  // a long run of empty rows (millions in a coarse R-MAT graph): search instead
+      for (int j = 0; j < 4; ++j) {
+        int64_t lo = cur, hi = n;  // off[lo] <= e < off[hi]
+        const int64_t e = ts + 4 * lane + j;
+        while (hi - lo > 1) {
+          const int64_t mid = (lo + hi) >> 1;
+          if (off[mid] <= e) lo = mid;
+          else hi = mid;
+        }
+        row[j] = lo;
+      }
+      cur = __shfl_sync(FULL, (long long)row[3], 31);
+      return;
+    }
     int64_t o[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -95,6 +109,22 @@ __device__ __forceinline__ void warp_tile_rows(const int64_t* __restrict__ off, 
   row[3] = cur + max(before, a3);
   cur += __shfl_sync(FULL, inc, 31);
   __syncwarp();  // the marks are cleared for the next tile
+}
+
+// The rows of the arcs ts + lane + 32 j, j = 0..3 (for stores that run along
+// the lanes): warp_tile_rows, then a pass through the marks.
+__device__ __forceinline__ void warp_tile_rows_strided(const int64_t* __restrict__ off, int64_t n, int64_t ts,
+                                                       int64_t& cur, int32_t* mark, int64_t row[4]) {
+  const int lane = threadIdx.x & 31;
+  const int64_t base = cur;
+  int64_t r[4];
+  warp_tile_rows(off, n, ts, cur, mark, r);
+  *reinterpret_cast<int4*>(mark + 4 * lane) =
+      make_int4((int32_t)(r[0] - base), (int32_t)(r[1] - base), (int32_t)(r[2] - base), (int32_t)(r[3] - base));
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < 4; ++j) row[j] = base + mark[lane + 32 * j];
+  __syncwarp();
 }
 
 // emit(r, sum) once for every row r with arcs among the tile's (a row that goes

@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(NTB, GROUP == 32 ? ((LOUV || !W::unit) ? 4 : 5
 }
 
 // The warp bin (degrees 33..t_warp): a warp takes vb (a power of two <= 32)
-// listed vertices at a time. Lane j < vb loads vertex j's header; the warp
+// listed vertices at a time, by the number listed. Lane j < vb loads vertex j's header; the warp
 // then scans each active vertex in turn (table inserts and evaluation as in
 // k_scan_group) and lane j keeps vertex j's best candidate. The decisions,
 // coins and move-list appends then run in parallel, one lane per vertex, and
@@ -248,8 +248,7 @@ __global__ void __launch_bounds__(NTB, GROUP == 32 ? ((LOUV || !W::unit) ? 4 : 5
 // warp so that its warps still fill the GPU.
 template <bool LOUV, class W, class V, bool NK>
 __global__ void __launch_bounds__(256, (LOUV || !W::unit) ? 4 : 5)
-    k_scan_warp(ScanCtx s, const int32_t* __restrict__ list, const unsigned long long* __restrict__ count_p,
-                int vb) {
+    k_scan_warp(ScanCtx s, const int32_t* __restrict__ list, const unsigned long long* __restrict__ count_p) {
   typedef typename KeyOf<LOUV, NK>::T K;
   constexpr int CAP = WARP_CAP_SLOTS, WPB = 256 / 32;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -267,6 +266,12 @@ __global__ void __launch_bounds__(256, (LOUV || !W::unit) ? 4 : 5)
   const int64_t count = (int64_t)*count_p;
   const int64_t warp = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * 256) >> 5;
+  // vertices per warp and step: 32, or the largest power of two that still
+  // gives every warp a step (late rounds list few vertices: sized by the whole
+  // bin, a few warps took up to 32 of them one after another, 79 us a round on
+  // the 1M-vertex LFR-style graph)
+  int vb = 32;
+  while (vb > 1 && count < nwarps * vb) vb >>= 1;
   int64_t n_act = 0, n_arcs = 0, n_cand = 0, n_def = 0, n_marcs = 0;
   for (int64_t base = warp * vb; base < count; base += nwarps * vb) {
     const int64_t i = base + lane;
@@ -881,9 +886,111 @@ __global__ void __launch_bounds__(NT) k_hub_eval(ScanCtx s) {
 // neighbours), so G of Eq. deltaQ equals the candidate key. PER threads work
 // on a vertex (a sub-warp tile, a warp, or the whole CTA); the decision, the
 // coin and the marking of a committed move's neighbours are those of the
-// general scan. No hub histogram is built or updated here: round 0 counts as
-// a heavy round, so every hub table is built at the start of round 1.
+// general scan (hubs: k_first_hubs). No hub histogram is built or updated
+// here: round 0 counts as a heavy round, so every hub table is built at the
+// start of round 1.
 constexpr int FIRST_MARK = 100;  // profile marks of first-round launches: FIRST_MARK + bin
+
+// The best candidate among the arcs [beg, end) of v that thread gl of PER
+// takes: four columns in flight, then their Sigma_tot, instead of one after
+// another.
+template <bool LOUV, class W, bool NK, int PER>
+__device__ __forceinline__ void first_best(const ScanCtx& s, int32_t v, int64_t beg, int64_t end, int gl, int64_t dv,
+                                           int64_t volv, typename KeyOf<LOUV, NK>::T& bk, int32_t& bc,
+                                           int64_t& n_cand) {
+  typedef typename KeyOf<LOUV, NK>::T K;
+  constexpr int U = PER >= 32 ? 4 : 1;  // a tile's vertex has at most PER arcs
+  for (int64_t e0 = beg + gl; e0 < end; e0 += U * PER) {
+    int32_t u[U];
+    int64_t wt[U], sg[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const int64_t e = e0 + (int64_t)j * PER;
+      u[j] = e < end ? __ldg(s.cols + e) : v;
+      wt[j] = e < end ? W::get(s.w, e) : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) sg[j] = LOUV && u[j] != v ? (int64_t)sig_of<NK>(s, u[j]) : 0;
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      if (u[j] == v) continue;
+      const K key = cand_key_sg<LOUV, NK>(sg[j], wt[j], dv, volv);
+      ++n_cand;
+      if (better(key, u[j], bk, bc)) {
+        bk = key;
+        bc = u[j];
+      }
+    }
+  }
+}
+
+// The same for hubs: a CTA per HUB_CHUNK arcs of a hub's row (a CTA per hub
+// made the largest row a serial chain: 1.8 of 3.9 ms of the first round at
+// R-MAT 22). The last item of a hub to finish combines the items' bests and
+// decides; k_hub_mark flags the neighbours of the hubs that move.
+template <bool LOUV, class W, bool NK>
+__global__ void __launch_bounds__(NT) k_first_hubs(ScanCtx s) {
+  typedef typename KeyOf<LOUV, NK>::T K;
+  __shared__ K red_k[NW];
+  __shared__ int32_t red_c[NW];
+  __shared__ int s_last;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int64_t n_act = 0, n_arcs = 0, n_cand = 0, n_def = 0, n_marcs = 0;
+  for (int64_t it = blockIdx.x; it < s.n_items; it += gridDim.x) {
+    const int32_t h = s.hub_item_hub[it];
+    const int32_t v = s.hub_list[h];
+    if (!is_active(s, v)) continue;  // uniform within the CTA
+    const int64_t a0 = s.hub_item_arc[it], rowend = s.off[v + 1];
+    const int64_t a1 = a0 + HUB_CHUNK < rowend ? a0 + HUB_CHUNK : rowend;
+    const int64_t dv = LOUV ? s.degw[v] : 0;
+    const int64_t volv = LOUV ? vol_of(s, v) : 0;
+    K bk = no_key<K>();
+    int32_t bc = NOCAND;
+    first_best<LOUV, W, NK, NT>(s, v, a0, a1, threadIdx.x, dv, volv, bk, bc, n_cand);
+    reduce_best(bk, bc, 32);
+    if (lane == 0) {
+      red_k[wid] = bk;
+      red_c[wid] = bc;
+    }
+    __syncthreads();
+    const int64_t i0 = s.hub_item_first[h], i1 = s.hub_item_first[h + 1];
+    if (threadIdx.x == 0) {
+      for (int w2 = 1; w2 < NW; ++w2)
+        if (better(red_k[w2], red_c[w2], bk, bc)) {
+          bk = red_k[w2];
+          bc = red_c[w2];
+        }
+      const i128 kk = (i128)bk;
+      s.hub_part[3 * it] = (int64_t)(kk >> 64);
+      s.hub_part[3 * it + 1] = (int64_t)(uint64_t)kk;
+      s.hub_part[3 * it + 2] = bc;
+      __threadfence();
+      s_last = atomicAdd(&s.hub_done[h], 1) == (int)(i1 - i0 - 1);
+    }
+    __syncthreads();
+    if (s_last && wid == 0) {  // one warp over the items' bests
+      __threadfence();
+      const volatile int64_t* part = s.hub_part;
+      K fk = no_key<K>();
+      int32_t fc = NOCAND;
+      for (int64_t p = i0 + lane; p < i1; p += 32) {
+        const i128 pk = (i128)(((unsigned __int128)(uint64_t)part[3 * p] << 64) | (uint64_t)part[3 * p + 1]);
+        const int32_t pc = (int32_t)part[3 * p + 2];
+        if (better((K)pk, pc, fk, fc)) {
+          fk = (K)pk;
+          fc = pc;
+        }
+      }
+      reduce_best(fk, fc, 32);
+      if (lane == 0) {
+        hub_decide<LOUV, NK>(s, h, v, v, fk, fc, false, 0, volv, n_act, n_arcs, n_def, n_marcs);
+        s.hub_done[h] = 0;
+      }
+    }
+    __syncthreads();
+  }
+  flush_counters(s, B_HUB, n_act, n_arcs, n_cand, n_def, n_marcs);
+}
 
 template <bool LOUV, class W, bool NK, int PER>
 __global__ void __launch_bounds__(NT) k_first_round(ScanCtx s, const int32_t* __restrict__ list,
@@ -916,17 +1023,7 @@ __global__ void __launch_bounds__(NT) k_first_round(ScanCtx s, const int32_t* __
     }
     K bk = no_key<K>();
     int32_t bc = NOCAND;
-    for (int64_t e = beg + gl; e < end; e += PER) {
-      const int32_t u = s.cols[e];
-      if (u == v) continue;
-      const int64_t wt = W::get(s.w, e);
-      const K key = LOUV ? cand_key<LOUV, NK>(s, u, wt, dv, volv) : K(wt);
-      ++n_cand;
-      if (better(key, u, bk, bc)) {
-        bk = key;
-        bc = u;
-      }
-    }
+    first_best<LOUV, W, NK, PER>(s, v, beg, end, gl, dv, volv, bk, bc, n_cand);
     reduce_best(bk, bc, TW);
     if constexpr (PER == NT) {
       if (lane == 0) {
@@ -1271,16 +1368,6 @@ unsigned wave_grid(KERN kernel, int nt, size_t smem, int64_t want) {
   return grid_cap(want, resident_ctas((const void*)kernel, nt, smem));
 }
 
-// Vertices per warp batch of k_scan_warp for a bin of cnt vertices: 32, or the
-// largest power of two that still gives every resident warp a batch.
-template <class KERN>
-int warp_batch(KERN kernel, size_t smem, int64_t cnt) {
-  const int64_t warps = (int64_t)resident_ctas((const void*)kernel, 256, smem) * 8;
-  int vb = 32;
-  while (vb > 1 && cnt < warps * vb) vb >>= 1;
-  return vb;
-}
-
 // Group-kernel configurations: (GROUP threads per vertex, CTA size, table slots).
 template <class V> constexpr size_t group_smem(int gpb, int cap) { return (size_t)gpb * cap * (sizeof(V) + 4 + 2); }
 template <class V> constexpr size_t warp_smem() { return group_smem<V>(8, WARP_CAP_SLOTS); }
@@ -1397,7 +1484,7 @@ int launch_first_round(cd_graph* g, ScanCtx& s, std::vector<std::pair<size_t, in
         case B_T4: CD_LAUNCH((k_first_round<LOUV, W, NK, 4><<<grid_cap((c + 63) / 64), NT, 0, st>>>(s, lst(b), dcnt(b), b))); break;
         case B_T8: CD_LAUNCH((k_first_round<LOUV, W, NK, 8><<<grid_cap((c + 31) / 32), NT, 0, st>>>(s, lst(b), dcnt(b), b))); break;
         case B_T16: CD_LAUNCH((k_first_round<LOUV, W, NK, 16><<<grid_cap((c + 15) / 16), NT, 0, st>>>(s, lst(b), dcnt(b), b))); break;
-        case B_HUB:
+        case B_HUB: CD_LAUNCH((k_first_hubs<LOUV, W, NK><<<grid_cap(g->hub_items, 152 * 8), NT, 0, st>>>(s))); break;
         case B_BLK4: CD_LAUNCH((k_first_round<LOUV, W, NK, NT><<<grid_cap(c), NT, 0, st>>>(s, lst(b), dcnt(b), b))); break;
         default: CD_LAUNCH((k_first_round<LOUV, W, NK, 32><<<grid_cap((c + NW - 1) / NW), NT, 0, st>>>(s, lst(b), dcnt(b), b))); break;
       }
@@ -1485,9 +1572,8 @@ int launch_round(cd_graph* g, ScanCtx& s, const int32_t* lists, const unsigned l
     {
       KTimer t(g, K_SCAN_WARP, 0.0, bs.s[3]);
       auto kern = k_scan_warp<LOUV, W, V, NK>;
-      const int vb = warp_batch(kern, warp_smem<V>(), cnt(B_WARP));
-      CD_LAUNCH((kern<<<wave_grid(kern, 256, warp_smem<V>(), (cnt(B_WARP) + 8 * vb - 1) / (8 * vb)), 256,
-                        warp_smem<V>(), bs.s[3]>>>(s, lst(B_WARP), dcnt(B_WARP), vb)));
+      CD_LAUNCH((kern<<<wave_grid(kern, 256, warp_smem<V>(), (cnt(B_WARP) + 7) / 8), 256,
+                        warp_smem<V>(), bs.s[3]>>>(s, lst(B_WARP), dcnt(B_WARP))));
     }
     if (g->ktiming) mark(B_WARP);
   }
