@@ -81,6 +81,34 @@ enum Kern {
 };
 extern const char* const kKernelNames[K_COUNT];
 
+// Hubs of the resident round loop (rounds.cu): at most RH_MAX_HUBS of them, on
+// graphs of at most RH_MAX_ARCS arcs. A hub that is examined has its label
+// histogram built in that round by items of RH_CHUNK arcs and read (and cleared)
+// by slices of RH_SLICE slots.
+constexpr int RH_CHUNK = 1024;
+constexpr int RH_SLICE = 2048;
+constexpr int64_t RH_MAX_HUBS = 4095;  // one CTA lays them out, with one entry more
+constexpr int64_t RH_MAX_ARCS = (int64_t)1 << 24;
+struct ResidentHubs {
+  int32_t nh = 0;
+  int32_t* v = nullptr;           // nh: vertex of each hub
+  int32_t* item = nullptr;        // nh+1: first item of each hub
+  int32_t* slice = nullptr;       // nh+1: first slice
+  int64_t* tab = nullptr;         // nh+1: first slot
+  int32_t* item_hub = nullptr;    // per item: hub
+  int32_t* slice_hub = nullptr;   // per slice: hub
+  unsigned long long* slot = nullptr;  // packed (label << 32 | count), or the counts when a deg_w reaches 2^32
+  int32_t* key = nullptr;         // the labels then (null: packed)
+  int64_t* part = nullptr;        // 3 per slice: best key (high, low) and community
+  int32_t* done = nullptr;        // nh: slices read this round
+  int32_t* has = nullptr;         // nh: the hub's own label was met
+  int64_t* cur = nullptr;         // nh: its weight
+  int32_t* moved = nullptr;       // nh: 1 + the round of its last move in this run
+  int32_t* to = nullptr;          // nh: that move
+  int32_t* from = nullptr;
+  void* mem[2] = {nullptr, nullptr};  // the two allocations
+};
+
 }  // namespace cd
 
 // The opaque handle.
@@ -93,7 +121,8 @@ struct cd_graph {
   int wkind = cd::W_UNIT;
   int64_t* degw = nullptr;  // n
 
-  // static degree bins
+  // static degree bins: counted when the graph is made; the lists and hub structures of the per-round kernels are
+  // made when those first run (ensure_bins)
   int32_t* bin_list = nullptr;           // n vertex ids grouped by bin
   int64_t bin_start[cd::NBINS + 1] = {};  // host copy of the bin offsets
   // frontier: the active vertices of a round, bin b at act_list + bin_start[b]
@@ -110,6 +139,8 @@ struct cd_graph {
   // is one word (label << 32 | count) when every deg_w < 2^32 ("packed"),
   // otherwise two words (label, count).
   int64_t nhubs = 0, hub_slots = 0, hub_items = 0, hub_eval_items = 0;
+  int64_t hub_arcs = 0;                    // arcs of the hubs
+  cd::ResidentHubs* rh = nullptr;          // the resident loop's hub tables (made when it first runs)
   int hub_wide = 0;                        // 1: two-word slots
   uint32_t* hub_pref = nullptr;        // per 32-vertex word: hubs with smaller vertex ids (hub number = rank)
   uint32_t* hub_bits = nullptr;            // (n+31)/32: bit v set iff v is a hub
@@ -219,6 +250,8 @@ int graph_adopt(cudaStream_t s, int64_t n, int64_t nnz, int64_t* off, int32_t* c
                 int wkind, cd_graph** out, int64_t* degw_pre = nullptr,
                 const unsigned long long* stats_pre = nullptr, const cd_graph* like = nullptr);
 int ensure_run_state(cd_graph* g);
+int ensure_bins(cd_graph* g);  // bin lists and hub structures of the per-round kernels
+int ensure_resident_hubs(cd_graph* g);
 // Recompute the degree bins and hub structures for new boundaries.
 int rebin(cd_graph* g, int t_warp, int t_hub);
 int check_labels(cd_graph* g, const int32_t* labels_dev);  // CD_EINVAL if out of [0, n)

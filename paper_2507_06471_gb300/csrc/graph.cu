@@ -119,18 +119,85 @@ __device__ __forceinline__ int bin_of(int64_t d, int t_warp = WARP_MAX, int t_hu
   return d <= BLK1_MAX ? B_BLK1 : B_BLK4;
 }
 
+// counts[NBINS]: arcs of the hubs.
 __global__ void k_bin_count(const int64_t* __restrict__ off, int64_t n, int t_warp, int t_hub,
                             unsigned long long* counts) {
-  __shared__ unsigned long long sb[NBINS];
-  if (threadIdx.x < NBINS) sb[threadIdx.x] = 0;
+  __shared__ unsigned long long sb[NBINS + 1];
+  if (threadIdx.x <= NBINS) sb[threadIdx.x] = 0;
   __syncthreads();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
     const int64_t d = off[v + 1] - off[v];
     if (d > 0) atomicAdd(&sb[bin_of(d, t_warp, t_hub)], 1ull);
+    if (d > t_hub) atomicAdd(&sb[NBINS], (unsigned long long)d);
   }
   __syncthreads();
-  if (threadIdx.x < NBINS && sb[threadIdx.x]) atomicAdd(&counts[threadIdx.x], sb[threadIdx.x]);
+  if (threadIdx.x <= NBINS && sb[threadIdx.x]) atomicAdd(&counts[threadIdx.x], sb[threadIdx.x]);
+}
+
+// The resident loop's hubs, in any order.
+__global__ void k_rh_collect(const int64_t* __restrict__ off, int64_t n, int t_hub, int32_t* __restrict__ v_out,
+                             int32_t* count) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride)
+    if (off[v + 1] - off[v] > t_hub) v_out[atomicAdd(count, 1)] = (int32_t)v;
+}
+
+// Items, slices and tables of nh <= RH_MAX_HUBS hubs: one CTA, four hubs a thread.
+__global__ void __launch_bounds__(1024) k_rh_layout(const int64_t* __restrict__ off, ResidentHubs r) {
+  __shared__ long long wsum[32][3];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  long long x[4][3], mine[3] = {0, 0, 0};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int h = threadIdx.x * 4 + q;
+    const int64_t d = h < r.nh ? off[r.v[h] + 1] - off[r.v[h]] : 0;
+    const int64_t cap = h < r.nh ? d + d / 2 + 64 : 0;  // at most two thirds full
+    x[q][0] = (d + RH_CHUNK - 1) / RH_CHUNK;
+    x[q][1] = (cap + RH_SLICE - 1) / RH_SLICE;
+    x[q][2] = cap;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) mine[c] += x[q][c];
+  }
+  long long inc[3] = {mine[0], mine[1], mine[2]};
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long y = __shfl_up_sync(FULL, inc[c], o);
+      if (lane >= o) inc[c] += y;
+    }
+  if (lane == 31)
+    for (int c = 0; c < 3; ++c) wsum[wid][c] = inc[c];
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int c = 0; c < 3; ++c) {
+      long long run = 0;
+      for (int w = 0; w < 32; ++w) {
+        const long long y = wsum[w][c];
+        wsum[w][c] = run;
+        run += y;
+      }
+    }
+  __syncthreads();
+  long long at[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) at[c] = wsum[wid][c] + inc[c] - mine[c];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int h = threadIdx.x * 4 + q;
+    if (h <= r.nh) {  // entry nh: the totals
+      r.item[h] = (int32_t)at[0];
+      r.slice[h] = (int32_t)at[1];
+      r.tab[h] = at[2];
+    }
+    if (h < r.nh) {
+      for (int i = 0; i < (int)x[q][0]; ++i) r.item_hub[at[0] + i] = h;
+      for (int i = 0; i < (int)x[q][1]; ++i) r.slice_hub[at[1] + i] = h;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) at[c] += x[q][c];
+  }
 }
 
 template <class OffT>
@@ -423,8 +490,11 @@ int read_status(cd_graph* g) {
   return st;
 }
 
+void free_resident_hubs(cd_graph* g);
+
 void free_arrays(cd_graph* g) {
   cudaStream_t s = g->stream;
+  free_resident_hubs(g);
   void* ps[] = {g->off,          g->cols,          g->w,            g->degw,         g->bin_list,
                 g->act_list,     g->act_cnt,       g->full_cnt,     g->act_ev,       g->act_small,
                 g->hub_cc,       g->hub_live,
@@ -443,8 +513,17 @@ void free_arrays(cd_graph* g) {
   if (g->h_ctr) cudaFreeHost(g->h_ctr);
 }
 
+void free_resident_hubs(cd_graph* g) {
+  if (!g->rh) return;
+  dev_free(g->rh->mem[0], g->stream);
+  dev_free(g->rh->mem[1], g->stream);
+  delete g->rh;
+  g->rh = nullptr;
+}
+
 void free_bins(cd_graph* g) {
   cudaStream_t s = g->stream;
+  free_resident_hubs(g);
   void* ps[] = {g->bin_list,     g->act_list,    g->act_cnt,      g->full_cnt,  g->act_ev,
                 g->act_small,    g->hub_cc,       g->hub_live,
                 g->hub_pref,      g->hub_bits,     g->hub_tab,   g->hub_slot,
@@ -488,7 +567,7 @@ void free_bins(cd_graph* g) {
   g->hub_lcnt = nullptr;
   g->hub_log = nullptr;
   g->hub_log_cap = 0;
-  g->nhubs = g->hub_slots = g->hub_items = g->hub_eval_items = 0;
+  g->nhubs = g->hub_arcs = g->hub_slots = g->hub_items = g->hub_eval_items = 0;
 }
 
 int build_bins(cd_graph* g);
@@ -504,23 +583,30 @@ int finish_graph(cd_graph* g, const unsigned long long* stats) {
   return build_bins(g);
 }
 
-// Degree bins for (t_warp, t_hub), and the hub histograms' layout.
+// Vertices per degree bin for (t_warp, t_hub).
 int build_bins(cd_graph* g) {
   cudaStream_t s = g->stream;
   int rc;
-  {
-    unsigned long long* d_cnt = nullptr;
-    unsigned long long h_cnt[NBINS] = {};
-    if ((rc = dev_alloc_t(&d_cnt, NBINS, s))) return rc;
-    CD_CHECK(cudaMemsetAsync(d_cnt, 0, NBINS * sizeof(unsigned long long), s));
-    if (g->n > 0)
-      CD_LAUNCH(k_bin_count<<<grid_for(g->n), NT, 0, s>>>(g->off, g->n, g->t_warp, g->t_hub, d_cnt));
-    CD_CHECK(cudaMemcpyAsync(h_cnt, d_cnt, sizeof(h_cnt), cudaMemcpyDeviceToHost, s));
-    CD_CHECK(cudaStreamSynchronize(s));
-    dev_free(d_cnt, s);
-    g->bin_start[0] = 0;
-    for (int b = 0; b < NBINS; ++b) g->bin_start[b + 1] = g->bin_start[b] + (int64_t)h_cnt[b];
-  }
+  unsigned long long* d_cnt = nullptr;
+  unsigned long long h_cnt[NBINS + 1] = {};
+  if ((rc = dev_alloc_t(&d_cnt, NBINS + 1, s))) return rc;
+  CD_CHECK(cudaMemsetAsync(d_cnt, 0, sizeof(h_cnt), s));
+  if (g->n > 0)
+    CD_LAUNCH(k_bin_count<<<grid_for(g->n), NT, 0, s>>>(g->off, g->n, g->t_warp, g->t_hub, d_cnt));
+  CD_CHECK(cudaMemcpyAsync(h_cnt, d_cnt, sizeof(h_cnt), cudaMemcpyDeviceToHost, s));
+  CD_CHECK(cudaStreamSynchronize(s));
+  dev_free(d_cnt, s);
+  g->bin_start[0] = 0;
+  for (int b = 0; b < NBINS; ++b) g->bin_start[b + 1] = g->bin_start[b] + (int64_t)h_cnt[b];
+  g->nhubs = (int64_t)h_cnt[B_HUB];
+  g->hub_arcs = (int64_t)h_cnt[NBINS];
+  return CD_OK;
+}
+
+// The bin lists, and the hub histograms' layout.
+int fill_bins(cd_graph* g) {
+  cudaStream_t s = g->stream;
+  int rc;
   int64_t listed = g->bin_start[NBINS];
   rc = dev_alloc_t(&g->bin_list, listed, s);
   if (rc) return rc;
@@ -538,8 +624,7 @@ int build_bins(cd_graph* g) {
                                                        g->bin_list));
   CD_CHECK(cudaGetLastError());
   // hubs: host-side layout of tables and work items
-  int64_t nh = g->bin_start[B_HUB + 1] - g->bin_start[B_HUB];
-  g->nhubs = nh;
+  const int64_t nh = g->nhubs;
   if (nh > 0) {
     {  // hubs in increasing vertex id (their number is their rank)
       std::vector<int32_t> hv(nh);
@@ -705,12 +790,76 @@ int ingest(cd_graph* g, int loops_twice, unsigned long long* stats_host) {
 int rebin(cd_graph* g, int t_warp, int t_hub) {
   if (t_warp < 32 || t_warp > WARP_MAX || t_hub < t_warp || t_hub > BLK4_MAX) return CD_EINVAL;
   g->bins_set = true;
-  if (t_warp == g->t_warp && t_hub == g->t_hub && g->bin_list) return CD_OK;
+  if (t_warp == g->t_warp && t_hub == g->t_hub) return CD_OK;
   CD_CHECK(cudaStreamSynchronize(g->stream));
   free_bins(g);
   g->t_warp = t_warp;
   g->t_hub = t_hub;
   return build_bins(g);
+}
+
+int ensure_bins(cd_graph* g) {
+  if (g->bin_list) return CD_OK;
+  const int rc = fill_bins(g);
+  if (rc) {  // nothing half made stays; the counts do
+    const int64_t nh = g->nhubs, ha = g->hub_arcs;
+    free_bins(g);
+    g->nhubs = nh;
+    g->hub_arcs = ha;
+  }
+  return rc;
+}
+
+int ensure_resident_hubs(cd_graph* g) {
+  if (g->rh) return CD_OK;
+  cudaStream_t s = g->stream;
+  const int64_t nh = g->nhubs, items = g->hub_arcs / RH_CHUNK + nh;
+  const int64_t slots = g->hub_arcs + g->hub_arcs / 2 + 64 * nh, slices = slots / RH_SLICE + nh;
+  const bool wide = g->max_degw >= ((int64_t)1 << 32);
+  ResidentHubs r;
+  r.nh = (int32_t)nh;
+  int rc;
+  // 8-byte arrays first
+  const size_t b8 = (size_t)((nh + 1) + 3 * slices + nh) * 8;
+  const size_t b4 = (size_t)(nh + 2 * (nh + 1) + items + slices + 5 * nh + 1) * 4;
+  if ((rc = dev_alloc(&r.mem[0], b8 + b4, s))) return rc;
+  if ((rc = dev_alloc(&r.mem[1], (size_t)slots * (wide ? 12 : 8), s))) {
+    dev_free(r.mem[0], s);
+    return rc;
+  }
+  r.tab = (int64_t*)r.mem[0];
+  r.part = r.tab + nh + 1;
+  r.cur = r.part + 3 * slices;
+  r.v = (int32_t*)(r.cur + nh);
+  r.item = r.v + nh;
+  r.slice = r.item + nh + 1;
+  r.item_hub = r.slice + nh + 1;
+  r.slice_hub = r.item_hub + items;
+  r.done = r.slice_hub + slices;
+  r.has = r.done + nh;
+  r.moved = r.has + nh;
+  r.to = r.moved + nh;
+  r.from = r.to + nh;
+  int32_t* count = r.from + nh;
+  r.slot = (unsigned long long*)r.mem[1];
+  r.key = wide ? (int32_t*)(r.slot + slots) : nullptr;
+  auto run = [&]() -> int {
+    CD_CHECK(cudaMemsetAsync(r.done, 0, (size_t)(2 * nh) * 4, s));  // done, has
+    CD_CHECK(cudaMemsetAsync(count, 0, 4, s));
+    CD_CHECK(cudaMemsetAsync(r.slot, wide ? 0 : 0xff, (size_t)slots * 8, s));
+    if (wide) CD_CHECK(cudaMemsetAsync(r.key, 0xff, (size_t)slots * 4, s));
+    CD_LAUNCH(k_rh_collect<<<grid_for(g->n), NT, 0, s>>>(g->off, g->n, g->t_hub, r.v, count));
+    CD_LAUNCH(k_rh_layout<<<1, 1024, 0, s>>>(g->off, r));
+    CD_CHECK(cudaGetLastError());
+    return CD_OK;
+  };
+  if ((rc = run())) {
+    dev_free(r.mem[0], s);
+    dev_free(r.mem[1], s);
+    return rc;
+  }
+  g->rh = new ResidentHubs(r);
+  return CD_OK;
 }
 
 int ensure_run_state(cd_graph* g) {

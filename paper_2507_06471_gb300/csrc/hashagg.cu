@@ -1,25 +1,38 @@
-// Louvain aggregation by hashing (Algorithm 3, Aggregation): the coarse
-// graph without a global sort of the arcs.
+// Louvain aggregation by hashing (Algorithm 3, Aggregation): the coarse graph
+// without a sort.
 //
-// 1. The n vertices are sorted by A = new(C[v]) (radix sort of n keys, not of
-//    m arcs), which lists every community's members together.
-// 2. An exclusive scan of the member degrees gives each community a contiguous
-//    segment of the arc space; every arc u->x of a member u writes
-//    (B = new(C[x]), w) into its community's segment (no atomics).
-// 3. Each segment is combined by hashing B: one warp for a segment of at most
-//    AG_WARP_MAX arcs, one CTA for at most AG_CTA_MAX, each with a
-//    shared-memory table; a larger segment is cut into AG_CHUNK-arc chunks,
-//    each combined in shared memory, whose distinct entries are then merged in
-//    a global table sized for the segment. The distinct (B, sum w) of a
-//    segment are written back at its start.
+// 1. A pass over the vertices notes each one's coarse vertex A = new(C[v]) and
+//    sums the arcs and deg_w of every A; a scan of the arc sums gives each
+//    community a contiguous segment of the arc space, and a second pass gives
+//    every member its place in the segment (any order: nothing depends on it).
+// 2. Every arc u->x of a member u writes (new(C[x]), w) into its place. The arcs
+//    are split evenly over the warps and taken in the graph's own order, so the
+//    columns are read and the segments written in runs (rowwalk.cuh).
+// 3. Each segment is combined by its keys: up to 8 or 32 arcs by as many lanes
+//    (a match, no table), up to 256 by a warp and up to AG_CTA_MAX by a CTA with
+//    a shared-memory table; a larger segment is cut into AG_CHUNK-arc chunks,
+//    each combined in shared memory, whose distinct entries are then merged in a
+//    global table sized for the segment. The distinct (B, sum w) of a segment
+//    are written back at its start.
 // 4. The segments are compacted into the coarse CSR (k rows, columns in no
-//    particular order, int64 weights; (A, A) collects every arc inside A,
-//    i.e. twice its internal weight, the internal convention for loops).
+//    particular order; (A, A) collects every arc inside A, i.e. twice its
+//    internal weight, the internal convention for loops).
+//
+// When vol(V) < 2^31 every weight and sum fits in 32 bits: the segments, the
+// tables (one 64-bit word a slot, one atomic a merge) and the coarse weights are
+// 32-bit then, 64-bit otherwise.
+//
+// Measured, R-MAT 22 weighted (1.3e8 arcs, 4.2e6 -> 2.7e6 vertices): a radix sort
+// of the vertices, a warp per member row and per community, 12 bytes an arc and
+// an ingest of the coarse arcs took 16.3 ms; this takes 5.3.
+//
 // The content of every row equals that of the sort-based aggregation; only the
 // order of columns inside a row differs, and no later step depends on it.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
+#include "rowwalk.cuh"
 
 namespace cd {
 namespace {
@@ -34,6 +47,10 @@ constexpr int AG_CCAP = 2 * AG_CTA_MAX;
 constexpr int AG_SLICE = 1024;     // global-table slots per extraction item (tables are multiples)
 constexpr int AG_CNT = 512;        // threads of the CTA-per-segment kernel
 constexpr int32_t AG_EMPTY = -1;
+constexpr unsigned long long AG_EMPTY_SLOT = ~0ull;
+
+// Counts on the device: segments per class, chunks, slots of the global tables.
+enum { AC_T8 = 0, AC_T32, AC_WARP, AC_CTA, AC_BIG, AC_CHUNKS, AC_SLOTS, AC_N };
 
 unsigned gcap(int64_t blocks, int64_t cap = 152 * 16) {
   if (blocks < 1) blocks = 1;
@@ -41,159 +58,264 @@ unsigned gcap(int64_t blocks, int64_t cap = 152 * 16) {
 }
 
 __device__ __forceinline__ unsigned lg_for(int64_t x) {  // smallest lg >= 1 with 2^lg >= x
-  unsigned lg = 1;
-  while (((int64_t)1 << lg) < x) ++lg;
-  return lg;
+  return x <= 2 ? 1 : 64 - __clzll((unsigned long long)(x - 1));
 }
 
 // ------------------------------------------------------------------ steps 1-2
 
-__global__ void k_ag_vkeys(const int32_t* __restrict__ labels, const int32_t* __restrict__ newid, int64_t n,
-                           uint64_t* __restrict__ key, int64_t* __restrict__ val) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-    key[v] = (uint64_t)newid[labels[v]];
-    val[v] = v;
+__global__ void __launch_bounds__(NT) k_ag_vertex(const int32_t* __restrict__ labels, const int32_t* __restrict__ newid,
+                                                  const int64_t* __restrict__ off, const int64_t* __restrict__ degw,
+                                                  int64_t n, int32_t* __restrict__ nl, unsigned long long* arcs,
+                                                  unsigned long long* cdegw) {
+  __shared__ CtaSums sa, sd;
+  sa.clear();
+  sd.clear();
+  __syncthreads();
+  const int64_t stride = (int64_t)gridDim.x * NT;
+  for (int64_t v = (int64_t)blockIdx.x * NT + threadIdx.x; v < n; v += stride) {
+    const int32_t a = newid[labels[v]];
+    const int64_t d = off[v + 1] - off[v];
+    nl[v] = a;
+    if (d > 0) {
+      sa.add(arcs, a, (unsigned long long)d);
+      sd.add(cdegw, a, (unsigned long long)degw[v]);
+    }
+  }
+  __syncthreads();
+  sa.flush(arcs);
+  sd.flush(cdegw);
+}
+
+// delta[v] = (place of v's first arc in the segments) - off[v]. The members of
+// one community that meet in a CTA take their places from one global atomic.
+constexpr int AP_VERTS = 8 * NT;  // vertices per step of a CTA
+__global__ void __launch_bounds__(NT) k_ag_place(const int32_t* __restrict__ nl, const int64_t* __restrict__ off,
+                                                 int64_t n, const int64_t* __restrict__ sstart,
+                                                 unsigned long long* taken, int64_t* __restrict__ delta) {
+  constexpr int SLOTS = 1024;
+  __shared__ unsigned long long tot[SLOTS];
+  __shared__ int32_t key[SLOTS];
+  for (int64_t v0 = (int64_t)blockIdx.x * AP_VERTS; v0 < n; v0 += (int64_t)gridDim.x * AP_VERTS) {
+    for (int i = threadIdx.x; i < SLOTS; i += NT) {
+      key[i] = AG_EMPTY;
+      tot[i] = 0;
+    }
+    __syncthreads();
+    int32_t a[8];
+    int16_t slot[8];
+    unsigned long long at[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int64_t v = v0 + q * NT + threadIdx.x;
+      a[q] = v < n ? nl[v] : -1;
+      at[q] = v < n ? (unsigned long long)(off[v + 1] - off[v]) : 0;
+      if (at[q] == 0) a[q] = -1;  // an isolated vertex has no place
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      slot[q] = -1;
+      if (a[q] < 0) continue;
+      unsigned h = ((uint32_t)a[q] * 2654435761u) >> 22;
+      for (int probe = 0; probe < 4; ++probe) {
+        int32_t c = *(volatile int32_t*)&key[h];
+        if (c == AG_EMPTY) c = atomicCAS(&key[h], AG_EMPTY, a[q]);
+        if (c == AG_EMPTY || c == a[q]) {
+          slot[q] = (int16_t)h;
+          break;
+        }
+        h = (h + 1) & (SLOTS - 1);
+      }
+      if (slot[q] >= 0) at[q] = atomicAdd(&tot[slot[q]], at[q]);
+      else at[q] = atomicAdd(&taken[a[q]], at[q]);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < SLOTS; i += NT)
+      if (key[i] != AG_EMPTY) tot[i] = atomicAdd(&taken[key[i]], tot[i]);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int64_t v = v0 + q * NT + threadIdx.x;
+      if (a[q] < 0) continue;
+      delta[v] = sstart[a[q]] + (int64_t)(at[q] + (slot[q] >= 0 ? tot[slot[q]] : 0)) - off[v];
+    }
+    __syncthreads();
   }
 }
 
-__global__ void k_ag_mdeg(const int64_t* __restrict__ off, const int64_t* __restrict__ mem, int64_t n,
-                          int64_t* __restrict__ md) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    const int64_t v = mem[i];
-    md[i] = off[v + 1] - off[v];
-  }
-}
-
-// sstart[A] = arc-space start of community A (its first member's prefix).
-__global__ void k_ag_heads(const uint64_t* __restrict__ skey, const int64_t* __restrict__ mpre, int64_t n,
-                           int64_t* __restrict__ sstart) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-    if (i == 0 || skey[i] != skey[i - 1]) sstart[skey[i]] = mpre[i];
-}
-
-// Warp per member: the member's arcs into its community's segment.
-template <class W>
+// The arcs into their segments.
+template <class W, class V>
 __global__ void __launch_bounds__(NT) k_ag_scatter(const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
-                                                   const void* w, const int32_t* __restrict__ labels,
-                                                   const int32_t* __restrict__ newid, const int64_t* __restrict__ mem,
-                                                   const int64_t* __restrict__ mpre, int64_t n,
-                                                   int32_t* __restrict__ ab, unsigned long long* __restrict__ aw) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * NT) >> 5;
-  for (int64_t i = warp; i < n; i += nwarps) {
-    const int64_t v = mem[i], base = mpre[i];
-    const int64_t beg = off[v], d = off[v + 1] - beg;
-    for (int64_t j = lane; j < d; j += 32) {
-      ab[base + j] = newid[labels[cols[beg + j]]];
-      aw[base + j] = (unsigned long long)W::get(w, beg + j);
+                                                   const void* w, int64_t n, int64_t m, int64_t piece,
+                                                   const int32_t* __restrict__ nl, const int64_t* __restrict__ delta,
+                                                   int32_t* __restrict__ ab, V* __restrict__ aw) {
+  __shared__ __align__(16) int32_t mark[NW][WALK_TILE];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t step = (((int64_t)gridDim.x * NT) >> 5) * piece;
+  for (int64_t e0 = (((int64_t)blockIdx.x * NT + threadIdx.x) >> 5) * piece; e0 < m; e0 += step) {  // uniform in the warp
+    const int64_t e1 = e0 + piece < m ? e0 + piece : m;
+    int64_t cur = warp_row_of(off, n, e0);
+    for (int64_t ts = e0; ts < e1; ts += WALK_TILE) {
+      int32_t b[4];
+      V x[4];
+      int64_t row[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int64_t e = ts + lane + 32 * j;
+        b[j] = e < e1 ? __ldg(cols + e) : -1;
+        x[j] = e < e1 ? (V)W::get(w, e) : 0;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) b[j] = b[j] >= 0 ? nl[b[j]] : -1;
+      warp_tile_rows_strided(off, n, ts, cur, mark[wid], row);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int64_t e = ts + lane + 32 * j;
+        if (e >= e1) continue;
+        const int64_t p = delta[row[j]] + e;
+        ab[p] = b[j];
+        aw[p] = x[j];
+      }
     }
   }
 }
 
 // ------------------------------------------------------------------ classes
 
-// cnt: [0] warp segments, [1] CTA segments, [2] large segments, [3] chunks.
-__global__ void k_ag_class_count(const int64_t* __restrict__ sstart, int64_t k, unsigned long long* cnt) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  unsigned long long c[4] = {0, 0, 0, 0};
-  for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < k; a += stride) {
-    const int64_t len = sstart[a + 1] - sstart[a];
-    if (len <= AG_WARP_MAX) {
-      ++c[0];
-    } else if (len <= AG_CTA_MAX) {
-      ++c[1];
-    } else {
-      ++c[2];
-      c[3] += (unsigned long long)((len + AG_CHUNK - 1) / AG_CHUNK);
-    }
-  }
-  for (int j = 0; j < 4; ++j)
-    if (c[j]) atomicAdd(&cnt[j], c[j]);
-}
-
-__global__ void k_ag_class_fill(const int64_t* __restrict__ sstart, int64_t k, unsigned long long* cur,
-                                int32_t* __restrict__ wl, int32_t* __restrict__ cl, int32_t* __restrict__ ll,
-                                int32_t* __restrict__ ch_seg, int64_t* __restrict__ ch_off) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < k; a += stride) {
-    const int64_t len = sstart[a + 1] - sstart[a];
-    if (len <= AG_WARP_MAX) {
-      wl[atomicAdd(&cur[0], 1ull)] = (int32_t)a;
-    } else if (len <= AG_CTA_MAX) {
-      cl[atomicAdd(&cur[1], 1ull)] = (int32_t)a;
-    } else {
-      ll[atomicAdd(&cur[2], 1ull)] = (int32_t)a;
-      const int64_t nc = (len + AG_CHUNK - 1) / AG_CHUNK;
-      const unsigned long long p = atomicAdd(&cur[3], (unsigned long long)nc);
-      for (int64_t j = 0; j < nc; ++j) {
-        ch_seg[p + j] = (int32_t)a;
-        ch_off[p + j] = j * AG_CHUNK;
+// The segments into their classes' lists; a CTA appends to each list once per step.
+constexpr int AF_SEGS = 8 * NT;
+__global__ void __launch_bounds__(NT) k_ag_classes(const int64_t* __restrict__ sstart, int64_t k,
+                                                   unsigned long long* cnt, int32_t* __restrict__ t8,
+                                                   int32_t* __restrict__ t32, int32_t* __restrict__ wl,
+                                                   int32_t* __restrict__ cl, int32_t* __restrict__ ll,
+                                                   int32_t* __restrict__ ch_seg, int64_t* __restrict__ ch_off) {
+  __shared__ int n_of[8];
+  __shared__ unsigned long long base[8];
+  const int lane = threadIdx.x & 31;
+  for (int64_t a0 = (int64_t)blockIdx.x * AF_SEGS; a0 < k; a0 += (int64_t)gridDim.x * AF_SEGS) {
+    if (threadIdx.x < 8) n_of[threadIdx.x] = 0;
+    __syncthreads();
+    int8_t cls[8];
+    int16_t rank[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int64_t a = a0 + q * NT + threadIdx.x;
+      const int64_t len = a < k ? sstart[a + 1] - sstart[a] : 0;
+      cls[q] = len == 0 ? -1 : len <= 8 ? AC_T8 : len <= 32 ? AC_T32 : len <= AG_WARP_MAX ? AC_WARP
+             : len <= AG_CTA_MAX ? AC_CTA : AC_BIG;
+      rank[q] = 0;
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        const unsigned m = __ballot_sync(FULL, cls[q] == c);
+        if (!m) continue;
+        int p = 0;
+        if (lane == 0) p = atomicAdd(&n_of[c], __popc(m));
+        p = __shfl_sync(FULL, p, 0);
+        if (cls[q] == c) rank[q] = (int16_t)(p + __popc(m & ((1u << lane) - 1u)));
+      }
+      if (cls[q] == AC_BIG) {
+        const int64_t nc = (len + AG_CHUNK - 1) / AG_CHUNK;
+        const unsigned long long p = atomicAdd(&cnt[AC_CHUNKS], (unsigned long long)nc);
+        for (int64_t j = 0; j < nc; ++j) {
+          ch_seg[p + j] = (int32_t)a;
+          ch_off[p + j] = j * AG_CHUNK;
+        }
       }
     }
+    __syncthreads();
+    if (threadIdx.x < 5 && n_of[threadIdx.x]) base[threadIdx.x] = atomicAdd(&cnt[threadIdx.x], (unsigned long long)n_of[threadIdx.x]);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      if (cls[q] < 0) continue;
+      int32_t* list = cls[q] == AC_T8 ? t8 : cls[q] == AC_T32 ? t32 : cls[q] == AC_WARP ? wl : cls[q] == AC_CTA ? cl : ll;
+      list[base[cls[q]] + rank[q]] = (int32_t)(a0 + q * NT + threadIdx.x);
+    }
+    __syncthreads();
   }
 }
 
 // ------------------------------------------------------------------ shared-memory combining
 
 // Open addressing in a 2^lg-slot table holding at most half that many keys,
-// so a free slot is always found; a claimed slot joins the occupied list.
-__device__ __forceinline__ void tab_insert(int32_t* keys, unsigned long long* vals, uint16_t* occ, int* occ_n,
-                                           unsigned lg, int32_t key, unsigned long long w) {
+// so a free slot is always found. A probe is a load; only an empty slot is
+// claimed with a compare-and-swap, and joins the occupied list.
+template <class V>
+__device__ __forceinline__ void tab_insert(int32_t* keys, V* vals, uint16_t* occ, int* occ_n,
+                                           unsigned lg, int32_t key, V w) {
   const unsigned mask = (1u << lg) - 1u;
   unsigned h = ((uint32_t)key * 2654435761u) >> (32 - lg);
   for (unsigned probe = 0; probe <= mask; ++probe) {
-    const int32_t prev = atomicCAS(&keys[h], AG_EMPTY, key);
-    if (prev == AG_EMPTY || prev == key) {
+    int32_t c = *(volatile int32_t*)&keys[h];
+    if (c == AG_EMPTY) {
+      c = atomicCAS(&keys[h], AG_EMPTY, key);
+      if (c == AG_EMPTY) {
+        occ[atomicAdd(occ_n, 1)] = (uint16_t)h;
+        c = key;
+      }
+    }
+    if (c == key) {
       atomicAdd(&vals[h], w);
-      if (prev == AG_EMPTY) occ[atomicAdd(occ_n, 1)] = (uint16_t)h;
       return;
     }
     h = (h + 1) & mask;
   }
 }
 
-// A warp inserts `len` entries starting at p: equal keys of one load are
-// combined first (match), so a key repeated across the warp costs one atomic.
-__device__ __forceinline__ void warp_insert(const int32_t* __restrict__ ab, const unsigned long long* __restrict__ aw,
-                                            int64_t p, int64_t len, int32_t* keys, unsigned long long* vals,
-                                            uint16_t* occ, int* occ_n, unsigned lg, unsigned long long* stage,
-                                            int lane) {
-  for (int64_t j = lane; j - lane < len; j += 32) {  // the whole warp iterates together
-    const bool ok = j < len;
-    const int32_t key = ok ? ab[p + j] : (int32_t)(0x80000000u | (unsigned)lane);
-    const unsigned long long wt = ok ? aw[p + j] : 0ull;
-    const unsigned peers = __match_any_sync(FULL, key);
-    stage[lane] = wt;
-    __syncwarp();
-    if (ok && (__ffs(peers) - 1) == lane) {
-      unsigned long long sum = 0;
-      unsigned m = peers;
-      while (m) {
-        sum += stage[__ffs(m) - 1];
-        m &= m - 1;
-      }
-      tab_insert(keys, vals, occ, occ_n, lg, key, sum);
+// TW lanes per segment of at most TW arcs: equal keys meet by a match, and the
+// first lane of each writes the sum.
+template <int TW, class V>
+__device__ __forceinline__ void tile_segments(const int64_t* __restrict__ sstart, const int32_t* __restrict__ list,
+                                              int64_t count, int64_t warp, int64_t nwarps, int32_t* ab, V* aw,
+                                              V* stage, int64_t* ucnt) {
+  const int lane = threadIdx.x & 31;
+  const int sub = lane & (TW - 1), tbase = lane - sub;
+  const unsigned tmask = (TW == 32 ? FULL : ((1u << (TW & 31)) - 1u)) << tbase;
+  constexpr int PER = 32 / TW;
+  for (int64_t q0 = warp * PER; q0 < count; q0 += nwarps * PER) {  // uniform in the warp
+    const int64_t q = q0 + lane / TW;
+    int64_t p = 0;
+    int len = 0;
+    int32_t a = 0;
+    if (q < count) {
+      a = list[q];
+      p = sstart[a];
+      len = (int)(sstart[a + 1] - p);
     }
+    const bool ok = sub < len;
+    const int32_t key = ok ? ab[p + sub] : (int32_t)(0x80000000u | (unsigned)lane);
+    const V w = ok ? aw[p + sub] : 0;
+    const unsigned peers = __match_any_sync(FULL, key) & tmask;
+    const int lead = __ffs(peers) - 1;
+    stage[lane] = 0;
+    __syncwarp();
+    if (ok) atomicAdd(&stage[lead], w);
+    __syncwarp();
+    const unsigned leads = __ballot_sync(FULL, ok && lead == lane) & tmask;
+    if (ok && lead == lane) {
+      const int r = __popc(leads & ((1u << lane) - 1u));
+      ab[p + r] = key;
+      aw[p + r] = stage[lane];
+    }
+    if (sub == 0 && q < count) ucnt[a] = __popc(leads);
     __syncwarp();
   }
 }
 
-// Warp per small segment: combine, then write the distinct entries back at
-// the segment start and record their number.
-__global__ void __launch_bounds__(NT) k_ag_warp(const int64_t* __restrict__ sstart, const int32_t* __restrict__ wl,
-                                                int64_t nw, int32_t* ab, unsigned long long* aw,
+// Segments of at most AG_WARP_MAX arcs: combine, write the distinct entries
+// back at the segment start and record their number.
+template <class V> constexpr size_t ag_warp_smem() { return (size_t)NW * AG_WCAP * (sizeof(V) + 4 + 2); }
+template <class V>
+__global__ void __launch_bounds__(NT) k_ag_warp(const int64_t* __restrict__ sstart, const int32_t* __restrict__ t8,
+                                                const int32_t* __restrict__ t32, const int32_t* __restrict__ wl,
+                                                const unsigned long long* __restrict__ cnt, int32_t* ab, V* aw,
                                                 int64_t* __restrict__ ucnt) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  unsigned long long* vals = (unsigned long long*)smem + (size_t)wid * AG_WCAP;
-  int32_t* keys = (int32_t*)(smem + (size_t)NW * AG_WCAP * 8) + (size_t)wid * AG_WCAP;
-  unsigned long long* stage = (unsigned long long*)(smem + (size_t)NW * AG_WCAP * 12) + (size_t)wid * 32;
-  uint16_t* occ = (uint16_t*)(smem + (size_t)NW * AG_WCAP * 12 + (size_t)NW * 32 * 8) + (size_t)wid * AG_WCAP;
+  V* vals = (V*)smem + (size_t)wid * AG_WCAP;
+  int32_t* keys = (int32_t*)(smem + (size_t)NW * AG_WCAP * sizeof(V)) + (size_t)wid * AG_WCAP;
+  uint16_t* occ = (uint16_t*)(smem + (size_t)NW * AG_WCAP * (sizeof(V) + 4)) + (size_t)wid * AG_WCAP;
   __shared__ int occ_n[NW];
+  __shared__ V stage[NW][32];
   for (int j = lane; j < AG_WCAP; j += 32) {
     keys[j] = AG_EMPTY;
     vals[j] = 0;
@@ -202,11 +324,25 @@ __global__ void __launch_bounds__(NT) k_ag_warp(const int64_t* __restrict__ ssta
   __syncwarp();
   const int64_t warp = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * NT) >> 5;
+  const int64_t nw = (int64_t)cnt[AC_WARP];
   for (int64_t q = warp; q < nw; q += nwarps) {
     const int32_t a = wl[q];
-    const int64_t p = sstart[a], len = sstart[a + 1] - p;
+    const int64_t p = sstart[a];
+    const int len = (int)(sstart[a + 1] - p);
     const unsigned lg = lg_for(2 * len);
-    warp_insert(ab, aw, p, len, keys, vals, occ, &occ_n[wid], lg, stage, lane);
+    for (int j0 = lane; j0 < len; j0 += 128) {
+      int32_t key[4];
+      V w[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool ok = j0 + 32 * u < len;
+        key[u] = ok ? ab[p + j0 + 32 * u] : AG_EMPTY;
+        w[u] = ok ? aw[p + j0 + 32 * u] : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (key[u] != AG_EMPTY) tab_insert(keys, vals, occ, &occ_n[wid], lg, key[u], w[u]);
+    }
     __syncwarp();
     const int nocc = occ_n[wid];
     for (int j = lane; j < nocc; j += 32) {
@@ -216,62 +352,62 @@ __global__ void __launch_bounds__(NT) k_ag_warp(const int64_t* __restrict__ ssta
       keys[slot] = AG_EMPTY;
       vals[slot] = 0;
     }
+    __syncwarp();
     if (lane == 0) {
       ucnt[a] = nocc;
       occ_n[wid] = 0;
     }
     __syncwarp();
   }
+  tile_segments<32, V>(sstart, t32, (int64_t)cnt[AC_T32], warp, nwarps, ab, aw, stage[wid], ucnt);
+  tile_segments<8, V>(sstart, t8, (int64_t)cnt[AC_T8], warp, nwarps, ab, aw, stage[wid], ucnt);
 }
 
-// CTA per block of up to AG_CTA_MAX arcs: a whole medium segment, or one chunk
-// of a large segment (then the chunk's distinct count goes to dch and to the
-// segment's upper bound ub).
-template <bool CHUNK>
-__global__ void __launch_bounds__(AG_CNT) k_ag_cta(const int64_t* __restrict__ sstart, const int32_t* __restrict__ list,
-                                               const int64_t* __restrict__ ch_off, int64_t nitems, int32_t* ab,
-                                               unsigned long long* aw, int64_t* __restrict__ ucnt,
-                                               int32_t* __restrict__ dch, unsigned long long* __restrict__ ub) {
+// CTA per block of up to AG_CTA_MAX arcs: first the chunks of the large
+// segments (a chunk's distinct count goes to dch and to the segment's upper
+// bound ub), then the whole medium segments.
+template <class V> constexpr size_t ag_cta_smem() { return (size_t)AG_CCAP * (sizeof(V) + 4 + 2); }
+template <class V>
+__global__ void __launch_bounds__(AG_CNT) k_ag_cta(const int64_t* __restrict__ sstart, const int32_t* __restrict__ cl,
+                                               const int32_t* __restrict__ ch_seg, const int64_t* __restrict__ ch_off,
+                                               const unsigned long long* __restrict__ cnt, int32_t* ab, V* aw,
+                                               int64_t* __restrict__ ucnt, int32_t* __restrict__ dch,
+                                               unsigned long long* __restrict__ ub) {
   extern __shared__ __align__(16) unsigned char smem[];
-  unsigned long long* vals = (unsigned long long*)smem;
-  int32_t* keys = (int32_t*)(smem + (size_t)AG_CCAP * 8);
-  unsigned long long* stage = (unsigned long long*)(smem + (size_t)AG_CCAP * 12) + (threadIdx.x >> 5) * 32;
-  uint16_t* occ = (uint16_t*)(smem + (size_t)AG_CCAP * 12 + (size_t)(AG_CNT / 32) * 32 * 8);
+  V* vals = (V*)smem;
+  int32_t* keys = (int32_t*)(smem + (size_t)AG_CCAP * sizeof(V));
+  uint16_t* occ = (uint16_t*)(smem + (size_t)AG_CCAP * (sizeof(V) + 4));
   __shared__ int occ_n;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t nch = (int64_t)cnt[AC_CHUNKS], items = nch + (int64_t)cnt[AC_CTA];
+  if (blockIdx.x >= items) return;
   for (int j = threadIdx.x; j < AG_CCAP; j += AG_CNT) {
     keys[j] = AG_EMPTY;
     vals[j] = 0;
   }
   if (threadIdx.x == 0) occ_n = 0;
   __syncthreads();
-  for (int64_t it = blockIdx.x; it < nitems; it += gridDim.x) {
-    const int32_t a = list[it];
-    int64_t p = sstart[a], len = sstart[a + 1] - p;
-    if (CHUNK) {
+  for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+    const bool chunk = it < nch;
+    const int32_t a = chunk ? ch_seg[it] : cl[it - nch];
+    int64_t p = sstart[a], left = sstart[a + 1] - p;
+    if (chunk) {
       p += ch_off[it];
-      len = len - ch_off[it] < AG_CHUNK ? len - ch_off[it] : AG_CHUNK;
+      left -= ch_off[it];
     }
+    const int len = left < AG_CHUNK ? (int)left : AG_CHUNK;
     const unsigned lg = lg_for(2 * len);
-    // warps take interleaved 32-entry rows of the block
-    for (int64_t j = (int64_t)wid * 32; j < len; j += AG_CNT) {
-      const int64_t jj = j + lane;
-      const bool ok = jj < len;
-      const int32_t key = ok ? ab[p + jj] : (int32_t)(0x80000000u | (unsigned)lane);
-      const unsigned long long wt = ok ? aw[p + jj] : 0ull;
-      const unsigned peers = __match_any_sync(FULL, key);
-      stage[lane] = wt;
-      __syncwarp();
-      if (ok && (__ffs(peers) - 1) == lane) {
-        unsigned long long sum = 0;
-        unsigned m = peers;
-        while (m) {
-          sum += stage[__ffs(m) - 1];
-          m &= m - 1;
-        }
-        tab_insert(keys, vals, occ, &occ_n, lg, key, sum);
+    for (int j0 = threadIdx.x; j0 < len; j0 += 4 * AG_CNT) {
+      int32_t key[4];
+      V w[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool ok = j0 + AG_CNT * u < len;
+        key[u] = ok ? ab[p + j0 + AG_CNT * u] : AG_EMPTY;
+        w[u] = ok ? aw[p + j0 + AG_CNT * u] : 0;
       }
-      __syncwarp();
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (key[u] != AG_EMPTY) tab_insert(keys, vals, occ, &occ_n, lg, key[u], w[u]);
     }
     __syncthreads();  // every entry read and inserted before the block is overwritten
     const int nocc = occ_n;
@@ -282,8 +418,9 @@ __global__ void __launch_bounds__(AG_CNT) k_ag_cta(const int64_t* __restrict__ s
       keys[slot] = AG_EMPTY;
       vals[slot] = 0;
     }
+    __syncthreads();
     if (threadIdx.x == 0) {
-      if (CHUNK) {
+      if (chunk) {
         dch[it] = nocc;
         atomicAdd(&ub[a], (unsigned long long)nocc);
       } else {
@@ -298,19 +435,21 @@ __global__ void __launch_bounds__(AG_CNT) k_ag_cta(const int64_t* __restrict__ s
 // ------------------------------------------------------------------ large segments
 
 // Global table of a large segment: 2^lg >= 2 x (its upper bound of distinct
-// keys) slots, at least AG_SLICE, placed at toff[a]; its slices are owned by a.
-__global__ void k_ag_tables_size(const int32_t* __restrict__ ll, int64_t nl, const unsigned long long* __restrict__ ub,
-                                 int32_t* __restrict__ tlg, int64_t* __restrict__ toff, unsigned long long* total) {
+// keys) slots, at least AG_SLICE, placed at toff[a].
+__global__ void k_ag_tables_size(const int32_t* __restrict__ ll, const unsigned long long* __restrict__ ub,
+                                 int32_t* __restrict__ tlg, int64_t* __restrict__ toff, unsigned long long* cnt) {
+  const int64_t nl = (int64_t)cnt[AC_BIG];
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nl; q += stride) {
     const int32_t a = ll[q];
     unsigned lg = lg_for(2 * (int64_t)ub[a]);
     if (lg < 10) lg = 10;  // AG_SLICE
     tlg[a] = (int32_t)lg;
-    toff[a] = (int64_t)atomicAdd(total, 1ull << lg);
+    toff[a] = (int64_t)atomicAdd(&cnt[AC_SLOTS], 1ull << lg);
   }
 }
 
+// A table's slices are owned by its segment.
 __global__ void k_ag_tables_own(const int32_t* __restrict__ ll, int64_t nl, const int32_t* __restrict__ tlg,
                                 const int64_t* __restrict__ toff, int32_t* __restrict__ owner) {
   for (int64_t q = blockIdx.x; q < nl; q += gridDim.x) {
@@ -320,30 +459,44 @@ __global__ void k_ag_tables_own(const int32_t* __restrict__ ll, int64_t nl, cons
   }
 }
 
-// CTA per chunk: its distinct entries into the segment's global table.
+// CTA per chunk: its distinct entries into the segment's global table. 32-bit
+// weights: a slot is one word (key << 32 | weight), claimed with its weight or
+// added to with one atomic; the sums stay below 2^31, so the weight never
+// carries into the key. 64-bit weights: key and weight in two arrays.
+template <class V>
 __global__ void __launch_bounds__(NT) k_ag_merge(const int64_t* __restrict__ sstart, const int32_t* __restrict__ ch_seg,
                                                  const int64_t* __restrict__ ch_off, const int32_t* __restrict__ dch,
                                                  int64_t nch, const int32_t* __restrict__ ab,
-                                                 const unsigned long long* __restrict__ aw,
+                                                 const V* __restrict__ aw,
                                                  const int32_t* __restrict__ tlg, const int64_t* __restrict__ toff,
-                                                 int32_t* gk, unsigned long long* gv) {
+                                                 unsigned long long* gs, int32_t* gk) {
   for (int64_t it = blockIdx.x; it < nch; it += gridDim.x) {
     const int32_t a = ch_seg[it];
     const int64_t p = sstart[a] + ch_off[it];
     const int d = dch[it];
     const unsigned lg = (unsigned)tlg[a];
     const uint64_t mask = ((uint64_t)1 << lg) - 1;
-    int32_t* keys = gk + toff[a];
-    unsigned long long* vals = gv + toff[a];
+    unsigned long long* slots = gs + toff[a];
     for (int j = threadIdx.x; j < d; j += NT) {
       const int32_t key = ab[p + j];
-      const unsigned long long w = aw[p + j];
+      const V w = aw[p + j];
       uint64_t h = ((uint64_t)(uint32_t)key * 0x9E3779B97F4A7C15ull) >> (64 - lg);
       for (uint64_t probe = 0; probe <= mask; ++probe) {
-        const int32_t prev = atomicCAS(&keys[h], AG_EMPTY, key);
-        if (prev == AG_EMPTY || prev == key) {
-          atomicAdd(&vals[h], w);
-          break;
+        if constexpr (sizeof(V) == 4) {
+          const unsigned long long mine = ((unsigned long long)(uint32_t)key << 32) | w;
+          unsigned long long c = *(volatile unsigned long long*)&slots[h];
+          if (c == AG_EMPTY_SLOT) c = atomicCAS(&slots[h], AG_EMPTY_SLOT, mine);
+          if (c == AG_EMPTY_SLOT) break;
+          if ((int32_t)(c >> 32) == key) {
+            atomicAdd(&slots[h], (unsigned long long)w);
+            break;
+          }
+        } else {
+          const int32_t prev = atomicCAS(&gk[toff[a] + h], AG_EMPTY, key);
+          if (prev == AG_EMPTY || prev == key) {
+            atomicAdd(&slots[h], (unsigned long long)w);
+            break;
+          }
         }
         h = (h + 1) & mask;
       }
@@ -353,191 +506,257 @@ __global__ void __launch_bounds__(NT) k_ag_merge(const int64_t* __restrict__ sst
 
 // CTA per AG_SLICE slots of the global tables: the live entries go back into
 // their segment (in any order).
+template <class V>
 __global__ void __launch_bounds__(NT) k_ag_extract(const int32_t* __restrict__ owner, int64_t nslices,
-                                                   const int32_t* __restrict__ gk, const unsigned long long* __restrict__ gv,
+                                                   const unsigned long long* __restrict__ gs, const int32_t* __restrict__ gk,
                                                    const int64_t* __restrict__ sstart, int32_t* ab,
-                                                   unsigned long long* aw, int64_t* ucnt) {
+                                                   V* aw, int64_t* ucnt) {
+  __shared__ int n_live;
+  __shared__ unsigned long long base;
   const int lane = threadIdx.x & 31;
+  constexpr int PER = AG_SLICE / NT;
   for (int64_t sl = blockIdx.x; sl < nslices; sl += gridDim.x) {
     const int32_t a = owner[sl];
     const int64_t p = sstart[a];
-    for (int j0 = 0; j0 < AG_SLICE; j0 += NT) {  // whole warps per step (the ballot needs them)
-      const int64_t slot = sl * AG_SLICE + j0 + threadIdx.x;
-      const int32_t key = gk[slot];
-      const bool live = key != AG_EMPTY;
-      const unsigned bal = __ballot_sync(FULL, live);
-      unsigned long long base = 0;
-      if (lane == 0 && bal) base = (unsigned long long)atomicAdd((unsigned long long*)&ucnt[a], (unsigned long long)__popc(bal));
-      base = __shfl_sync(FULL, base, 0);
-      if (live) {
-        const int64_t q = p + (int64_t)base + __popc(bal & ((1u << lane) - 1u));
-        ab[q] = key;
-        aw[q] = gv[slot];
+    if (threadIdx.x == 0) n_live = 0;
+    __syncthreads();
+    int32_t key[PER];
+    V w[PER];
+    int at[PER];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int64_t slot = sl * AG_SLICE + q * NT + threadIdx.x;
+      const unsigned long long x = gs[slot];
+      if constexpr (sizeof(V) == 4) key[q] = x == AG_EMPTY_SLOT ? AG_EMPTY : (int32_t)(x >> 32);
+      else key[q] = gk[slot];
+      w[q] = (V)x;
+    }
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const unsigned bal = __ballot_sync(FULL, key[q] != AG_EMPTY);
+      int b = 0;
+      if (lane == 0 && bal) b = atomicAdd(&n_live, __popc(bal));
+      at[q] = __shfl_sync(FULL, b, 0) + __popc(bal & ((1u << lane) - 1u));
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) base = n_live ? atomicAdd((unsigned long long*)&ucnt[a], (unsigned long long)n_live) : 0;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < PER; ++q)
+      if (key[q] != AG_EMPTY) {
+        ab[p + (int64_t)base + at[q]] = key[q];
+        aw[p + (int64_t)base + at[q]] = w[q];
+      }
+    __syncthreads();
+  }
+}
+
+// ------------------------------------------------------------------ coarse CSR
+
+// delta[A] = (start of A's segment) - (start of its coarse row); the number of empty rows.
+__global__ void __launch_bounds__(NT) k_ag_rows(const int64_t* __restrict__ sstart, const int64_t* __restrict__ coff,
+                                                int64_t k, int64_t* __restrict__ delta, const unsigned long long* cdegw,
+                                                unsigned long long* stat) {
+  __shared__ unsigned long long s_max;
+  __shared__ int s_iso;
+  if (threadIdx.x == 0) {
+    s_max = 0;
+    s_iso = 0;
+  }
+  __syncthreads();
+  int iso = 0;
+  unsigned long long mx = 0;
+  const int64_t stride = (int64_t)gridDim.x * NT;
+  for (int64_t a = (int64_t)blockIdx.x * NT + threadIdx.x; a < k; a += stride) {
+    const int64_t c = coff[a];
+    delta[a] = sstart[a] - c;
+    if (coff[a + 1] == c) ++iso;
+    mx = cdegw[a] > mx ? cdegw[a] : mx;
+  }
+  if (iso) atomicAdd(&s_iso, iso);
+  if (mx) atomicMax(&s_max, mx);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (s_iso) atomicAdd(&stat[0], (unsigned long long)s_iso);
+    if (s_max) atomicMax(&stat[1], s_max);
+  }
+}
+
+// The distinct entries into the coarse rows, split evenly by entries.
+template <class V, class WOUT>
+__global__ void __launch_bounds__(NT) k_ag_compact(const int64_t* __restrict__ coff, int64_t k, int64_t nseg,
+                                                   int64_t piece, const int64_t* __restrict__ delta,
+                                                   const int32_t* __restrict__ ab, const V* __restrict__ aw,
+                                                   int32_t* __restrict__ ccols, WOUT* __restrict__ cw) {
+  __shared__ __align__(16) int32_t mark[NW][WALK_TILE];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t step = (((int64_t)gridDim.x * NT) >> 5) * piece;
+  for (int64_t e0 = (((int64_t)blockIdx.x * NT + threadIdx.x) >> 5) * piece; e0 < nseg; e0 += step) {  // uniform in the warp
+    const int64_t e1 = e0 + piece < nseg ? e0 + piece : nseg;
+    int64_t cur = warp_row_of(coff, k, e0);
+    for (int64_t ts = e0; ts < e1; ts += WALK_TILE) {
+      int64_t row[4];
+      warp_tile_rows_strided(coff, k, ts, cur, mark[wid], row);
+      int32_t c[4];
+      V x[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int64_t e = ts + lane + 32 * j;
+        if (e >= e1) continue;
+        const int64_t p = delta[row[j]] + e;
+        c[j] = ab[p];
+        x[j] = aw[p];
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int64_t e = ts + lane + 32 * j;
+        if (e >= e1) continue;
+        ccols[e] = c[j];
+        cw[e] = (WOUT)x[j];
       }
     }
   }
 }
 
-// Warp per community: its distinct entries into the coarse CSR.
-__global__ void __launch_bounds__(NT) k_ag_compact(const int64_t* __restrict__ sstart, const int64_t* __restrict__ ucnt,
-                                                   const int64_t* __restrict__ coff, int64_t k,
-                                                   const int32_t* __restrict__ ab, const unsigned long long* __restrict__ aw,
-                                                   int32_t* __restrict__ ccols, int64_t* __restrict__ cw) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * NT) >> 5;
-  for (int64_t a = warp; a < k; a += nwarps) {
-    const int64_t p = sstart[a], d = ucnt[a], o = coff[a];
-    for (int64_t j = lane; j < d; j += 32) {
-      ccols[o + j] = ab[p + j];
-      cw[o + j] = (int64_t)aw[p + j];
-    }
-  }
-}
-
-}  // namespace
-
-// Inside aggregate_hash: a CUDA error frees the scratch before returning.
+// Inside aggregate_as: a CUDA error frees the scratch before returning.
 #define AG_CHECK(call)                                         \
   do {                                                         \
     cudaError_t _e = (call);                                   \
     if (_e != cudaSuccess) return fail(set_cuda_error(_e));    \
   } while (0)
 
-int aggregate_hash(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_dev, int64_t k,
-                   cd_graph** coarse_out) {
+// V: type of the segments' weights. 32-bit ones become the coarse graph's own.
+template <class V>
+int aggregate_as(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_dev, int64_t k, cd_graph** coarse_out) {
+  constexpr bool NARROW = sizeof(V) == 4;
   cudaStream_t s = g->stream;
   const int64_t n = g->n, m = g->nnz;
-  const int bits = [&] {
-    int b = 0;
-    while (((int64_t)1 << b) < k) ++b;
-    return b;
-  }();
   int rc = CD_OK;
   // scratch
-  uint64_t *vk = nullptr, *vk2 = nullptr;
-  int64_t *vv = nullptr, *vv2 = nullptr, *mpre = nullptr, *sstart = nullptr, *ucnt = nullptr, *coff = nullptr;
-  int64_t *tot = nullptr, *ch_off = nullptr, *toff = nullptr;
-  int32_t *ab = nullptr, *wl = nullptr, *cl = nullptr, *ll = nullptr, *ch_seg = nullptr, *dch = nullptr;
-  int32_t *tlg = nullptr, *owner = nullptr, *gk = nullptr;
-  unsigned long long *aw = nullptr, *cnt = nullptr, *ub = nullptr, *gv = nullptr;
-  int64_t* coarse_off = nullptr;
+  int32_t *nl = nullptr, *ab = nullptr, *lists = nullptr, *ch_seg = nullptr, *dch = nullptr, *tlg = nullptr;
+  int32_t *owner = nullptr, *gk = nullptr;
+  int64_t *delta = nullptr, *sstart = nullptr, *ch_off = nullptr, *toff = nullptr, *ucnt = nullptr;
+  unsigned long long *arcs = nullptr, *cnt = nullptr, *ub = nullptr, *gs = nullptr;
+  V* aw = nullptr;
+  // the coarse graph
+  int64_t *coarse_off = nullptr, *cdegw = nullptr;
   int32_t* ccols = nullptr;
-  int64_t* cw = nullptr;
+  void* cw = nullptr;
   auto cleanup = [&]() {
-    void* ps[] = {vk, vk2, vv, vv2, mpre, sstart, ucnt, coff, tot, ch_off, toff, ab, wl, cl, ll, ch_seg, dch,
-                  tlg, owner, gk, aw, cnt, ub, gv};
+    void* ps[] = {nl, ab, lists, ch_seg, dch, tlg, owner, gk, delta, sstart, ch_off, toff, arcs, cnt, ub, gs, aw};
     for (void* p : ps) dev_free(p, s);
   };
   auto fail = [&](int r) {
     cleanup();
     dev_free(coarse_off, s);
+    dev_free(cdegw, s);
     dev_free(ccols, s);
     dev_free(cw, s);
     return r;
   };
-  if ((rc = dev_alloc_t(&vk, n, s)) || (rc = dev_alloc_t(&vk2, n, s)) || (rc = dev_alloc_t(&vv, n, s)) ||
-      (rc = dev_alloc_t(&vv2, n, s)) || (rc = dev_alloc_t(&mpre, n, s)) || (rc = dev_alloc_t(&sstart, k + 1, s)) ||
-      (rc = dev_alloc_t(&ucnt, k, s)) || (rc = dev_alloc_t(&coff, k, s)) || (rc = dev_alloc_t(&tot, 1, s)) ||
-      (rc = dev_alloc_t(&ab, m, s)) || (rc = dev_alloc_t(&aw, m, s)) || (rc = dev_alloc_t(&cnt, 8, s)))
+  const int64_t max_big = m / (AG_CTA_MAX + 1) + 1;           // large segments at most
+  const int64_t max_chunks = m / AG_CHUNK + max_big;          // their chunks at most
+  const int64_t max_cta = m / (AG_WARP_MAX + 1) + 1;          // CTA segments at most
+  const int64_t max_warp = std::min(k, m / 33 + 1), max_t32 = std::min(k, m / 9 + 1), max_t8 = std::min(k, m + 1);
+  if ((rc = dev_alloc_t(&nl, n, s)) || (rc = dev_alloc_t(&delta, std::max(n, k), s)) ||
+      (rc = dev_alloc_t(&arcs, 2 * k, s)) || (rc = dev_alloc_t(&cdegw, k, s)) ||
+      (rc = dev_alloc_t(&sstart, k + 1, s)) || (rc = dev_alloc_t(&cnt, AC_N + 2, s)) ||
+      (rc = dev_alloc_t(&ab, m, s)) || (rc = dev_alloc_t(&aw, m, s)) ||
+      (rc = dev_alloc_t(&lists, max_t8 + max_t32 + max_warp + max_cta + max_big, s)) ||
+      (rc = dev_alloc_t(&ch_seg, max_chunks, s)) || (rc = dev_alloc_t(&ch_off, max_chunks, s)) ||
+      (rc = dev_alloc_t(&dch, max_chunks, s)) || (rc = dev_alloc_t(&coarse_off, k + 1, s)))
     return fail(rc);
+  ucnt = (int64_t*)arcs + k;  // one array, cleared together
+  int32_t *t8 = lists, *t32 = t8 + max_t8, *wl = t32 + max_t32, *cl = wl + max_warp, *ll = cl + max_cta;
   const int wbytes = g->wkind == W_UNIT ? 0 : g->wkind == W_I32 ? 4 : 8;
-
-  // 1-2: members by community, segments, scatter
-  uint64_t* sk = vk;
-  int64_t* sv = vv;
+  const unsigned gv = gcap((n + NT - 1) / NT, 152 * 8);
   {
-    KTimer t(g, K_SORT, (double)n * 32 * ((bits + 7) / 8));
-    if (n > 0) CD_LAUNCH(k_ag_vkeys<<<gcap((n + NT - 1) / NT), NT, 0, s>>>(labels_dev, newid_dev, n, vk, vv));
-    if ((rc = radix_sort_pairs(vk, vv, vk2, vv2, n, bits, s, &sk, &sv))) return fail(rc);
-  }
-  {
-    KTimer t(g, K_AGG_EMIT, (double)n * (8 + 16 + 8 + 8) + (double)m * (4 + 4 + 4 + wbytes + 4 + 8));
-    if (n > 0) CD_LAUNCH(k_ag_mdeg<<<gcap((n + NT - 1) / NT), NT, 0, s>>>(g->off, sv, n, mpre));
-    if ((rc = exclusive_scan_i64(mpre, mpre, n, tot, s))) return fail(rc);
-    if (n > 0) CD_LAUNCH(k_ag_heads<<<gcap((n + NT - 1) / NT), NT, 0, s>>>(sk, mpre, n, sstart));
-    AG_CHECK(cudaMemcpyAsync(sstart + k, tot, 8, cudaMemcpyDeviceToDevice, s));
+    KTimer t(g, K_AGG_EMIT, (double)n * (4 + 4 + 8 + 8 + 4 + 8) + (double)m * (4 + 4 + wbytes + 4 + sizeof(V)));
+    AG_CHECK(cudaMemsetAsync(arcs, 0, 2 * k * 8, s));
+    AG_CHECK(cudaMemsetAsync(cdegw, 0, k * 8, s));
+    CD_LAUNCH(k_ag_vertex<<<gv, NT, 0, s>>>(labels_dev, newid_dev, g->off, g->degw, n, nl, arcs,
+                                            (unsigned long long*)cdegw));
+    if ((rc = exclusive_scan_i64((const int64_t*)arcs, sstart, k, sstart + k, s))) return fail(rc);
+    AG_CHECK(cudaMemsetAsync(arcs, 0, k * 8, s));  // now the places taken per community
+    CD_LAUNCH(k_ag_place<<<gcap((n + AP_VERTS - 1) / AP_VERTS, 152 * 6), NT, 0, s>>>(nl, g->off, n, sstart, arcs, delta));
     if (m > 0) {
-      const unsigned gr = gcap((n + NW - 1) / NW);
+      const unsigned gr = gcap((m + 8 * WALK_TILE - 1) / (8 * WALK_TILE), 152 * 8);
+      const int64_t piece = walk_piece(m, (int64_t)gr * NW);
       if (g->wkind == W_UNIT)
-        CD_LAUNCH(k_ag_scatter<WUnit><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, labels_dev, newid_dev, sv, mpre, n, ab, aw));
+        CD_LAUNCH((k_ag_scatter<WUnit, V><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, m, piece, nl, delta, ab, aw)));
       else if (g->wkind == W_I32)
-        CD_LAUNCH(k_ag_scatter<WI32><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, labels_dev, newid_dev, sv, mpre, n, ab, aw));
+        CD_LAUNCH((k_ag_scatter<WI32, V><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, m, piece, nl, delta, ab, aw)));
       else
-        CD_LAUNCH(k_ag_scatter<WI64><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, labels_dev, newid_dev, sv, mpre, n, ab, aw));
+        CD_LAUNCH((k_ag_scatter<WI64, V><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, m, piece, nl, delta, ab, aw)));
     }
   }
-  // the vertex-sort buffers are no longer needed
-  dev_free(vk, s);
-  dev_free(vk2, s);
-  dev_free(vv, s);
-  dev_free(vv2, s);
-  vk = vk2 = nullptr;
-  vv = vv2 = nullptr;
-
+  unsigned long long h[AC_N + 2] = {};  // the counts; then empty rows, largest deg_w
   int64_t nseg = 0;
   {
-    KTimer t(g, K_AGG_REDUCE, (double)m * 2 * (4 + 8) + (double)k * 32);
-    // 3: classes
-    unsigned long long h[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    AG_CHECK(cudaMemsetAsync(cnt, 0, 8 * sizeof(unsigned long long), s));
-    if (k > 0) CD_LAUNCH(k_ag_class_count<<<gcap((k + NT - 1) / NT), NT, 0, s>>>(sstart, k, cnt));
-    AG_CHECK(cudaMemcpyAsync(h, cnt, 4 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-    AG_CHECK(cudaStreamSynchronize(s));
-    const int64_t nw = (int64_t)h[0], nc = (int64_t)h[1], nl = (int64_t)h[2], nch = (int64_t)h[3];
-    if ((rc = dev_alloc_t(&wl, nw, s)) || (rc = dev_alloc_t(&cl, nc, s)) || (rc = dev_alloc_t(&ll, nl, s)) ||
-        (rc = dev_alloc_t(&ch_seg, nch, s)) || (rc = dev_alloc_t(&ch_off, nch, s)) || (rc = dev_alloc_t(&dch, nch, s)))
-      return fail(rc);
-    AG_CHECK(cudaMemsetAsync(cnt, 0, 8 * sizeof(unsigned long long), s));
-    if (k > 0) CD_LAUNCH(k_ag_class_fill<<<gcap((k + NT - 1) / NT), NT, 0, s>>>(sstart, k, cnt, wl, cl, ll, ch_seg, ch_off));
-    if (nl > 0) {
+    KTimer t(g, K_AGG_REDUCE, (double)m * 2 * (4 + sizeof(V)) + (double)k * 32);
+    AG_CHECK(cudaMemsetAsync(cnt, 0, (AC_N + 2) * sizeof(unsigned long long), s));
+    const bool big = m > AG_CTA_MAX;  // there may be large segments
+    if (big) {
       if ((rc = dev_alloc_t(&ub, k, s)) || (rc = dev_alloc_t(&tlg, k, s)) || (rc = dev_alloc_t(&toff, k, s)))
         return fail(rc);
       AG_CHECK(cudaMemsetAsync(ub, 0, k * sizeof(unsigned long long), s));
-      AG_CHECK(cudaMemsetAsync(ucnt, 0, k * sizeof(int64_t), s));  // large segments count by atomics
     }
-    const size_t wsm = (size_t)NW * AG_WCAP * 12 + (size_t)NW * 32 * 8 + (size_t)NW * AG_WCAP * 2;
-    const size_t csm = (size_t)AG_CCAP * 12 + (size_t)(AG_CNT / 32) * 32 * 8 + (size_t)AG_CCAP * 2;
-    AG_CHECK(cudaFuncSetAttribute(k_ag_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm));
-    AG_CHECK(cudaFuncSetAttribute(k_ag_cta<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
-    AG_CHECK(cudaFuncSetAttribute(k_ag_cta<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
-    if (nw > 0) CD_LAUNCH(k_ag_warp<<<gcap((nw + NW - 1) / NW, 152 * 4), NT, wsm, s>>>(sstart, wl, nw, ab, aw, ucnt));
-    if (nc > 0)
-      CD_LAUNCH(k_ag_cta<false><<<gcap(nc, 152 * 2), AG_CNT, csm, s>>>(sstart, cl, nullptr, nc, ab, aw, ucnt, nullptr, nullptr));
-    if (nl > 0) {
-      CD_LAUNCH(k_ag_cta<true><<<gcap(nch, 152 * 2), AG_CNT, csm, s>>>(sstart, ch_seg, ch_off, nch, ab, aw, ucnt, dch, ub));
-      AG_CHECK(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
-      CD_LAUNCH(k_ag_tables_size<<<gcap((nl + NT - 1) / NT), NT, 0, s>>>(ll, nl, ub, tlg, toff, cnt));
-      unsigned long long slots = 0;
-      AG_CHECK(cudaMemcpyAsync(&slots, cnt, sizeof(slots), cudaMemcpyDeviceToHost, s));
+    AG_CHECK(cudaFuncSetAttribute(k_ag_warp<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ag_warp_smem<V>()));
+    AG_CHECK(cudaFuncSetAttribute(k_ag_cta<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ag_cta_smem<V>()));
+    if (m > 0) {
+      CD_LAUNCH(k_ag_classes<<<gcap((k + AF_SEGS - 1) / AF_SEGS, 152 * 8), NT, 0, s>>>(sstart, k, cnt, t8, t32, wl, cl, ll,
+                                                                                    ch_seg, ch_off));
+      if (m > AG_WARP_MAX)
+        CD_LAUNCH(k_ag_cta<V><<<gcap(max_cta + max_chunks, 152 * 2), AG_CNT, ag_cta_smem<V>(), s>>>(
+            sstart, cl, ch_seg, ch_off, cnt, ab, aw, ucnt, dch, ub));
+      CD_LAUNCH(k_ag_warp<V><<<gcap((k + NW - 1) / NW, 152 * 4), NT, ag_warp_smem<V>(), s>>>(sstart, t8, t32, wl, cnt, ab,
+                                                                                          aw, ucnt));
+    }
+    if (big) {
+      CD_LAUNCH(k_ag_tables_size<<<gcap((max_big + NT - 1) / NT), NT, 0, s>>>(ll, ub, tlg, toff, cnt));
+      AG_CHECK(cudaMemcpyAsync(h, cnt, AC_N * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
       AG_CHECK(cudaStreamSynchronize(s));
-      const int64_t nslices = (int64_t)slots / AG_SLICE;
-      if ((rc = dev_alloc_t(&gk, (int64_t)slots, s)) || (rc = dev_alloc_t(&gv, (int64_t)slots, s)) ||
-          (rc = dev_alloc_t(&owner, nslices, s)))
-        return fail(rc);
-      AG_CHECK(cudaMemsetAsync(gk, 0xff, slots * sizeof(int32_t), s));
-      AG_CHECK(cudaMemsetAsync(gv, 0, slots * sizeof(unsigned long long), s));
-      CD_LAUNCH(k_ag_tables_own<<<gcap(nl, 152 * 8), NT, 0, s>>>(ll, nl, tlg, toff, owner));
-      CD_LAUNCH(k_ag_merge<<<gcap(nch, 152 * 8), NT, 0, s>>>(sstart, ch_seg, ch_off, dch, nch, ab, aw, tlg, toff, gk, gv));
-      CD_LAUNCH(k_ag_extract<<<gcap(nslices, 152 * 8), NT, 0, s>>>(owner, nslices, gk, gv, sstart, ab, aw, ucnt));
+      const int64_t nlarge = (int64_t)h[AC_BIG], nch = (int64_t)h[AC_CHUNKS], slots = (int64_t)h[AC_SLOTS];
+      if (nlarge > 0) {
+        const int64_t nslices = slots / AG_SLICE;
+        if ((rc = dev_alloc_t(&gs, slots, s)) || (!NARROW && (rc = dev_alloc_t(&gk, slots, s))) ||
+            (rc = dev_alloc_t(&owner, nslices, s)))
+          return fail(rc);
+        AG_CHECK(cudaMemsetAsync(gs, NARROW ? 0xff : 0, slots * sizeof(unsigned long long), s));
+        if (!NARROW) AG_CHECK(cudaMemsetAsync(gk, 0xff, slots * sizeof(int32_t), s));
+        CD_LAUNCH(k_ag_tables_own<<<gcap(nlarge, 152 * 8), NT, 0, s>>>(ll, nlarge, tlg, toff, owner));
+        CD_LAUNCH(k_ag_merge<V><<<gcap(nch, 152 * 8), NT, 0, s>>>(sstart, ch_seg, ch_off, dch, nch, ab, aw, tlg, toff, gs,
+                                                               gk));
+        CD_LAUNCH(k_ag_extract<V><<<gcap(nslices, 152 * 8), NT, 0, s>>>(owner, nslices, gs, gk, sstart, ab, aw, ucnt));
+      }
     }
-    // 4: compact into the coarse CSR
-    if ((rc = exclusive_scan_i64(ucnt, coff, k, tot, s))) return fail(rc);
-    AG_CHECK(cudaMemcpyAsync(&nseg, tot, 8, cudaMemcpyDeviceToHost, s));
+    // 4: the coarse CSR
+    if ((rc = exclusive_scan_i64(ucnt, coarse_off, k, coarse_off + k, s))) return fail(rc);
+    CD_LAUNCH(k_ag_rows<<<gcap((k + NT - 1) / NT, 152 * 8), NT, 0, s>>>(sstart, coarse_off, k, delta,
+                                                                      (const unsigned long long*)cdegw, cnt + AC_N));
+    AG_CHECK(cudaMemcpyAsync(&nseg, coarse_off + k, 8, cudaMemcpyDeviceToHost, s));
+    AG_CHECK(cudaMemcpyAsync(h + AC_N, cnt + AC_N, 16, cudaMemcpyDeviceToHost, s));
     AG_CHECK(cudaStreamSynchronize(s));
-    if ((rc = dev_alloc_t(&coarse_off, k + 1, s)) || (rc = dev_alloc_t(&ccols, nseg + COL_PAD, s)) ||
-        (rc = dev_alloc_t(&cw, nseg, s)))
+    if ((rc = dev_alloc_t(&ccols, nseg + COL_PAD, s)) ||
+        (rc = dev_alloc(&cw, (size_t)std::max<int64_t>(nseg, 1) * (NARROW ? 4 : 8), s)))
       return fail(rc);
-    AG_CHECK(cudaMemcpyAsync(coarse_off, coff, k * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-    AG_CHECK(cudaMemcpyAsync(coarse_off + k, tot, 8, cudaMemcpyDeviceToDevice, s));
     AG_CHECK(cudaMemsetAsync(ccols + nseg, 0, COL_PAD * sizeof(int32_t), s));
-    if (k > 0 && nseg > 0)
-      CD_LAUNCH(k_ag_compact<<<gcap((k + NW - 1) / NW), NT, 0, s>>>(sstart, ucnt, coff, k, ab, aw, ccols, cw));
+    if (nseg > 0) {
+      const unsigned gr = gcap((nseg + 8 * WALK_TILE - 1) / (8 * WALK_TILE), 152 * 8);
+      const int64_t piece = walk_piece(nseg, (int64_t)gr * NW);
+      typedef typename std::conditional<NARROW, int32_t, int64_t>::type WOUT;
+      CD_LAUNCH((k_ag_compact<V, WOUT><<<gr, NT, 0, s>>>(coarse_off, k, nseg, piece, delta, ab, aw, ccols, (WOUT*)cw)));
+    }
     if (cudaGetLastError() != cudaSuccess) return fail(CD_ECUDA);
   }
   cleanup();
+  // what an ingest of the coarse arcs would find: aggregation keeps vol(V), and deg_w was summed above
+  unsigned long long stats[INGEST_STATS] = {};
+  stats[0] = (unsigned long long)g->vol;
+  stats[2] = h[AC_N];
+  stats[3] = h[AC_N + 1];
   cd_graph* c = nullptr;
-  rc = graph_adopt(s, k, nseg, coarse_off, ccols, cw, W_I64, &c, nullptr, nullptr, g);
+  rc = graph_adopt(s, k, nseg, coarse_off, ccols, cw, NARROW ? W_I32 : W_I64, &c, cdegw, stats, g);
   if (rc) return rc;
   c->timing = g->timing;
   c->ktiming = g->ktiming;
@@ -547,5 +766,12 @@ int aggregate_hash(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_
 }
 
 #undef AG_CHECK
+
+}  // namespace
+
+int aggregate_hash(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_dev, int64_t k, cd_graph** coarse_out) {
+  if (g->vol < ((int64_t)1 << 31)) return aggregate_as<uint32_t>(g, labels_dev, newid_dev, k, coarse_out);
+  return aggregate_as<unsigned long long>(g, labels_dev, newid_dev, k, coarse_out);
+}
 
 }  // namespace cd

@@ -108,6 +108,28 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(In in, int64_t n, co
   }
 }
 
+// One tile: the whole scan in one launch (small graphs and late levels are
+// launch bound).
+template <class T, class In>
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_one(In in, int64_t n, T* out, int64_t* total) {
+  const int64_t base = (int64_t)threadIdx.x * SCAN_ITEMS;
+  T v[SCAN_ITEMS];
+  T s = 0;
+#pragma unroll
+  for (int j = 0; j < SCAN_ITEMS; ++j) {
+    v[j] = base + j < n ? in(base + j) : T(0);
+    s += v[j];
+  }
+  __shared__ T tot;
+  T ex = block_exclusive_scan<T, SCAN_THREADS>(s, &tot);
+#pragma unroll
+  for (int j = 0; j < SCAN_ITEMS; ++j) {
+    if (base + j < n) out[base + j] = ex;
+    ex += v[j];
+  }
+  if (threadIdx.x == 0 && total) *total = (int64_t)tot;
+}
+
 template <class T, class In>
 int scan_impl(In in, T* out, int64_t n, int64_t* total_dev, cudaStream_t s) {
   if (n <= 0) {
@@ -115,6 +137,11 @@ int scan_impl(In in, T* out, int64_t n, int64_t* total_dev, cudaStream_t s) {
     return CD_OK;
   }
   int64_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
+  if (nb == 1) {
+    CD_LAUNCH(k_scan_one<T, In><<<1, SCAN_THREADS, 0, s>>>(in, n, out, total_dev));
+    CD_CHECK(cudaGetLastError());
+    return CD_OK;
+  }
   T* sums = nullptr;
   int rc = dev_alloc_t(&sums, nb, s);
   if (rc) return rc;

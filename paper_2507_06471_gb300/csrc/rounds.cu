@@ -1,5 +1,5 @@
 // The round loop of a run or Louvain level as one resident kernel, for graphs
-// without hubs: every round of Label Propagation (Algorithm 1) or local moving
+// without hubs or with few of them: every round of Label Propagation (Algorithm 1) or local moving
 // (Algorithm 2), synchronous, with the decisions, coins, counters and stop
 // tests of the per-round kernels in scan.cu (the results are the same).
 //
@@ -12,15 +12,22 @@
 // How: one cooperative launch of at most one wave of 256-thread CTAs. The
 // vertices are dealt out in units of 1 to 32 consecutive ids round robin, so
 // that every CTA gets an even share of whatever is active. In a round a CTA
-//   1. takes its vertices' flags (clearing them: the map is the next round's
-//      for the other parity), sorts the flagged ones by degree bin into a list in
+//   1. takes its vertices' flags, sorts the flagged ones by degree bin into a list in
 //      shared memory and scans them: a half CTA per vertex of degree t_warp+1
 //      to 1,024, warps for degree 33..t_warp and 4/8/16/32-lane tiles below
 //      (tasks taken from a counter in shared memory, longest first); it marks
 //      the neighbours of its moves in the next map and keeps its moves;
 //   2. meets the others at a barrier whose one atomic per CTA also sums moved +
 //      deferred (the stop test);
-//   3. applies its moves (labels, Sigma_tot, sizes) and meets the others again.
+//   3. applies its moves (labels, Sigma_tot, sizes), clears its part of the map
+//      it read, and meets the others again.
+// Hubs (degree above t_hub) that are examined in a round have their label
+// histograms built in step 1, by items of 1,024 arcs dealt out over the half
+// CTAs (combined in shared memory, then added to the hub's table in global
+// memory); after the first barrier the tables are read by slices, cleared while
+// read, and the last slice of a hub decides; a third barrier then comes before
+// step 3. The per-round kernels keep the histograms from round to round instead,
+// which pays on large graphs: see resident_rounds_apply.
 // The grid has at most as many CTAs as are resident at once (cooperative
 // launch), so the barrier's waits end; they are bounded all the same.
 //
@@ -52,28 +59,30 @@ struct LoopCtx {
   int32_t lgu;
   uint32_t* flag0;  // read in even rounds, written in odd ones
   uint32_t* flag1;
-  int32_t max_iter, first_rows, t_warp, per_graph;
+  int32_t max_iter, first_rows, t_warp, t_hub, per_graph;
   int64_t threshold;
   int32_t* last_change;       // per_graph: 1 + the last round in which a vertex of the graph wanted to move
-  unsigned long long* bar;    // two words per round, zero
+  unsigned long long* bar;    // three words per round, zero
   unsigned long long* head;   // HEAD words, then TRACE_COLS per round, zero
   uint32_t* sigma32;          // NK: Sigma_tot
+  ResidentHubs rh;            // rh.nh = 0: none
 };
 
-// Every CTA arrives once; `add` is summed over the CTAs. False: a wait ran out.
-__device__ __forceinline__ bool grid_meet(unsigned long long* word, unsigned add, unsigned long long& sum,
-                                          int32_t* status) {
+// Every CTA arrives once; `add` (changed vertices, < 2^32 in all) and `hubs`
+// are summed over the CTAs (at most 2^15). False: a wait ran out.
+__device__ __forceinline__ bool grid_meet(unsigned long long* word, unsigned add, unsigned hubs, unsigned& sum,
+                                          unsigned& hub_sum, int32_t* status) {
   __shared__ unsigned long long got;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    atomicAdd(word, (1ull << 40) | add);
+    atomicAdd(word, (1ull << 48) | ((unsigned long long)hubs << 32) | add);
     unsigned long long x;
     int64_t polls = 0;
     do {
       asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(word) : "memory");
-    } while ((x >> 40) < gridDim.x && ++polls < WAIT_LIMIT);
-    if ((x >> 40) < gridDim.x) {
+    } while ((x >> 48) < gridDim.x && ++polls < WAIT_LIMIT);
+    if ((x >> 48) < gridDim.x) {
       atomicCAS(status, 0, CD_ETIMEOUT);
       x = ~0ull;
     }
@@ -82,7 +91,8 @@ __device__ __forceinline__ bool grid_meet(unsigned long long* word, unsigned add
   }
   __syncthreads();
   const unsigned long long x = got;
-  sum = x & ((1ull << 40) - 1);
+  sum = (unsigned)x;
+  hub_sum = (unsigned)(x >> 32) & 0xffffu;
   return x != ~0ull;
 }
 
@@ -330,6 +340,99 @@ struct Scan {
   }
 };
 
+__device__ __forceinline__ bool flagged(const uint32_t* map, int32_t v) {
+  return !map || ((__ldcg(map + (v >> 5)) >> (v & 31)) & 1u);
+}
+
+// Add `w` arcs of `label` to hub h's table.
+template <class V>
+__device__ __forceinline__ void rh_add(const ResidentHubs& r, int64_t base, int64_t cap, int32_t label, V w) {
+  int64_t at = hub_home(label, cap);
+  for (int64_t probe = 0; probe < cap; ++probe) {  // at most two thirds of the slots fill: always ends
+    if constexpr (sizeof(V) == 4) {
+      unsigned long long* p = r.slot + base + at;
+      unsigned long long x = *(volatile unsigned long long*)p;
+      if (x == SLOT_EMPTY) {
+        x = atomicCAS(p, SLOT_EMPTY, ((unsigned long long)(uint32_t)label << 32) | w);
+        if (x == SLOT_EMPTY) return;
+      }
+      if ((int32_t)(x >> 32) == label) {
+        atomicAdd(p, (unsigned long long)w);
+        return;
+      }
+    } else {
+      int32_t x = *(volatile int32_t*)(r.key + base + at);
+      if (x == EMPTY) x = atomicCAS(r.key + base + at, EMPTY, label);
+      if (x == EMPTY || x == label) {
+        atomicAdd(r.slot + base + at, (unsigned long long)w);
+        return;
+      }
+    }
+    at = at + 1 == cap ? 0 : at + 1;
+  }
+}
+
+// The items of examined hubs that fall to this half CTA: build. Returns whether there was one.
+template <class W, class V>
+__device__ __forceinline__ bool rh_build(const ScanCtx& s, const ResidentHubs& r, const uint32_t* map, int half,
+                                         int32_t* keys, V* vals, uint16_t* occ, int* occ_n) {
+  const int gl = threadIdx.x & 127;
+  const int n_items = r.item[r.nh];
+  bool any = false;
+  for (int it = blockIdx.x * 2 + half; it < n_items; it += gridDim.x * 2) {
+    const int h = __ldg(r.item_hub + it);
+    const int32_t v = __ldg(r.v + h);
+    if (!flagged(map, v) || (s.gfrozen && s.gfrozen[s.gid[v]])) continue;  // uniform in the half CTA
+    any = true;
+    const int64_t beg = __ldg(s.off + v) + (int64_t)(it - __ldg(r.item + h)) * RH_CHUNK, row_end = __ldg(s.off + v + 1);
+    const int64_t end = beg + RH_CHUNK < row_end ? beg + RH_CHUNK : row_end;
+    const int64_t base = __ldg(r.tab + h), cap = __ldg(r.tab + h + 1) - base;
+    group_insert<W, V, 128>(s, v, beg, end, gl, keys, vals, occ, occ_n, 11);
+    half_sync(half);
+    const int n = *occ_n;
+    for (int j = gl; j < n; j += 128) {
+      const int q = occ[j];
+      const int32_t label = keys[q];
+      const V w = vals[q];
+      keys[q] = EMPTY;
+      vals[q] = 0;
+      rh_add<V>(r, base, cap, label, w);
+    }
+    half_sync(half);
+    if (gl == 0) *occ_n = 0;
+    half_sync(half);
+  }
+  return any;
+}
+static_assert(RH_CHUNK <= BLK1_MAX, "an item fits a half CTA's table");
+
+// One move per lane with `ok`: vertex v from community `from` to `to`.
+template <bool LOUV, bool NK>
+__device__ __forceinline__ void apply_moves(const ScanCtx& s, const LoopCtx& L, bool ok, int32_t v, int32_t to,
+                                            int32_t from, int64_t* stage) {
+  const int lane = threadIdx.x & 31;
+  if (ok) s.C_w[v] = to;
+  if constexpr (LOUV) {
+    const int64_t d = ok ? __ldg(s.degw + v) : 0;
+    // one atomic per distinct community of the warp: popular targets would serialise
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      const int32_t key = side ? from : to;
+      const unsigned peers = __match_any_sync(FULL, key);
+      stage[lane] = side ? -d : d;
+      __syncwarp();
+      if (key >= 0 && (__ffs(peers) - 1) == lane) {
+        int64_t sum = 0;
+        for (unsigned m = peers; m; m &= m - 1) sum += stage[__ffs(m) - 1];
+        if constexpr (NK) atomicAdd(&L.sigma32[key], (uint32_t)sum);
+        else atomicAdd((unsigned long long*)&s.sigma_w[key], (unsigned long long)sum);
+        atomicAdd(&s.csize_w[key], side ? -__popc(peers) : __popc(peers));
+      }
+      __syncwarp();
+    }
+  }
+}
+
 template <class V> constexpr size_t loop_smem() {
   return (size_t)PNW * PCAP * (sizeof(V) + 4 + 2) + (size_t)PNW * 32 * 8 + (size_t)CH_VERTS * 4;
 }
@@ -344,6 +447,9 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
   __shared__ int bincnt[2][8];  // by parity of the step: vertices per bin, then [7]: next task
   __shared__ int n_mv;
   __shared__ unsigned long long sums[5];
+  __shared__ int hub_moves, s_last;
+  __shared__ typename S::K red_k[PNW];
+  __shared__ int32_t red_c[PNW];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, half = tid >> 7;
   V* vals0 = (V*)smem;
   int32_t* keys0 = (int32_t*)(smem + (size_t)PNW * PCAP * sizeof(V));
@@ -366,14 +472,37 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
   const int64_t mv_stride = L.n32;
   int step = 0;
   int32_t round = 0;
+  // the CTA's counters of a round, added to the round's trace row; returns moved + deferred
+  auto account = [&](const Tally& t, int more_moves) -> unsigned {
+    unsigned long long c[5] = {t.act, t.arcs, t.cand, t.def, t.marcs};
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) c[q] += __shfl_xor_sync(FULL, c[q], o);
+      if (lane == 0 && c[q]) atomicAdd(&sums[q], c[q]);
+    }
+    __syncthreads();
+    const int nm = more_moves ? hub_moves : n_mv;
+    const unsigned changed = (unsigned)nm + (unsigned)sums[3];
+    if (tid < 6) {
+      const unsigned long long x = tid == 0 ? sums[0] : tid == 1 ? sums[1] : tid == 2 ? (unsigned long long)nm
+                                 : tid == 3 ? sums[3] : tid == 4 ? sums[2] : sums[4];
+      if (x) atomicAdd(&L.head[HEAD + (int64_t)round * TRACE_COLS + tid], x);
+    }
+    return changed;
+  };
   for (; round < L.max_iter;) {
     uint32_t* cur_map = round & 1 ? L.flag1 : L.flag0;
     uint32_t* nxt_map = round & 1 ? L.flag0 : L.flag1;
     const bool frontier = s.mark != 0;
-    if (tid == 0) n_mv = 0;
+    if (tid == 0) n_mv = hub_moves = 0;
     if (tid < 5) sums[tid] = 0;
     const S sc{s, L, round, round == 0 && L.first_rows, frontier ? nxt_map : nullptr, mv, mv_stride, &n_mv};
     Tally t;
+    bool hubs_here = false;
+    if (L.rh.nh)
+      hubs_here = rh_build<W, V>(s, L.rh, frontier ? cur_map : nullptr, half, keys0 + half * 4 * PCAP,
+                                 vals0 + half * 4 * PCAP, occ0 + half * 4 * PCAP, &occ_n[half * 4]);
     for (int64_t c0 = 0; c0 < my_verts; c0 += CH_VERTS) {
       // the lane's vertices of this step, c0 + (wid CH_PER_WARP + k) 32 + lane of the CTA's, and their flags
       int32_t vk[CH_PER_WARP];  // -1: not flagged
@@ -391,13 +520,6 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
       for (int k = 0; k < CH_PER_WARP; ++k) {
         if (vk[k] < 0) continue;
         const int32_t v = vk[k];
-        if (frontier && (v & (U - 1)) == 0) {  // the unit's flags are taken
-          const uint32_t mask = (U == 32 ? FULL : ((1u << U) - 1u)) << (v & 31);
-          if (fw[k] & mask) {
-            if (U == 32) cur_map[v >> 5] = 0;
-            else atomicAnd(&cur_map[v >> 5], ~mask);
-          }
-        }
         if ((fw[k] >> (v & 31)) & 1u) any = true;
         else vk[k] = -1;
       }
@@ -414,6 +536,7 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
         if (vk[k] >= 0) {
           const int32_t v = vk[k];
           deg[k] = (int)(__ldg(s.off + v + 1) - __ldg(s.off + v));
+          if (deg[k] > L.t_hub) deg[k] = 0;  // hubs: by items
           if (s.gfrozen && s.gfrozen[s.gid[v]]) deg[k] = 0;
         }
       }
@@ -486,61 +609,169 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
       }
       ++step;
     }
-    // the CTA's counters
-    unsigned long long c[5] = {t.act, t.arcs, t.cand, t.def, t.marcs};
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) c[q] += __shfl_xor_sync(FULL, c[q], o);
-      if (lane == 0 && c[q]) atomicAdd(&sums[q], c[q]);
-    }
-    __syncthreads();
+    hubs_here = __syncthreads_or(hubs_here);
+    const unsigned changed = account(t, 0);
     const int nm = n_mv;
-    const unsigned changed = (unsigned)nm + (unsigned)sums[3];
-    if (tid < 6) {
-      const unsigned long long x = tid == 0 ? sums[0] : tid == 1 ? sums[1] : tid == 2 ? (unsigned long long)nm
-                                 : tid == 3 ? sums[3] : tid == 4 ? sums[2] : sums[4];
-      if (x) atomicAdd(&L.head[HEAD + (int64_t)round * TRACE_COLS + tid], x);
+    unsigned total, hubs, none;
+    if (!grid_meet(L.bar + 3 * (int64_t)round, changed, hubs_here, total, hubs, s.status)) return;
+    if (hubs) {  // the same in every CTA: read the hubs' tables
+      const ResidentHubs& r = L.rh;
+      if (tid < 5) sums[tid] = 0;
+      __syncthreads();
+      Tally th;
+      const int n_slices = r.slice[r.nh];
+      for (int q = (int)b; q < n_slices; q += (int)G) {
+        const int h = __ldg(r.slice_hub + q);
+        const int32_t v = __ldg(r.v + h);
+        if (!flagged(frontier ? cur_map : nullptr, v) || (s.gfrozen && s.gfrozen[s.gid[v]])) continue;  // uniform
+        const int32_t cur = s.C[v];
+        const int64_t dv = LOUV ? __ldg(s.degw + v) : 0;
+        const int64_t volv = LOUV ? vol_of(s, v) : 0;
+        const int first_slice = __ldg(r.slice + h), slices = __ldg(r.slice + h + 1) - first_slice;
+        const int64_t base = __ldg(r.tab + h), cap = __ldg(r.tab + h + 1) - base;
+        const int64_t s0 = (int64_t)(q - first_slice) * RH_SLICE, s1 = s0 + RH_SLICE < cap ? s0 + RH_SLICE : cap;
+        typename S::K bk = no_key<typename S::K>();
+        int32_t bc = NOCAND;
+        for (int64_t e0 = s0 + tid; e0 < s1; e0 += 4 * PNT) {
+          int32_t c[4];
+          int64_t k[4], sg[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int64_t e = e0 + (int64_t)j * PNT;
+            c[j] = -1;
+            k[j] = 0;
+            if (e >= s1) continue;
+            if constexpr (sizeof(V) == 4) {
+              const unsigned long long x = __ldcg(r.slot + base + e);
+              if (x != SLOT_EMPTY) {
+                c[j] = (int32_t)(x >> 32);
+                k[j] = (int64_t)(uint32_t)x;
+                r.slot[base + e] = SLOT_EMPTY;
+              }
+            } else {
+              c[j] = __ldcg(r.key + base + e);
+              if (c[j] != EMPTY) {
+                k[j] = (int64_t)__ldcg(r.slot + base + e);
+                r.key[base + e] = EMPTY;
+                r.slot[base + e] = 0;
+              }
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) sg[j] = LOUV && c[j] >= 0 ? sig_of<NK>(s, c[j]) : 0;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (c[j] < 0) continue;
+            ++th.cand;
+            if (c[j] == cur) {
+              r.cur[h] = k[j];
+              r.has[h] = 1;
+              if (LOUV) continue;
+            }
+            const typename S::K key = cand_key_sg<LOUV, NK>(sg[j], k[j], dv, volv);
+            if (better(key, c[j], bk, bc)) {
+              bk = key;
+              bc = c[j];
+            }
+          }
+        }
+        reduce_best(bk, bc, 32);
+        if (lane == 0) {
+          red_k[wid] = bk;
+          red_c[wid] = bc;
+        }
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+          for (int w = 1; w < PNW; ++w)
+            if (better(red_k[w], red_c[w], bk, bc)) {
+              bk = red_k[w];
+              bc = red_c[w];
+            }
+          const i128 kk = (i128)bk;
+          r.part[3 * (int64_t)q] = (int64_t)(kk >> 64);
+          r.part[3 * (int64_t)q + 1] = (int64_t)(uint64_t)kk;
+          r.part[3 * (int64_t)q + 2] = bc;
+          __threadfence();
+          s_last = atomicAdd(&r.done[h], 1) == slices - 1;
+        }
+        __syncthreads();
+        if (s_last && wid == 0) {  // the hub's last slice: decide
+          __threadfence();
+          const volatile int64_t* part = r.part;
+          typename S::K fk = no_key<typename S::K>();
+          int32_t fc = NOCAND;
+          for (int p = first_slice + lane; p < first_slice + slices; p += 32) {
+            const i128 pk = (i128)(((unsigned __int128)(uint64_t)part[3 * (int64_t)p] << 64) |
+                                   (uint64_t)part[3 * (int64_t)p + 1]);
+            const int32_t pc = (int32_t)part[3 * (int64_t)p + 2];
+            if (better((typename S::K)pk, pc, fk, fc)) {
+              fk = (typename S::K)pk;
+              fc = pc;
+            }
+          }
+          reduce_best(fk, fc, 32);
+          if (lane == 0) {
+            const bool hc = *((volatile int32_t*)&r.has[h]) != 0;
+            const int64_t kc = hc ? *((volatile int64_t*)&r.cur[h]) : 0;
+            const int32_t target = decide<LOUV, NK>(s, v, cur, fk, fc, hc, kc, volv);
+            const uint32_t d = (uint32_t)(__ldg(s.off + v + 1) - __ldg(s.off + v));
+            ++th.act;
+            th.arcs += d;
+            if (target != cur) {
+              if (frontier) set_flag(nxt_map, v);
+              if (L.per_graph) L.last_change[s.gid[v]] = round + 1;
+              if (commit_coin(s.seed, s.level, round, local_id(s, v))) {
+                r.moved[h] = round + 1;
+                r.to[h] = target;
+                r.from[h] = cur;
+                atomicAdd(&hub_moves, 1);
+                th.marcs += d;
+              } else {
+                ++th.def;
+              }
+            }
+            r.done[h] = 0;
+            r.has[h] = 0;
+          }
+        }
+        __syncthreads();  // red_k, s_last
+      }
+      const unsigned more = account(th, 1);
+      unsigned hub_total;
+      if (!grid_meet(L.bar + 3 * (int64_t)round + 1, more, 0, hub_total, none, s.status)) return;
+      total += hub_total;
+      // the neighbours of the moved hubs
+      if (frontier) {
+        const int n_items = r.item[r.nh];
+        for (int it = (int)b; it < n_items; it += (int)G) {
+          const int h = __ldg(r.item_hub + it);
+          if (__ldcg(r.moved + h) != round + 1) continue;
+          const int32_t v = __ldg(r.v + h);
+          const int64_t beg = __ldg(s.off + v) + (int64_t)(it - __ldg(r.item + h)) * RH_CHUNK;
+          const int64_t row_end = __ldg(s.off + v + 1), end = beg + RH_CHUNK < row_end ? beg + RH_CHUNK : row_end;
+          for (int64_t e = beg + tid; e < end; e += PNT) set_flag(nxt_map, __ldg(s.cols + e));
+        }
+      }
+      // and their moves, dealt out over the warps of the grid
+      for (int64_t h0 = (b * PNW + wid) * 32; h0 < r.nh; h0 += G * PNW * 32) {
+        const int64_t h = h0 + lane;
+        const bool ok = h < r.nh && __ldcg(r.moved + h) == round + 1;
+        const int32_t v = ok ? r.v[h] : 0, to = ok ? __ldcg(r.to + h) : -1, from = ok ? __ldcg(r.from + h) : -1;
+        apply_moves<LOUV, NK>(s, L, ok, v, to, from, stage);
+      }
     }
-    unsigned long long total, none;
-    if (!grid_meet(L.bar + 2 * (int64_t)round, changed, total, s.status)) return;
-    // the moves
+    // the moves, and the flags that were read
     for (int base = wid * 32; base < nm; base += PNT) {
       const int i = base + lane;
       const bool ok = i < nm;
-      int32_t v = 0, to = -1, from = -1;
-      if (ok) {
-        v = mv[i];
-        to = mv[mv_stride + i];
-        s.C_w[v] = to;
-      }
-      if constexpr (LOUV) {
-        int64_t d = 0;
-        if (ok) {
-          from = mv[2 * mv_stride + i];
-          d = __ldg(s.degw + v);
-        }
-        // one atomic per distinct community of the warp: popular targets would serialise
-#pragma unroll
-        for (int side = 0; side < 2; ++side) {
-          const int32_t key = side ? from : to;
-          const unsigned peers = __match_any_sync(FULL, key);
-          stage[lane] = side ? -d : d;
-          __syncwarp();
-          if (key >= 0 && (__ffs(peers) - 1) == lane) {
-            int64_t sum = 0;
-            for (unsigned m = peers; m; m &= m - 1) sum += stage[__ffs(m) - 1];
-            if constexpr (NK) atomicAdd(&L.sigma32[key], (uint32_t)sum);
-            else atomicAdd((unsigned long long*)&s.sigma_w[key], (unsigned long long)sum);
-            atomicAdd(&s.csize_w[key], side ? -__popc(peers) : __popc(peers));
-          }
-          __syncwarp();
-        }
-      }
+      apply_moves<LOUV, NK>(s, L, ok, ok ? mv[i] : 0, ok ? mv[mv_stride + i] : -1, ok ? mv[2 * mv_stride + i] : -1, stage);
     }
+    if (frontier)
+      for (int64_t w = b * PNT + tid; w < L.nwords; w += G * PNT) cur_map[w] = 0;
     ++round;
     if (LOUV ? total == 0 : (int64_t)total <= L.threshold) break;
-    if (round < L.max_iter && !grid_meet(L.bar + 2 * (int64_t)round - 1, 0, none, s.status)) return;
+    if (round < L.max_iter && !grid_meet(L.bar + 3 * (int64_t)round - 1, 0, 0, total, none, s.status)) return;
   }
   if (b == 0 && tid == 0) L.head[0] = (unsigned long long)round;
 }
@@ -572,6 +803,7 @@ __global__ void __launch_bounds__(PNT) k_rounds_init(LoopCtx L, int32_t* C, int6
   for (int64_t i = tid; i < zero_words; i += stride) L.bar[i] = 0;  // the header and the trace follow the barrier words
   if (L.per_graph)
     for (int64_t i = tid; i < L.per_graph; i += stride) L.last_change[i] = 0;
+  for (int64_t i = tid; i < L.rh.nh; i += stride) L.rh.moved[i] = 0;
 }
 
 int loop_sms() {
@@ -647,7 +879,8 @@ ScanCtx loop_ctx(cd_graph* g, const RunOpts& o, bool louv, bool nk) {
 }  // namespace
 
 bool resident_rounds_apply(const cd_graph* g, const RunOpts& o, bool per_graph_stop) {
-  return o.device_loop && !g->timing && !o.async_mode && o.max_iter > 0 && g->n > 0 && g->nhubs == 0 &&
+  return o.device_loop && !g->timing && !o.async_mode && o.max_iter > 0 && g->n > 0 &&
+         (g->nhubs == 0 || (g->nhubs <= RH_MAX_HUBS && g->nnz <= RH_MAX_ARCS)) &&
          g->bin_start[B_BLK4 + 1] == g->bin_start[B_BLK4] && (!per_graph_stop || (o.threshold == 0 && o.use_frontier));
 }
 
@@ -669,10 +902,15 @@ int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, i
   L.max_iter = o.max_iter;
   L.first_rows = singletons && g->cols_distinct;
   L.t_warp = g->t_warp;
+  L.t_hub = g->t_hub;
+  if (g->nhubs > 0) {
+    if ((rc = ensure_resident_hubs(g))) return rc;
+    L.rh = *g->rh;
+  }
   L.threshold = o.threshold;
   L.per_graph = per_graph ? (int32_t)g->nb : 0;
   L.sigma32 = nk ? g->sigma32 : nullptr;
-  const int64_t words = 2 * (int64_t)o.max_iter + HEAD + (int64_t)TRACE_COLS * o.max_iter;
+  const int64_t words = 3 * (int64_t)o.max_iter + HEAD + (int64_t)TRACE_COLS * o.max_iter;
   unsigned long long* work = nullptr;
   if ((rc = dev_alloc_t(&work, words, st))) return rc;
   if (per_graph && (rc = dev_alloc_t(&L.last_change, g->nb, st))) {
@@ -680,7 +918,7 @@ int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, i
     return rc;
   }
   L.bar = work;
-  L.head = work + 2 * (int64_t)o.max_iter;
+  L.head = work + 3 * (int64_t)o.max_iter;
   std::vector<unsigned long long> h;
   std::vector<int32_t> hl;
   int32_t status = 0;

@@ -1899,6 +1899,7 @@ int run_rounds(cd_graph* g, const RunOpts& o, bool louv, int64_t* moves_out, int
   const int64_t n = g->n;
   const bool per_graph_stop = o.batched && graph_rounds != nullptr;
   if (!g->h_ctr) CD_CHECK(cudaMallocHost(&g->h_ctr, C_COUNT * sizeof(int64_t)));
+  if (int rcb = ensure_bins(g)) return rcb;
   std::vector<int64_t> h_gcnt;
   std::vector<uint8_t> h_frozen;
   if (per_graph_stop) {
@@ -2266,7 +2267,7 @@ int cd_autotune(cd_graph* g, const cd_params* p, int32_t rounds, int32_t* t_warp
   for (int i = 0; i < 3 && !rc; ++i)
     for (int j = 0; j < 4 && !rc; ++j) {
       if (th[j] < tw[i]) continue;
-      if ((rc = rebin(g, tw[i], th[j]))) break;
+      if ((rc = rebin(g, tw[i], th[j])) || (rc = ensure_bins(g))) break;
       RunOpts o = opts_from(p, 0);
       o.max_iter = rounds;
       cudaEventRecord(a, g->stream);

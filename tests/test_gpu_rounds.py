@@ -59,6 +59,24 @@ def test_equals_host_loop_and_oracle(n, wmax, loops):
     assert np.array_equal(got[10], lab) and got[11] == lv and abs(got[12] - q) <= 1e-12 * max(1.0, abs(q))
 
 
+@pytest.mark.parametrize("wmax,loops", [(1, 0), (9, 30), (2_000_000_000, 0)])
+@pytest.mark.parametrize("degs", [[1025], [2047, 2048, 2049, 1024], [9000, 1300, 4097], [1030] * 40 + EDGES])
+def test_hubs(degs, wmax, loops):
+    g = degrees_graph(12_000, degs, sum(degs), wmax, loops)
+    got = check(g, {})
+    off, cols, w = g.numpy()
+    lab, tr = oracle.lpa(off, cols, w)
+    assert np.array_equal(got[0], lab) and got[1] == tr.rounds
+    lab, lv, q, _ = oracle.louvain(off, cols, w)
+    assert np.array_equal(got[10], lab) and got[11] == lv and abs(got[12] - q) <= 1e-12 * max(1.0, abs(q))
+
+
+def test_hub_parameters():
+    g = degrees_graph(6000, [5000, 1100, 1024], 8, 3)
+    for params in ({"use_frontier": 0}, {"threshold": 40}, {"tie_keep_current": 0}, {"max_iter": 2}):
+        check(g, params)
+
+
 @pytest.mark.parametrize("params", [{"use_frontier": 0}, {"threshold": 40}, {"tie_keep_current": 0}, {"max_iter": 1},
                                     {"max_iter": 300, "sched_seed": 77}, {"singleton_rule": 0}])
 def test_parameters(params):
@@ -67,7 +85,7 @@ def test_parameters(params):
 
 def test_batched_equals_host_loop():
     import paper_2507_06471_gb300 as cd
-    graphs = [degrees_graph(n, [d for d in EDGES if d < n // 2], n, 4) for n in (1, 2, 40, 700, 33, 1500, 64, 3)]
+    graphs = [degrees_graph(n, [d for d in EDGES + [1500] if d < n // 2], n, 4) for n in (1, 2, 40, 700, 33, 4000, 64, 3)]
     packed, vstart = synth.pack_batch(graphs)
     G = cd.Graph(packed.off.cuda(), packed.cols.cuda(), packed.w.cuda())
     G.set_batches(vstart)
