@@ -145,7 +145,7 @@ struct cd_graph {
   uint32_t* hub_pref = nullptr;        // per 32-vertex word: hubs with smaller vertex ids (hub number = rank)
   uint32_t* hub_bits = nullptr;            // (n+31)/32: bit v set iff v is a hub
   int64_t* hub_tab = nullptr;              // nhubs+1
-  int64_t* hub_cc = nullptr;               // nhubs: slots in use, [0, hub_cc) of the allocation (rest empty)
+  int64_t* hub_cc = nullptr;               // nhubs: slots in use, [0, hub_cc) of the allocation
   int32_t* hub_live = nullptr;             // nhubs: live entries counted by the evaluate items of a round
   unsigned long long* hub_slot = nullptr;  // hub_slots words (x2 when wide)
   int32_t* hub_item_hub = nullptr;         // per build/mark item (HUB_CHUNK arcs): hub
@@ -167,7 +167,10 @@ struct cd_graph {
   int32_t* hub_mlist = nullptr;            // hub_items: mark items queued this round
   unsigned long long* hub_lcnt = nullptr;  // 2: queued build and mark items
   int32_t* hub_cl = nullptr;               // 5 x nhubs: hubs rebuilt per build class
-  unsigned long long* hub_ccnt = nullptr;  // 5: their counts
+  unsigned long long* hub_ccnt = nullptr;  // 7: their counts, and those of the two lists of hub_pl
+  int32_t* hub_nl = nullptr;               // nhubs: live entries at the last evaluation in this run (-1: none yet)
+  int64_t* hub_nc = nullptr;               // nhubs: slots a rebuild lays out
+  int32_t* hub_pl = nullptr;               // 2 x nhubs: hubs prepared by a CTA; rebuilds that overflowed
   unsigned long long* hub_log = nullptr;   // per round: hub-histogram updates (hub, old, new, w) to apply
   int64_t hub_log_cap = 0;
   int64_t max_degw = 0;            // largest deg_w (selects 32-bit table counters)

@@ -503,6 +503,7 @@ void free_arrays(cd_graph* g) {
                 g->hub_ev_first, g->hub_part,      g->hub_cur,      g->hub_hascur,   g->hub_done,
                 g->hub_mv,       g->hub_rb,       g->hub_used,     g->hub_item_first,
                 g->hub_flist,    g->hub_fcnt,     g->hub_cl,       g->hub_ccnt,
+                g->hub_nl,       g->hub_nc,       g->hub_pl,
                 g->hub_blist,    g->hub_mlist,     g->hub_lcnt,     g->C,            g->sigma,        g->csize,
                 g->hub_log,
                 g->sigma32,
@@ -531,7 +532,7 @@ void free_bins(cd_graph* g) {
                 g->hub_part,     g->hub_cur,     g->hub_hascur,   g->hub_done,  g->hub_mv,
                 g->hub_rb,       g->hub_used,     g->hub_item_first, g->hub_blist,
                 g->hub_flist,    g->hub_fcnt,     g->hub_cl,       g->hub_ccnt,
-                g->hub_mlist,    g->hub_lcnt,     g->hub_log};
+                g->hub_mlist,    g->hub_lcnt,     g->hub_log,      g->hub_nl,    g->hub_nc,      g->hub_pl};
   for (void* p : ps) dev_free(p, s);
   g->bin_list = nullptr;
   g->act_list = nullptr;
@@ -566,6 +567,8 @@ void free_bins(cd_graph* g) {
   g->hub_mlist = nullptr;
   g->hub_lcnt = nullptr;
   g->hub_log = nullptr;
+  g->hub_nl = g->hub_pl = nullptr;
+  g->hub_nc = nullptr;
   g->hub_log_cap = 0;
   g->nhubs = g->hub_arcs = g->hub_slots = g->hub_items = g->hub_eval_items = 0;
 }
@@ -692,7 +695,10 @@ int fill_bins(cd_graph* g) {
     if ((rc = dev_alloc_t(&g->hub_flist, 2 * nh, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_fcnt, 2, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_cl, 5 * nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_ccnt, 5, s))) return rc;
+    if ((rc = dev_alloc_t(&g->hub_ccnt, 7, s))) return rc;
+    if ((rc = dev_alloc_t(&g->hub_nl, nh, s))) return rc;
+    if ((rc = dev_alloc_t(&g->hub_nc, nh, s))) return rc;
+    if ((rc = dev_alloc_t(&g->hub_pl, 2 * nh, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_used, nh, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_item_first, nh + 1, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_blist, g->hub_items, s))) return rc;
@@ -716,7 +722,7 @@ int fill_bins(cd_graph* g) {
     CD_CHECK(cudaMemsetAsync(g->hub_used, 0, nh * 4, s));
     CD_CHECK(cudaMemsetAsync(g->hub_lcnt, 0, 2 * 8, s));
     CD_CHECK(cudaMemsetAsync(g->hub_fcnt, 0, 2 * 8, s));
-    CD_CHECK(cudaMemsetAsync(g->hub_ccnt, 0, 5 * 8, s));
+    CD_CHECK(cudaMemsetAsync(g->hub_ccnt, 0, 7 * 8, s));
     CD_CHECK(cudaMemsetAsync(g->hub_cur, 0, nh * 8, s));
     CD_CHECK(cudaMemsetAsync(g->hub_hascur, 0, nh * 4, s));
     CD_CHECK(cudaMemsetAsync(g->hub_done, 0, nh * 4, s));

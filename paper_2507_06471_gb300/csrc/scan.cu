@@ -382,36 +382,92 @@ constexpr int HUB_PREP_SLOTS = 12288;  // shared-memory slots of a compaction (l
 constexpr size_t HUB_PREP_SMEM = (size_t)HUB_PREP_SLOTS * 8;
 
 // A hub's table in use is [0, cc) of its allocation of A = 1.5 deg + 64
-// slots; the slots past cc are empty. A rebuild from the row takes all of A
-// (the number of distinct labels is not known before it). When an evaluation
+// slots. A rebuild from the row lays out 2 live + HUB_SLACK slots, from the live
+// entries its last evaluation counted: a neighbourhood rarely comes to hold many
+// more distinct labels from one round to the next, and the table is then written
+// and read at the size of what it holds, and built by fewer CTAs (level 1 of
+// R-MAT 26 holds 1.1e8 live entries after six rounds in 1.8e9 slots). The first
+// rebuild of a run takes all of A; one that runs out of slots is repeated with
+// all of A by k_hub_retry and k_hub_build. When an evaluation
 // finds at most a quarter of the slots in use holding live entries, the hub
 // is queued for compaction, which rehashes them into 2 live + 64 slots. Late
 // in a level most hubs' neighbours sit in few communities, so an evaluation
 // then reads a few hundred slots instead of 1.5 deg.
+constexpr int64_t HUB_SLACK = 256;
+constexpr int HUB_FULL_PROBES = 512;     // a rebuild that probes further counts as out of slots
 constexpr int64_t HUB_SHRINK_MIN = 512;  // tables in use this small are left as they are
 __device__ __forceinline__ void hub_maybe_shrink(const ScanCtx& s, int32_t h, int64_t cc, int64_t live) {
   if (!s.hub_wide && cc > HUB_SHRINK_MIN && live * 4 < cc && 3 * live + 64 <= HUB_PREP_SLOTS && s.hub_rb[h] == 0)
     hub_flag(s, h, HUB_COMPACT);
 }
 
-// Start of a round, a CTA per hub flagged in the previous round (every hub in
-// round 0). COMPACT (packed slots): the live entries (count > 0) are listed at
-// the top of shared memory and rehashed below them into a table of 2 live + 64
-// slots (at most the allocation), which is written back with coalesced stores
-// (the slots it no longer uses are cleared). REBUILD, or too many live entries
-// for shared memory: the table goes back to its whole allocation, is cleared
-// (unless a cluster build overwrites it whole) and the hub's build is queued.
+// Start of a round, a thread per hub flagged in the previous round (every hub
+// after a heavy one): a rebuild that one CTA or a cluster can lay out goes to its
+// build class; compactions, and tables too large for shared memory, to the list
+// k_hub_prepare takes a CTA each for. (A CTA per flagged hub for this alone took
+// 0.8 ms in a heavy round of R-MAT 24.)
+__global__ void __launch_bounds__(NT) k_hub_sort(ScanCtx s) {
+  const int64_t nf = (int64_t)*(volatile const unsigned long long*)s.hub_fcnt_r;
+  const int64_t stride = (int64_t)gridDim.x * NT;
+  for (int64_t q = (int64_t)blockIdx.x * NT + threadIdx.x; q < nf; q += stride) {
+    const int32_t h = s.hub_flist_r[q];
+    const int64_t cap = s.hub_tab[h + 1] - s.hub_tab[h];
+    int c = -1;
+    if (!s.hub_wide && s.hub_rb[h] != HUB_COMPACT) {
+      const int64_t nl = s.hub_nl[h];
+      const int64_t nc = nl >= 0 && 2 * nl + HUB_SLACK < cap ? 2 * nl + HUB_SLACK : cap;
+      c = hub_class(nc);
+      if (c >= 0) {
+        s.hub_nc[h] = nc;
+        s.hub_used[h] = 0;
+        s.hub_rb[h] = HUB_REBUILD;  // cleared by the build
+      }
+    }
+    const int list = c >= 0 ? c : 5;
+    int32_t* to = c >= 0 ? s.hub_cl + (int64_t)c * s.nhubs : s.hub_pl;
+    to[(int64_t)atomicAdd(&s.hub_ccnt[list], 1ull)] = h;
+  }
+}
+
+// Clear hub h's whole allocation and queue its items for k_hub_build (one CTA).
+__device__ __forceinline__ void hub_clear(const ScanCtx& s, int32_t h, int64_t cap) {
+  __shared__ unsigned long long pos;
+  const int64_t base = s.hub_tab[h];
+  const int64_t i0 = s.hub_item_first[h], ni = s.hub_item_first[h + 1] - i0;
+  for (int64_t i = threadIdx.x; i < cap; i += NT) {
+    if (!s.hub_wide) {
+      s.hub_slot[base + i] = SLOT_EMPTY;
+    } else {
+      s.hub_slot[2 * (base + i)] = SLOT_EMPTY;
+      s.hub_slot[2 * (base + i) + 1] = 0;
+    }
+  }
+  if (threadIdx.x == 0) {
+    atomicAdd(&s.ctr[C_HUB_PSLOTS], (unsigned long long)cap);
+    s.hub_cc[h] = cap;
+    s.hub_used[h] = 0;
+    s.hub_rb[h] = HUB_REBUILD;  // cleared once built (start of the evaluate kernel)
+    pos = atomicAdd(&s.hub_lcnt[0], (unsigned long long)ni);
+  }
+  __syncthreads();
+  for (int64_t j = threadIdx.x; j < ni; j += NT) s.hub_blist[pos + j] = (int32_t)(i0 + j);
+}
+
+// A CTA per hub k_hub_sort listed. COMPACT (packed slots): the live entries
+// (count > 0) are listed at the top of shared memory and rehashed below them
+// into a table of 2 live + 64 slots (at most the allocation), which is written
+// back with coalesced stores. Too many live entries for that, or a table too
+// large for a cluster: the table goes back to its whole allocation and is
+// rebuilt, by a build class or, cleared here, by items.
 __global__ void __launch_bounds__(NT) k_hub_prepare(ScanCtx s) {
   extern __shared__ __align__(16) unsigned char smem[];
   unsigned long long* T = (unsigned long long*)smem;
-  __shared__ unsigned long long pos;
   __shared__ int n_live;
-  const int64_t nf = (int64_t)*(volatile const unsigned long long*)s.hub_fcnt_r;
+  const int64_t nf = (int64_t)*(volatile const unsigned long long*)&s.hub_ccnt[5];
   for (int64_t q = blockIdx.x; q < nf; q += gridDim.x) {
-    const int32_t h = s.hub_flist_r[q];
+    const int32_t h = s.hub_pl[q];
     const int64_t base = s.hub_tab[h], cap = s.hub_tab[h + 1] - base;  // the allocation
     const int64_t cc = s.hub_cc[h];                                     // slots in use
-    const int64_t i0 = s.hub_item_first[h], ni = s.hub_item_first[h + 1] - i0;
     if (s.hub_rb[h] == HUB_COMPACT && !s.hub_wide) {  // uniform in the CTA
       if (threadIdx.x == 0) n_live = 0;
       __syncthreads();
@@ -437,7 +493,6 @@ __global__ void __launch_bounds__(NT) k_hub_prepare(ScanCtx s) {
         }
         __syncthreads();
         for (int64_t i = threadIdx.x; i < nc; i += NT) s.hub_slot[base + i] = T[i];
-        for (int64_t i = nc + threadIdx.x; i < cc; i += NT) s.hub_slot[base + i] = SLOT_EMPTY;
         if (threadIdx.x == 0) {
           s.hub_cc[h] = nc;
           s.hub_used[h] = (int32_t)nl;
@@ -451,7 +506,7 @@ __global__ void __launch_bounds__(NT) k_hub_prepare(ScanCtx s) {
     if (!s.hub_wide && hub_class(cap) >= 0) {  // one CTA or a cluster builds it and writes the whole table
       if (threadIdx.x == 0) {
         const int c = hub_class(cap);
-        s.hub_cc[h] = cap;
+        s.hub_nc[h] = cap;
         s.hub_used[h] = 0;
         s.hub_rb[h] = HUB_REBUILD;  // cleared by the cluster once built
         s.hub_cl[(int64_t)c * s.nhubs + (int64_t)atomicAdd(&s.hub_ccnt[c], 1ull)] = h;
@@ -459,49 +514,44 @@ __global__ void __launch_bounds__(NT) k_hub_prepare(ScanCtx s) {
       __syncthreads();
       continue;
     }
-    {  // giant or two-word hubs: cleared here (the slots past cc are empty already),
-       // built by items with global inserts
-      const int64_t clr = s.hub_wide ? cap : cc;
-      if (threadIdx.x == 0) atomicAdd(&s.ctr[C_HUB_PSLOTS], (unsigned long long)clr);
-      for (int64_t i = threadIdx.x; i < clr; i += NT) {
-        if (!s.hub_wide) {
-          s.hub_slot[base + i] = SLOT_EMPTY;
-        } else {
-          s.hub_slot[2 * (base + i)] = SLOT_EMPTY;
-          s.hub_slot[2 * (base + i) + 1] = 0;
-        }
-      }
-    }
-    if (threadIdx.x == 0) {
-      s.hub_cc[h] = cap;
-      s.hub_used[h] = 0;
-      s.hub_rb[h] = HUB_REBUILD;  // cleared once built (start of the evaluate kernel)
-      pos = atomicAdd(&s.hub_lcnt[0], (unsigned long long)ni);
-    }
+    hub_clear(s, h, cap);
     __syncthreads();
-    for (int64_t j = threadIdx.x; j < ni; j += NT) s.hub_blist[pos + j] = (int32_t)(i0 + j);
+  }
+}
+
+// Rebuilds that ran out of slots: their tables cleared whole, their items queued.
+__global__ void __launch_bounds__(NT) k_hub_retry(ScanCtx s) {
+  const int64_t nf = (int64_t)*(volatile const unsigned long long*)&s.hub_ccnt[6];
+  for (int64_t q = blockIdx.x; q < nf; q += gridDim.x) {
+    const int32_t h = s.hub_pl[s.nhubs + q];
+    hub_clear(s, h, s.hub_tab[h + 1] - s.hub_tab[h]);
     __syncthreads();
   }
 }
 
 constexpr int HUB_NT = 512;
 
-// A hub table of at most C x hub_cl_slots(C) packed slots is rebuilt from the
-// hub's row by a cluster of C CTAs: the table is laid out in its final hash
-// order across the cluster's shared memories (CTA p holds slots
-// [p S, (p+1) S)), every arc's label is added there (remote slots through
-// distributed shared memory), and each CTA then writes its part with
-// coalesced stores. No global atomics. In shared memory a slot is two 32-bit
-// words, the label and its count (packed tables have every count < 2^32), so
-// a probe past an occupied slot is a plain 32-bit load, only an empty slot is
-// claimed with a compare-and-swap, and the count takes a 32-bit add.
+// A hub table of at most C x SLOTS packed slots is rebuilt from the hub's row
+// by a cluster of C CTAs: the table is laid out in its final hash order across
+// the cluster's shared memories (CTA p holds slots [p S, (p+1) S)), every arc's
+// label is added there (remote slots through distributed shared memory), and
+// each CTA then writes its part with coalesced stores. No global atomics. In
+// shared memory a slot is two 32-bit words, the label and its count (packed
+// tables have every count < 2^32), so a probe past an occupied slot is a plain
+// 32-bit load, only an empty slot is claimed with a compare-and-swap, and the
+// count takes a 32-bit add.
+//
+// One CTA adds every arc by itself; in a cluster the equal labels of a warp are
+// combined first, since each addition may cross to another SM.
+// Returns 1 for a claimed slot, 0 for a label met before, -1 if none was found.
 template <int C>
-__device__ __forceinline__ bool hub_cl_insert(cg::cluster_group& cl, int32_t* K, uint32_t* V, int64_t cap,
-                                              int64_t S, int32_t lbl, uint32_t sum) {
+__device__ __forceinline__ int hub_cl_insert(cg::cluster_group& cl, int32_t* K, uint32_t* V, int64_t cap,
+                                             int64_t S, int32_t lbl, uint32_t sum) {
   const uint32_t home = (uint32_t)hub_home(lbl, cap);
+  const int lim = cap < HUB_FULL_PROBES ? (int)cap : HUB_FULL_PROBES;
   if constexpr (C == 1) {  // the whole table is local
     uint32_t slot = home;
-    for (int64_t probe = 0; probe < cap; ++probe) {  // at most 2/3 of the slots fill: always ends
+    for (int probe = 0; probe < lim; ++probe) {
       int32_t k = *(volatile int32_t*)&K[slot];
       if (k == EMPTY) k = atomicCAS(&K[slot], EMPTY, lbl);
       if (k == EMPTY || k == lbl) {
@@ -514,7 +564,7 @@ __device__ __forceinline__ bool hub_cl_insert(cg::cluster_group& cl, int32_t* K,
     // slot = owner * S + local (tables here are < 2^32 slots); probing steps
     // local and carries into the next owner, wrapping at cap
     uint32_t owner = home / (uint32_t)S, local = home - owner * (uint32_t)S;
-    for (int64_t probe = 0; probe < cap; ++probe) {  // at most 2/3 of the slots fill: always ends
+    for (int probe = 0; probe < lim; ++probe) {
       int32_t* pk = cl.map_shared_rank(K + local, owner);
       int32_t k = *(volatile int32_t*)pk;
       if (k == EMPTY) k = atomicCAS(pk, EMPTY, lbl);
@@ -528,7 +578,7 @@ __device__ __forceinline__ bool hub_cl_insert(cg::cluster_group& cl, int32_t* K,
       }
     }
   }
-  return false;
+  return -1;
 }
 
 template <class W, int CI>
@@ -538,7 +588,8 @@ __global__ void __cluster_dims__(HubClass<CI>::C, 1, 1) __launch_bounds__(HubCla
   extern __shared__ __align__(16) unsigned char hsm[];  // SLOTS keys, then as many counts
   int32_t* K = (int32_t*)hsm;
   uint32_t* V = (uint32_t*)(hsm + (size_t)SLOTS * 4);
-  __shared__ uint32_t st_w[NTB / 32][32];
+  __shared__ uint32_t st_w[C == 1 || W::unit ? 1 : NTB / 32][32];
+  __shared__ int full;  // rank 0's: this hub ran out of slots
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -549,17 +600,19 @@ __global__ void __cluster_dims__(HubClass<CI>::C, 1, 1) __launch_bounds__(HubCla
     K[i] = EMPTY;
     V[i] = 0;
   }
+  if (threadIdx.x == 0) full = 0;
   if constexpr (C == 1) __syncthreads(); else cl.sync();
   for (int64_t q = blockIdx.x / C; q < n; q += gridDim.x / C) {  // uniform in the cluster
     const int32_t h = list[q];
     const int32_t v = s.hub_list[h];
-    const int64_t base = s.hub_tab[h], cap = s.hub_tab[h + 1] - base;
+    const int64_t base = s.hub_tab[h], cap = s.hub_nc[h];
     const int64_t S = (cap + C - 1) / C;  // slots per CTA
     const int64_t mine = cap - rank * S < S ? cap - rank * S : S;
     const int64_t beg = s.off[v], end = s.off[v + 1];
     const int64_t share = (end - beg + C - 1) / C;
     const int64_t a0 = beg + rank * share, a1 = a0 + share < end ? a0 + share : end;
     int claimed = 0;
+    bool over = false;
     constexpr int U = 4;  // arcs per thread per step: their loads and gathers are in flight together
     for (int64_t e0 = a0; e0 < a1; e0 += (int64_t)U * NTB) {  // whole CTAs iterate together
       int32_t nb[U], lbl[U];
@@ -568,7 +621,7 @@ __global__ void __cluster_dims__(HubClass<CI>::C, 1, 1) __launch_bounds__(HubCla
       for (int j = 0; j < U; ++j) {
         const int64_t e = e0 + (int64_t)j * NTB + threadIdx.x;
         const bool has = e < a1;
-        nb[j] = has ? s.cols[e] : v;
+        nb[j] = has ? __ldg(s.cols + e) : v;
         w[j] = (has && nb[j] != v) ? (uint32_t)W::get(s.w, e) : 0u;
       }
 #pragma unroll
@@ -576,42 +629,63 @@ __global__ void __cluster_dims__(HubClass<CI>::C, 1, 1) __launch_bounds__(HubCla
         lbl[j] = w[j] ? s.C[nb[j]] : (int32_t)(0x80000000u | (unsigned)lane);
 #pragma unroll
       for (int j = 0; j < U; ++j) {
-        const bool cand = lbl[j] >= 0;
-        const unsigned peers = __match_any_sync(FULL, lbl[j]);
-        uint32_t sum;
-        if constexpr (W::unit) {
-          sum = (uint32_t)__popc(peers);
+        int got = 0;
+        if constexpr (C == 1) {
+          if (lbl[j] >= 0) got = hub_cl_insert<C>(cl, K, V, cap, S, lbl[j], w[j]);
         } else {
-          st_w[wid][lane] = w[j];
-          __syncwarp();
-          sum = 0;
-          unsigned m = peers;
-          while (m) {
-            sum += st_w[wid][__ffs(m) - 1];
-            m &= m - 1;
+          const unsigned peers = __match_any_sync(FULL, lbl[j]);
+          uint32_t sum;
+          if constexpr (W::unit) {
+            sum = (uint32_t)__popc(peers);
+          } else {
+            const int lead = __ffs(peers) - 1;
+            st_w[wid][lane] = 0;
+            __syncwarp();
+            atomicAdd(&st_w[wid][lead], w[j]);
+            __syncwarp();
+            sum = st_w[wid][lane];
+            __syncwarp();
           }
-          __syncwarp();
+          if (lbl[j] >= 0 && (__ffs(peers) - 1) == lane) got = hub_cl_insert<C>(cl, K, V, cap, S, lbl[j], sum);
         }
-        if (cand && (__ffs(peers) - 1) == lane && hub_cl_insert<C>(cl, K, V, cap, S, lbl[j], sum)) ++claimed;
+        if (got > 0) ++claimed;
+        over = over || got < 0;
       }
     }
+    if (over) {
+      if constexpr (C == 1) full = 1;
+      else *cl.map_shared_rank(&full, 0) = 1;
+    }
     if constexpr (C == 1) __syncthreads(); else cl.sync();  // every insert is done
+    const bool ran_out = C == 1 ? full != 0 : *(volatile int*)cl.map_shared_rank(&full, 0) != 0;
     for (int64_t i = threadIdx.x; i < mine; i += NTB) {
       const int32_t k = K[i];
-      s.hub_slot[base + rank * S + i] =
-          k == EMPTY ? SLOT_EMPTY : (((unsigned long long)(uint32_t)k << 32) | (unsigned long long)V[i]);
+      if (!ran_out)
+        s.hub_slot[base + rank * S + i] =
+            k == EMPTY ? SLOT_EMPTY : (((unsigned long long)(uint32_t)k << 32) | (unsigned long long)V[i]);
       K[i] = EMPTY;
       V[i] = 0;
     }
+    if (!ran_out) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) claimed += __shfl_xor_sync(FULL, claimed, o);
-    if (lane == 0 && claimed) atomicAdd(&s.hub_used[h], claimed);
+      for (int o = 16; o > 0; o >>= 1) claimed += __shfl_xor_sync(FULL, claimed, o);
+      if (lane == 0 && claimed) atomicAdd(&s.hub_used[h], claimed);
+    }
     if (rank == 0 && threadIdx.x == 0) {
-      s.hub_rb[h] = 0;
       atomicAdd(&s.ctr[C_HUB_BARCS], (unsigned long long)(end - beg));
-      atomicAdd(&s.ctr[C_HUB_BSLOTS], (unsigned long long)cap);
+      if (ran_out) {
+        s.hub_pl[s.nhubs + (int64_t)atomicAdd(&s.hub_ccnt[6], 1ull)] = h;
+      } else {
+        s.hub_cc[h] = cap;
+        s.hub_rb[h] = 0;
+        atomicAdd(&s.ctr[C_HUB_BSLOTS], (unsigned long long)cap);
+      }
     }
     if constexpr (C == 1) __syncthreads(); else cl.sync();  // parts cleared before the next hub's inserts
+    if (ran_out) {
+      if (threadIdx.x == 0) full = 0;
+      if constexpr (C == 1) __syncthreads(); else cl.sync();
+    }
   }
 }
 constexpr int HUB_CAP = 2 * HUB_CHUNK;
@@ -748,6 +822,7 @@ __global__ void __launch_bounds__(NT) k_hub_eval_small(ScanCtx s) {
     if (lane == 0) {
       hub_decide<LOUV, NK>(s, h, v, cur, bk, bc, hm != 0, kc, volv, n_act, n_arcs, n_def, n_marcs);
       hub_maybe_shrink(s, h, cap, nl);
+      s.hub_nl[h] = (int32_t)nl;
     }
   }
   flush_counters(s, B_HUB, n_act, n_arcs, n_cand, n_def, n_marcs);
@@ -863,7 +938,9 @@ __global__ void __launch_bounds__(NT) k_hub_eval(ScanCtx s) {
       const bool hc = *((volatile int32_t*)&s.hub_hascur[h]) != 0;
       const int64_t kc = hc ? *((volatile int64_t*)&s.hub_cur[h]) : 0;
       hub_decide<LOUV, NK>(s, h, v, cur, fk, fc, hc, kc, volv, n_act, n_arcs, n_def, n_marcs);
-      hub_maybe_shrink(s, h, cap, *(volatile int32_t*)&s.hub_live[h]);
+      const int32_t live = *(volatile int32_t*)&s.hub_live[h];
+      hub_maybe_shrink(s, h, cap, live);
+      s.hub_nl[h] = live;
       s.hub_live[h] = 0;
       s.hub_done[h] = 0;
       s.hub_cur[h] = 0;
@@ -1514,11 +1591,8 @@ int launch_round(cd_graph* g, ScanCtx& s, const int32_t* lists, const unsigned l
   if (cnt(B_HUB) > 0) {
     {
       KTimer t(g, K_HUB_PREP);  // compactions, and clears of the tables rebuilt below
+      CD_LAUNCH(k_hub_sort<<<grid_cap((g->nhubs + NT - 1) / NT, 152 * 4), NT, 0, st>>>(s));
       CD_LAUNCH(k_hub_prepare<<<grid_cap(g->nhubs, 152 * 2), NT, HUB_PREP_SMEM, st>>>(s));
-      // the examined hubs' evaluate work, by the table sizes the preparation left
-      CD_CHECK(cudaMemsetAsync(g->act_cnt + NBINS, 0, 2 * sizeof(unsigned long long), st));
-      CD_LAUNCH(k_hub_route<<<grid_cap((g->nhubs + NT - 1) / NT), NT, 0, st>>>(s, g->act_ev, g->act_small,
-                                                                             g->act_cnt + NBINS));
     }
     if (g->ktiming) marks.push_back({g->pending.size() - 1, -2});
     {
@@ -1528,7 +1602,12 @@ int launch_round(cd_graph* g, ScanCtx& s, const int32_t* lists, const unsigned l
       CD_LAUNCH((k_hub_build_cl<W, 2><<<304, HUB_NT, hub_cl_smem<2>(), st>>>(s)));
       CD_LAUNCH((k_hub_build_cl<W, 3><<<304, HUB_NT, hub_cl_smem<3>(), st>>>(s)));
       CD_LAUNCH((k_hub_build_cl<W, 4><<<304, HUB_NT, hub_cl_smem<4>(), st>>>(s)));
+      CD_LAUNCH(k_hub_retry<<<152, NT, 0, st>>>(s));
       CD_LAUNCH(k_hub_build<W, V><<<grid_cap(g->hub_items, 152 * 3), HUB_NT, hub_smem<V>(), st>>>(s));
+      // the examined hubs' evaluate work, by the sizes of their tables
+      CD_CHECK(cudaMemsetAsync(g->act_cnt + NBINS, 0, 2 * sizeof(unsigned long long), st));
+      CD_LAUNCH(k_hub_route<<<grid_cap((g->nhubs + NT - 1) / NT), NT, 0, st>>>(s, g->act_ev, g->act_small,
+                                                                             g->act_cnt + NBINS));
     }
     if (g->ktiming) marks.push_back({g->pending.size() - 1, -1});
   }
@@ -1681,6 +1760,9 @@ ScanCtx static_ctx(cd_graph* g, const RunOpts& o, bool louv, bool use_s32, bool 
   s.hub_lcnt = g->hub_lcnt;
   s.hub_cl = g->hub_cl;
   s.hub_ccnt = g->hub_ccnt;
+  s.hub_nl = g->hub_nl;
+  s.hub_nc = g->hub_nc;
+  s.hub_pl = g->hub_pl;
   s.n_items = g->hub_items;
   s.nhubs = g->nhubs;
   s.n_ev_items = g->hub_eval_items;
@@ -1801,7 +1883,7 @@ int device_rounds(cd_graph* g, const RunOpts& o, bool louv, bool use_s32, bool p
     if (nh > 0) {
       CD_CHECK(cudaMemsetAsync(g->hub_mv, 0, 3 * nh * sizeof(int32_t), cap));
       CD_CHECK(cudaMemsetAsync(g->hub_lcnt, 0, 2 * sizeof(unsigned long long), cap));
-      CD_CHECK(cudaMemsetAsync(g->hub_ccnt, 0, HUB_NCLASS * sizeof(unsigned long long), cap));
+      CD_CHECK(cudaMemsetAsync(g->hub_ccnt, 0, (HUB_NCLASS + 2) * sizeof(unsigned long long), cap));
       CD_CHECK(cudaMemsetAsync(cntB, 0, sizeof(unsigned long long), cap));
     }
     CD_LAUNCH(k_loop_begin<<<1, 1, 0, cap>>>(dl, n, louv ? HUB_SKIP_DIV : HUB_SKIP_DIV_LPA, nh > 0));
@@ -1910,6 +1992,7 @@ int run_rounds(cd_graph* g, const RunOpts& o, bool louv, int64_t* moves_out, int
   }
   int rc = CD_OK;
   if (g->nhubs > 0) {  // every histogram is built from the starting labels in round 0
+    CD_CHECK(cudaMemsetAsync(g->hub_nl, 0xff, g->nhubs * sizeof(int32_t), st));
     CD_LAUNCH(k_fill_i32<<<grid_cap((g->nhubs + NT - 1) / NT), NT, 0, st>>>(g->hub_rb, g->nhubs, 1));
     CD_LAUNCH(k_iota_i32<<<grid_cap((g->nhubs + NT - 1) / NT), NT, 0, st>>>(g->hub_flist + g->nhubs, g->nhubs));
     const unsigned long long nh = (unsigned long long)g->nhubs;
@@ -1955,7 +2038,7 @@ int run_rounds(cd_graph* g, const RunOpts& o, bool louv, int64_t* moves_out, int
     if (g->nhubs > 0) {
       CD_CHECK(cudaMemsetAsync(g->hub_mv, 0, 3 * g->nhubs * sizeof(int32_t), st));
       CD_CHECK(cudaMemsetAsync(g->hub_lcnt, 0, 2 * sizeof(unsigned long long), st));
-      CD_CHECK(cudaMemsetAsync(g->hub_ccnt, 0, HUB_NCLASS * sizeof(unsigned long long), st));
+      CD_CHECK(cudaMemsetAsync(g->hub_ccnt, 0, (HUB_NCLASS + 2) * sizeof(unsigned long long), st));
       CD_CHECK(cudaMemsetAsync(g->hub_fcnt + (r & 1), 0, sizeof(unsigned long long), st));
     }
     ScanCtx s = static_ctx(g, o, louv, use_s32, per_graph_stop);

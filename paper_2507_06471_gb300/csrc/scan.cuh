@@ -127,12 +127,15 @@ struct ScanCtx {
   const int32_t* hub_flist_r;        // hubs flagged in the previous round
   const unsigned long long* hub_fcnt_r;
   int32_t* hub_used;                 // per hub: slots claimed since its last build
+  int32_t* hub_nl;                   // per hub: live entries at its last evaluation in this run, -1: none yet
+  int64_t* hub_nc;                   // per hub: slots its rebuild of this round lays out
+  int32_t* hub_pl;                   // nhubs: hubs a CTA prepares this round; then nhubs: rebuilds that overflowed
   const int64_t* hub_item_first;     // nhubs+1: first build/mark item of each hub
   int32_t* hub_blist;                // build items of the hubs being rebuilt this round
   int32_t* hub_mlist;                // mark items of the hubs that moved this round
   unsigned long long* hub_lcnt;      // [0] build items, [1] mark items
   int32_t* hub_cl;                   // 5 x nhubs: hubs rebuilt per build class (one CTA small/large, clusters of 2, 4, 8)
-  unsigned long long* hub_ccnt;      // 5: their counts
+  unsigned long long* hub_ccnt;      // 5: their counts; [5], [6]: those of hub_pl's two lists
   const int32_t* ev_list;            // evaluate items (of large hubs) to run this round
   const unsigned long long* ev_cnt;  // their number
   const int32_t* small_list;         // small hubs (one warp each) to evaluate this round
