@@ -446,8 +446,9 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
   __shared__ int occ_n[PNW];
   __shared__ int bincnt[2][8];  // by parity of the step: vertices per bin, then [7]: next task
   __shared__ int n_mv;
-  __shared__ unsigned long long sums[5];
+  __shared__ uint32_t sums[5];  // a CTA has at most 2^31 / 152 vertices of at most 1,024 arcs
   __shared__ int hub_moves, s_last;
+  __shared__ int start[PNW][8];
   __shared__ typename S::K red_k[PNW];
   __shared__ int32_t red_c[PNW];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, half = tid >> 7;
@@ -466,7 +467,7 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
   // this CTA's units: blockIdx.x + i gridDim.x; its moves have room for all their vertices
   const int64_t G = gridDim.x, b = blockIdx.x;
   const int U = 1 << L.lgu;
-  const int64_t my_verts = (L.nunits / G + (b < L.nunits % G ? 1 : 0)) << L.lgu;
+  const uint32_t my_verts = (uint32_t)(L.nunits / G + (b < L.nunits % G ? 1 : 0)) << L.lgu;
   const int64_t mv_at = (b * (L.nunits / G) + (b < L.nunits % G ? b : L.nunits % G)) << L.lgu;
   int32_t* mv = s.mv_v + mv_at;
   const int64_t mv_stride = L.n32;
@@ -474,16 +475,17 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
   int32_t round = 0;
   // the CTA's counters of a round, added to the round's trace row; returns moved + deferred
   auto account = [&](const Tally& t, int more_moves) -> unsigned {
-    unsigned long long c[5] = {t.act, t.arcs, t.cand, t.def, t.marcs};
+    if (__any_sync(FULL, t.act | t.cand)) {
+      const uint32_t c[5] = {t.act, t.arcs, t.cand, t.def, t.marcs};  // a warp's arcs of a round stay below 2^32
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) c[q] += __shfl_xor_sync(FULL, c[q], o);
-      if (lane == 0 && c[q]) atomicAdd(&sums[q], c[q]);
+      for (int q = 0; q < 5; ++q) {
+        const uint32_t x = __reduce_add_sync(FULL, c[q]);
+        if (lane == 0 && x) atomicAdd(&sums[q], x);
+      }
     }
     __syncthreads();
     const int nm = more_moves ? hub_moves : n_mv;
-    const unsigned changed = (unsigned)nm + (unsigned)sums[3];
+    const unsigned changed = (unsigned)nm + sums[3];
     if (tid < 6) {
       const unsigned long long x = tid == 0 ? sums[0] : tid == 1 ? sums[1] : tid == 2 ? (unsigned long long)nm
                                  : tid == 3 ? sums[3] : tid == 4 ? sums[2] : sums[4];
@@ -503,74 +505,63 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
     if (L.rh.nh)
       hubs_here = rh_build<W, V>(s, L.rh, frontier ? cur_map : nullptr, half, keys0 + half * 4 * PCAP,
                                  vals0 + half * 4 * PCAP, occ0 + half * 4 * PCAP, &occ_n[half * 4]);
-    for (int64_t c0 = 0; c0 < my_verts; c0 += CH_VERTS) {
-      // the lane's vertices of this step, c0 + (wid CH_PER_WARP + k) 32 + lane of the CTA's, and their flags
-      int32_t vk[CH_PER_WARP];  // -1: not flagged
-      uint32_t fw[CH_PER_WARP];
+    for (uint32_t c0 = 0; c0 < my_verts; c0 += CH_VERTS) {
+      // the lane's vertices of this step, c0 + (wid CH_PER_WARP + k) 32 + lane of
+      // the CTA's: -1 where not flagged. A warp without one skips what follows,
+      // and so does a group of 32 in it: late rounds have few, and this sorting
+      // was most of a small graph's instructions.
+      const uint32_t i0 = (uint32_t)c0 + wid * CH_PER_WARP * 32 + lane;
+      int32_t vk[CH_PER_WARP];
 #pragma unroll
       for (int k = 0; k < CH_PER_WARP; ++k) {
-        const int64_t i = c0 + (wid * CH_PER_WARP + k) * 32 + lane;
-        const int64_t v = ((b + (i >> L.lgu) * G) << L.lgu) + (i & (U - 1));
-        vk[k] = i < my_verts && v < L.n ? (int32_t)v : -1;
-        fw[k] = FULL;
-        if (frontier && vk[k] >= 0) fw[k] = __ldcg(cur_map + (v >> 5));
+        vk[k] = -1;
+        const uint32_t i = i0 + 32 * k;
+        if (i - lane >= my_verts) continue;  // uniform in the warp
+        const uint32_t v = (((uint32_t)b + (i >> L.lgu) * (uint32_t)G) << L.lgu) + (i & (U - 1));
+        if (i < my_verts && v < (uint32_t)L.n) vk[k] = (int32_t)v;
       }
-      bool any = false;
+      if (frontier) {
+        uint32_t fw[CH_PER_WARP];
 #pragma unroll
-      for (int k = 0; k < CH_PER_WARP; ++k) {
-        if (vk[k] < 0) continue;
-        const int32_t v = vk[k];
-        if ((fw[k] >> (v & 31)) & 1u) any = true;
-        else vk[k] = -1;
+        for (int k = 0; k < CH_PER_WARP; ++k) fw[k] = vk[k] >= 0 ? __ldcg(cur_map + (vk[k] >> 5)) : 0;
+#pragma unroll
+        for (int k = 0; k < CH_PER_WARP; ++k)
+          if (!((fw[k] >> (vk[k] & 31)) & 1u)) vk[k] = -1;
       }
+      unsigned some = 0;  // the groups of 32 with a flagged vertex
+#pragma unroll
+      for (int k = 0; k < CH_PER_WARP; ++k) some |= __any_sync(FULL, vk[k] >= 0) ? 1u << k : 0u;
       int* cnt = bincnt[step & 1];
-      if (!__syncthreads_or(any)) continue;
-      // degree bins; the vertex's rank inside its bin of the warp
-      int deg[CH_PER_WARP];
-      int8_t bin[CH_PER_WARP];
-      int16_t rank[CH_PER_WARP];
-      int wcnt[PBINS] = {0, 0, 0, 0, 0, 0};
+      if (!__syncthreads_or(some != 0)) continue;
+      // degree bins, and the vertex's rank inside its bin
+      int slot[CH_PER_WARP];  // bin << 16 | rank, -1: none
 #pragma unroll
       for (int k = 0; k < CH_PER_WARP; ++k) {
-        deg[k] = 0;
+        slot[k] = -1;
+        if (!((some >> k) & 1u)) continue;
         if (vk[k] >= 0) {
           const int32_t v = vk[k];
-          deg[k] = (int)(__ldg(s.off + v + 1) - __ldg(s.off + v));
-          if (deg[k] > L.t_hub) deg[k] = 0;  // hubs: by items
-          if (s.gfrozen && s.gfrozen[s.gid[v]]) deg[k] = 0;
+          int64_t d = __ldg(s.off + v + 1) - __ldg(s.off + v);
+          if (s.gfrozen && s.gfrozen[s.gid[v]]) d = 0;
+          if (d > 0 && d <= L.t_hub) {  // hubs: by items
+            const int bin = d <= 4 ? 5 : d <= 8 ? 4 : d <= 16 ? 3 : d <= 32 ? 2 : d <= L.t_warp ? 1 : 0;
+            slot[k] = (bin << 16) | atomicAdd(&cnt[bin], 1);
+          }
         }
       }
-#pragma unroll
-      for (int k = 0; k < CH_PER_WARP; ++k) {
-        const int d = deg[k];
-        bin[k] = d == 0 ? -1 : d <= 4 ? 5 : d <= 8 ? 4 : d <= 16 ? 3 : d <= 32 ? 2 : d <= L.t_warp ? 1 : 0;
-        rank[k] = 0;
-        if (!__any_sync(FULL, d != 0)) continue;
-#pragma unroll
-        for (int q = 0; q < PBINS; ++q) {
-          const unsigned m = __ballot_sync(FULL, bin[k] == q);
-          if (bin[k] == q) rank[k] = (int16_t)(wcnt[q] + __popc(m & ((1u << lane) - 1u)));
-          wcnt[q] += __popc(m);
-        }
-      }
-      int mine = 0;
-#pragma unroll
-      for (int q = 0; q < PBINS; ++q)
-        if (lane == q) mine = wcnt[q];
-      int at = 0;
-      if (lane < PBINS && mine) at = atomicAdd(&cnt[lane], mine);
       __syncthreads();
       int first_of[PBINS + 1];  // where each bin starts in the list
       first_of[0] = 0;
 #pragma unroll
       for (int q = 0; q < PBINS; ++q) first_of[q + 1] = first_of[q] + cnt[q];
+      if (some) {
 #pragma unroll
-      for (int q = 0; q < PBINS; ++q)
-        if (lane == q) at += first_of[q];
+        for (int q = 0; q < PBINS; ++q)
+          if (lane == q) start[wid][q] = first_of[q];
+        __syncwarp();
 #pragma unroll
-      for (int k = 0; k < CH_PER_WARP; ++k) {
-        const int p = __shfl_sync(FULL, at, bin[k] < 0 ? 0 : bin[k]) + rank[k];
-        if (bin[k] >= 0) list[p] = vk[k];
+        for (int k = 0; k < CH_PER_WARP; ++k)
+          if (slot[k] >= 0) list[start[wid][slot[k] >> 16] + (slot[k] & 0xffff)] = vk[k];
       }
       if (tid < 8) bincnt[(step + 1) & 1][tid] = 0;  // the next step's
       __syncthreads();
