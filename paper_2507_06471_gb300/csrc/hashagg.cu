@@ -93,7 +93,8 @@ __global__ void __launch_bounds__(NT) k_ag_place(const int32_t* __restrict__ nl,
                                                  int64_t n, const int64_t* __restrict__ sstart,
                                                  unsigned long long* taken, int64_t* __restrict__ delta) {
   constexpr int SLOTS = 1024;
-  __shared__ unsigned long long tot[SLOTS];
+  __shared__ uint32_t tot[SLOTS];  // 32-bit shared atomics: 64-bit ones take 25 times as long
+  __shared__ unsigned long long base[SLOTS];
   __shared__ int32_t key[SLOTS];
   for (int64_t v0 = (int64_t)blockIdx.x * AP_VERTS; v0 < n; v0 += (int64_t)gridDim.x * AP_VERTS) {
     for (int i = threadIdx.x; i < SLOTS; i += NT) {
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(NT) k_ag_place(const int32_t* __restrict__ nl,
       slot[q] = -1;
       if (a[q] < 0) continue;
       unsigned h = ((uint32_t)a[q] * 2654435761u) >> 22;
-      for (int probe = 0; probe < 4; ++probe) {
+      for (int probe = 0; probe < 4 && at[q] < (1u << 21); ++probe) {  // 2,048 such degrees stay below 2^32
         int32_t c = *(volatile int32_t*)&key[h];
         if (c == AG_EMPTY) c = atomicCAS(&key[h], AG_EMPTY, a[q]);
         if (c == AG_EMPTY || c == a[q]) {
@@ -125,18 +126,18 @@ __global__ void __launch_bounds__(NT) k_ag_place(const int32_t* __restrict__ nl,
         }
         h = (h + 1) & (SLOTS - 1);
       }
-      if (slot[q] >= 0) at[q] = atomicAdd(&tot[slot[q]], at[q]);
+      if (slot[q] >= 0) at[q] = atomicAdd(&tot[slot[q]], (uint32_t)at[q]);
       else at[q] = atomicAdd(&taken[a[q]], at[q]);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < SLOTS; i += NT)
-      if (key[i] != AG_EMPTY) tot[i] = atomicAdd(&taken[key[i]], tot[i]);
+      if (key[i] != AG_EMPTY) base[i] = atomicAdd(&taken[key[i]], (unsigned long long)tot[i]);
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const int64_t v = v0 + q * NT + threadIdx.x;
       if (a[q] < 0) continue;
-      delta[v] = sstart[a[q]] + (int64_t)(at[q] + (slot[q] >= 0 ? tot[slot[q]] : 0)) - off[v];
+      delta[v] = sstart[a[q]] + (int64_t)(at[q] + (slot[q] >= 0 ? base[slot[q]] : 0)) - off[v];
     }
     __syncthreads();
   }

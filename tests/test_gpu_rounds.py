@@ -71,6 +71,17 @@ def test_hubs(degs, wmax, loops):
     assert np.array_equal(got[10], lab) and got[11] == lv and abs(got[12] - q) <= 1e-12 * max(1.0, abs(q))
 
 
+@pytest.mark.parametrize("n,k,p_in,p_out,wmax", [(4000, 4, "0.3", "0.02", 1), (4000, 1, "0.15", "0", 5), (3500, 40, "0.9", "0.08", 3)])
+def test_many_wide_rows(n, k, p_in, p_out, wmax):
+    # rows of 257 to 1,024 arcs in every CTA: few labels each, and so many that the warps' tables overflow
+    g = synth.sbm(n, k, p_in, p_out, seed=n + k, wmax=wmax)
+    got = check(g, {"max_iter": 12})
+    off, cols, w = g.numpy()
+    assert int((np.diff(off) > 256).sum()) == n
+    lab, moves, tr = oracle.local_move(off, cols, w, max_iter=12)
+    assert np.array_equal(got[3], lab) and got[4] == moves
+
+
 def test_hub_parameters():
     g = degrees_graph(6000, [5000, 1100, 1024], 8, 3)
     for params in ({"use_frontier": 0}, {"threshold": 40}, {"tie_keep_current": 0}, {"max_iter": 2}):
