@@ -270,6 +270,7 @@ struct RunOpts {
   int async_mode = 0;  // committed moves take effect at once (the coin still defers half of them)
   bool singleton_start = false;  // the run starts from C[v] = v (Sigma_tot = deg_w, sizes 1)
   bool device_loop = false;      // the round loop runs on the device where that is possible and pays
+  int share = 1;                 // a resident loop takes 1 / share of the GPU at most
   bool graph_loop = false;       // graphs with hubs: rounds after the first run as one captured graph (batched runs)
   bool device_loop_all = false;  // ... in every run
 };
@@ -286,7 +287,10 @@ int run_local_move(cd_graph* g, const RunOpts& o, int init_given, int64_t* moves
 RunOpts opts_from(const cd_params* p, int32_t level);
 // cd_params.device_loop of the server's workers when the caller left the
 // default: resident loops, but no captured graphs (several workers
-// instantiating graphs at once cost more than the read-backs they save).
+// instantiating graphs at once cost more than the read-backs they save). The
+// low bits hold the number of workers: a resident loop takes that share of the
+// GPU at most, so that the workers' loops run side by side. Loops that fill the
+// GPU run one after another, and most of a loop's time is latency.
 constexpr int32_t LOOP_NO_GRAPH = 0x10000;
 
 // rounds.cu: the whole round loop as one resident kernel (graphs without hubs).

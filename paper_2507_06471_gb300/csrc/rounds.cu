@@ -805,7 +805,7 @@ int loop_sms() {
 }
 
 template <bool LOUV, class W, class V, bool NK>
-int launch_loop(cd_graph* g, const ScanCtx& s, LoopCtx L) {
+int launch_loop(cd_graph* g, const ScanCtx& s, LoopCtx L, int share) {
   static std::atomic<int> resident{0};  // CTAs at once; the same for every thread that gets here
   auto kern = k_rounds<LOUV, W, V, NK>;
   constexpr size_t sm = loop_smem<V>();
@@ -817,7 +817,7 @@ int launch_loop(cd_graph* g, const ScanCtx& s, LoopCtx L) {
     r = std::max(1, per) * loop_sms();
     resident.store(r);
   }
-  const int64_t grid = std::max<int64_t>(1, std::min(std::min<int64_t>(r, L.n), g->nnz / ARCS_PER_CTA));
+  const int64_t grid = std::max<int64_t>(1, std::min(std::min<int64_t>(std::max(1, r / share), L.n), g->nnz / ARCS_PER_CTA));
   // the largest units that still give every CTA four
   L.lgu = 5;
   while (L.lgu > 0 && (L.n >> L.lgu) < 4 * grid) --L.lgu;
@@ -829,13 +829,13 @@ int launch_loop(cd_graph* g, const ScanCtx& s, LoopCtx L) {
 }
 
 template <bool LOUV, bool NK>
-int dispatch_loop(cd_graph* g, const ScanCtx& s, const LoopCtx& L) {
+int dispatch_loop(cd_graph* g, const ScanCtx& s, const LoopCtx& L, int share) {
   const bool v32 = g->max_degw < ((int64_t)1 << 32);
   if (g->wkind == W_UNIT)
-    return v32 ? launch_loop<LOUV, WUnit, uint32_t, NK>(g, s, L) : launch_loop<LOUV, WUnit, unsigned long long, NK>(g, s, L);
+    return v32 ? launch_loop<LOUV, WUnit, uint32_t, NK>(g, s, L, share) : launch_loop<LOUV, WUnit, unsigned long long, NK>(g, s, L, share);
   if (g->wkind == W_I32)
-    return v32 ? launch_loop<LOUV, WI32, uint32_t, NK>(g, s, L) : launch_loop<LOUV, WI32, unsigned long long, NK>(g, s, L);
-  return v32 ? launch_loop<LOUV, WI64, uint32_t, NK>(g, s, L) : launch_loop<LOUV, WI64, unsigned long long, NK>(g, s, L);
+    return v32 ? launch_loop<LOUV, WI32, uint32_t, NK>(g, s, L, share) : launch_loop<LOUV, WI32, unsigned long long, NK>(g, s, L, share);
+  return v32 ? launch_loop<LOUV, WI64, uint32_t, NK>(g, s, L, share) : launch_loop<LOUV, WI64, unsigned long long, NK>(g, s, L, share);
 }
 
 // The parts of the context the resident kernel uses (no hubs, no counters).
@@ -919,8 +919,8 @@ int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, i
     CD_LAUNCH(k_rounds_init<<<gi, PNT, 0, st>>>(L, g->C, g->sigma, g->csize, g->degw, louv ? 1 : 0, singletons ? 1 : 0,
                                                 words));
     const ScanCtx s = loop_ctx(g, o, louv, nk);
-    int r = !louv ? dispatch_loop<false, false>(g, s, L) : nk ? dispatch_loop<true, true>(g, s, L)
-                                                              : dispatch_loop<true, false>(g, s, L);
+    int r = !louv ? dispatch_loop<false, false>(g, s, L, o.share) : nk ? dispatch_loop<true, true>(g, s, L, o.share)
+                                                              : dispatch_loop<true, false>(g, s, L, o.share);
     if (r) return r;
     CD_CHECK(cudaGetLastError());
     // the header and the rounds of a usual run in one copy

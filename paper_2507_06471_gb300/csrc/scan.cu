@@ -2273,7 +2273,9 @@ RunOpts opts_from(const cd_params* p, int32_t level) {
   o.level = level;
   o.async_mode = p->asynchronous ? 1 : 0;
   o.device_loop = p->device_loop != 0;
-  o.graph_loop = p->device_loop != 0 && p->device_loop != LOOP_NO_GRAPH;
+  const bool served = p->device_loop > LOOP_NO_GRAPH && p->device_loop <= LOOP_NO_GRAPH + 64;
+  o.graph_loop = p->device_loop != 0 && !served;
+  o.share = served ? p->device_loop - LOOP_NO_GRAPH : 1;
   o.device_loop_all = p->device_loop == 2;
   return o;
 }

@@ -220,7 +220,7 @@ int cd_server_create(const cd_params* p, int32_t slots, int64_t mem_budget_bytes
   // by default (1) the workers' calls use resident loops but no captured
   // graphs: several workers capturing and instantiating round graphs at once
   // cost more than the round trips they save (2 still forces them)
-  if (s->params.device_loop == 1) s->params.device_loop = cd::LOOP_NO_GRAPH;
+  if (s->params.device_loop == 1) s->params.device_loop = cd::LOOP_NO_GRAPH + slots;
   cudaGetDevice(&s->device);
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
