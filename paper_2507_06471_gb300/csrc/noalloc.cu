@@ -97,6 +97,15 @@ __global__ void __launch_bounds__(NT) k_noalloc_pass(const int64_t* __restrict__
   unsigned long long my_in = 0, my_vol = 0;
   for (int64_t e0 = m0 + (tid >> 5) * piece; e0 < m1; e0 += (threads >> 5) * piece) {  // uniform in the warp
     const int64_t e1 = e0 + piece < m1 ? e0 + piece : m1;
+    int32_t un[4], xn[4];  // the next tile's columns and weights, in flight during this one's
+    auto load = [&](int64_t e) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        un[j] = e + j < e1 ? cols[e + j] : -1;
+        xn[j] = UNIT || e + j >= e1 ? 1 : w[e + j];
+      }
+    };
+    load(e0 + 4 * lane);
     int64_t cur = cd::warp_row_of(off, n, e0);
     for (int64_t ts = e0; ts < e1; ts += cd::WALK_TILE) {
       const int64_t e = ts + 4 * lane;
@@ -106,9 +115,10 @@ __global__ void __launch_bounds__(NT) k_noalloc_pass(const int64_t* __restrict__
       unsigned long long val[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        u[j] = e + j < e1 ? cols[e + j] : -1;
-        x[j] = UNIT || e + j >= e1 ? 1 : (long long)w[e + j];
+        u[j] = un[j];
+        x[j] = xn[j];
       }
+      if (ts + cd::WALK_TILE < e1) load(e + cd::WALK_TILE);
       cd::warp_tile_rows(off, n, ts, cur, mark[wid], row);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -190,11 +200,11 @@ extern "C" int cd_modularity_noalloc(const int64_t* off, const int32_t* cols, co
   if (rc) return rc;
   CD_CHECK(cudaMemsetAsync(scratch, 0, (size_t)(kCtlWords + n) * sizeof(unsigned long long), s));
   if (n > 0) {
-    // from 1,024 arcs or vertices a CTA up to one CTA per SM (latency), then 8,192 (each popular community
+    // from 1,024 arcs or vertices a CTA up to two CTAs per SM (latency), then 4,096 (each popular community
     // costs a CTA one atomic), 8 CTAs per SM at most
     const int64_t work = nnz > n ? nnz : n;
     int64_t blocks = (work + 1023) / 1024;
-    if (blocks > 152) blocks = work / 8192 < 152 ? 152 : work / 8192 < 152 * 8 ? work / 8192 : 152 * 8;
+    if (blocks > 304) blocks = work / 4096 < 304 ? 304 : work / 4096 < 152 * 8 ? work / 4096 : 152 * 8;
     const unsigned grid = (unsigned)blocks;
     if (w)
       CD_LAUNCH(k_noalloc_pass<false><<<grid, NT, 0, s>>>(off, cols, w, labels, n, nnz, scratch));
