@@ -79,9 +79,11 @@ __device__ __forceinline__ bool grid_meet(unsigned long long* word, unsigned add
     atomicAdd(word, (1ull << 48) | ((unsigned long long)hubs << 32) | add);
     unsigned long long x;
     int64_t polls = 0;
-    do {
+    for (;;) {
       asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(word) : "memory");
-    } while ((x >> 48) < gridDim.x && ++polls < WAIT_LIMIT);
+      if ((x >> 48) >= gridDim.x || ++polls >= WAIT_LIMIT) break;
+      __nanosleep(40);  // arrivals go to the same word
+    }
     if ((x >> 48) < gridDim.x) {
       atomicCAS(status, 0, CD_ETIMEOUT);
       x = ~0ull;
@@ -433,6 +435,69 @@ __device__ __forceinline__ void apply_moves(const ScanCtx& s, const LoopCtx& L, 
   }
 }
 
+// Step 1's sorting: the flagged ones of the CTA's vertices c0 .. c0 + NG PNT into
+// `list` by degree bin, with the bins' starts in first_of (cnt: vertices per
+// bin, zero before). False: none. A warp without one skips what follows, and so
+// does a group of 32 in it: late rounds have few, and this was most of a small
+// graph's instructions.
+template <int NG>
+__device__ __forceinline__ bool collect(const ScanCtx& s, const LoopCtx& L, const uint32_t* map, uint32_t c0,
+                                        uint32_t my_verts, int* cnt, int* start, int32_t* list,
+                                        int first_of[PBINS + 1]) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint32_t i0 = c0 + wid * NG * 32 + lane;
+  int32_t vk[NG];
+#pragma unroll
+  for (int k = 0; k < NG; ++k) {
+    vk[k] = -1;
+    const uint32_t i = i0 + 32 * k;
+    if (i - lane >= my_verts) continue;  // uniform in the warp
+    const uint32_t v = ((blockIdx.x + (i >> L.lgu) * gridDim.x) << L.lgu) + (i & ((1u << L.lgu) - 1u));
+    if (i < my_verts && v < (uint32_t)L.n) vk[k] = (int32_t)v;
+  }
+  if (map) {
+    uint32_t fw[NG];
+#pragma unroll
+    for (int k = 0; k < NG; ++k) fw[k] = vk[k] >= 0 ? __ldcg(map + (vk[k] >> 5)) : 0;
+#pragma unroll
+    for (int k = 0; k < NG; ++k)
+      if (!((fw[k] >> (vk[k] & 31)) & 1u)) vk[k] = -1;
+  }
+  unsigned some = 0;  // the groups of 32 with a flagged vertex
+#pragma unroll
+  for (int k = 0; k < NG; ++k) some |= __any_sync(FULL, vk[k] >= 0) ? 1u << k : 0u;
+  if (!__syncthreads_or(some != 0)) return false;
+  int slot[NG];  // bin << 16 | rank, -1: none
+#pragma unroll
+  for (int k = 0; k < NG; ++k) {
+    slot[k] = -1;
+    if (!((some >> k) & 1u)) continue;
+    if (vk[k] >= 0) {
+      const int32_t v = vk[k];
+      int64_t d = __ldg(s.off + v + 1) - __ldg(s.off + v);
+      if (s.gfrozen && s.gfrozen[s.gid[v]]) d = 0;
+      if (d > 0 && d <= L.t_hub) {  // hubs: by items
+        const int bin = d <= 4 ? 5 : d <= 8 ? 4 : d <= 16 ? 3 : d <= 32 ? 2 : d <= L.t_warp ? 1 : 0;
+        slot[k] = (bin << 16) | atomicAdd(&cnt[bin], 1);
+      }
+    }
+  }
+  __syncthreads();
+  first_of[0] = 0;
+#pragma unroll
+  for (int q = 0; q < PBINS; ++q) first_of[q + 1] = first_of[q] + cnt[q];
+  if (some) {
+#pragma unroll
+    for (int q = 0; q < PBINS; ++q)
+      if (lane == q) start[q] = first_of[q];
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < NG; ++k)
+      if (slot[k] >= 0) list[start[slot[k] >> 16] + (slot[k] & 0xffff)] = vk[k];
+  }
+  return true;
+}
+
 template <class V> constexpr size_t loop_smem() {
   return (size_t)PNW * PCAP * (sizeof(V) + 4 + 2) + (size_t)PNW * 32 * 8 + (size_t)CH_VERTS * 4;
 }
@@ -466,7 +531,6 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
   __syncthreads();
   // this CTA's units: blockIdx.x + i gridDim.x; its moves have room for all their vertices
   const int64_t G = gridDim.x, b = blockIdx.x;
-  const int U = 1 << L.lgu;
   const uint32_t my_verts = (uint32_t)(L.nunits / G + (b < L.nunits % G ? 1 : 0)) << L.lgu;
   const int64_t mv_at = (b * (L.nunits / G) + (b < L.nunits % G ? b : L.nunits % G)) << L.lgu;
   int32_t* mv = s.mv_v + mv_at;
@@ -506,63 +570,13 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
       hubs_here = rh_build<W, V>(s, L.rh, frontier ? cur_map : nullptr, half, keys0 + half * 4 * PCAP,
                                  vals0 + half * 4 * PCAP, occ0 + half * 4 * PCAP, &occ_n[half * 4]);
     for (uint32_t c0 = 0; c0 < my_verts; c0 += CH_VERTS) {
-      // the lane's vertices of this step, c0 + (wid CH_PER_WARP + k) 32 + lane of
-      // the CTA's: -1 where not flagged. A warp without one skips what follows,
-      // and so does a group of 32 in it: late rounds have few, and this sorting
-      // was most of a small graph's instructions.
-      const uint32_t i0 = (uint32_t)c0 + wid * CH_PER_WARP * 32 + lane;
-      int32_t vk[CH_PER_WARP];
-#pragma unroll
-      for (int k = 0; k < CH_PER_WARP; ++k) {
-        vk[k] = -1;
-        const uint32_t i = i0 + 32 * k;
-        if (i - lane >= my_verts) continue;  // uniform in the warp
-        const uint32_t v = (((uint32_t)b + (i >> L.lgu) * (uint32_t)G) << L.lgu) + (i & (U - 1));
-        if (i < my_verts && v < (uint32_t)L.n) vk[k] = (int32_t)v;
-      }
-      if (frontier) {
-        uint32_t fw[CH_PER_WARP];
-#pragma unroll
-        for (int k = 0; k < CH_PER_WARP; ++k) fw[k] = vk[k] >= 0 ? __ldcg(cur_map + (vk[k] >> 5)) : 0;
-#pragma unroll
-        for (int k = 0; k < CH_PER_WARP; ++k)
-          if (!((fw[k] >> (vk[k] & 31)) & 1u)) vk[k] = -1;
-      }
-      unsigned some = 0;  // the groups of 32 with a flagged vertex
-#pragma unroll
-      for (int k = 0; k < CH_PER_WARP; ++k) some |= __any_sync(FULL, vk[k] >= 0) ? 1u << k : 0u;
       int* cnt = bincnt[step & 1];
-      if (!__syncthreads_or(some != 0)) continue;
-      // degree bins, and the vertex's rank inside its bin
-      int slot[CH_PER_WARP];  // bin << 16 | rank, -1: none
-#pragma unroll
-      for (int k = 0; k < CH_PER_WARP; ++k) {
-        slot[k] = -1;
-        if (!((some >> k) & 1u)) continue;
-        if (vk[k] >= 0) {
-          const int32_t v = vk[k];
-          int64_t d = __ldg(s.off + v + 1) - __ldg(s.off + v);
-          if (s.gfrozen && s.gfrozen[s.gid[v]]) d = 0;
-          if (d > 0 && d <= L.t_hub) {  // hubs: by items
-            const int bin = d <= 4 ? 5 : d <= 8 ? 4 : d <= 16 ? 3 : d <= 32 ? 2 : d <= L.t_warp ? 1 : 0;
-            slot[k] = (bin << 16) | atomicAdd(&cnt[bin], 1);
-          }
-        }
-      }
-      __syncthreads();
       int first_of[PBINS + 1];  // where each bin starts in the list
-      first_of[0] = 0;
-#pragma unroll
-      for (int q = 0; q < PBINS; ++q) first_of[q + 1] = first_of[q] + cnt[q];
-      if (some) {
-#pragma unroll
-        for (int q = 0; q < PBINS; ++q)
-          if (lane == q) start[wid][q] = first_of[q];
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < CH_PER_WARP; ++k)
-          if (slot[k] >= 0) list[start[wid][slot[k] >> 16] + (slot[k] & 0xffff)] = vk[k];
-      }
+      const bool any = my_verts - c0 <= PNT
+                           ? collect<1>(s, L, frontier ? cur_map : nullptr, c0, my_verts, cnt, start[wid], list, first_of)
+                           : collect<CH_PER_WARP>(s, L, frontier ? cur_map : nullptr, c0, my_verts, cnt, start[wid], list,
+                                                  first_of);
+      if (!any) continue;
       if (tid < 8) bincnt[(step + 1) & 1][tid] = 0;  // the next step's
       __syncthreads();
       // half CTAs
