@@ -40,6 +40,45 @@ __global__ void k_fix_unused(const uint8_t* __restrict__ used, int64_t n, int32_
     if (!used[c]) newid[c] = -1;
 }
 
+// Renumbering of at most RN_SMALL communities in one launch (one CTA): used
+// flags in shared memory, their exclusive scan, -1 for unused ids.
+constexpr int RN_SMALL = 8192;
+__global__ void __launch_bounds__(1024) k_renumber_small(const int32_t* __restrict__ labels, int n, int32_t* newid,
+                                                         int64_t* total) {
+  __shared__ uint8_t used[RN_SMALL];
+  __shared__ int wsum[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  constexpr int PER = RN_SMALL / 1024;
+  for (int i = threadIdx.x; i < RN_SMALL / 4; i += 1024) ((uint32_t*)used)[i] = 0;
+  __syncthreads();
+  for (int v = threadIdx.x; v < n; v += 1024) used[labels[v]] = 1;
+  __syncthreads();
+  int mine = 0;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) mine += used[threadIdx.x * PER + j];
+  int inc = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(FULL, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) wsum[wid] = inc;
+  __syncthreads();
+  int before = 0, all = 0;
+  for (int w = 0; w < 32; ++w) {
+    if (w < wid) before += wsum[w];
+    all += wsum[w];
+  }
+  int at = before + inc - mine;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int c = threadIdx.x * PER + j;
+    if (c < n) newid[c] = used[c] ? at : -1;
+    at += used[c];
+  }
+  if (threadIdx.x == 0) *total = all;
+}
+
 // Warp per vertex: one (key, weight) pair per arc.
 template <class W>
 __global__ void __launch_bounds__(NT) k_agg_emit(const int64_t* __restrict__ off,
@@ -205,13 +244,15 @@ int renumber(cd_graph* g, const int32_t* labels_dev, int32_t* newid_dev, int64_t
   }
   uint8_t* used = nullptr;
   int64_t* total = nullptr;
-  int rc = dev_alloc_t(&used, n, s);
-  if (!rc) rc = dev_alloc_t(&total, 1, s);
-  if (rc) {
-    dev_free(used, s);
-    return rc;
-  }
-  {
+  Arena scratch;
+  scratch.add(&total, 1);
+  scratch.add(&used, n > RN_SMALL ? n : 1);
+  int rc = scratch.make(s);
+  if (rc) return rc;
+  if (n <= RN_SMALL) {
+    KTimer t(g, K_RENUMBER, (double)n * (4 + 1 + 1 + 4 + 1));
+    CD_LAUNCH(k_renumber_small<<<1, 1024, 0, s>>>(labels_dev, (int)n, newid_dev, total));
+  } else {
     KTimer t(g, K_RENUMBER, (double)n * (4 + 1 + 1 + 4 + 1));
     CD_CHECK(cudaMemsetAsync(used, 0, n, s));
     CD_LAUNCH(k_mark_used<<<grid_cap((n + NT - 1) / NT), NT, 0, s>>>(labels_dev, n, used));
@@ -224,8 +265,7 @@ int renumber(cd_graph* g, const int32_t* labels_dev, int32_t* newid_dev, int64_t
     *k_out = k;
   else if (!rc)
     rc = set_cuda_error(cudaGetLastError());
-  dev_free(used, s);
-  dev_free(total, s);
+  scratch.free(s);
   return rc;
 }
 
@@ -327,18 +367,13 @@ int modularity(cd_graph* g, const int32_t* labels_dev, double* q_out) {
     if (!rc) *q_out = 0.0;
     return rc;
   }
-  unsigned long long *volc = nullptr, *acc = nullptr;
-  int rc = dev_alloc_t(&volc, n, s);
-  if (!rc) rc = dev_alloc_t(&acc, 4, s);
-  if (rc) {
-    dev_free(volc, s);
-    return rc;
-  }
+  unsigned long long* acc = nullptr;  // 4 words, then the communities' volumes: cleared together
+  if (int rc = dev_alloc_t(&acc, 4 + n, s)) return rc;
+  unsigned long long* volc = acc + 4;
   {
     const int wbytes = g->wkind == W_UNIT ? 0 : g->wkind == W_I32 ? 4 : 8;
     KTimer t(g, K_MODULARITY, (double)n * (8 + 4 + 4 + 8 + 8 + 8) + (double)g->nnz * (4 + 4 + wbytes));
-    cudaMemsetAsync(volc, 0, n * 8, s);
-    cudaMemsetAsync(acc, 0, 4 * 8, s);
+    cudaMemsetAsync(acc, 0, (4 + n) * 8, s);
     CD_LAUNCH(k_mod_vol<<<grid_cap((n + NT - 1) / NT, 152 * 8), NT, 0, s>>>(labels_dev, g->degw, n, volc, acc));
     CD_LAUNCH(k_mod_sq<<<grid_cap((n + NT - 1) / NT, 152 * 4), NT, 0, s>>>(volc, n, acc));
     const int64_t m = g->nnz;
@@ -355,7 +390,6 @@ int modularity(cd_graph* g, const int32_t* labels_dev, double* q_out) {
   CD_CHECK(cudaGetLastError());
   CD_CHECK(cudaMemcpyAsync(h, acc, sizeof(h), cudaMemcpyDeviceToHost, s));
   CD_CHECK(cudaStreamSynchronize(s));
-  dev_free(volc, s);
   dev_free(acc, s);
   if (h[3]) return CD_EINVAL;
   const unsigned __int128 S = ((unsigned __int128)h[1] << 64) | h[0];

@@ -179,10 +179,11 @@ struct cd_graph {
   int t_hub = cd::BLOCK_MAX;       // degrees t_warp+1..t_hub: 128 threads (512 above 1024); above: hub
   bool bins_set = false;           // thresholds chosen by cd_graph_set_bins / cd_autotune (kept by coarse graphs)
 
-  // run state (allocated on first use)
+  // run state (one allocation, made on first use; the pointers below are parts of it)
+  void* run_mem = nullptr;
   int32_t* C = nullptr;
   int64_t* sigma = nullptr;
-  uint32_t* sigma32 = nullptr;  // 32-bit copy for the gathers (allocated on first use)
+  uint32_t* sigma32 = nullptr;  // 32-bit copy for the gathers
   int32_t* csize = nullptr;
   uint32_t* flag[2] = {nullptr, nullptr};  // needCheck / tmpNeedCheck bitmaps (n bits each)
 
@@ -232,6 +233,27 @@ template <class T>
 int dev_alloc_t(T** p, int64_t count, cudaStream_t s) {
   return dev_alloc((void**)p, (size_t)(count > 0 ? count : 1) * sizeof(T), s);
 }
+// Several arrays from one allocation: small graphs spend a microsecond on each
+// allocation and each release. add() every array, then make() sets the pointers.
+struct Arena {
+  std::vector<std::pair<void**, size_t>> parts;
+  size_t bytes = 0;
+  void* mem = nullptr;
+  template <class T>
+  void add(T** p, int64_t count) {
+    parts.push_back({(void**)p, bytes});
+    bytes += ((size_t)(count > 0 ? count : 1) * sizeof(T) + 255) / 256 * 256;
+  }
+  int make(cudaStream_t s) {
+    const int rc = dev_alloc(&mem, bytes, s);
+    for (auto& x : parts) *x.first = rc ? nullptr : (char*)mem + x.second;
+    return rc;
+  }
+  void free(cudaStream_t s) {
+    dev_free(mem, s);
+    mem = nullptr;
+  }
+};
 
 // profiling helpers: bracket a launch with events when per-kernel timing is on
 struct KTimer {
@@ -247,11 +269,24 @@ void profile_reset(cd_graph* g);
 int profile_flush(cd_graph* g);  // syncs, accumulates pending events
 
 // graph.cu
+// Degree bin of a row of d > 0 arcs.
+__host__ __device__ __forceinline__ int bin_of(int64_t d, int t_warp = WARP_MAX, int t_hub = BLOCK_MAX) {
+  if (d <= 4) return B_T4;
+  if (d <= 8) return B_T8;
+  if (d <= 16) return B_T16;
+  if (d <= 32) return B_T32;
+  if (d <= t_warp) return B_WARP;
+  if (d > t_hub) return B_HUB;
+  return d <= BLK1_MAX ? B_BLK1 : B_BLK4;
+}
+// bins_pre: NBINS + 1 words, the vertices per degree bin for the thresholds of `like` (or the defaults) and the arcs
+// of the hubs, if the caller counted them.
 constexpr int INGEST_STATS = 5 + NBINS;  // words of the ingest statistics: [0] vol, [2] isolated, [3] largest deg_w, ...
 // Takes ownership of device arrays in the internal convention (loop arcs 2L).
 int graph_adopt(cudaStream_t s, int64_t n, int64_t nnz, int64_t* off, int32_t* cols, void* w,
                 int wkind, cd_graph** out, int64_t* degw_pre = nullptr,
-                const unsigned long long* stats_pre = nullptr, const cd_graph* like = nullptr);
+                const unsigned long long* stats_pre = nullptr, const cd_graph* like = nullptr,
+                const unsigned long long* bins_pre = nullptr);
 int ensure_run_state(cd_graph* g);
 int ensure_bins(cd_graph* g);  // bin lists and hub structures of the per-round kernels
 int ensure_resident_hubs(cd_graph* g);

@@ -109,16 +109,6 @@ constexpr int NSTATS = INGEST_STATS;
 
 __device__ __forceinline__ void fail(int32_t* status, int code) { atomicCAS(status, 0, code); }
 
-__device__ __forceinline__ int bin_of(int64_t d, int t_warp = WARP_MAX, int t_hub = BLOCK_MAX) {
-  if (d <= 4) return B_T4;
-  if (d <= 8) return B_T8;
-  if (d <= 16) return B_T16;
-  if (d <= 32) return B_T32;
-  if (d <= t_warp) return B_WARP;
-  if (d > t_hub) return B_HUB;
-  return d <= BLK1_MAX ? B_BLK1 : B_BLK4;
-}
-
 // counts[NBINS]: arcs of the hubs.
 __global__ void k_bin_count(const int64_t* __restrict__ off, int64_t n, int t_warp, int t_hub,
                             unsigned long long* counts) {
@@ -200,13 +190,13 @@ __global__ void __launch_bounds__(1024) k_rh_layout(const int64_t* __restrict__ 
   }
 }
 
+// `in` may be `out` (64-bit offsets are checked where they were copied to).
 template <class OffT>
-__global__ void k_offsets_check(const OffT* __restrict__ in, int64_t n, int64_t nnz,
-                                int64_t* __restrict__ out, int32_t* status) {
+__global__ void k_offsets_check(const OffT* in, int64_t n, int64_t nnz, int64_t* out, int32_t* status) {
   int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= n; i += stride) {
     int64_t a = (int64_t)in[i];
-    out[i] = a;
+    if (sizeof(OffT) != 8) out[i] = a;
     if (a < 0 || a > nnz) fail(status, CD_ENOTSYM);
     if (i < n && (int64_t)in[i + 1] < a) fail(status, CD_ENOTSYM);
     if (i == 0 && a != 0) fail(status, CD_ENOTSYM);
@@ -504,11 +494,8 @@ void free_arrays(cd_graph* g) {
                 g->hub_mv,       g->hub_rb,       g->hub_used,     g->hub_item_first,
                 g->hub_flist,    g->hub_fcnt,     g->hub_cl,       g->hub_ccnt,
                 g->hub_nl,       g->hub_nc,       g->hub_pl,
-                g->hub_blist,    g->hub_mlist,     g->hub_lcnt,     g->C,            g->sigma,        g->csize,
-                g->hub_log,
-                g->sigma32,
-                g->flag[0],      g->flag[1],       g->mv_v,
-                g->ctr,          g->status,        g->gid,          g->gbase,        g->gvol,
+                g->hub_blist,    g->hub_mlist,     g->hub_lcnt,     g->hub_log,
+                g->run_mem,      g->status,        g->gid,          g->gbase,        g->gvol,
                 g->gfrozen,      g->gcnt};
   for (void* p : ps) dev_free(p, s);
   if (g->h_ctr) cudaFreeHost(g->h_ctr);
@@ -575,15 +562,24 @@ void free_bins(cd_graph* g) {
 
 int build_bins(cd_graph* g);
 
+void take_bins(cd_graph* g, const unsigned long long* cnt) {
+  g->bin_start[0] = 0;
+  for (int b = 0; b < NBINS; ++b) g->bin_start[b + 1] = g->bin_start[b] + (int64_t)cnt[b];
+  g->nhubs = (int64_t)cnt[B_HUB];
+  g->hub_arcs = (int64_t)cnt[NBINS];
+}
+
 // Scalars, bins and hub structures of a graph whose CSR, weights and deg_w
 // are in place; stats from k_ingest.
-int finish_graph(cd_graph* g, const unsigned long long* stats) {
+int finish_graph(cd_graph* g, const unsigned long long* stats, const unsigned long long* bins) {
   g->cols_distinct = stats[ST_UNSORTED] == 0;  // strictly increasing rows; aggregation sets it for coarse rows
   g->vol = (int64_t)stats[0];
   g->n_isolated = (int64_t)stats[2];
   g->max_degw = (int64_t)stats[3];
   if (stats[0] >= (1ull << 62)) return CD_EOVERFLOW;
-  return build_bins(g);
+  if (!bins) return build_bins(g);
+  take_bins(g, bins);
+  return CD_OK;
 }
 
 // Vertices per degree bin for (t_warp, t_hub).
@@ -599,10 +595,7 @@ int build_bins(cd_graph* g) {
   CD_CHECK(cudaMemcpyAsync(h_cnt, d_cnt, sizeof(h_cnt), cudaMemcpyDeviceToHost, s));
   CD_CHECK(cudaStreamSynchronize(s));
   dev_free(d_cnt, s);
-  g->bin_start[0] = 0;
-  for (int b = 0; b < NBINS; ++b) g->bin_start[b + 1] = g->bin_start[b] + (int64_t)h_cnt[b];
-  g->nhubs = (int64_t)h_cnt[B_HUB];
-  g->hub_arcs = (int64_t)h_cnt[NBINS];
+  take_bins(g, h_cnt);
   return CD_OK;
 }
 
@@ -745,21 +738,17 @@ int fill_bins(cd_graph* g) {
   return CD_OK;
 }
 
-int ingest(cd_graph* g, int loops_twice, unsigned long long* stats_host) {
+int ingest(cd_graph* g, int loops_twice, unsigned long long* stats_host, int32_t* status_host) {
   cudaStream_t s = g->stream;
-  unsigned long long* d_stats = nullptr;
-  int rc = dev_alloc_t(&d_stats, NSTATS, s);
-  if (rc) return rc;
-  CD_CHECK(cudaMemsetAsync(d_stats, 0, (NSTATS) * sizeof(unsigned long long), s));
-  int32_t* big = nullptr;
-  unsigned long long* nbig = nullptr;
   const int64_t big_cap = g->nnz / (INGEST_WARP + 1) + 1;  // rows longer than INGEST_WARP arcs, at most
-  if ((rc = dev_alloc_t(&big, big_cap, s)) || (rc = dev_alloc_t(&nbig, 1, s))) {
-    dev_free(big, s);
-    dev_free(d_stats, s);
-    return rc;
-  }
-  CD_CHECK(cudaMemsetAsync(nbig, 0, sizeof(unsigned long long), s));
+  unsigned long long* d_stats = nullptr;  // the statistics, then the number of listed rows
+  int32_t* big = nullptr;
+  Arena scratch;
+  scratch.add(&d_stats, NSTATS + 1);
+  scratch.add(&big, big_cap);
+  if (int rc = scratch.make(s)) return rc;
+  unsigned long long* nbig = d_stats + NSTATS;
+  CD_CHECK(cudaMemsetAsync(d_stats, 0, (NSTATS + 1) * sizeof(unsigned long long), s));
   {
     KTimer t(g, K_UPLOAD, (double)g->nnz * (4 + (g->wkind == W_I32 ? 4 : g->wkind == W_I64 ? 8 : 0)) +
                               (double)g->n * 16);
@@ -781,12 +770,11 @@ int ingest(cd_graph* g, int loops_twice, unsigned long long* stats_host) {
 #undef CD_INGEST
     }
   }
-  dev_free(big, s);
-  dev_free(nbig, s);
   CD_CHECK(cudaGetLastError());
   CD_CHECK(cudaMemcpyAsync(stats_host, d_stats, (NSTATS) * sizeof(unsigned long long),
                            cudaMemcpyDeviceToHost, s));
-  dev_free(d_stats, s);
+  CD_CHECK(cudaMemcpyAsync(status_host, g->status, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  scratch.free(s);
   CD_CHECK(cudaStreamSynchronize(s));
   return CD_OK;
 }
@@ -870,18 +858,21 @@ int ensure_resident_hubs(cd_graph* g) {
 
 int ensure_run_state(cd_graph* g) {
   if (g->C) return CD_OK;
-  cudaStream_t s = g->stream;
-  int rc;
-  if ((rc = dev_alloc_t(&g->C, g->n, s))) return rc;
-  if ((rc = dev_alloc_t(&g->sigma, g->n, s))) return rc;
-  if ((rc = dev_alloc_t(&g->csize, g->n, s))) return rc;
-  if ((rc = dev_alloc_t(&g->flag[0], (g->n + 31) / 32 + 1, s))) return rc;
-  if ((rc = dev_alloc_t(&g->flag[1], (g->n + 31) / 32 + 1, s))) return rc;
   const int64_t n32 = (g->n + 31) / 32 * 32;
-  if ((rc = dev_alloc_t(&g->mv_v, 3 * n32, s))) return rc;
+  Arena a;
+  a.add(&g->C, g->n);
+  a.add(&g->sigma, g->n);
+  a.add(&g->csize, g->n);
+  a.add(&g->sigma32, g->vol < ((int64_t)1 << 31) ? g->n : 1);
+  a.add(&g->flag[0], n32 / 32 + 1);
+  a.add(&g->flag[1], n32 / 32 + 1);
+  a.add(&g->mv_v, 3 * n32);
+  a.add(&g->ctr, C_COUNT);
+  const int rc = a.make(g->stream);
+  if (rc) return rc;
+  g->run_mem = a.mem;
   g->mv_c = g->mv_v + n32;
   g->mv_a = g->mv_v + 2 * n32;
-  if ((rc = dev_alloc_t(&g->ctr, C_COUNT, s))) return rc;
   return CD_OK;
 }
 
@@ -898,7 +889,7 @@ int check_labels(cd_graph* g, const int32_t* labels_dev) {
 // too; otherwise deg_w is computed as the plain row sum.
 int graph_adopt(cudaStream_t s, int64_t n, int64_t nnz, int64_t* off, int32_t* cols, void* w,
                 int wkind, cd_graph** out, int64_t* degw_pre, const unsigned long long* stats_pre,
-                const cd_graph* like) {
+                const cd_graph* like, const unsigned long long* bins_pre) {
   cd_graph* g = new cd_graph();
   if (like) {
     g->t_warp = like->t_warp;
@@ -906,6 +897,7 @@ int graph_adopt(cudaStream_t s, int64_t n, int64_t nnz, int64_t* off, int32_t* c
     g->bins_set = like->bins_set;
     if (!g->bins_set && nnz >= COARSE_HUB_ARCS && g->t_hub > COARSE_T_HUB && g->t_warp <= COARSE_T_HUB)
       g->t_hub = COARSE_T_HUB;
+    if (g->t_hub != like->t_hub) bins_pre = nullptr;  // counted for the other threshold
   }
   g->stream = s;
   g->n = n;
@@ -923,11 +915,9 @@ int graph_adopt(cudaStream_t s, int64_t n, int64_t nnz, int64_t* off, int32_t* c
     memcpy(stats, stats_pre, sizeof(stats));
   } else {
     if (!rc) rc = dev_alloc_t(&g->degw, n, s);
-    if (!rc) rc = ingest(g, 0, stats);
-    if (!rc) {
-      int st = read_status(g);
-      if (st) rc = st;
-    }
+    int32_t st = 0;
+    if (!rc) rc = ingest(g, 0, stats, &st);
+    if (!rc) rc = st;
   }
   // 64-bit weights whose every row sum (loops doubled included) is below 2^31
   // are kept in 32 bits: every arc weight is at most its row's deg_w
@@ -941,7 +931,7 @@ int graph_adopt(cudaStream_t s, int64_t n, int64_t nnz, int64_t* off, int32_t* c
       g->wkind = W_I32;
     }
   }
-  if (!rc) rc = finish_graph(g, stats);
+  if (!rc) rc = finish_graph(g, stats, bins_pre);
   if (rc) {
     free_arrays(g);
     delete g;
@@ -1013,7 +1003,7 @@ int cd_csr_upload(const void* offsets, int offsets_is_i64, const int32_t* cols, 
   if (!rc && cudaMemsetAsync(d_cols + nnz, 0, COL_PAD * sizeof(int32_t), s) != cudaSuccess) rc = CD_ECUDA;
   if (!rc && w) rc = dev_alloc_t(&d_w, nnz, s);
   size_t ob = (size_t)(n + 1) * (offsets_is_i64 ? 8 : 4);
-  if (!rc) rc = dev_alloc(&d_off_in, ob, s);
+  if (!rc && !offsets_is_i64) rc = dev_alloc(&d_off_in, ob, s);
   auto cleanup = [&]() {
     dev_free(d_cols, s);
     dev_free(d_off, s);
@@ -1026,7 +1016,7 @@ int cd_csr_upload(const void* offsets, int offsets_is_i64, const int32_t* cols, 
     return rc;
   }
   if (cudaMemsetAsync(tmp.status, 0, 4, s) != cudaSuccess ||
-      cudaMemcpyAsync(d_off_in, offsets, ob, kind, s) != cudaSuccess ||
+      cudaMemcpyAsync(offsets_is_i64 ? (void*)d_off : d_off_in, offsets, ob, kind, s) != cudaSuccess ||
       (nnz > 0 && cudaMemcpyAsync(d_cols, cols, (size_t)nnz * 4, kind, s) != cudaSuccess) ||
       (w && nnz > 0 && cudaMemcpyAsync(d_w, w, (size_t)nnz * 4, kind, s) != cudaSuccess)) {
     int e = set_cuda_error(cudaGetLastError());
@@ -1034,7 +1024,7 @@ int cd_csr_upload(const void* offsets, int offsets_is_i64, const int32_t* cols, 
     return e;
   }
   if (offsets_is_i64)
-    CD_LAUNCH(k_offsets_check<int64_t><<<grid_for(n + 1), NT, 0, s>>>((const int64_t*)d_off_in, n, nnz, d_off,
+    CD_LAUNCH(k_offsets_check<int64_t><<<grid_for(n + 1), NT, 0, s>>>(d_off, n, nnz, d_off,
                                                             tmp.status));
   else
     CD_LAUNCH(k_offsets_check<int32_t><<<grid_for(n + 1), NT, 0, s>>>((const int32_t*)d_off_in, n, nnz, d_off,
@@ -1059,10 +1049,8 @@ int cd_csr_upload(const void* offsets, int offsets_is_i64, const int32_t* cols, 
   tmp.wkind = d_w ? W_I32 : W_UNIT;
   rc = dev_alloc_t(&tmp.degw, n, s);
   unsigned long long stats[NSTATS] = {};
-  if (!rc) rc = ingest(&tmp, 1, stats);
-  if (!rc && cudaMemcpyAsync(&st, tmp.status, 4, cudaMemcpyDeviceToHost, s) == cudaSuccess &&
-      cudaStreamSynchronize(s) == cudaSuccess && st)
-    rc = st;
+  if (!rc) rc = ingest(&tmp, 1, stats, &st);
+  if (!rc) rc = st;
   dev_free(tmp.status, s);
   tmp.status = nullptr;
   if (rc) {
@@ -1093,7 +1081,11 @@ int cd_csr_upload(const void* offsets, int offsets_is_i64, const int32_t* cols, 
     wint = w64;
     wk = W_I64;
   }
-  return graph_adopt(s, n, nnz, d_off, d_cols, wint, wk, out, tmp.degw, stats);
+  // the ingest counted the degree bins, but not the arcs of the hubs
+  unsigned long long bins[NBINS + 1] = {};
+  for (int b = 0; b < NBINS; ++b) bins[b] = stats[4 + b];
+  return graph_adopt(s, n, nnz, d_off, d_cols, wint, wk, out, tmp.degw, stats, nullptr,
+                     bins[B_HUB] == 0 ? bins : nullptr);
 }
 
 int cd_graph_free(cd_graph* g) {

@@ -29,6 +29,7 @@
 // The content of every row equals that of the sort-based aggregation; only the
 // order of columns inside a row differs, and no later step depends on it.
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "common.cuh"
@@ -554,32 +555,38 @@ __global__ void __launch_bounds__(NT) k_ag_extract(const int32_t* __restrict__ o
 
 // ------------------------------------------------------------------ coarse CSR
 
-// delta[A] = (start of A's segment) - (start of its coarse row); the number of empty rows.
+// delta[A] = (start of A's segment) - (start of its coarse row); stat: the number
+// of empty rows, the largest deg_w, the rows per degree bin and the hubs' arcs.
 __global__ void __launch_bounds__(NT) k_ag_rows(const int64_t* __restrict__ sstart, const int64_t* __restrict__ coff,
                                                 int64_t k, int64_t* __restrict__ delta, const unsigned long long* cdegw,
-                                                unsigned long long* stat) {
-  __shared__ unsigned long long s_max;
-  __shared__ int s_iso;
-  if (threadIdx.x == 0) {
-    s_max = 0;
-    s_iso = 0;
-  }
+                                                int t_warp, int t_hub, unsigned long long* stat) {
+  __shared__ unsigned long long s_max, s_hub;
+  __shared__ int s_bin[NBINS + 1];  // [NBINS]: empty
+  if (threadIdx.x <= NBINS) s_bin[threadIdx.x] = 0;
+  if (threadIdx.x == 0) s_max = s_hub = 0;
   __syncthreads();
-  int iso = 0;
   unsigned long long mx = 0;
   const int64_t stride = (int64_t)gridDim.x * NT;
   for (int64_t a = (int64_t)blockIdx.x * NT + threadIdx.x; a < k; a += stride) {
-    const int64_t c = coff[a];
+    const int64_t c = coff[a], d = coff[a + 1] - c;
     delta[a] = sstart[a] - c;
-    if (coff[a + 1] == c) ++iso;
+    const int b = d == 0 ? NBINS : bin_of(d, t_warp, t_hub);
+    atomicAdd(&s_bin[b], 1);
+    if (b == B_HUB) atomicAdd(&s_hub, (unsigned long long)d);
     mx = cdegw[a] > mx ? cdegw[a] : mx;
   }
-  if (iso) atomicAdd(&s_iso, iso);
-  if (mx) atomicMax(&s_max, mx);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long y = __shfl_xor_sync(FULL, mx, o);
+    mx = y > mx ? y : mx;
+  }
+  if ((threadIdx.x & 31) == 0 && mx) atomicMax(&s_max, mx);
   __syncthreads();
+  if (threadIdx.x < NBINS && s_bin[threadIdx.x]) atomicAdd(&stat[2 + threadIdx.x], (unsigned long long)s_bin[threadIdx.x]);
   if (threadIdx.x == 0) {
-    if (s_iso) atomicAdd(&stat[0], (unsigned long long)s_iso);
+    if (s_bin[NBINS]) atomicAdd(&stat[0], (unsigned long long)s_bin[NBINS]);
     if (s_max) atomicMax(&stat[1], s_max);
+    if (s_hub) atomicAdd(&stat[2 + NBINS], s_hub);
   }
 }
 
@@ -634,18 +641,20 @@ int aggregate_as(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_de
   const int64_t n = g->n, m = g->nnz;
   int rc = CD_OK;
   // scratch
-  int32_t *nl = nullptr, *ab = nullptr, *lists = nullptr, *ch_seg = nullptr, *dch = nullptr, *tlg = nullptr;
-  int32_t *owner = nullptr, *gk = nullptr;
-  int64_t *delta = nullptr, *sstart = nullptr, *ch_off = nullptr, *toff = nullptr, *ucnt = nullptr;
-  unsigned long long *arcs = nullptr, *cnt = nullptr, *ub = nullptr, *gs = nullptr;
-  V* aw = nullptr;
+  Arena scratch;
+  int32_t *nl, *ab, *t8, *t32, *wl, *cl, *ll, *ch_seg, *dch, *tlg, *owner = nullptr, *gk = nullptr;
+  int64_t *delta, *sstart, *ch_off, *toff, *ucnt;
+  unsigned long long *arcs, *cnt, *ub, *gs = nullptr;
+  V* aw;
   // the coarse graph
   int64_t *coarse_off = nullptr, *cdegw = nullptr;
   int32_t* ccols = nullptr;
   void* cw = nullptr;
   auto cleanup = [&]() {
-    void* ps[] = {nl, ab, lists, ch_seg, dch, tlg, owner, gk, delta, sstart, ch_off, toff, arcs, cnt, ub, gs, aw};
-    for (void* p : ps) dev_free(p, s);
+    scratch.free(s);
+    dev_free(gs, s);
+    dev_free(gk, s);
+    dev_free(owner, s);
   };
   auto fail = [&](int r) {
     cleanup();
@@ -658,22 +667,33 @@ int aggregate_as(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_de
   const int64_t max_big = m / (AG_CTA_MAX + 1) + 1;           // large segments at most
   const int64_t max_chunks = m / AG_CHUNK + max_big;          // their chunks at most
   const int64_t max_cta = m / (AG_WARP_MAX + 1) + 1;          // CTA segments at most
-  const int64_t max_warp = std::min(k, m / 33 + 1), max_t32 = std::min(k, m / 9 + 1), max_t8 = std::min(k, m + 1);
-  if ((rc = dev_alloc_t(&nl, n, s)) || (rc = dev_alloc_t(&delta, std::max(n, k), s)) ||
-      (rc = dev_alloc_t(&arcs, 2 * k, s)) || (rc = dev_alloc_t(&cdegw, k, s)) ||
-      (rc = dev_alloc_t(&sstart, k + 1, s)) || (rc = dev_alloc_t(&cnt, AC_N + 2, s)) ||
-      (rc = dev_alloc_t(&ab, m, s)) || (rc = dev_alloc_t(&aw, m, s)) ||
-      (rc = dev_alloc_t(&lists, max_t8 + max_t32 + max_warp + max_cta + max_big, s)) ||
-      (rc = dev_alloc_t(&ch_seg, max_chunks, s)) || (rc = dev_alloc_t(&ch_off, max_chunks, s)) ||
-      (rc = dev_alloc_t(&dch, max_chunks, s)) || (rc = dev_alloc_t(&coarse_off, k + 1, s)))
+  const bool big = m > AG_CTA_MAX;                            // there may be large segments
+  scratch.add(&nl, n);
+  scratch.add(&delta, std::max(n, k));
+  scratch.add(&arcs, 3 * k);  // arcs per community, distinct entries, upper bounds: cleared together
+  scratch.add(&sstart, k + 1);
+  scratch.add(&cnt, AC_N + 2 + NBINS + 1);
+  scratch.add(&ab, m);
+  scratch.add(&aw, m);
+  scratch.add(&t8, std::min(k, m + 1));
+  scratch.add(&t32, std::min(k, m / 9 + 1));
+  scratch.add(&wl, std::min(k, m / 33 + 1));
+  scratch.add(&cl, max_cta);
+  scratch.add(&ll, max_big);
+  scratch.add(&ch_seg, max_chunks);
+  scratch.add(&ch_off, max_chunks);
+  scratch.add(&dch, max_chunks);
+  scratch.add(&tlg, big ? k : 1);
+  scratch.add(&toff, big ? k : 1);
+  if ((rc = scratch.make(s)) || (rc = dev_alloc_t(&cdegw, k, s)) || (rc = dev_alloc_t(&coarse_off, k + 1, s)))
     return fail(rc);
-  ucnt = (int64_t*)arcs + k;  // one array, cleared together
-  int32_t *t8 = lists, *t32 = t8 + max_t8, *wl = t32 + max_t32, *cl = wl + max_warp, *ll = cl + max_cta;
+  ucnt = (int64_t*)arcs + k;
+  ub = arcs + 2 * k;
   const int wbytes = g->wkind == W_UNIT ? 0 : g->wkind == W_I32 ? 4 : 8;
   const unsigned gv = gcap((n + NT - 1) / NT, 152 * 8);
   {
     KTimer t(g, K_AGG_EMIT, (double)n * (4 + 4 + 8 + 8 + 4 + 8) + (double)m * (4 + 4 + wbytes + 4 + sizeof(V)));
-    AG_CHECK(cudaMemsetAsync(arcs, 0, 2 * k * 8, s));
+    AG_CHECK(cudaMemsetAsync(arcs, 0, 3 * k * 8, s));
     AG_CHECK(cudaMemsetAsync(cdegw, 0, k * 8, s));
     CD_LAUNCH(k_ag_vertex<<<gv, NT, 0, s>>>(labels_dev, newid_dev, g->off, g->degw, n, nl, arcs,
                                             (unsigned long long*)cdegw));
@@ -691,19 +711,17 @@ int aggregate_as(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_de
         CD_LAUNCH((k_ag_scatter<WI64, V><<<gr, NT, 0, s>>>(g->off, g->cols, g->w, n, m, piece, nl, delta, ab, aw)));
     }
   }
-  unsigned long long h[AC_N + 2] = {};  // the counts; then empty rows, largest deg_w
+  unsigned long long h[AC_N + 2 + NBINS + 1] = {};  // the counts; then empty rows, largest deg_w, degree bins, hub arcs
   int64_t nseg = 0;
   {
     KTimer t(g, K_AGG_REDUCE, (double)m * 2 * (4 + sizeof(V)) + (double)k * 32);
-    AG_CHECK(cudaMemsetAsync(cnt, 0, (AC_N + 2) * sizeof(unsigned long long), s));
-    const bool big = m > AG_CTA_MAX;  // there may be large segments
-    if (big) {
-      if ((rc = dev_alloc_t(&ub, k, s)) || (rc = dev_alloc_t(&tlg, k, s)) || (rc = dev_alloc_t(&toff, k, s)))
-        return fail(rc);
-      AG_CHECK(cudaMemsetAsync(ub, 0, k * sizeof(unsigned long long), s));
+    AG_CHECK(cudaMemsetAsync(cnt, 0, sizeof(h), s));
+    static std::atomic<bool> attrs{false};  // idempotent; threads may race here
+    if (!attrs) {
+      AG_CHECK(cudaFuncSetAttribute(k_ag_warp<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ag_warp_smem<V>()));
+      AG_CHECK(cudaFuncSetAttribute(k_ag_cta<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ag_cta_smem<V>()));
+      attrs = true;
     }
-    AG_CHECK(cudaFuncSetAttribute(k_ag_warp<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ag_warp_smem<V>()));
-    AG_CHECK(cudaFuncSetAttribute(k_ag_cta<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ag_cta_smem<V>()));
     if (m > 0) {
       CD_LAUNCH(k_ag_classes<<<gcap((k + AF_SEGS - 1) / AF_SEGS, 152 * 8), NT, 0, s>>>(sstart, k, cnt, t8, t32, wl, cl, ll,
                                                                                     ch_seg, ch_off));
@@ -734,9 +752,9 @@ int aggregate_as(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_de
     // 4: the coarse CSR
     if ((rc = exclusive_scan_i64(ucnt, coarse_off, k, coarse_off + k, s))) return fail(rc);
     CD_LAUNCH(k_ag_rows<<<gcap((k + NT - 1) / NT, 152 * 8), NT, 0, s>>>(sstart, coarse_off, k, delta,
-                                                                      (const unsigned long long*)cdegw, cnt + AC_N));
+                                                                      (const unsigned long long*)cdegw, g->t_warp, g->t_hub, cnt + AC_N));
     AG_CHECK(cudaMemcpyAsync(&nseg, coarse_off + k, 8, cudaMemcpyDeviceToHost, s));
-    AG_CHECK(cudaMemcpyAsync(h + AC_N, cnt + AC_N, 16, cudaMemcpyDeviceToHost, s));
+    AG_CHECK(cudaMemcpyAsync(h + AC_N, cnt + AC_N, (2 + NBINS + 1) * 8, cudaMemcpyDeviceToHost, s));
     AG_CHECK(cudaStreamSynchronize(s));
     if ((rc = dev_alloc_t(&ccols, nseg + COL_PAD, s)) ||
         (rc = dev_alloc(&cw, (size_t)std::max<int64_t>(nseg, 1) * (NARROW ? 4 : 8), s)))
@@ -757,7 +775,7 @@ int aggregate_as(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_de
   stats[2] = h[AC_N];
   stats[3] = h[AC_N + 1];
   cd_graph* c = nullptr;
-  rc = graph_adopt(s, k, nseg, coarse_off, ccols, cw, NARROW ? W_I32 : W_I64, &c, cdegw, stats, g);
+  rc = graph_adopt(s, k, nseg, coarse_off, ccols, cw, NARROW ? W_I32 : W_I64, &c, cdegw, stats, g, h + AC_N + 2);
   if (rc) return rc;
   c->timing = g->timing;
   c->ktiming = g->ktiming;

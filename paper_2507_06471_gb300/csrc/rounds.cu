@@ -897,7 +897,6 @@ int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, i
   const bool per_graph = graph_rounds != nullptr;
   const bool nk = louv && g->vol < ((int64_t)1 << 31);
   int rc;
-  if (nk && !g->sigma32 && (rc = dev_alloc_t(&g->sigma32, g->n, st))) return rc;
   LoopCtx L{};
   L.n = g->n;
   L.nwords = (g->n + 31) / 32;
@@ -917,11 +916,10 @@ int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, i
   L.sigma32 = nk ? g->sigma32 : nullptr;
   const int64_t words = 3 * (int64_t)o.max_iter + HEAD + (int64_t)TRACE_COLS * o.max_iter;
   unsigned long long* work = nullptr;
-  if ((rc = dev_alloc_t(&work, words, st))) return rc;
-  if (per_graph && (rc = dev_alloc_t(&L.last_change, g->nb, st))) {
-    dev_free(work, st);
-    return rc;
-  }
+  Arena scratch;
+  scratch.add(&work, words);
+  if (per_graph) scratch.add(&L.last_change, g->nb);
+  if ((rc = scratch.make(st))) return rc;
   L.bar = work;
   L.head = work + 3 * (int64_t)o.max_iter;
   std::vector<unsigned long long> h;
@@ -956,8 +954,7 @@ int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, i
     return status;
   };
   rc = run();
-  dev_free(work, st);
-  dev_free(L.last_change, st);
+  scratch.free(st);
   if (rc) return rc;
   const int32_t rounds = (int32_t)h[0];
   int64_t moves = 0;

@@ -2009,10 +2009,6 @@ int run_rounds(cd_graph* g, const RunOpts& o, bool louv, int64_t* moves_out, int
   // 32-bit Sigma_tot copy for the gathers (synchronous Louvain, vol(V) < 2^31)
   const bool use_s32 = louv && !o.async_mode && g->vol < ((int64_t)1 << 31) && n > 0;
   if (use_s32) {
-    if (!g->sigma32) {
-      int rc2 = dev_alloc_t(&g->sigma32, n, st);
-      if (rc2) return rc2;
-    }
     CD_LAUNCH(k_sigma32_all<<<grid_cap((n + NT - 1) / NT), NT, 0, st>>>(g->sigma, n, g->sigma32));
   }
   // round 0 from the rows when every vertex starts alone and no row repeats a
