@@ -136,10 +136,13 @@ __global__ void __launch_bounds__(NT) k_bmod_internal(const int64_t* __restrict_
   int32_t b = -1;
   for (int64_t e0 = (((int64_t)blockIdx.x * NT + threadIdx.x) >> 5) * piece; e0 < m; e0 += step) {  // uniform in the warp
     const int64_t e1 = e0 + piece < m ? e0 + piece : m;
+    auto columns = [&](int64_t e) { return e < e1 ? __ldg(reinterpret_cast<const int4*>(cols + e)) : make_int4(0, 0, 0, 0); };
+    int4 next = columns(e0 + 4 * lane);  // a tile ahead
     int64_t cur = warp_row_of(off, n, e0);
     for (int64_t ts = e0; ts < e1; ts += WALK_TILE) {
       const int64_t e = ts + 4 * lane;
-      const int4 c4 = e < e1 ? __ldg(reinterpret_cast<const int4*>(cols + e)) : make_int4(0, 0, 0, 0);
+      const int4 c4 = next;
+      next = columns(e + WALK_TILE);
       const int32_t cs[4] = {c4.x, c4.y, c4.z, c4.w};
       int32_t lc[4], lr[4], br[4];
       int64_t row[4];

@@ -155,6 +155,9 @@ __global__ void __launch_bounds__(NT) k_ag_scatter(const int64_t* __restrict__ o
   const int64_t step = (((int64_t)gridDim.x * NT) >> 5) * piece;
   for (int64_t e0 = (((int64_t)blockIdx.x * NT + threadIdx.x) >> 5) * piece; e0 < m; e0 += step) {  // uniform in the warp
     const int64_t e1 = e0 + piece < m ? e0 + piece : m;
+    int32_t bn[4];  // columns a tile ahead
+#pragma unroll
+    for (int j = 0; j < 4; ++j) bn[j] = e0 + lane + 32 * j < e1 ? __ldg(cols + e0 + lane + 32 * j) : -1;
     int64_t cur = warp_row_of(off, n, e0);
     for (int64_t ts = e0; ts < e1; ts += WALK_TILE) {
       int32_t b[4];
@@ -163,7 +166,8 @@ __global__ void __launch_bounds__(NT) k_ag_scatter(const int64_t* __restrict__ o
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int64_t e = ts + lane + 32 * j;
-        b[j] = e < e1 ? __ldg(cols + e) : -1;
+        b[j] = bn[j];
+        bn[j] = e + WALK_TILE < e1 ? __ldg(cols + e + WALK_TILE) : -1;
         x[j] = e < e1 ? (V)W::get(w, e) : 0;
       }
 #pragma unroll
