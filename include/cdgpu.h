@@ -72,15 +72,19 @@ typedef struct cd_params {
                                (the deferral coin still applies: without it adjacent vertices swap
                                labels in lockstep); results vary from run to run. 0 (default):
                                synchronous rounds, reproducible */
-  int32_t device_loop;      /* Where the round loop runs. 1 (default): in batched runs (cd_batch_*) the
-                               rounds after the first of a run or Louvain level run as one captured CUDA
-                               graph (a conditional WHILE node whose body is one round; the round number,
-                               the stop tests and the trace stay on the device), so a level costs one
-                               graph launch and no per-round host synchronisation; other runs keep the
-                               host loop (building a graph per level costs more than the few round trips
-                               of a small graph saves). 2: every run uses the device loop. 0: the host
-                               loop everywhere (one read-back per round). Results are identical in every
-                               mode; timing != 0 always uses the host loop (it records per-round events) */
+  int32_t device_loop;      /* Where the round loop runs. 1 (default): on the device where that pays. All
+                               rounds of a run or Louvain level run as one resident kernel on graphs
+                               without hubs (vertices of more than t_hub arcs) and on graphs of at most
+                               2^24 arcs with at most 4,095 of them; on larger ones, and in batched runs
+                               (cd_batch_*), the rounds after the first run as one captured CUDA graph (a
+                               conditional WHILE node whose body is one round) if at least 2^22 arcs and
+                               max_iter > 16 make the graph worth its making; others keep the host loop.
+                               The round number, the stop tests and the trace stay on the device, so a
+                               level costs one launch and no per-round host synchronisation. 2: runs that
+                               are not resident always take the captured graph. 0: the host loop
+                               everywhere (one read-back per round). Results are identical in every mode;
+                               timing != 0 (per-round events) and the asynchronous mode are never
+                               resident, and timing != 0 always uses the host loop */
 } cd_params;
 
 /* Per-round record of the last run on a graph (cd_trace_get). */
@@ -227,9 +231,9 @@ typedef struct cd_request_result {
 } cd_request_result;
 
 /* Start a server on the current device with parameters p (copied; timing is
- * ignored; device_loop = 1 keeps the host loop in the workers' packed calls,
- * where concurrent graph instantiation costs more than it saves, and 2 still
- * uses the device loop everywhere), 1 <= slots <= 64 workers, a device-memory budget in bytes (<= 0:
+ * ignored; device_loop = 1 means resident loops of 1 / slots of the GPU but no
+ * captured graphs in the workers, where concurrent graph instantiation costs
+ * more than it saves; 2 still uses captured graphs), 1 <= slots <= 64 workers, a device-memory budget in bytes (<= 0:
  * 80% of the free memory now), the packing limits small_n and batch_arcs
  * (0 turns packing off). Errors: CD_EINVAL, CD_ECUDA. */
 int cd_server_create(const cd_params* p, int32_t slots, int64_t mem_budget_bytes, int64_t small_n,

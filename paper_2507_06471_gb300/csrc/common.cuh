@@ -72,6 +72,13 @@ enum Ctr {
   C_HUB_PSLOTS,                      // table slots cleared, or read and written by compactions
   C_COUNT
 };
+// The words cleared at the start of a round: the counters, then the active
+// vertices per bin and the routed hub work, the queued build and mark items, the
+// hubs per build class and of the two lists of hub_pl.
+constexpr int R_ACT = C_COUNT;
+constexpr int R_HUB_ITEMS = R_ACT + NBINS + 2;
+constexpr int R_HUB_CLASS = R_HUB_ITEMS + 2;
+constexpr int R_WORDS = R_HUB_CLASS + 7;
 
 // Per-kernel profiling slots.
 enum Kern {
@@ -127,7 +134,7 @@ struct cd_graph {
   int64_t bin_start[cd::NBINS + 1] = {};  // host copy of the bin offsets
   // frontier: the active vertices of a round, bin b at act_list + bin_start[b]
   int32_t* act_list = nullptr;
-  unsigned long long* act_cnt = nullptr;   // NBINS+2: active per bin (hub bin: hub numbers), then the
+  unsigned long long* act_cnt = nullptr;   // NBINS+2 (part of ctr): active per bin (hub bin: hub numbers), then the
                                            // evaluate items and small hubs routed this round
   unsigned long long* full_cnt = nullptr;  // NBINS+2: the same for every listed vertex
   int32_t* act_ev = nullptr;               // evaluate items of the examined hubs with large tables in use
@@ -157,7 +164,7 @@ struct cd_graph {
   int64_t* hub_cur = nullptr;              // nhubs: weight into the hub's own label
   int32_t* hub_hascur = nullptr;           // nhubs
   int32_t* hub_done = nullptr;             // nhubs: finished evaluate items this round
-  int32_t* hub_mv = nullptr;               // 3 x nhubs: moved flag, old label, new label
+  int32_t* hub_mv = nullptr;               // 2 x nhubs: old and new label of a hub that moved this round
   int32_t* hub_rb = nullptr;               // nhubs: 1 = rebuild this hub's table from its row
   int32_t* hub_flist = nullptr;            // 2 x nhubs: hubs flagged in even / odd rounds
   unsigned long long* hub_fcnt = nullptr;  // 2: their counts
@@ -165,9 +172,9 @@ struct cd_graph {
   int64_t* hub_item_first = nullptr;       // nhubs+1: first build/mark item of each hub
   int32_t* hub_blist = nullptr;            // hub_items: build items queued this round
   int32_t* hub_mlist = nullptr;            // hub_items: mark items queued this round
-  unsigned long long* hub_lcnt = nullptr;  // 2: queued build and mark items
+  unsigned long long* hub_lcnt = nullptr;  // 2: queued build and mark items (part of ctr)
   int32_t* hub_cl = nullptr;               // 5 x nhubs: hubs rebuilt per build class
-  unsigned long long* hub_ccnt = nullptr;  // 7: their counts, and those of the two lists of hub_pl
+  unsigned long long* hub_ccnt = nullptr;  // 7: their counts, and those of the two lists of hub_pl (part of ctr)
   int32_t* hub_nl = nullptr;               // nhubs: live entries at the last evaluation in this run (-1: none yet)
   int64_t* hub_nc = nullptr;               // nhubs: slots a rebuild lays out
   int32_t* hub_pl = nullptr;               // 2 x nhubs: hubs prepared by a CTA; rebuilds that overflowed
@@ -190,7 +197,7 @@ struct cd_graph {
   int32_t* mv_v = nullptr;  // committed moves: vertex, new label, old label (three parts of one
   int32_t* mv_c = nullptr;  // array, each n rounded up to whole flag words)
   int32_t* mv_a = nullptr;
-  int64_t* ctr = nullptr;      // device counters
+  int64_t* ctr = nullptr;      // R_WORDS device counters, cleared at the start of a round
   int64_t* h_ctr = nullptr;    // pinned host copy
   int32_t* status = nullptr;   // device status word (0 = ok)
 
@@ -327,6 +334,14 @@ RunOpts opts_from(const cd_params* p, int32_t level);
 // GPU at most, so that the workers' loops run side by side. Loops that fill the
 // GPU run one after another, and most of a loop's time is latency.
 constexpr int32_t LOOP_NO_GRAPH = 0x10000;
+
+// A solo run on a graph with hubs of at least GRAPH_LOOP_ARCS arcs and with at
+// least GRAPH_LOOP_ROUNDS rounds to go takes the captured graph too: its launches
+// follow one another without the host's gaps and read-backs (LPA 19.7 -> 18.7 ms
+// and Louvain 135 -> 129 ms on R-MAT 22, 8.6 -> 7.5 and 65.5 -> 61.7 ms on R-MAT
+// 20), which pays for making the graph (about 0.4 ms) from some ten rounds on.
+constexpr int64_t GRAPH_LOOP_ARCS = (int64_t)1 << 22;
+constexpr int32_t GRAPH_LOOP_ROUNDS = 16;
 
 // rounds.cu: the whole round loop as one resident kernel (graphs without hubs).
 bool resident_rounds_apply(const cd_graph* g, const RunOpts& o, bool per_graph_stop);

@@ -486,15 +486,15 @@ void free_arrays(cd_graph* g) {
   cudaStream_t s = g->stream;
   free_resident_hubs(g);
   void* ps[] = {g->off,          g->cols,          g->w,            g->degw,         g->bin_list,
-                g->act_list,     g->act_cnt,       g->full_cnt,     g->act_ev,       g->act_small,
+                g->act_list,     g->full_cnt,     g->act_ev,       g->act_small,
                 g->hub_cc,       g->hub_live,
                 g->hub_pref,      g->hub_bits,      g->hub_tab,       g->hub_slot,
                 g->hub_item_hub,  g->hub_item_arc, g->hub_ev_hub,   g->hub_ev_slot,
                 g->hub_ev_first, g->hub_part,      g->hub_cur,      g->hub_hascur,   g->hub_done,
                 g->hub_mv,       g->hub_rb,       g->hub_used,     g->hub_item_first,
-                g->hub_flist,    g->hub_fcnt,     g->hub_cl,       g->hub_ccnt,
+                g->hub_flist,    g->hub_fcnt,     g->hub_cl,
                 g->hub_nl,       g->hub_nc,       g->hub_pl,
-                g->hub_blist,    g->hub_mlist,     g->hub_lcnt,     g->hub_log,
+                g->hub_blist,    g->hub_mlist,     g->hub_log,
                 g->run_mem,      g->status,        g->gid,          g->gbase,        g->gvol,
                 g->gfrozen,      g->gcnt};
   for (void* p : ps) dev_free(p, s);
@@ -512,18 +512,17 @@ void free_resident_hubs(cd_graph* g) {
 void free_bins(cd_graph* g) {
   cudaStream_t s = g->stream;
   free_resident_hubs(g);
-  void* ps[] = {g->bin_list,     g->act_list,    g->act_cnt,      g->full_cnt,  g->act_ev,
+  void* ps[] = {g->bin_list,     g->act_list,    g->full_cnt,  g->act_ev,
                 g->act_small,    g->hub_cc,       g->hub_live,
                 g->hub_pref,      g->hub_bits,     g->hub_tab,   g->hub_slot,
                 g->hub_item_hub, g->hub_item_arc, g->hub_ev_hub,  g->hub_ev_slot, g->hub_ev_first,
                 g->hub_part,     g->hub_cur,     g->hub_hascur,   g->hub_done,  g->hub_mv,
                 g->hub_rb,       g->hub_used,     g->hub_item_first, g->hub_blist,
-                g->hub_flist,    g->hub_fcnt,     g->hub_cl,       g->hub_ccnt,
-                g->hub_mlist,    g->hub_lcnt,     g->hub_log,      g->hub_nl,    g->hub_nc,      g->hub_pl};
+                g->hub_flist,    g->hub_fcnt,     g->hub_cl,
+                g->hub_mlist,    g->hub_log,      g->hub_nl,    g->hub_nc,      g->hub_pl};
   for (void* p : ps) dev_free(p, s);
   g->bin_list = nullptr;
   g->act_list = nullptr;
-  g->act_cnt = nullptr;
   g->full_cnt = nullptr;
   g->act_ev = nullptr;
   g->act_small = nullptr;
@@ -547,12 +546,10 @@ void free_bins(cd_graph* g) {
   g->hub_flist = nullptr;
   g->hub_fcnt = nullptr;
   g->hub_cl = nullptr;
-  g->hub_ccnt = nullptr;
   g->hub_used = nullptr;
   g->hub_item_first = nullptr;
   g->hub_blist = nullptr;
   g->hub_mlist = nullptr;
-  g->hub_lcnt = nullptr;
   g->hub_log = nullptr;
   g->hub_nl = g->hub_pl = nullptr;
   g->hub_nc = nullptr;
@@ -607,7 +604,6 @@ int fill_bins(cd_graph* g) {
   rc = dev_alloc_t(&g->bin_list, listed, s);
   if (rc) return rc;
   if ((rc = dev_alloc_t(&g->act_list, listed, s))) return rc;
-  if ((rc = dev_alloc_t(&g->act_cnt, NBINS + 2, s))) return rc;
   if ((rc = dev_alloc_t(&g->full_cnt, NBINS + 2, s))) return rc;
   int64_t* d_base = nullptr;
   unsigned long long* d_cur = nullptr;
@@ -683,12 +679,11 @@ int fill_bins(cd_graph* g) {
     if ((rc = dev_alloc_t(&g->hub_cur, nh, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_hascur, nh, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_done, nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_mv, 3 * nh, s))) return rc;
+    if ((rc = dev_alloc_t(&g->hub_mv, 2 * nh, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_rb, nh, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_flist, 2 * nh, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_fcnt, 2, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_cl, 5 * nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_ccnt, 7, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_nl, nh, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_nc, nh, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_pl, 2 * nh, s))) return rc;
@@ -696,7 +691,6 @@ int fill_bins(cd_graph* g) {
     if ((rc = dev_alloc_t(&g->hub_item_first, nh + 1, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_blist, g->hub_items, s))) return rc;
     if ((rc = dev_alloc_t(&g->hub_mlist, g->hub_items, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_lcnt, 2, s))) return rc;
     {  // a round applies at most hub_arcs / HUB_LOG_DIV logged updates (random probes
        // into the tables cost about as much as rebuilding the hubs); the hub of
        // every update beyond that budget is rebuilt from its row instead
@@ -713,9 +707,7 @@ int fill_bins(cd_graph* g) {
     CD_CHECK(cudaMemcpyAsync(g->hub_item_first, item_first.data(), (nh + 1) * 8, cudaMemcpyHostToDevice, s));
     CD_CHECK(cudaMemsetAsync(g->hub_rb, 0, nh * 4, s));
     CD_CHECK(cudaMemsetAsync(g->hub_used, 0, nh * 4, s));
-    CD_CHECK(cudaMemsetAsync(g->hub_lcnt, 0, 2 * 8, s));
     CD_CHECK(cudaMemsetAsync(g->hub_fcnt, 0, 2 * 8, s));
-    CD_CHECK(cudaMemsetAsync(g->hub_ccnt, 0, 7 * 8, s));
     CD_CHECK(cudaMemsetAsync(g->hub_cur, 0, nh * 8, s));
     CD_CHECK(cudaMemsetAsync(g->hub_hascur, 0, nh * 4, s));
     CD_CHECK(cudaMemsetAsync(g->hub_done, 0, nh * 4, s));
@@ -867,10 +859,13 @@ int ensure_run_state(cd_graph* g) {
   a.add(&g->flag[0], n32 / 32 + 1);
   a.add(&g->flag[1], n32 / 32 + 1);
   a.add(&g->mv_v, 3 * n32);
-  a.add(&g->ctr, C_COUNT);
+  a.add(&g->ctr, R_WORDS);
   const int rc = a.make(g->stream);
   if (rc) return rc;
   g->run_mem = a.mem;
+  g->act_cnt = (unsigned long long*)g->ctr + R_ACT;
+  g->hub_lcnt = (unsigned long long*)g->ctr + R_HUB_ITEMS;
+  g->hub_ccnt = (unsigned long long*)g->ctr + R_HUB_CLASS;
   g->mv_c = g->mv_v + n32;
   g->mv_a = g->mv_v + 2 * n32;
   return CD_OK;

@@ -750,9 +750,8 @@ __device__ __forceinline__ void hub_decide(const ScanCtx& s, int32_t h, int32_t 
   if (target != cur && !def) {
     n_marcs += s.off[v + 1] - s.off[v];
     atomicAdd(&s.ctr[C_HUB_MARCS], (unsigned long long)(s.off[v + 1] - s.off[v]));
-    s.hub_mv[3 * h] = 1;
-    s.hub_mv[3 * h + 1] = cur;
-    s.hub_mv[3 * h + 2] = target;
+    s.hub_mv[2 * h] = cur;
+    s.hub_mv[2 * h + 1] = target;
     const int64_t i0 = s.hub_item_first[h], ni = s.hub_item_first[h + 1] - i0;
     const unsigned long long pos = atomicAdd(&s.hub_lcnt[1], (unsigned long long)ni);
     for (int64_t j = 0; j < ni; ++j) s.hub_mlist[pos + j] = (int32_t)(i0 + j);
@@ -1351,7 +1350,7 @@ __global__ void __launch_bounds__(NT) k_hub_mark(ScanCtx s) {
   for (int64_t q = blockIdx.x; q < nm; q += gridDim.x) {
     const int32_t it = s.hub_mlist[q];
     const int32_t h = s.hub_item_hub[it];
-    const int32_t A = s.hub_mv[3 * h + 1], c = s.hub_mv[3 * h + 2];
+    const int32_t A = s.hub_mv[2 * h], c = s.hub_mv[2 * h + 1];
     const int32_t v = s.hub_list[h];
     const int64_t a0 = s.hub_item_arc[it];
     const int64_t rowend = s.off[v + 1];
@@ -1605,7 +1604,6 @@ int launch_round(cd_graph* g, ScanCtx& s, const int32_t* lists, const unsigned l
       CD_LAUNCH(k_hub_retry<<<152, NT, 0, st>>>(s));
       CD_LAUNCH(k_hub_build<W, V><<<grid_cap(g->hub_items, 152 * 3), HUB_NT, hub_smem<V>(), st>>>(s));
       // the examined hubs' evaluate work, by the sizes of their tables
-      CD_CHECK(cudaMemsetAsync(g->act_cnt + NBINS, 0, 2 * sizeof(unsigned long long), st));
       CD_LAUNCH(k_hub_route<<<grid_cap((g->nhubs + NT - 1) / NT), NT, 0, st>>>(s, g->act_ev, g->act_small,
                                                                              g->act_cnt + NBINS));
     }
@@ -1874,21 +1872,17 @@ int device_rounds(cd_graph* g, const RunOpts& o, bool louv, bool use_s32, bool p
   // one round, enqueued on the capture stream (the launch helpers use g->stream)
   g->stream = cap;
   rc = [&]() -> int {
-    CD_CHECK(cudaMemsetAsync(g->ctr, 0, C_COUNT * sizeof(int64_t), cap));
+    CD_CHECK(cudaMemsetAsync(g->ctr, 0, R_WORDS * sizeof(int64_t), cap));
     if (per_graph_stop) {
       CD_CHECK(cudaMemsetAsync(g->gcnt, 0, g->nb * sizeof(int64_t), cap));
       CD_CHECK(cudaMemsetAsync(&dl->alive, 0, sizeof(unsigned long long), cap));
     }
     if (o.use_frontier && n > 0) CD_CHECK(cudaMemsetAsync(fnxt, 0, fbytes, cap));
     if (nh > 0) {
-      CD_CHECK(cudaMemsetAsync(g->hub_mv, 0, 3 * nh * sizeof(int32_t), cap));
-      CD_CHECK(cudaMemsetAsync(g->hub_lcnt, 0, 2 * sizeof(unsigned long long), cap));
-      CD_CHECK(cudaMemsetAsync(g->hub_ccnt, 0, (HUB_NCLASS + 2) * sizeof(unsigned long long), cap));
       CD_CHECK(cudaMemsetAsync(cntB, 0, sizeof(unsigned long long), cap));
     }
     CD_LAUNCH(k_loop_begin<<<1, 1, 0, cap>>>(dl, n, louv ? HUB_SKIP_DIV : HUB_SKIP_DIV_LPA, nh > 0));
     if (compact) {
-      CD_CHECK(cudaMemsetAsync(g->act_cnt, 0, (NBINS + 2) * sizeof(unsigned long long), cap));
       BinBounds bb;
       for (int b = 0; b <= NBINS; ++b) bb.b[b] = g->bin_start[b];
       CD_LAUNCH(k_compact<<<wave_grid(k_compact, NT, 0, (g->bin_start[NBINS] + NT - 1) / NT), NT, 0, cap>>>(
@@ -2020,7 +2014,9 @@ int run_rounds(cd_graph* g, const RunOpts& o, bool louv, int64_t* moves_out, int
     for (auto& e : ev) cudaEventCreate(&e);
   // rounds after the first as one captured graph (a device-side loop) unless
   // per-round events are wanted
-  const bool dev_loop = o.graph_loop && !g->timing && (o.batched || o.device_loop_all);
+  const bool dev_loop = o.graph_loop && !g->timing &&
+                        (o.batched || o.device_loop_all ||
+                         (g->nnz >= GRAPH_LOOP_ARCS && o.max_iter > GRAPH_LOOP_ROUNDS));
   for (int32_t r = 0; r < o.max_iter && rc == CD_OK; ++r) {
     if (r > 0 && dev_loop) {
       rc = device_rounds(g, o, louv, use_s32, per_graph_stop, r, fcur, fnxt, prev_moves, total_moves, rounds,
@@ -2028,13 +2024,10 @@ int run_rounds(cd_graph* g, const RunOpts& o, bool louv, int64_t* moves_out, int
       break;
     }
     if (g->timing) cudaEventRecord(ev[0], st);
-    CD_CHECK(cudaMemsetAsync(g->ctr, 0, C_COUNT * sizeof(int64_t), st));
+    CD_CHECK(cudaMemsetAsync(g->ctr, 0, R_WORDS * sizeof(int64_t), st));
     if (per_graph_stop) CD_CHECK(cudaMemsetAsync(g->gcnt, 0, g->nb * sizeof(int64_t), st));
     if (o.use_frontier && n > 0) CD_CHECK(cudaMemsetAsync(fnxt, 0, fbytes, st));
     if (g->nhubs > 0) {
-      CD_CHECK(cudaMemsetAsync(g->hub_mv, 0, 3 * g->nhubs * sizeof(int32_t), st));
-      CD_CHECK(cudaMemsetAsync(g->hub_lcnt, 0, 2 * sizeof(unsigned long long), st));
-      CD_CHECK(cudaMemsetAsync(g->hub_ccnt, 0, (HUB_NCLASS + 2) * sizeof(unsigned long long), st));
       CD_CHECK(cudaMemsetAsync(g->hub_fcnt + (r & 1), 0, sizeof(unsigned long long), st));
     }
     ScanCtx s = static_ctx(g, o, louv, use_s32, per_graph_stop);
@@ -2065,7 +2058,6 @@ int run_rounds(cd_graph* g, const RunOpts& o, bool louv, int64_t* moves_out, int
     s.hub_act_cnt = nullptr;
     if (o.use_frontier && r > 0 && g->bin_start[NBINS] > 0) {
       KTimer t(g, K_FRONTIER, (double)g->bin_start[NBINS] * (4 + 1 + 4));
-      CD_CHECK(cudaMemsetAsync(g->act_cnt, 0, (NBINS + 2) * sizeof(unsigned long long), st));
       BinBounds bb;
       for (int b = 0; b <= NBINS; ++b) bb.b[b] = g->bin_start[b];
       CD_LAUNCH(k_compact<<<wave_grid(k_compact, NT, 0, (g->bin_start[NBINS] + NT - 1) / NT), NT, 0, st>>>(
