@@ -129,7 +129,8 @@ struct cd_graph {
   int64_t* degw = nullptr;  // n
 
   // static degree bins: counted when the graph is made; the lists and hub structures of the per-round kernels are
-  // made when those first run (ensure_bins)
+  // made when those first run (ensure_bins), in two allocations (bin_mem)
+  void* bin_mem[2] = {nullptr, nullptr};
   int32_t* bin_list = nullptr;           // n vertex ids grouped by bin
   int64_t bin_start[cd::NBINS + 1] = {};  // host copy of the bin offsets
   // frontier: the active vertices of a round, bin b at act_list + bin_start[b]

@@ -376,9 +376,14 @@ __global__ void __launch_bounds__(NT) k_double_loops(const int64_t* __restrict__
     }
 }
 
+struct BinBase {
+  int64_t b[NBINS + 1];
+};
+
+// The listed vertices by bin; cursor comes back with the vertices per bin. The
+// hubs are only counted here (k_hub_list lists them in order).
 __global__ void __launch_bounds__(NT) k_bin_fill(const int64_t* __restrict__ off, int64_t n, int t_warp,
-                                                 int t_hub, const int64_t* __restrict__ bin_base,
-                                                 unsigned long long* cursor,
+                                                 int t_hub, BinBase base, unsigned long long* cursor,
                                                  int32_t* __restrict__ list) {
   const int lane = threadIdx.x & 31;
   int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -397,42 +402,70 @@ __global__ void __launch_bounds__(NT) k_bin_fill(const int64_t* __restrict__ off
       unsigned long long pos = 0;
       int first = __ffs(m) - 1;
       if (lane == first) pos = atomicAdd(&cursor[bb], (unsigned long long)__popc(m));
+      if (bb == B_HUB) continue;
       pos = __shfl_sync(FULL, pos, first);
-      if (b == bb) list[bin_base[bb] + (int64_t)pos + __popc(m & ((1u << lane) - 1u))] = (int32_t)v;
+      if (b == bb) list[base.b[bb] + (int64_t)pos + __popc(m & ((1u << lane) - 1u))] = (int32_t)v;
     }
-  }
-}
-
-__global__ void k_hub_bits(const int32_t* __restrict__ hubs, int64_t nh, uint32_t* hub_bits) {
-  int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (h < nh) {
-    const int32_t v = hubs[h];
-    atomicOr(&hub_bits[v >> 5], 1u << (v & 31));
   }
 }
 
 // Hubs are numbered in increasing vertex id, so the number of vertex u is its
 // rank among the hubs: hub_pref[u / 32] (hubs below 32 (u / 32)) plus the hub
-// bits below u in its word. hub_pref[w] = lower bound of 32 w in the sorted list.
-__global__ void k_hub_pref(const int32_t* __restrict__ hubs, int64_t nh, int64_t nwords, uint32_t* hub_pref) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nwords; w += stride) {
-    int64_t lo = 0, hi = nh;  // first hub with vertex >= 32 w
-    while (lo < hi) {
-      const int64_t mid = (lo + hi) / 2;
-      if ((int64_t)hubs[mid] < 32 * w) lo = mid + 1; else hi = mid;
+// bits below u in its word. The bits and their counts per word, a warp per word:
+__global__ void __launch_bounds__(NT) k_hub_words(const int64_t* __restrict__ off, int64_t n, int t_hub,
+                                                  uint32_t* __restrict__ bits, int64_t* __restrict__ count) {
+  const int lane = threadIdx.x & 31;
+  const int64_t words = (n + 31) / 32, nwarps = ((int64_t)gridDim.x * NT) >> 5;
+  for (int64_t w = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 5; w < words; w += nwarps) {
+    const int64_t v = 32 * w + lane;
+    const unsigned m = __ballot_sync(FULL, v < n && off[v + 1] - off[v] > t_hub);
+    if (lane == 0) {
+      bits[w] = m;
+      count[w] = __popc(m);
     }
-    hub_pref[w] = (uint32_t)lo;
   }
 }
 
-__global__ void k_gather_rows(const int64_t* __restrict__ off, const int32_t* __restrict__ vs,
-                              int64_t m, int64_t* __restrict__ out) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < m) {
-    int32_t v = vs[i];
-    out[2 * i] = off[v];
-    out[2 * i + 1] = off[v + 1];
+// The hubs in order, and each one's table slots, build/mark items and evaluate
+// items (scanned into the offsets of each afterwards).
+__global__ void k_hub_list(const int64_t* __restrict__ off, int64_t words, const uint32_t* __restrict__ bits,
+                           const int64_t* __restrict__ pref, uint32_t* __restrict__ hub_pref,
+                           int32_t* __restrict__ hubs, int64_t* __restrict__ cap, int64_t* __restrict__ items,
+                           int64_t* __restrict__ evs) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < words; w += stride) {
+    int64_t h = pref[w];
+    hub_pref[w] = (uint32_t)h;
+    for (uint32_t m = bits[w]; m; m &= m - 1, ++h) {
+      const int64_t v = 32 * w + __ffs(m) - 1;
+      const int64_t d = off[v + 1] - off[v];
+      const int64_t c = d + d / 2 + 64;  // live labels <= deg; the rest absorbs labels that come and go
+      hubs[h] = (int32_t)v;
+      cap[h] = c;
+      items[h] = (d + HUB_CHUNK - 1) / HUB_CHUNK;
+      evs[h] = (c + HUB_SLICE - 1) / HUB_SLICE;
+    }
+  }
+}
+
+// Warp per hub: its items.
+__global__ void __launch_bounds__(NT) k_hub_items(const int64_t* __restrict__ off, const int32_t* __restrict__ hubs,
+                                                  int64_t nh, const int64_t* __restrict__ item_first,
+                                                  const int64_t* __restrict__ ev_first, int32_t* __restrict__ item_hub,
+                                                  int64_t* __restrict__ item_arc, int32_t* __restrict__ ev_hub,
+                                                  int64_t* __restrict__ ev_slot) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nwarps = ((int64_t)gridDim.x * NT) >> 5;
+  for (int64_t h = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 5; h < nh; h += nwarps) {
+    const int64_t beg = off[hubs[h]], i0 = item_first[h], i1 = item_first[h + 1], e0 = ev_first[h], e1 = ev_first[h + 1];
+    for (int64_t i = i0 + lane; i < i1; i += 32) {
+      item_hub[i] = (int32_t)h;
+      item_arc[i] = beg + (i - i0) * HUB_CHUNK;
+    }
+    for (int64_t e = e0 + lane; e < e1; e += 32) {
+      ev_hub[e] = (int32_t)h;
+      ev_slot[e] = (e - e0) * HUB_SLICE;
+    }
   }
 }
 
@@ -485,18 +518,8 @@ void free_resident_hubs(cd_graph* g);
 void free_arrays(cd_graph* g) {
   cudaStream_t s = g->stream;
   free_resident_hubs(g);
-  void* ps[] = {g->off,          g->cols,          g->w,            g->degw,         g->bin_list,
-                g->act_list,     g->full_cnt,     g->act_ev,       g->act_small,
-                g->hub_cc,       g->hub_live,
-                g->hub_pref,      g->hub_bits,      g->hub_tab,       g->hub_slot,
-                g->hub_item_hub,  g->hub_item_arc, g->hub_ev_hub,   g->hub_ev_slot,
-                g->hub_ev_first, g->hub_part,      g->hub_cur,      g->hub_hascur,   g->hub_done,
-                g->hub_mv,       g->hub_rb,       g->hub_used,     g->hub_item_first,
-                g->hub_flist,    g->hub_fcnt,     g->hub_cl,
-                g->hub_nl,       g->hub_nc,       g->hub_pl,
-                g->hub_blist,    g->hub_mlist,     g->hub_log,
-                g->run_mem,      g->status,        g->gid,          g->gbase,        g->gvol,
-                g->gfrozen,      g->gcnt};
+  void* ps[] = {g->off,  g->cols,  g->w,    g->degw,    g->bin_mem[0], g->bin_mem[1], g->run_mem, g->status,
+                g->gid,  g->gbase, g->gvol, g->gfrozen, g->gcnt};
   for (void* p : ps) dev_free(p, s);
   if (g->h_ctr) cudaFreeHost(g->h_ctr);
 }
@@ -512,15 +535,10 @@ void free_resident_hubs(cd_graph* g) {
 void free_bins(cd_graph* g) {
   cudaStream_t s = g->stream;
   free_resident_hubs(g);
-  void* ps[] = {g->bin_list,     g->act_list,    g->full_cnt,  g->act_ev,
-                g->act_small,    g->hub_cc,       g->hub_live,
-                g->hub_pref,      g->hub_bits,     g->hub_tab,   g->hub_slot,
-                g->hub_item_hub, g->hub_item_arc, g->hub_ev_hub,  g->hub_ev_slot, g->hub_ev_first,
-                g->hub_part,     g->hub_cur,     g->hub_hascur,   g->hub_done,  g->hub_mv,
-                g->hub_rb,       g->hub_used,     g->hub_item_first, g->hub_blist,
-                g->hub_flist,    g->hub_fcnt,     g->hub_cl,
-                g->hub_mlist,    g->hub_log,      g->hub_nl,    g->hub_nc,      g->hub_pl};
-  for (void* p : ps) dev_free(p, s);
+  for (void*& p : g->bin_mem) {
+    dev_free(p, s);
+    p = nullptr;
+  }
   g->bin_list = nullptr;
   g->act_list = nullptr;
   g->full_cnt = nullptr;
@@ -599,134 +617,86 @@ int build_bins(cd_graph* g) {
 // The bin lists, and the hub histograms' layout.
 int fill_bins(cd_graph* g) {
   cudaStream_t s = g->stream;
-  int rc;
-  int64_t listed = g->bin_start[NBINS];
-  rc = dev_alloc_t(&g->bin_list, listed, s);
+  const int64_t listed = g->bin_start[NBINS], nh = g->nhubs, words = (g->n + 31) / 32;
+  int64_t* count = nullptr;  // hubs per word, then their prefix
+  Arena a;
+  a.add(&g->bin_list, listed);
+  a.add(&g->act_list, listed);
+  a.add(&g->full_cnt, NBINS + 2);
+  const size_t zero0 = a.bytes;  // cleared from here ...
+  if (nh > 0) {
+    a.add(&g->hub_live, nh);
+    a.add(&g->hub_rb, nh);
+    a.add(&g->hub_used, nh);
+    a.add(&g->hub_fcnt, 2);
+    a.add(&g->hub_hascur, nh);
+    a.add(&g->hub_done, nh);
+    a.add(&g->hub_cur, nh);
+  }
+  const size_t zero1 = a.bytes;  // ... to here
+  if (nh > 0) {
+    a.add(&g->act_small, nh);  // any hub whose table in use is small
+    a.add(&g->hub_cc, nh);
+    a.add(&g->hub_pref, words);
+    a.add(&g->hub_bits, words);
+    a.add(&g->hub_tab, nh + 1);
+    a.add(&g->hub_ev_first, nh + 1);
+    a.add(&g->hub_item_first, nh + 1);
+    a.add(&g->hub_mv, 2 * nh);
+    a.add(&g->hub_flist, 2 * nh);
+    a.add(&g->hub_cl, 5 * nh);
+    a.add(&g->hub_nl, nh);
+    a.add(&g->hub_nc, nh);
+    a.add(&g->hub_pl, 2 * nh);
+    a.add(&count, words);
+  }
+  int rc = a.make(s);
   if (rc) return rc;
-  if ((rc = dev_alloc_t(&g->act_list, listed, s))) return rc;
-  if ((rc = dev_alloc_t(&g->full_cnt, NBINS + 2, s))) return rc;
-  int64_t* d_base = nullptr;
-  unsigned long long* d_cur = nullptr;
-  if ((rc = dev_alloc_t(&d_base, NBINS, s))) return rc;
-  if ((rc = dev_alloc_t(&d_cur, NBINS, s))) return rc;
-  CD_CHECK(cudaMemcpyAsync(d_base, g->bin_start, NBINS * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-  CD_CHECK(cudaMemsetAsync(d_cur, 0, NBINS * sizeof(unsigned long long), s));
+  g->bin_mem[0] = a.mem;
+  BinBase base;
+  for (int b = 0; b <= NBINS; ++b) base.b[b] = g->bin_start[b];
+  CD_CHECK(cudaMemsetAsync(g->full_cnt, 0, (NBINS + 2) * sizeof(unsigned long long), s));
   if (g->n > 0)
-    CD_LAUNCH(k_bin_fill<<<grid_for(g->n), NT, 0, s>>>(g->off, g->n, g->t_warp, g->t_hub, d_base, d_cur,
+    CD_LAUNCH(k_bin_fill<<<grid_for(g->n), NT, 0, s>>>(g->off, g->n, g->t_warp, g->t_hub, base, g->full_cnt,
                                                        g->bin_list));
   CD_CHECK(cudaGetLastError());
-  // hubs: host-side layout of tables and work items
-  const int64_t nh = g->nhubs;
-  if (nh > 0) {
-    {  // hubs in increasing vertex id (their number is their rank)
-      std::vector<int32_t> hv(nh);
-      int32_t* dl = g->bin_list + g->bin_start[B_HUB];
-      CD_CHECK(cudaMemcpyAsync(hv.data(), dl, nh * 4, cudaMemcpyDeviceToHost, s));
-      CD_CHECK(cudaStreamSynchronize(s));
-      std::sort(hv.begin(), hv.end());
-      CD_CHECK(cudaMemcpyAsync(dl, hv.data(), nh * 4, cudaMemcpyHostToDevice, s));
-      CD_CHECK(cudaStreamSynchronize(s));  // hv dies here
-    }
-    int64_t* d_rows = nullptr;
-    if ((rc = dev_alloc_t(&d_rows, 2 * nh, s))) return rc;
-    CD_LAUNCH(k_gather_rows<<<(unsigned)((nh + 255) / 256), 256, 0, s>>>(g->off, g->bin_list + g->bin_start[B_HUB],
-                                                              nh, d_rows));
-    std::vector<int64_t> rows(2 * nh);
-    CD_CHECK(cudaMemcpyAsync(rows.data(), d_rows, 2 * nh * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    CD_CHECK(cudaStreamSynchronize(s));
-    dev_free(d_rows, s);
-    std::vector<int64_t> tab(nh + 1, 0), item_arc, ev_first(nh + 1, 0), ev_slot, item_first(nh + 1, 0);
-    std::vector<int32_t> item_hub, ev_hub;
-    std::vector<int64_t> cc(nh);
-    for (int64_t h = 0; h < nh; ++h) {
-      int64_t beg = rows[2 * h], deg = rows[2 * h + 1] - beg;
-      int64_t cap = deg + deg / 2 + 64;  // live labels <= deg; the rest absorbs labels that come and go
-      tab[h + 1] = tab[h] + cap;
-      item_first[h] = (int64_t)item_hub.size();
-      for (int64_t a = 0; a < deg; a += HUB_CHUNK) {
-        item_hub.push_back((int32_t)h);
-        item_arc.push_back(beg + a);
-      }
-      ev_first[h] = (int64_t)ev_hub.size();
-      for (int64_t e = 0; e < cap; e += HUB_SLICE) {
-        ev_hub.push_back((int32_t)h);
-        ev_slot.push_back(e);
-      }
-    }
-    ev_first[nh] = (int64_t)ev_hub.size();
-    item_first[nh] = (int64_t)item_hub.size();
-    g->hub_slots = tab[nh];
-    g->hub_items = (int64_t)item_hub.size();
-    g->hub_eval_items = (int64_t)ev_hub.size();
-    if ((rc = dev_alloc_t(&g->act_ev, g->hub_eval_items, s))) return rc;
-    if ((rc = dev_alloc_t(&g->act_small, nh, s))) return rc;  // any hub whose table in use is small
-    if ((rc = dev_alloc_t(&g->hub_cc, nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_live, nh, s))) return rc;
-    for (int64_t h = 0; h < nh; ++h) cc[h] = tab[h + 1] - tab[h];  // every table starts at its allocation
-    CD_CHECK(cudaMemcpyAsync(g->hub_cc, cc.data(), nh * 8, cudaMemcpyHostToDevice, s));
-    CD_CHECK(cudaMemsetAsync(g->hub_live, 0, nh * 4, s));
-    if ((rc = dev_alloc_t(&g->hub_pref, (g->n + 31) / 32, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_bits, (g->n + 31) / 32, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_tab, nh + 1, s))) return rc;
-    g->hub_wide = g->max_degw >= ((int64_t)1 << 32) ? 1 : 0;
-    if ((rc = dev_alloc_t(&g->hub_slot, g->hub_slots * (1 + g->hub_wide), s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_item_hub, g->hub_items, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_item_arc, g->hub_items, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_ev_hub, g->hub_eval_items, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_ev_slot, g->hub_eval_items, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_ev_first, nh + 1, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_part, 3 * std::max(g->hub_eval_items, g->hub_items), s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_cur, nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_hascur, nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_done, nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_mv, 2 * nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_rb, nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_flist, 2 * nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_fcnt, 2, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_cl, 5 * nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_nl, nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_nc, nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_pl, 2 * nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_used, nh, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_item_first, nh + 1, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_blist, g->hub_items, s))) return rc;
-    if ((rc = dev_alloc_t(&g->hub_mlist, g->hub_items, s))) return rc;
-    {  // a round applies at most hub_arcs / HUB_LOG_DIV logged updates (random probes
-       // into the tables cost about as much as rebuilding the hubs); the hub of
-       // every update beyond that budget is rebuilt from its row instead
-      const int64_t hub_arcs = tab[nh] * 2 / 3;
-      g->hub_log_cap = std::max<int64_t>(1, hub_arcs / HUB_LOG_DIV);
-      if ((rc = dev_alloc_t(&g->hub_log, 2 * g->hub_log_cap, s))) return rc;
-    }
-    CD_CHECK(cudaMemcpyAsync(g->hub_tab, tab.data(), (nh + 1) * 8, cudaMemcpyHostToDevice, s));
-    CD_CHECK(cudaMemcpyAsync(g->hub_item_hub, item_hub.data(), item_hub.size() * 4, cudaMemcpyHostToDevice, s));
-    CD_CHECK(cudaMemcpyAsync(g->hub_item_arc, item_arc.data(), item_arc.size() * 8, cudaMemcpyHostToDevice, s));
-    CD_CHECK(cudaMemcpyAsync(g->hub_ev_hub, ev_hub.data(), ev_hub.size() * 4, cudaMemcpyHostToDevice, s));
-    CD_CHECK(cudaMemcpyAsync(g->hub_ev_slot, ev_slot.data(), ev_slot.size() * 8, cudaMemcpyHostToDevice, s));
-    CD_CHECK(cudaMemcpyAsync(g->hub_ev_first, ev_first.data(), (nh + 1) * 8, cudaMemcpyHostToDevice, s));
-    CD_CHECK(cudaMemcpyAsync(g->hub_item_first, item_first.data(), (nh + 1) * 8, cudaMemcpyHostToDevice, s));
-    CD_CHECK(cudaMemsetAsync(g->hub_rb, 0, nh * 4, s));
-    CD_CHECK(cudaMemsetAsync(g->hub_used, 0, nh * 4, s));
-    CD_CHECK(cudaMemsetAsync(g->hub_fcnt, 0, 2 * 8, s));
-    CD_CHECK(cudaMemsetAsync(g->hub_cur, 0, nh * 8, s));
-    CD_CHECK(cudaMemsetAsync(g->hub_hascur, 0, nh * 4, s));
-    CD_CHECK(cudaMemsetAsync(g->hub_done, 0, nh * 4, s));
-    CD_CHECK(cudaMemsetAsync(g->hub_bits, 0, (g->n + 31) / 32 * 4, s));
-    CD_LAUNCH(k_hub_bits<<<(unsigned)((nh + 255) / 256), 256, 0, s>>>(g->bin_list + g->bin_start[B_HUB], nh,
-                                                                      g->hub_bits));
-    CD_LAUNCH(k_hub_pref<<<grid_for((g->n + 31) / 32), NT, 0, s>>>(g->bin_list + g->bin_start[B_HUB], nh,
-                                                                   (g->n + 31) / 32, g->hub_pref));
-    CD_CHECK(cudaStreamSynchronize(s));  // the host vectors above die here
-  }
-  {
-    unsigned long long full[NBINS + 2];
-    for (int b = 0; b < NBINS; ++b) full[b] = (unsigned long long)(g->bin_start[b + 1] - g->bin_start[b]);
-    full[NBINS] = full[NBINS + 1] = 0;  // hub evaluate work is routed per round
-    CD_CHECK(cudaMemcpyAsync(g->full_cnt, full, sizeof(full), cudaMemcpyHostToDevice, s));
-    CD_CHECK(cudaStreamSynchronize(s));  // `full` lives on this stack frame
-  }
-  dev_free(d_base, s);
-  dev_free(d_cur, s);
+  if (nh == 0) return CD_OK;
+  // hubs: their list, tables and work items, laid out on the device (one read-back, the totals)
+  int32_t* hubs = g->bin_list + g->bin_start[B_HUB];
+  CD_LAUNCH(k_hub_words<<<grid_for(words * 32), NT, 0, s>>>(g->off, g->n, g->t_hub, g->hub_bits, count));
+  if ((rc = exclusive_scan_i64(count, count, words, nullptr, s))) return rc;
+  CD_LAUNCH(k_hub_list<<<grid_for(words), NT, 0, s>>>(g->off, words, g->hub_bits, count, g->hub_pref, hubs, g->hub_cc,
+                                                      g->hub_nc, g->hub_cur));
+  if ((rc = exclusive_scan_i64(g->hub_cc, g->hub_tab, nh, g->hub_tab + nh, s)) ||
+      (rc = exclusive_scan_i64(g->hub_nc, g->hub_item_first, nh, g->hub_item_first + nh, s)) ||
+      (rc = exclusive_scan_i64(g->hub_cur, g->hub_ev_first, nh, g->hub_ev_first + nh, s)))
+    return rc;
+  CD_CHECK(cudaMemcpyAsync(&g->hub_slots, g->hub_tab + nh, 8, cudaMemcpyDeviceToHost, s));
+  CD_CHECK(cudaMemcpyAsync(&g->hub_items, g->hub_item_first + nh, 8, cudaMemcpyDeviceToHost, s));
+  CD_CHECK(cudaMemcpyAsync(&g->hub_eval_items, g->hub_ev_first + nh, 8, cudaMemcpyDeviceToHost, s));
+  CD_CHECK(cudaMemsetAsync((char*)a.mem + zero0, 0, zero1 - zero0, s));
+  CD_CHECK(cudaStreamSynchronize(s));
+  g->hub_wide = g->max_degw >= ((int64_t)1 << 32) ? 1 : 0;
+  // a round applies at most hub_arcs / HUB_LOG_DIV logged updates (random probes
+  // into the tables cost about as much as rebuilding the hubs); the hub of
+  // every update beyond that budget is rebuilt from its row instead
+  g->hub_log_cap = std::max<int64_t>(1, g->hub_slots * 2 / 3 / HUB_LOG_DIV);
+  Arena w;
+  w.add(&g->act_ev, g->hub_eval_items);
+  w.add(&g->hub_slot, g->hub_slots * (1 + g->hub_wide));
+  w.add(&g->hub_item_hub, g->hub_items);
+  w.add(&g->hub_item_arc, g->hub_items);
+  w.add(&g->hub_ev_hub, g->hub_eval_items);
+  w.add(&g->hub_ev_slot, g->hub_eval_items);
+  w.add(&g->hub_part, 3 * std::max(g->hub_eval_items, g->hub_items));
+  w.add(&g->hub_blist, g->hub_items);
+  w.add(&g->hub_mlist, g->hub_items);
+  w.add(&g->hub_log, 2 * g->hub_log_cap);
+  if ((rc = w.make(s))) return rc;
+  g->bin_mem[1] = w.mem;
+  CD_LAUNCH(k_hub_items<<<grid_for(nh * 32), NT, 0, s>>>(g->off, hubs, nh, g->hub_item_first, g->hub_ev_first,
+                                                         g->hub_item_hub, g->hub_item_arc, g->hub_ev_hub, g->hub_ev_slot));
+  CD_CHECK(cudaGetLastError());
   return CD_OK;
 }
 

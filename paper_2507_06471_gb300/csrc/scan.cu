@@ -471,11 +471,16 @@ __global__ void __launch_bounds__(NT) k_hub_prepare(ScanCtx s) {
     if (s.hub_rb[h] == HUB_COMPACT && !s.hub_wide) {  // uniform in the CTA
       if (threadIdx.x == 0) n_live = 0;
       __syncthreads();
-      for (int64_t i = threadIdx.x; i < cc; i += NT) {
-        const unsigned long long x = s.hub_slot[base + i];
-        if (x == SLOT_EMPTY || (x & 0xffffffffull) == 0) continue;
-        const int j = atomicAdd(&n_live, 1);
-        if (j < HUB_PREP_SLOTS) T[HUB_PREP_SLOTS - 1 - j] = x;  // the live list grows down from the top
+      for (int64_t i0 = threadIdx.x; i0 < cc; i0 += 8 * NT) {
+        unsigned long long x[8];  // in flight together
+#pragma unroll
+        for (int q = 0; q < 8; ++q) x[q] = i0 + q * NT < cc ? s.hub_slot[base + i0 + q * NT] : SLOT_EMPTY;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          if (x[q] == SLOT_EMPTY || (x[q] & 0xffffffffull) == 0) continue;
+          const int j = atomicAdd(&n_live, 1);
+          if (j < HUB_PREP_SLOTS) T[HUB_PREP_SLOTS - 1 - j] = x[q];  // the live list grows down from the top
+        }
       }
       __syncthreads();
       const int64_t nl = n_live;
