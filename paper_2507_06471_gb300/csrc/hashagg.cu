@@ -9,8 +9,10 @@
 //    are split evenly over the warps and taken in the graph's own order, so the
 //    columns are read and the segments written in runs (rowwalk.cuh).
 // 3. Each segment is combined by its keys: up to 8 or 32 arcs by as many lanes
-//    (a match, no table), up to 256 by a warp and up to AG_CTA_MAX by a CTA with
-//    a shared-memory table; a larger segment is cut into AG_CHUNK-arc chunks,
+//    (a match, no table), up to 256 by a warp and up to AG_MID_MAX and AG_CTA_MAX
+//    by CTAs of 128 and 512 threads with a shared-memory table (512 threads for a
+//    few hundred arcs are mostly barriers: 1.58 ms of the case below with one
+//    size); a larger segment is cut into AG_CHUNK-arc chunks,
 //    each combined in shared memory, whose distinct entries are then merged in a
 //    global table sized for the segment. The distinct (B, sum w) of a segment
 //    are written back at its start.
@@ -41,17 +43,17 @@ namespace {
 constexpr int NT = 256;
 constexpr int NW = NT / 32;
 constexpr int AG_WARP_MAX = 256;   // arcs of a segment combined by one warp (512-slot table)
-constexpr int AG_CTA_MAX = 4096;   // by one CTA (8192-slot table)
+constexpr int AG_MID_MAX = 1024;   // by a CTA of 128 threads (2048-slot table)
+constexpr int AG_CTA_MAX = 4096;   // by one of 512 (8192-slot table)
 constexpr int AG_CHUNK = 4096;     // arcs per chunk of a larger segment
 constexpr int AG_WCAP = 2 * AG_WARP_MAX;
-constexpr int AG_CCAP = 2 * AG_CTA_MAX;
 constexpr int AG_SLICE = 1024;     // global-table slots per extraction item (tables are multiples)
-constexpr int AG_CNT = 512;        // threads of the CTA-per-segment kernel
 constexpr int32_t AG_EMPTY = -1;
 constexpr unsigned long long AG_EMPTY_SLOT = ~0ull;
 
 // Counts on the device: segments per class, chunks, slots of the global tables.
-enum { AC_T8 = 0, AC_T32, AC_WARP, AC_CTA, AC_BIG, AC_CHUNKS, AC_SLOTS, AC_N };
+enum { AC_T8 = 0, AC_T32, AC_WARP, AC_MID, AC_CTA, AC_BIG, AC_CHUNKS, AC_SLOTS, AC_N };
+constexpr int AC_LISTS = 6;  // the first ones have a list of segments each
 
 unsigned gcap(int64_t blocks, int64_t cap = 152 * 16) {
   if (blocks < 1) blocks = 1;
@@ -192,7 +194,8 @@ constexpr int AF_SEGS = 8 * NT;
 __global__ void __launch_bounds__(NT) k_ag_classes(const int64_t* __restrict__ sstart, int64_t k,
                                                    unsigned long long* cnt, int32_t* __restrict__ t8,
                                                    int32_t* __restrict__ t32, int32_t* __restrict__ wl,
-                                                   int32_t* __restrict__ cl, int32_t* __restrict__ ll,
+                                                   int32_t* __restrict__ ml, int32_t* __restrict__ cl,
+                                                   int32_t* __restrict__ ll,
                                                    int32_t* __restrict__ ch_seg, int64_t* __restrict__ ch_off) {
   __shared__ int n_of[8];
   __shared__ unsigned long long base[8];
@@ -207,10 +210,10 @@ __global__ void __launch_bounds__(NT) k_ag_classes(const int64_t* __restrict__ s
       const int64_t a = a0 + q * NT + threadIdx.x;
       const int64_t len = a < k ? sstart[a + 1] - sstart[a] : 0;
       cls[q] = len == 0 ? -1 : len <= 8 ? AC_T8 : len <= 32 ? AC_T32 : len <= AG_WARP_MAX ? AC_WARP
-             : len <= AG_CTA_MAX ? AC_CTA : AC_BIG;
+             : len <= AG_MID_MAX ? AC_MID : len <= AG_CTA_MAX ? AC_CTA : AC_BIG;
       rank[q] = 0;
 #pragma unroll
-      for (int c = 0; c < 5; ++c) {
+      for (int c = 0; c < AC_LISTS; ++c) {
         const unsigned m = __ballot_sync(FULL, cls[q] == c);
         if (!m) continue;
         int p = 0;
@@ -228,12 +231,13 @@ __global__ void __launch_bounds__(NT) k_ag_classes(const int64_t* __restrict__ s
       }
     }
     __syncthreads();
-    if (threadIdx.x < 5 && n_of[threadIdx.x]) base[threadIdx.x] = atomicAdd(&cnt[threadIdx.x], (unsigned long long)n_of[threadIdx.x]);
+    if (threadIdx.x < AC_LISTS && n_of[threadIdx.x]) base[threadIdx.x] = atomicAdd(&cnt[threadIdx.x], (unsigned long long)n_of[threadIdx.x]);
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       if (cls[q] < 0) continue;
-      int32_t* list = cls[q] == AC_T8 ? t8 : cls[q] == AC_T32 ? t32 : cls[q] == AC_WARP ? wl : cls[q] == AC_CTA ? cl : ll;
+      int32_t* list = cls[q] == AC_T8 ? t8 : cls[q] == AC_T32 ? t32 : cls[q] == AC_WARP ? wl
+                    : cls[q] == AC_MID ? ml : cls[q] == AC_CTA ? cl : ll;
       list[base[cls[q]] + rank[q]] = (int32_t)(a0 + q * NT + threadIdx.x);
     }
     __syncthreads();
@@ -369,22 +373,23 @@ __global__ void __launch_bounds__(NT) k_ag_warp(const int64_t* __restrict__ ssta
   tile_segments<8, V>(sstart, t8, (int64_t)cnt[AC_T8], warp, nwarps, ab, aw, stage[wid], ucnt);
 }
 
-// CTA per block of up to AG_CTA_MAX arcs: first the chunks of the large
-// segments (a chunk's distinct count goes to dch and to the segment's upper
-// bound ub), then the whole medium segments.
-template <class V> constexpr size_t ag_cta_smem() { return (size_t)AG_CCAP * (sizeof(V) + 4 + 2); }
-template <class V>
-__global__ void __launch_bounds__(AG_CNT) k_ag_cta(const int64_t* __restrict__ sstart, const int32_t* __restrict__ cl,
+// CTA of TH threads per block of up to MAX arcs: first (with 512 threads) the
+// chunks of the large segments (a chunk's distinct count goes to dch and to the
+// segment's upper bound ub), then the whole segments of `list`.
+template <class V, int MAX> constexpr size_t ag_cta_smem() { return (size_t)2 * MAX * (sizeof(V) + 4 + 2); }
+template <class V, int TH, int MAX, int CLASS>
+__global__ void __launch_bounds__(TH) k_ag_cta(const int64_t* __restrict__ sstart, const int32_t* __restrict__ cl,
                                                const int32_t* __restrict__ ch_seg, const int64_t* __restrict__ ch_off,
                                                const unsigned long long* __restrict__ cnt, int32_t* ab, V* aw,
                                                int64_t* __restrict__ ucnt, int32_t* __restrict__ dch,
                                                unsigned long long* __restrict__ ub) {
   extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int AG_CNT = TH, AG_CCAP = 2 * MAX;
   V* vals = (V*)smem;
   int32_t* keys = (int32_t*)(smem + (size_t)AG_CCAP * sizeof(V));
   uint16_t* occ = (uint16_t*)(smem + (size_t)AG_CCAP * (sizeof(V) + 4));
   __shared__ int occ_n;
-  const int64_t nch = (int64_t)cnt[AC_CHUNKS], items = nch + (int64_t)cnt[AC_CTA];
+  const int64_t nch = CLASS == AC_CTA ? (int64_t)cnt[AC_CHUNKS] : 0, items = nch + (int64_t)cnt[CLASS];
   if (blockIdx.x >= items) return;
   for (int j = threadIdx.x; j < AG_CCAP; j += AG_CNT) {
     keys[j] = AG_EMPTY;
@@ -400,7 +405,7 @@ __global__ void __launch_bounds__(AG_CNT) k_ag_cta(const int64_t* __restrict__ s
       p += ch_off[it];
       left -= ch_off[it];
     }
-    const int len = left < AG_CHUNK ? (int)left : AG_CHUNK;
+    const int len = left < MAX ? (int)left : MAX;
     const unsigned lg = lg_for(2 * len);
     for (int j0 = threadIdx.x; j0 < len; j0 += 4 * AG_CNT) {
       int32_t key[4];
@@ -646,7 +651,7 @@ int aggregate_as(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_de
   int rc = CD_OK;
   // scratch
   Arena scratch;
-  int32_t *nl, *ab, *t8, *t32, *wl, *cl, *ll, *ch_seg, *dch, *tlg, *owner = nullptr, *gk = nullptr;
+  int32_t *nl, *ab, *t8, *t32, *wl, *ml, *cl, *ll, *ch_seg, *dch, *tlg, *owner = nullptr, *gk = nullptr;
   int64_t *delta, *sstart, *ch_off, *toff, *ucnt;
   unsigned long long *arcs, *cnt, *ub, *gs = nullptr;
   V* aw;
@@ -670,7 +675,8 @@ int aggregate_as(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_de
   };
   const int64_t max_big = m / (AG_CTA_MAX + 1) + 1;           // large segments at most
   const int64_t max_chunks = m / AG_CHUNK + max_big;          // their chunks at most
-  const int64_t max_cta = m / (AG_WARP_MAX + 1) + 1;          // CTA segments at most
+  const int64_t max_mid = std::min(k, m / (AG_WARP_MAX + 1) + 1);  // segments of each CTA class at most
+  const int64_t max_cta = std::min(k, m / (AG_MID_MAX + 1) + 1);
   const bool big = m > AG_CTA_MAX;                            // there may be large segments
   scratch.add(&nl, n);
   scratch.add(&delta, std::max(n, k));
@@ -682,6 +688,7 @@ int aggregate_as(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_de
   scratch.add(&t8, std::min(k, m + 1));
   scratch.add(&t32, std::min(k, m / 9 + 1));
   scratch.add(&wl, std::min(k, m / 33 + 1));
+  scratch.add(&ml, max_mid);
   scratch.add(&cl, max_cta);
   scratch.add(&ll, max_big);
   scratch.add(&ch_seg, max_chunks);
@@ -721,17 +728,23 @@ int aggregate_as(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_de
     KTimer t(g, K_AGG_REDUCE, (double)m * 2 * (4 + sizeof(V)) + (double)k * 32);
     AG_CHECK(cudaMemsetAsync(cnt, 0, sizeof(h), s));
     static std::atomic<bool> attrs{false};  // idempotent; threads may race here
+    auto mid = k_ag_cta<V, 128, AG_MID_MAX, AC_MID>;
+    auto cta = k_ag_cta<V, 512, AG_CTA_MAX, AC_CTA>;
+    constexpr size_t msm = ag_cta_smem<V, AG_MID_MAX>(), csm = ag_cta_smem<V, AG_CTA_MAX>();
     if (!attrs) {
       AG_CHECK(cudaFuncSetAttribute(k_ag_warp<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ag_warp_smem<V>()));
-      AG_CHECK(cudaFuncSetAttribute(k_ag_cta<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ag_cta_smem<V>()));
+      AG_CHECK(cudaFuncSetAttribute(mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msm));
+      AG_CHECK(cudaFuncSetAttribute(cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
       attrs = true;
     }
     if (m > 0) {
-      CD_LAUNCH(k_ag_classes<<<gcap((k + AF_SEGS - 1) / AF_SEGS, 152 * 8), NT, 0, s>>>(sstart, k, cnt, t8, t32, wl, cl, ll,
-                                                                                    ch_seg, ch_off));
+      CD_LAUNCH(k_ag_classes<<<gcap((k + AF_SEGS - 1) / AF_SEGS, 152 * 8), NT, 0, s>>>(sstart, k, cnt, t8, t32, wl, ml, cl,
+                                                                                    ll, ch_seg, ch_off));
+      if (m > AG_MID_MAX)
+        CD_LAUNCH((cta<<<gcap(max_cta + max_chunks, 152 * 2), 512, csm, s>>>(sstart, cl, ch_seg, ch_off, cnt, ab, aw, ucnt,
+                                                                             dch, ub)));
       if (m > AG_WARP_MAX)
-        CD_LAUNCH(k_ag_cta<V><<<gcap(max_cta + max_chunks, 152 * 2), AG_CNT, ag_cta_smem<V>(), s>>>(
-            sstart, cl, ch_seg, ch_off, cnt, ab, aw, ucnt, dch, ub));
+        CD_LAUNCH((mid<<<gcap(max_mid, 152 * 10), 128, msm, s>>>(sstart, ml, ch_seg, ch_off, cnt, ab, aw, ucnt, dch, ub)));
       CD_LAUNCH(k_ag_warp<V><<<gcap((k + NW - 1) / NW, 152 * 4), NT, ag_warp_smem<V>(), s>>>(sstart, t8, t32, wl, cnt, ab,
                                                                                           aw, ucnt));
     }
