@@ -345,7 +345,7 @@ def kernel_group(name: str) -> str:
     base = m.group(1)
     rest = name[m.end():]
     targs = rest[1:rest.find(">")].split(",") if rest.startswith("<") else []
-    if base in ("k_hub_prepare", "k_hub_route"):
+    if base in ("k_hub_sort", "k_hub_prepare", "k_hub_retry", "k_hub_route"):
         return "hub_prepare"
     if base in ("k_hub_build_cl", "k_hub_build"):
         return "hub_build"
@@ -359,7 +359,9 @@ def kernel_group(name: str) -> str:
         return "scan_tile" + targs[0].strip()
     if base == "k_scan_warp":
         return "scan_warp"
-    if base == "k_first_round":
+    if base in ("k_rounds", "k_rounds_init"):
+        return "resident round loop"
+    if base in ("k_first_round", "k_first_hubs"):
         return "first round (every bin)"
     if base == "k_compact":
         return "frontier"

@@ -298,6 +298,7 @@ int graph_adopt(cudaStream_t s, int64_t n, int64_t nnz, int64_t* off, int32_t* c
 int ensure_run_state(cd_graph* g);
 int ensure_bins(cd_graph* g);  // bin lists and hub structures of the per-round kernels
 int ensure_resident_hubs(cd_graph* g);
+void drop_resident_hubs(cd_graph* g);
 // Recompute the degree bins and hub structures for new boundaries.
 int rebin(cd_graph* g, int t_warp, int t_hub);
 int check_labels(cd_graph* g, const int32_t* labels_dev);  // CD_EINVAL if out of [0, n)

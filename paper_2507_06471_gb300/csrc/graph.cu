@@ -766,6 +766,8 @@ int ensure_bins(cd_graph* g) {
   return rc;
 }
 
+void drop_resident_hubs(cd_graph* g) { free_resident_hubs(g); }
+
 int ensure_resident_hubs(cd_graph* g) {
   if (g->rh) return CD_OK;
   cudaStream_t s = g->stream;

@@ -1,13 +1,18 @@
 // The round loop of a run or Louvain level as one resident kernel, for graphs
-// without hubs or with few of them: every round of Label Propagation (Algorithm 1) or local moving
-// (Algorithm 2), synchronous, with the decisions, coins, counters and stop
-// tests of the per-round kernels in scan.cu (the results are the same).
+// without hubs or with few of them: every round of Label Propagation
+// (Algorithm 1) or local moving (Algorithm 2), synchronous, with the decisions,
+// coins, counters and stop tests of the per-round kernels in scan.cu (the
+// results are the same).
 //
 // Why: a round of a small graph, or a late round of a large one, examines few
 // vertices, and its time is latency: a dozen launches of 3 to 8 us each, a
 // compaction over all n list entries, a read-back and a synchronisation. The
 // 10,000-vertex planted partition took 49 us a round that way (43 rounds, 2.1
-// ms), the 1M-vertex LFR-style graph 165 us (233 rounds, 38.5 ms).
+// ms), the 1M-vertex LFR-style graph 165 us (233 rounds, 38.5 ms). So: 12 us a
+// round (0.50 ms) and 75 us (17.4 ms). What bounds a small round is then the
+// chain of one warp's work (flags, offsets, columns, labels, Sigma_tot: dependent
+// loads) and the two barriers; what bounds a large one is the instructions of the
+// table inserts.
 //
 // How: one cooperative launch of at most one wave of 256-thread CTAs. The
 // vertices are dealt out in units of 1 to 32 consecutive ids round robin, so
@@ -46,9 +51,14 @@ constexpr int PCAP = WARP_CAP_SLOTS;      // table slots per warp; four warps' t
 static_assert(4 * PCAP == BLK1_CAP_SLOTS, "a half CTA's table is its four warps' tables");
 constexpr int CH_VERTS = 2048;            // vertices a CTA takes per step
 constexpr int CH_PER_WARP = CH_VERTS / PNT;
-// Arcs per CTA at least: a small graph gets fewer CTAs, which meet faster.
+// Arcs per CTA at least (or vertices enough for a step): a small graph gets fewer CTAs, which meet faster.
 constexpr int64_t ARCS_PER_CTA = 512;
 constexpr int PBINS = 6;                  // task order: half CTA, warp, 32, 16, 8, 4 lanes
+// Isolated vertices at most, where they are the majority: the resident loop looks
+// at every vertex's flag each round, the per-round kernels' lists leave them out.
+// LPA with 1e6 arcs among 1e5 vertices: 2.85 -> 1.76 ms with 1e7 vertices in all,
+// 3.08 -> 5.58 ms with 5e7.
+constexpr int64_t MAX_ISOLATED = (int64_t)1 << 23;
 constexpr int TRACE_COLS = 8;             // examined, arcs, moved, deferred, candidates, arcs of moved, -, -
 constexpr int HEAD = 8;                   // int64 words before the trace: rounds, moves, status
 constexpr int64_t WAIT_LIMIT = (int64_t)1 << 24;  // polls of one barrier (seconds), then CD_ETIMEOUT
@@ -831,7 +841,8 @@ int launch_loop(cd_graph* g, const ScanCtx& s, LoopCtx L, int share) {
     r = std::max(1, per) * loop_sms();
     resident.store(r);
   }
-  const int64_t grid = std::max<int64_t>(1, std::min(std::min<int64_t>(std::max(1, r / share), L.n), g->nnz / ARCS_PER_CTA));
+  const int64_t useful = std::max(g->nnz / ARCS_PER_CTA, L.n / CH_VERTS);
+  const int64_t grid = std::max<int64_t>(1, std::min(std::min<int64_t>(std::max(1, r / share), L.n), useful));
   // the largest units that still give every CTA four
   L.lgu = 5;
   while (L.lgu > 0 && (L.n >> L.lgu) < 4 * grid) --L.lgu;
@@ -885,6 +896,7 @@ ScanCtx loop_ctx(cd_graph* g, const RunOpts& o, bool louv, bool nk) {
 
 bool resident_rounds_apply(const cd_graph* g, const RunOpts& o, bool per_graph_stop) {
   return o.device_loop && !g->timing && !o.async_mode && o.max_iter > 0 && g->n > 0 &&
+         g->n_isolated <= std::max(g->n - g->n_isolated, MAX_ISOLATED) &&
          (g->nhubs == 0 || (g->nhubs <= RH_MAX_HUBS && g->nnz <= RH_MAX_ARCS)) &&
          g->bin_start[B_BLK4 + 1] == g->bin_start[B_BLK4] && (!per_graph_stop || (o.threshold == 0 && o.use_frontier));
 }
@@ -955,7 +967,11 @@ int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, i
   };
   rc = run();
   scratch.free(st);
-  if (rc) return rc;
+  if (rc) {  // the hubs' tables may hold entries of the round that was cut short
+    drop_resident_hubs(g);
+    if (status) cudaMemsetAsync(g->status, 0, sizeof(int32_t), st);
+    return rc;
+  }
   const int32_t rounds = (int32_t)h[0];
   int64_t moves = 0;
   for (int32_t r = 0; r < rounds; ++r) {

@@ -9,7 +9,7 @@
 // 16-byte column load): the rows that start inside the tile are marked in
 // shared memory and a running maximum turns the marks into the row of each arc.
 // Sum over the arcs inside communities, R-MAT scale 23 (2.6e8 arcs): 6.57 ms
-// with a warp per row, 1.21 ms so (0.78 ms is what gathering 2.6e8 labels from
+// with a warp per row, 1.05 ms so (0.78 ms is what gathering 2.6e8 labels from
 // L2 takes by itself, at one 32-byte sector per clock and SM).
 #pragma once
 #include "common.cuh"

@@ -1,4 +1,4 @@
-"""Aggregation at the edges of its segment classes (8, 32, 256 and 4,096 arcs, chunks of 4,096 above), with 32- and
+"""Aggregation at the edges of its segment classes (8, 32, 256, 1,024 and 4,096 arcs, chunks of 4,096 above), with 32- and
 64-bit weights, loops and isolated vertices, against a plain numpy summation. Integers: equal."""
 import numpy as np
 import pytest
@@ -19,7 +19,7 @@ def graph(n, m, seed, wmax, loops):
 
 
 @pytest.mark.parametrize("wmax,loops", [(1, 0), (6, 40), (1_000_000, 7)])
-@pytest.mark.parametrize("sizes", [[1, 7, 8, 9, 31, 32, 33, 255, 256, 257], [4095, 4096, 4097, 8193, 3, 1], [30000, 9, 300]])
+@pytest.mark.parametrize("sizes", [[1, 7, 8, 9, 31, 32, 33, 255, 256, 257], [1023, 1024, 1025, 2, 511], [4095, 4096, 4097, 8193, 3, 1], [30000, 9, 300]])
 def test_segment_edges(sizes, wmax, loops):
     import paper_2507_06471_gb300 as cd
     n = 12_000

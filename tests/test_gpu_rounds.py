@@ -107,3 +107,16 @@ def test_batched_equals_host_loop():
         assert np.array_equal(a[0].cpu().numpy(), b[0].cpu().numpy()) and np.array_equal(a[1], b[1])
         assert np.array_equal(a[2], b[2])
     G.close()
+
+
+@pytest.mark.parametrize("isolated", [100_000, (1 << 23), (1 << 23) + 1])
+def test_mostly_isolated(isolated):
+    # both sides of the line from which graphs of isolated vertices take the per-round kernels
+    import torch
+    g = degrees_graph(2000, [300, 40, 17], 4, 3)
+    alone = int((np.diff(g.numpy()[0]) == 0).sum())
+    tail = torch.full((isolated - alone,), int(g.off[-1]), dtype=g.off.dtype)
+    got = check(type("G", (), {"off": torch.cat([g.off, tail]), "cols": g.cols, "w": g.w}), {})
+    n = len(got[0])
+    lab, tr = oracle.lpa(*g.numpy())
+    assert np.array_equal(got[0], np.concatenate([lab, np.arange(2000, n)])) and got[1] == tr.rounds
