@@ -180,7 +180,8 @@ struct CtaSums {
       lo[i] = hi[i] = 0;
     }
   }
-  __device__ __forceinline__ void add(unsigned long long* global, int32_t k, unsigned long long x) {
+  // The slot the sum went to, -1: straight to the global array.
+  __device__ __forceinline__ int add(unsigned long long* global, int32_t k, unsigned long long x) {
     unsigned h = ((uint32_t)k * 2654435761u) >> 23;
     for (int probe = 0; probe < 4; ++probe) {
       int32_t c = *(volatile int32_t*)&key[h];
@@ -189,11 +190,12 @@ struct CtaSums {
         const uint32_t xl = (uint32_t)x, old = atomicAdd(&lo[h], xl);
         const uint32_t up = (uint32_t)(x >> 32) + (old + xl < old ? 1u : 0u);
         if (up) atomicAdd(&hi[h], up);
-        return;
+        return (int)h;
       }
       h = (h + 1) & (SLOTS - 1);
     }
     atomicAdd(&global[k], x);
+    return -1;
   }
   __device__ __forceinline__ void flush(unsigned long long* global) {  // after __syncthreads()
     for (int i = threadIdx.x; i < SLOTS; i += blockDim.x)
