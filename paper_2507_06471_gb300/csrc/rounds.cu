@@ -54,6 +54,12 @@ constexpr int CH_PER_WARP = CH_VERTS / PNT;
 // Arcs per CTA at least (or vertices enough for a step): a small graph gets fewer CTAs, which meet faster.
 constexpr int64_t ARCS_PER_CTA = 512;
 constexpr int PBINS = 6;                  // task order: half CTA, warp, 32, 16, 8, 4 lanes
+// Arcs of a loop that takes a share of the GPU (the server's workers) at most:
+// larger graphs are bound by the work of their rounds, and the per-round kernels
+// of several workers fill the GPU better. 256 requests of up to 2e6 vertices,
+// four workers: 67 requests/s with every loop on a quarter of the GPU, 105 with
+// the large ones on all of it (graphs without hubs), 120 so.
+constexpr int64_t SHARED_LOOP_ARCS = (int64_t)1 << 22;
 // Isolated vertices at most, where they are the majority: the resident loop looks
 // at every vertex's flag each round, the per-round kernels' lists leave them out.
 // LPA with 1e6 arcs among 1e5 vertices: 2.85 -> 1.76 ms with 1e7 vertices in all,
@@ -897,6 +903,7 @@ ScanCtx loop_ctx(cd_graph* g, const RunOpts& o, bool louv, bool nk) {
 bool resident_rounds_apply(const cd_graph* g, const RunOpts& o, bool per_graph_stop) {
   return o.device_loop && !g->timing && !o.async_mode && o.max_iter > 0 && g->n > 0 &&
          g->n_isolated <= std::max(g->n - g->n_isolated, MAX_ISOLATED) &&
+         (o.share <= 1 || g->nnz <= SHARED_LOOP_ARCS) &&
          (g->nhubs == 0 || (g->nhubs <= RH_MAX_HUBS && g->nnz <= RH_MAX_ARCS)) &&
          g->bin_start[B_BLK4 + 1] == g->bin_start[B_BLK4] && (!per_graph_stop || (o.threshold == 0 && o.use_frontier));
 }
