@@ -372,6 +372,13 @@ __host__ __device__ constexpr int hub_class(int64_t cap) {
   return cap <= HUB_CL0_SLOTS ? 0 : cap <= HUB_CL1_SLOTS ? 1 : cap <= 2 * HUB_CL_SLOTS ? 2
        : cap <= 4 * HUB_CL_SLOTS ? 3 : cap <= 8 * HUB_CL_SLOTS ? 4 : -1;
 }
+// The least build class of a row whose allocation is `cap` slots (1.5 per arc): up
+// to 8,192 arcs for 256 threads, about 32,768 per CTA of 512 above. By the size of
+// the table alone a row of a million arcs with few labels went to 256 threads,
+// which the whole build then waited for (R-MAT 24: step 511 -> 500 ms).
+__host__ __device__ constexpr int hub_row_class(int64_t cap) {
+  return cap <= 12 << 10 ? 0 : cap <= 48 << 10 ? 1 : cap <= 96 << 10 ? 2 : cap <= 192 << 10 ? 3 : 4;
+}
 template <int CI> struct HubClass;  // CTAs per cluster, threads per CTA, table slots per CTA
 template <> struct HubClass<0> { static constexpr int C = 1, NT = 256, SLOTS = HUB_CL0_SLOTS; };
 template <> struct HubClass<1> { static constexpr int C = 1, NT = 512, SLOTS = HUB_CL1_SLOTS; };
@@ -421,6 +428,7 @@ __global__ void __launch_bounds__(NT) k_hub_sort(ScanCtx s) {
       const int64_t nc = nl >= 0 && 2 * nl + HUB_SLACK < cap ? 2 * nl + HUB_SLACK : cap;
       c = hub_class(nc);
       if (c >= 0) {
+        c = c > hub_row_class(cap) ? c : hub_row_class(cap);
         s.hub_nc[h] = nc;
         s.hub_used[h] = 0;
         s.hub_rb[h] = HUB_REBUILD;  // cleared by the build
