@@ -45,7 +45,7 @@ __global__ void k_fix_unused(const uint8_t* __restrict__ used, int64_t n, int32_
 constexpr int RN_SMALL = 8192;
 __global__ void __launch_bounds__(1024) k_renumber_small(const int32_t* __restrict__ labels, int n, int32_t* newid,
                                                          int64_t* total) {
-  __shared__ uint8_t used[RN_SMALL];
+  __shared__ __align__(4) uint8_t used[RN_SMALL];  // cleared by words
   __shared__ int wsum[32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   constexpr int PER = RN_SMALL / 1024;
