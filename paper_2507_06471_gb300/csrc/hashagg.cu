@@ -31,7 +31,6 @@
 // The content of every row equals that of the sort-based aggregation; only the
 // order of columns inside a row differs, and no later step depends on it.
 #include <algorithm>
-#include <atomic>
 #include <type_traits>
 
 #include "common.cuh"
@@ -727,15 +726,15 @@ int aggregate_as(cd_graph* g, const int32_t* labels_dev, const int32_t* newid_de
   {
     KTimer t(g, K_AGG_REDUCE, (double)m * 2 * (4 + sizeof(V)) + (double)k * 32);
     AG_CHECK(cudaMemsetAsync(cnt, 0, sizeof(h), s));
-    static std::atomic<bool> attrs{false};  // idempotent; threads may race here
+    static PerDevice attrs;
     auto mid = k_ag_cta<V, 128, AG_MID_MAX, AC_MID>;
     auto cta = k_ag_cta<V, 512, AG_CTA_MAX, AC_CTA>;
     constexpr size_t msm = ag_cta_smem<V, AG_MID_MAX>(), csm = ag_cta_smem<V, AG_CTA_MAX>();
-    if (!attrs) {
+    if (!attrs.get()) {
       AG_CHECK(cudaFuncSetAttribute(k_ag_warp<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ag_warp_smem<V>()));
       AG_CHECK(cudaFuncSetAttribute(mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msm));
       AG_CHECK(cudaFuncSetAttribute(cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
-      attrs = true;
+      attrs.set(1);
     }
     if (m > 0) {
       CD_LAUNCH(k_ag_classes<<<gcap((k + AF_SEGS - 1) / AF_SEGS, 152 * 8), NT, 0, s>>>(sstart, k, cnt, t8, t32, wl, ml, cl,

@@ -39,7 +39,6 @@
 // Sigma_tot is kept in 32 bits when vol(V) < 2^31 (integers: exact), in 64
 // otherwise.
 #include <algorithm>
-#include <atomic>
 
 #include "scan.cuh"
 
@@ -836,16 +835,16 @@ int loop_sms() {
 
 template <bool LOUV, class W, class V, bool NK>
 int launch_loop(cd_graph* g, const ScanCtx& s, LoopCtx L, int share) {
-  static std::atomic<int> resident{0};  // CTAs at once; the same for every thread that gets here
+  static PerDevice resident;  // CTAs at once
   auto kern = k_rounds<LOUV, W, V, NK>;
   constexpr size_t sm = loop_smem<V>();
-  int r = resident.load();
+  int r = resident.get();
   if (r == 0) {
     CD_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     int per = 0;
     CD_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, PNT, sm));
     r = std::max(1, per) * loop_sms();
-    resident.store(r);
+    resident.set(r);
   }
   const int64_t useful = std::max(g->nnz / ARCS_PER_CTA, L.n / CH_VERTS);
   const int64_t grid = std::max<int64_t>(1, std::min(std::min<int64_t>(std::max(1, r / share), L.n), useful));

@@ -1482,8 +1482,8 @@ template <class V> constexpr size_t hub_smem() { return group_smem<V>(1, HUB_CAP
 
 template <bool LOUV, class W, class V, bool NK>
 int set_smem_attrs() {
-  static std::atomic<bool> done{false};  // idempotent; threads may race here
-  if (done) return CD_OK;
+  static PerDevice done;
+  if (done.get()) return CD_OK;
   CD_CHECK(cudaFuncSetAttribute(k_scan_warp<LOUV, W, V, NK>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)warp_smem<V>()));
   CD_CHECK(cudaFuncSetAttribute(k_scan_group<LOUV, W, V, 512, 512, BLK4_CAP_SLOTS, B_BLK4, false, NK>,
@@ -1498,7 +1498,7 @@ int set_smem_attrs() {
   CD_CHECK(cudaFuncSetAttribute(k_hub_build_cl<W, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hub_cl_smem<4>()));
   CD_CHECK(cudaFuncSetAttribute(k_hub_build<W, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)hub_smem<V>()));
-  done = true;
+  done.set(1);
   return CD_OK;
 }
 
