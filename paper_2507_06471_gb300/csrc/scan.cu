@@ -457,7 +457,7 @@ __device__ __forceinline__ void hub_clear(const ScanCtx& s, int32_t h, int64_t c
     atomicAdd(&s.ctr[C_HUB_PSLOTS], (unsigned long long)cap);
     s.hub_cc[h] = cap;
     s.hub_used[h] = 0;
-    s.hub_rb[h] = HUB_REBUILD;  // cleared once built (start of the evaluate kernel)
+    s.hub_rb[h] = HUB_REBUILD;  // cleared once built (k_hub_route)
     pos = atomicAdd(&s.hub_lcnt[0], (unsigned long long)ni);
   }
   __syncthreads();
@@ -856,14 +856,6 @@ __global__ void __launch_bounds__(NT) k_hub_eval(ScanCtx s) {
   __shared__ unsigned s_live;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (threadIdx.x == 0) s_live = 0;
-  {
-    const int64_t nb = (int64_t)*(volatile unsigned long long*)&s.hub_lcnt[0];
-    for (int64_t q = (int64_t)blockIdx.x * NT + threadIdx.x; q < nb; q += (int64_t)gridDim.x * NT) {
-      const int32_t it = s.hub_blist[q];
-      const int32_t h = s.hub_item_hub[it];
-      if (s.hub_item_first[h] == it) s.hub_rb[h] = 0;
-    }
-  }
   __syncthreads();
   int64_t n_act = 0, n_arcs = 0, n_cand = 0, n_def = 0, n_marcs = 0;
   const int64_t n_ev = (int64_t)*s.ev_cnt;
@@ -1284,10 +1276,20 @@ __global__ void __launch_bounds__(NT) k_compact(ScanCtx s, const int32_t* __rest
 // tables after this round's preparation: a hub with at most HUB_SMALL slots in
 // use goes to the one-warp list, a larger one's first ceil(cc / HUB_SLICE)
 // items to the item list. cnt[0] and cnt[1] count them (zeroed before).
+// It also ends the rebuild of the hubs built by items: between the builds and the
+// bins' scans, which run beside the evaluation and may flag a hub again (log
+// full). Cleared any later, such a flag would be taken for the old one: the hub
+// not queued, the flag gone and the lost updates never made good.
 __global__ void __launch_bounds__(NT) k_hub_route(ScanCtx s, int32_t* __restrict__ ev, int32_t* __restrict__ small,
                                                   unsigned long long* __restrict__ cnt) {
   const int64_t n = s.hub_act ? (int64_t)*s.hub_act_cnt : s.nhubs;
+  const int64_t nb = (int64_t)*(volatile unsigned long long*)&s.hub_lcnt[0];
   const int64_t stride = (int64_t)gridDim.x * NT;
+  for (int64_t q = (int64_t)blockIdx.x * NT + threadIdx.x; q < nb; q += stride) {
+    const int32_t it = s.hub_blist[q];
+    const int32_t h = s.hub_item_hub[it];
+    if (s.hub_item_first[h] == it) s.hub_rb[h] = 0;
+  }
   for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n; i += stride) {
     const int32_t h = s.hub_act ? s.hub_act[i] : (int32_t)i;
     const int64_t cc = s.hub_cc[h];
