@@ -76,6 +76,7 @@ __device__ __forceinline__ void warp_tile_rows(const int64_t* __restrict__ off, 
         row[j] = lo;
       }
       cur = __shfl_sync(FULL, (long long)row[3], 31);
+      __syncwarp();  // as below: lanes have written marks, and shuffles order no memory
       return;
     }
     int64_t o[4];

@@ -65,3 +65,39 @@ def test_batched_modularity_of_many_graphs_per_tile():
         assert np.array_equal(lab[vstart[b]:vstart[b + 1]], olab) and levels[b] == olv
         assert abs(q[b] - oq) <= 1e-12
     G.close()
+
+
+@pytest.mark.parametrize("run", [511, 512, 543, 544, 545, 546, 577, 700, 5000])
+@pytest.mark.parametrize("wmax", [1, 6])
+def test_long_runs_of_empty_rows(run, wmax):
+    # more rows start inside one tile than a warp marks: it searches the offsets instead, at the first and the last arcs
+    # of a tile, in tiles that follow one another, and before tiles that mark again
+    import paper_2507_06471_gb300 as cd
+    rng = np.random.default_rng(run + wmax)
+    edges, at = [], 0
+    for deg in (1, 2, 126, 127, 128, 129, 3, 1, 300, 1, 1, 1):  # a vertex joined to the `deg` ones after it, then the run
+        edges += [(at, at + 1 + i) for i in range(deg)]
+        at += deg + 1 + run
+    n = at + 1
+    edges.append((0, n - 1))
+    ws = rng.integers(1, wmax + 1, len(edges)).tolist() if wmax > 1 else None
+    g = synth.from_edge_list(n, edges, ws, {int(v): 2 for v in rng.choice(n, 7, replace=False)})
+    off, cols, w = g.numpy()
+    dw = None if g.w is None else g.w.cuda()
+    for _ in range(3):
+        G = cd.Graph(g.off.cuda(), g.cols.cuda(), dw)
+        for lab in (np.arange(n), rng.integers(0, 3, n), np.arange(n) // 7):
+            lab = lab.astype(np.int32)
+            q = oracle.modularity(off, cols, w, lab)[0]
+            dl = torch.from_numpy(lab).cuda()
+            assert abs(G.modularity(dl) - q) <= 1e-12 * max(1.0, abs(q))
+            assert abs(cd.cd_modularity_noalloc(g.off.cuda(), g.cols.cuda(), dw, dl) - q) <= 1e-12 * max(1.0, abs(q))
+            k, newid, coff, ccols, cw = oracle.aggregate(off, cols, w, lab)
+            C, kg = G.aggregate(dl)
+            goff, gcols, gw = C.download()
+            assert kg == k and np.array_equal(goff, coff)
+            for a, b in zip(goff[:-1], goff[1:]):
+                i, j = np.argsort(gcols[a:b]), np.argsort(ccols[a:b])
+                assert np.array_equal(gcols[a:b][i], ccols[a:b][j]) and np.array_equal(gw[a:b][i], cw[a:b][j])
+            C.close()
+        G.close()
