@@ -440,8 +440,9 @@ __global__ void __launch_bounds__(NT) k_hub_sort(ScanCtx s) {
   }
 }
 
-// Clear hub h's whole allocation and queue its items for k_hub_build (one CTA).
-__device__ __forceinline__ void hub_clear(const ScanCtx& s, int32_t h, int64_t cap) {
+// Clear hub h's whole allocation and queue its items for k_hub_build (one CTA);
+// the slots are counted in counter `ctr`.
+__device__ __forceinline__ void hub_clear(const ScanCtx& s, int32_t h, int64_t cap, int ctr) {
   __shared__ unsigned long long pos;
   const int64_t base = s.hub_tab[h];
   const int64_t i0 = s.hub_item_first[h], ni = s.hub_item_first[h + 1] - i0;
@@ -454,7 +455,7 @@ __device__ __forceinline__ void hub_clear(const ScanCtx& s, int32_t h, int64_t c
     }
   }
   if (threadIdx.x == 0) {
-    atomicAdd(&s.ctr[C_HUB_PSLOTS], (unsigned long long)cap);
+    atomicAdd(&s.ctr[ctr], (unsigned long long)cap);
     s.hub_cc[h] = cap;
     s.hub_used[h] = 0;
     s.hub_rb[h] = HUB_REBUILD;  // cleared once built (k_hub_route)
@@ -530,7 +531,7 @@ __global__ void __launch_bounds__(NT) k_hub_prepare(ScanCtx s) {
       __syncthreads();
       continue;
     }
-    hub_clear(s, h, cap);
+    hub_clear(s, h, cap, C_HUB_PSLOTS);
     __syncthreads();
   }
 }
@@ -540,7 +541,7 @@ __global__ void __launch_bounds__(NT) k_hub_retry(ScanCtx s) {
   const int64_t nf = (int64_t)*(volatile const unsigned long long*)&s.hub_ccnt[6];
   for (int64_t q = blockIdx.x; q < nf; q += gridDim.x) {
     const int32_t h = s.hub_pl[s.nhubs + q];
-    hub_clear(s, h, s.hub_tab[h + 1] - s.hub_tab[h]);
+    hub_clear(s, h, s.hub_tab[h + 1] - s.hub_tab[h], C_HUB_BSLOTS);  // part of the builds, and timed with them
     __syncthreads();
   }
 }
