@@ -75,13 +75,13 @@ typedef struct cd_params {
   int32_t device_loop;      /* Where the round loop runs. 1 (default): on the device where that pays. All
                                rounds of a run or Louvain level run as one resident kernel on graphs
                                without hubs (vertices of more than t_hub arcs) and on graphs of at most
-                               2^24 arcs with at most 4,095 of them; on larger ones, and in batched runs
-                               (cd_batch_*), the rounds after the first run as one captured CUDA graph (a
-                               conditional WHILE node whose body is one round) if at least 2^22 arcs and
-                               max_iter > 16 make the graph worth its making; others keep the host loop.
+                               2^24 arcs with at most 4,095 of them; otherwise the rounds after the first
+                               run as one captured CUDA graph (a conditional WHILE node whose body is one
+                               round) in batched runs (cd_batch_*), and in others if at least 2^22 arcs and
+                               max_iter > 16 make the graph worth its making; the rest keeps the host loop.
                                The round number, the stop tests and the trace stay on the device, so a
-                               level costs one launch and no per-round host synchronisation. 2: runs that
-                               are not resident always take the captured graph. 0: the host loop
+                               level costs one launch and no per-round host synchronisation. 2: the
+                               captured graph in every run, also where 1 is resident. 0: the host loop
                                everywhere (one read-back per round). Results are identical in every mode;
                                timing != 0 (per-round events) and the asynchronous mode are never
                                resident, and timing != 0 always uses the host loop */

@@ -337,8 +337,8 @@ struct RunOpts {
   bool singleton_start = false;  // the run starts from C[v] = v (Sigma_tot = deg_w, sizes 1)
   bool device_loop = false;      // the round loop runs on the device where that is possible and pays
   int share = 1;                 // a resident loop takes 1 / share of the GPU at most
-  bool graph_loop = false;       // graphs with hubs: rounds after the first run as one captured graph (batched runs)
-  bool device_loop_all = false;  // ... in every run
+  bool graph_loop = false;       // rounds after the first as one captured graph, where that pays
+  bool device_loop_all = false;  // ... in every run, those of the resident loop included
 };
 // Algorithm 1 / Algorithm 2 round loops on g->C (device). Louvain: g->C holds
 // the initial partition; sigma/csize are rebuilt from it.

@@ -900,7 +900,7 @@ ScanCtx loop_ctx(cd_graph* g, const RunOpts& o, bool louv, bool nk) {
 }  // namespace
 
 bool resident_rounds_apply(const cd_graph* g, const RunOpts& o, bool per_graph_stop) {
-  return o.device_loop && !g->timing && !o.async_mode && o.max_iter > 0 && g->n > 0 &&
+  return o.device_loop && !o.device_loop_all && !g->timing && !o.async_mode && o.max_iter > 0 && g->n > 0 &&
          g->n_isolated <= std::max(g->n - g->n_isolated, MAX_ISOLATED) &&
          (o.share <= 1 || g->nnz <= SHARED_LOOP_ARCS) &&
          (g->nhubs == 0 || (g->nhubs <= RH_MAX_HUBS && g->nnz <= RH_MAX_ARCS)) &&

@@ -1,0 +1,77 @@
+"""The three forms of the round loop (one resident kernel, one captured graph, the host loop) on graphs small enough for
+the resident one: which form a run takes, and equal results of the captured one with every kind of hub table and key.
+Integers: everything must be equal."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+KEYS = ("level", "round", "active", "arcs", "moved", "deferred", "cands", "moved_arcs")
+
+
+def hub_graph(wmax, loops):
+    """Two hubs (1,500 and 3,000 arcs) over a planted partition, weights up to wmax, loops on some vertices."""
+    rng = np.random.default_rng(wmax % 1000 + loops)
+    base = synth.sbm(6000, 60, "0.08", "0.0005", seed=9)
+    bu = np.repeat(np.arange(base.n), np.diff(base.off.numpy()))
+    edges = {(int(a), int(b)) for a, b in zip(bu, base.cols.numpy()) if a < b}
+    for hub, d in ((0, 1500), (1, 3000)):
+        edges |= {(hub, int(x)) for x in rng.choice(np.arange(2, base.n), d, replace=False)}
+    edges = sorted(edges)
+    ws = rng.integers(max(1, wmax // 2), wmax + 1, len(edges)).tolist() if wmax > 1 else None
+    lo = {int(v): int(rng.integers(1, wmax + 1)) for v in rng.choice(base.n, loops, replace=False)} if loops else None
+    return synth.from_edge_list(base.n, edges, ws, lo)
+
+
+def upload(g):
+    import paper_2507_06471_gb300 as cd
+    return cd.Graph(g.off.cuda(), g.cols.cuda(), None if g.w is None else g.w.cuda())
+
+
+def run(G, loop, call, **params):
+    """(results, kernels launched) of one call."""
+    import paper_2507_06471_gb300 as cd
+    before = cd.cd_launch_count()
+    out = getattr(G, call)(device_loop=loop, **params)
+    launches = cd.cd_launch_count() - before
+    out = [x.cpu().numpy() if torch.is_tensor(x) else x for x in out]
+    return out, [{k: t[k] for k in KEYS} for t in G.trace()], launches
+
+
+# packed tables; loops; 128-bit keys with packed tables (vol(V) >= 2^31 but every deg_w < 2^32); two-word tables
+@pytest.mark.parametrize("wmax,loops", [(1, 0), (7, 40), (100_000, 0), (2_000_000_000, 3)])
+@pytest.mark.parametrize("call", ["lpa", "local_move", "louvain"])
+def test_captured_graph(wmax, loops, call):
+    g = hub_graph(wmax, loops)
+    off, cols, w = g.numpy()
+    dw, vol = oracle.degw(off, cols, w)
+    assert (vol >= 2**31) == (wmax >= 100_000) and (dw.max() >= 2**32) == (wmax > 10**9)
+    G = upload(g)
+    for loop in (0, 1, 2):  # lays the structures of the form out
+        getattr(G, call)(device_loop=loop)
+    res = {loop: run(G, loop, call) for loop in (0, 1, 2)}
+    few = {loop: run(G, loop, call, max_iter=4) for loop in (0, 1, 2)}
+    G.close()
+    for r in (res, few):
+        for loop in (1, 2):
+            for a, b in zip(r[loop][0], r[0][0]):
+                assert np.array_equal(a, b)
+            assert r[loop][1] == r[0][1]
+    if call != "louvain":
+        # launches: the resident loop's two kernels, a captured graph's however many rounds it runs, the host loop's more
+        # with every round
+        assert res[1][2] == few[1][2] <= 3 < few[2][2] == res[2][2] < res[0][2]
+        assert few[0][2] < res[0][2]
+    if call == "lpa":
+        lab, tr = oracle.lpa(off, cols, w)
+        assert np.array_equal(res[2][0][0], lab) and res[2][0][1] == tr.rounds
+    elif call == "local_move":
+        lab, moves, tr = oracle.local_move(off, cols, w)
+        assert np.array_equal(res[2][0][0], lab) and res[2][0][1:] == [moves, tr.rounds]
+    else:
+        lab, lv, q, _ = oracle.louvain(off, cols, w)
+        assert np.array_equal(res[2][0][0], lab) and res[2][0][1] == lv
