@@ -186,6 +186,11 @@ struct cd_graph {
   bool cols_distinct = false;      // no row repeats a column (strictly increasing input rows, or coarse rows)
   int t_warp = cd::WARP_MAX;       // degrees 33..t_warp: a warp per vertex
   int t_hub = cd::BLOCK_MAX;       // degrees t_warp+1..t_hub: 128 threads (512 above 1024); above: hub
+  // Graphs of the server's workers, unless its caller chose a loop: the number of workers (0: not served). They use
+  // resident loops, but no captured graphs (several workers instantiating graphs at once cost more than the read-backs
+  // they save), and a resident loop takes 1 / workers of the GPU at most, so that the workers' loops run side by side:
+  // loops that fill the GPU run one after another, and most of a loop's time is latency. Coarse graphs inherit it.
+  int workers = 0;
   bool bins_set = false;           // thresholds chosen by cd_graph_set_bins / cd_autotune (kept by coarse graphs)
 
   // run state (one allocation, made on first use; the pointers below are parts of it)
@@ -336,9 +341,7 @@ struct RunOpts {
   int async_mode = 0;  // committed moves take effect at once (the coin still defers half of them)
   bool singleton_start = false;  // the run starts from C[v] = v (Sigma_tot = deg_w, sizes 1)
   bool device_loop = false;      // the round loop runs on the device where that is possible and pays
-  int share = 1;                 // a resident loop takes 1 / share of the GPU at most
-  bool graph_loop = false;       // rounds after the first as one captured graph, where that pays
-  bool device_loop_all = false;  // ... in every run, those of the resident loop included
+  bool device_loop_all = false;  // ... as one captured graph in every run, those of the resident loop included
 };
 // Algorithm 1 / Algorithm 2 round loops on g->C (device). Louvain: g->C holds
 // the initial partition; sigma/csize are rebuilt from it.
@@ -351,14 +354,6 @@ void release_batches(cd_graph* g);
 int run_local_move(cd_graph* g, const RunOpts& o, int init_given, int64_t* moves_out,
                    int32_t* rounds_out);
 RunOpts opts_from(const cd_params* p, int32_t level);
-// cd_params.device_loop of the server's workers when the caller left the
-// default: resident loops, but no captured graphs (several workers
-// instantiating graphs at once cost more than the read-backs they save). The
-// low bits hold the number of workers: a resident loop takes that share of the
-// GPU at most, so that the workers' loops run side by side. Loops that fill the
-// GPU run one after another, and most of a loop's time is latency.
-constexpr int32_t LOOP_NO_GRAPH = 0x10000;
-
 // A solo run on a graph with hubs of at least GRAPH_LOOP_ARCS arcs and with at
 // least GRAPH_LOOP_ROUNDS rounds to go takes the captured graph too: its launches
 // follow one another without the host's gaps and read-backs (LPA 19.7 -> 18.7 ms

@@ -840,6 +840,7 @@ int graph_adopt(cudaStream_t s, int64_t n, int64_t nnz, int64_t* off, int32_t* c
     g->t_warp = like->t_warp;
     g->t_hub = like->t_hub;
     g->bins_set = like->bins_set;
+    g->workers = like->workers;
     if (!g->bins_set && nnz >= COARSE_HUB_ARCS && g->t_hub > COARSE_T_HUB && g->t_warp <= COARSE_T_HUB)
       g->t_hub = COARSE_T_HUB;
     if (g->t_hub != like->t_hub) bins_pre = nullptr;  // counted for the other threshold

@@ -834,7 +834,7 @@ int loop_sms() {
 }
 
 template <bool LOUV, class W, class V, bool NK>
-int launch_loop(cd_graph* g, const ScanCtx& s, LoopCtx L, int share) {
+int launch_loop(cd_graph* g, const ScanCtx& s, LoopCtx L) {
   static PerDevice resident;  // CTAs at once
   auto kern = k_rounds<LOUV, W, V, NK>;
   constexpr size_t sm = loop_smem<V>();
@@ -847,7 +847,7 @@ int launch_loop(cd_graph* g, const ScanCtx& s, LoopCtx L, int share) {
     resident.set(r);
   }
   const int64_t useful = std::max(g->nnz / ARCS_PER_CTA, L.n / CH_VERTS);
-  const int64_t grid = std::max<int64_t>(1, std::min(std::min<int64_t>(std::max(1, r / share), L.n), useful));
+  const int64_t grid = std::max<int64_t>(1, std::min(std::min<int64_t>(std::max(1, r / std::max(1, g->workers)), L.n), useful));
   // the largest units that still give every CTA four
   L.lgu = 5;
   while (L.lgu > 0 && (L.n >> L.lgu) < 4 * grid) --L.lgu;
@@ -859,13 +859,13 @@ int launch_loop(cd_graph* g, const ScanCtx& s, LoopCtx L, int share) {
 }
 
 template <bool LOUV, bool NK>
-int dispatch_loop(cd_graph* g, const ScanCtx& s, const LoopCtx& L, int share) {
+int dispatch_loop(cd_graph* g, const ScanCtx& s, const LoopCtx& L) {
   const bool v32 = g->max_degw < ((int64_t)1 << 32);
   if (g->wkind == W_UNIT)
-    return v32 ? launch_loop<LOUV, WUnit, uint32_t, NK>(g, s, L, share) : launch_loop<LOUV, WUnit, unsigned long long, NK>(g, s, L, share);
+    return v32 ? launch_loop<LOUV, WUnit, uint32_t, NK>(g, s, L) : launch_loop<LOUV, WUnit, unsigned long long, NK>(g, s, L);
   if (g->wkind == W_I32)
-    return v32 ? launch_loop<LOUV, WI32, uint32_t, NK>(g, s, L, share) : launch_loop<LOUV, WI32, unsigned long long, NK>(g, s, L, share);
-  return v32 ? launch_loop<LOUV, WI64, uint32_t, NK>(g, s, L, share) : launch_loop<LOUV, WI64, unsigned long long, NK>(g, s, L, share);
+    return v32 ? launch_loop<LOUV, WI32, uint32_t, NK>(g, s, L) : launch_loop<LOUV, WI32, unsigned long long, NK>(g, s, L);
+  return v32 ? launch_loop<LOUV, WI64, uint32_t, NK>(g, s, L) : launch_loop<LOUV, WI64, unsigned long long, NK>(g, s, L);
 }
 
 // The parts of the context the resident kernel uses (no hubs, no counters).
@@ -902,7 +902,7 @@ ScanCtx loop_ctx(cd_graph* g, const RunOpts& o, bool louv, bool nk) {
 bool resident_rounds_apply(const cd_graph* g, const RunOpts& o, bool per_graph_stop) {
   return o.device_loop && !o.device_loop_all && !g->timing && !o.async_mode && o.max_iter > 0 && g->n > 0 &&
          g->n_isolated <= std::max(g->n - g->n_isolated, MAX_ISOLATED) &&
-         (o.share <= 1 || g->nnz <= SHARED_LOOP_ARCS) &&
+         (g->workers <= 1 || g->nnz <= SHARED_LOOP_ARCS) &&
          (g->nhubs == 0 || (g->nhubs <= RH_MAX_HUBS && g->nnz <= RH_MAX_ARCS)) &&
          g->bin_start[B_BLK4 + 1] == g->bin_start[B_BLK4] && (!per_graph_stop || (o.threshold == 0 && o.use_frontier));
 }
@@ -949,8 +949,8 @@ int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, i
     CD_LAUNCH(k_rounds_init<<<gi, PNT, 0, st>>>(L, g->C, g->sigma, g->csize, g->degw, louv ? 1 : 0, singletons ? 1 : 0,
                                                 words));
     const ScanCtx s = loop_ctx(g, o, louv, nk);
-    int r = !louv ? dispatch_loop<false, false>(g, s, L, o.share) : nk ? dispatch_loop<true, true>(g, s, L, o.share)
-                                                              : dispatch_loop<true, false>(g, s, L, o.share);
+    int r = !louv ? dispatch_loop<false, false>(g, s, L) : nk ? dispatch_loop<true, true>(g, s, L)
+                                                              : dispatch_loop<true, false>(g, s, L);
     if (r) return r;
     CD_CHECK(cudaGetLastError());
     // the header and the rounds of a usual run in one copy

@@ -2046,9 +2046,10 @@ int run_rounds(cd_graph* g, const RunOpts& o, bool louv, int64_t* moves_out, int
     for (auto& e : ev) cudaEventCreate(&e);
   // rounds after the first as one captured graph (a device-side loop) unless
   // per-round events are wanted
-  const bool dev_loop = o.graph_loop && !g->timing &&
-                        (o.batched || o.device_loop_all ||
-                         (g->nnz >= GRAPH_LOOP_ARCS && o.max_iter > GRAPH_LOOP_ROUNDS));
+  const bool dev_loop = o.device_loop && !g->timing &&
+                        (o.device_loop_all ||
+                         (g->workers == 0 &&
+                          (o.batched || (g->nnz >= GRAPH_LOOP_ARCS && o.max_iter > GRAPH_LOOP_ROUNDS))));
   for (int32_t r = 0; r < o.max_iter && rc == CD_OK; ++r) {
     if (r > 0 && dev_loop) {
       rc = device_rounds(g, o, louv, use_s32, per_graph_stop, r, fcur, fnxt, prev_moves, total_moves, rounds,
@@ -2294,9 +2295,6 @@ RunOpts opts_from(const cd_params* p, int32_t level) {
   o.level = level;
   o.async_mode = p->asynchronous ? 1 : 0;
   o.device_loop = p->device_loop != 0;
-  const bool served = p->device_loop > LOOP_NO_GRAPH && p->device_loop <= LOOP_NO_GRAPH + 64;
-  o.graph_loop = p->device_loop != 0 && !served;
-  o.share = served ? p->device_loop - LOOP_NO_GRAPH : 1;
   o.device_loop_all = p->device_loop == 2;
   return o;
 }

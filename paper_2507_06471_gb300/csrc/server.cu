@@ -67,11 +67,15 @@ int64_t estimate_bytes(int64_t n, int64_t nnz) {
   return 64 * nnz + 96 * n + (16ll << 20);
 }
 
+// cd_graph.workers of a request's graph: a caller's own choice of loop stands.
+int worker_loops(const cd_server* s) { return s->params.device_loop == 1 ? s->slots : 0; }
+
 void solve_one(cd_server* s, cudaStream_t st, Request& r) {
   cd_graph* g = nullptr;
   int rc = cd_csr_upload(r.off.data(), 1, r.cols.data(), r.w.empty() ? nullptr : r.w.data(), r.n, r.nnz, 0, st, &g);
   r.labels.assign(r.n, 0);
   if (!rc) {
+    g->workers = worker_loops(s);
     if (r.kind == CD_REQ_LPA)
       rc = cd_lpa_run(g, &s->params, r.labels.data(), 0, &r.iters);
     else
@@ -101,7 +105,10 @@ void solve_packed(cd_server* s, cudaStream_t st, std::vector<std::shared_ptr<Req
   }
   cd_graph* g = nullptr;
   int rc = cd_csr_upload(off.data(), 1, cols.data(), weighted ? w.data() : nullptr, n, nnz, 0, st, &g);
-  if (!rc) rc = cd_graph_set_batches(g, vstart.data(), B, 0);
+  if (!rc) {
+    g->workers = worker_loops(s);
+    rc = cd_graph_set_batches(g, vstart.data(), B, 0);
+  }
   std::vector<int32_t> lab(n, 0), iters(B, 0);
   std::vector<double> q(B, 0.0);
   if (!rc) {
@@ -217,10 +224,6 @@ int cd_server_create(const cd_params* p, int32_t slots, int64_t mem_budget_bytes
   cd_server* s = new cd_server();
   s->params = *p;
   s->params.timing = 0;
-  // by default (1) the workers' calls use resident loops but no captured
-  // graphs: several workers capturing and instantiating round graphs at once
-  // cost more than the round trips they save (2 still forces them)
-  if (s->params.device_loop == 1) s->params.device_loop = cd::LOOP_NO_GRAPH + slots;
   cudaGetDevice(&s->device);
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {

@@ -75,3 +75,20 @@ def test_captured_graph(wmax, loops, call):
     else:
         lab, lv, q, _ = oracle.louvain(off, cols, w)
         assert np.array_equal(res[2][0][0], lab) and res[2][0][1] == lv
+
+
+@pytest.mark.parametrize("loop", [3, -1, 0x10001, 0x10004, 0x10040])
+def test_other_values_of_device_loop_are_the_default(loop):
+    # no value of the public field stands for the serving engine's workers, which take no captured graphs
+    import paper_2507_06471_gb300 as cd
+    graphs = [synth.sbm(n, 5, "0.2", "0.002", seed=n, wmax=3) for n in (300, 900, 80)]
+    packed, vstart = synth.pack_batch(graphs)
+    G = cd.Graph(packed.off.cuda(), packed.cols.cuda(), packed.w.cuda())
+    G.set_batches(vstart)
+    G.batch_lpa(threshold=3)
+    want, trace, launches = run(G, 1, "batch_lpa", threshold=3)
+    got = run(G, loop, "batch_lpa", threshold=3)
+    host = run(G, 0, "batch_lpa", threshold=3)
+    G.close()
+    assert np.array_equal(got[0][0], want[0]) and list(got[0][1]) == list(want[1]) and got[1] == trace
+    assert got[2] == launches != host[2]
