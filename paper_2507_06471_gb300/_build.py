@@ -13,6 +13,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libcdgpu.so")
 SRCS = ["prims.cu", "graph.cu", "scan.cu", "rounds.cu", "aggregate.cu", "batch.cu", "noalloc.cu", "server.cu", "hashagg.cu"]
 HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "rowwalk.cuh"), os.path.join(CSRC, "scan.cuh"),
+           os.path.join(CSRC, "perdevice.h"),
            os.path.join(ROOT, "include", "cdgpu.h")]
 FLAGS = ["-std=c++17", "-O3", "-gencode", "arch=compute_103a,code=sm_103a", "-lineinfo",
          "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include")]

@@ -2,12 +2,12 @@
 #pragma once
 #include <cuda_runtime.h>
 
-#include <atomic>
 #include <cstdint>
 #include <string>
 #include <vector>
 
 #include "cdgpu.h"
+#include "perdevice.h"
 
 namespace cd {
 
@@ -247,27 +247,6 @@ template <class T>
 int dev_alloc_t(T** p, int64_t count, cudaStream_t s) {
   return dev_alloc((void**)p, (size_t)(count > 0 ? count : 1) * sizeof(T), s);
 }
-// A number per device, 0 at first: what a kernel's attributes and occupancy give
-// holds for the device they were asked on. Every thread would set the same value.
-class PerDevice {
-  static constexpr int MAX_DEVICES = 64;  // past it nothing is kept
-  std::atomic<int> v_[MAX_DEVICES] = {};
-  static int current() {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    return dev;
-  }
-
- public:
-  int get() const {
-    const int d = current();
-    return d < MAX_DEVICES ? v_[d].load() : 0;
-  }
-  void set(int x) {
-    const int d = current();
-    if (d < MAX_DEVICES) v_[d].store(x);
-  }
-};
 // Several arrays from one allocation: small graphs spend a microsecond on each
 // allocation and each release. add() every array, then make() sets the pointers.
 struct Arena {

@@ -10,8 +10,6 @@
 #include <cstdio>
 #include <cstring>
 
-#include <mutex>
-
 #include "common.cuh"
 #include "rowwalk.cuh"
 
@@ -37,17 +35,16 @@ int set_cuda_error(cudaError_t e) {
 }
 
 int dev_alloc(void** p, size_t bytes, cudaStream_t s) {
-  // keep freed blocks in the device's default pool (threads may race here)
-  static std::once_flag pool_set;
-  std::call_once(pool_set, [] {
-    int dev = 0;
-    cudaGetDevice(&dev);
+  // keep freed blocks in the device's default pool (threads that race here set the same)
+  static PerDevice pool_set;
+  if (!pool_set.get()) {
     cudaMemPool_t pool;
-    if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
+    if (cudaDeviceGetDefaultMemPool(&pool, current_device()) == cudaSuccess) {
       uint64_t thr = UINT64_MAX;
       cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
     }
-  });
+    pool_set.set(1);
+  }
   cudaError_t e = cudaMallocAsync(p, bytes, s);
   if (e != cudaSuccess) {
     *p = nullptr;

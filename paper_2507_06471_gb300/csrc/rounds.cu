@@ -827,9 +827,8 @@ __global__ void __launch_bounds__(PNT) k_rounds_init(LoopCtx L, int32_t* C, int6
 }
 
 int loop_sms() {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, current_device());
   return sms;
 }
 

@@ -1454,17 +1454,17 @@ unsigned grid_cap(int64_t blocks, int64_t cap = 152 * 16) {
 }
 
 // CTAs of `kernel` resident on the device at once (occupancy x SMs), cached
-// per kernel. Scan grids are capped to this: a grid-stride loop over one wave
+// per device and kernel. Scan grids are capped to this: a grid-stride loop over one wave
 // has no partly filled second wave.
 int resident_ctas(const void* kernel, int nt, size_t smem) {
   static std::mutex mu;
-  static std::unordered_map<const void*, int> cache;
+  static ByDevice<std::unordered_map<const void*, int>> caches;
   std::lock_guard<std::mutex> lock(mu);
+  auto& cache = caches.here();
   auto it = cache.find(kernel);
   if (it != cache.end()) return it->second;
-  int dev = 0, sms = 0, per = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int sms = 0, per = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, current_device());
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, nt, smem);
   const int r = std::max(1, per) * std::max(1, sms);
   cache[kernel] = r;
@@ -1525,27 +1525,6 @@ struct BinStreams {
   cudaStream_t s[4];
   bool on = false;
 };
-
-// The auxiliary streams and their events belong to the calling host thread
-// (created on its first use), so handles cost no stream creation and the
-// server's worker threads never share them.
-struct AuxStreams {
-  cudaStream_t s[3] = {nullptr, nullptr, nullptr};
-  cudaEvent_t fork = nullptr, join[3] = {nullptr, nullptr, nullptr};
-  bool ok = false;
-  AuxStreams() {
-    ok = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) == cudaSuccess;
-    for (int i = 0; i < 3 && ok; ++i)
-      ok = cudaStreamCreateWithFlags(&s[i], cudaStreamNonBlocking) == cudaSuccess &&
-           cudaEventCreateWithFlags(&join[i], cudaEventDisableTiming) == cudaSuccess;
-    if (!ok) cudaGetLastError();
-  }
-};
-
-AuxStreams& aux_streams() {
-  static thread_local AuxStreams a;
-  return a;
-}
 
 BinStreams fork_bins(cd_graph* g, bool concurrent) {
   BinStreams b;
@@ -1874,13 +1853,13 @@ int device_rounds(cd_graph* g, const RunOpts& o, bool louv, bool use_s32, bool p
   cudaGraphExec_t exec = nullptr;
   // capture happens on a stream of this thread's own (never the legacy
   // default stream, which cannot be captured); the graph runs on g->stream
-  static thread_local cudaStream_t cap = nullptr;
+  cudaStream_t cap = nullptr;
   cudaGraphConditionalHandle handle;
   auto cleanup = [&]() {
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
   };
-  cudaError_t e = cap ? cudaSuccess : cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+  cudaError_t e = capture_stream(&cap);
   if (e == cudaSuccess) e = cudaGraphCreate(&graph, 0);
   if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&handle, graph, 1, cudaGraphCondAssignDefault);
   if (e == cudaSuccess) {
