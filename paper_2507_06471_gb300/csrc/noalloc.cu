@@ -127,11 +127,11 @@ __global__ void __launch_bounds__(NT) k_noalloc_pass(const int64_t* __restrict__
           row[j] = -1;
           continue;
         }
-        if (x[j] < 1) na_fail(&ctl[5], CD_EINVAL);
-        if (u[j] < 0 || u[j] >= n) {
+        if (u[j] < 0 || u[j] >= n) {  // reported before the arc's weight
           na_fail(&ctl[5], CD_EBOUNDS);
           continue;
         }
+        if (x[j] < 1) na_fail(&ctl[5], CD_EINVAL);
         val[j] = (unsigned long long)(u[j] == row[j] ? 2 * x[j] : x[j]);
         my_vol += val[j];
         if (labels[u[j]] == labels[row[j]]) my_in += val[j];

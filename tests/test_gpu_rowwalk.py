@@ -101,3 +101,18 @@ def test_long_runs_of_empty_rows(run, wmax):
                 assert np.array_equal(gcols[a:b][i], ccols[a:b][j]) and np.array_equal(gw[a:b][i], cw[a:b][j])
             C.close()
         G.close()
+
+
+@pytest.mark.parametrize("arc", [0, 3, 127, 128, 300])
+def test_noalloc_reports_a_bad_column_before_a_bad_weight(arc):
+    import paper_2507_06471_gb300 as cd
+    g = _star_mix(300, 0, 250, 3, 5, 0)
+    off, lab = g.off.cuda(), torch.zeros(300, dtype=torch.int32, device="cuda")
+    for col, weight, status in ((-1, 0, cd.CD_EBOUNDS), (300, -7, cd.CD_EBOUNDS), (300, 2, cd.CD_EBOUNDS), (None, 0, cd.CD_EINVAL)):
+        cols, w = g.cols.clone(), g.w.clone()
+        if col is not None:
+            cols[arc] = col
+        w[arc] = weight
+        with pytest.raises(cd.CDError) as e:
+            cd.cd_modularity_noalloc(off, cols.cuda(), w.cuda(), lab)
+        assert e.value.status == status
