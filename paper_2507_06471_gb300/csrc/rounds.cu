@@ -62,7 +62,10 @@ constexpr int64_t SHARED_LOOP_ARCS = (int64_t)1 << 22;
 // Isolated vertices at most, where they are the majority: the resident loop looks
 // at every vertex's flag each round, the per-round kernels' lists leave them out.
 // LPA with 1e6 arcs among 1e5 vertices: 2.85 -> 1.76 ms with 1e7 vertices in all,
-// 3.08 -> 5.58 ms with 5e7.
+// 3.08 -> 5.58 ms with 5e7. Graphs of few isolated vertices need no such line: the
+// lists then hold every vertex and are gone through every round too (1e8 vertices
+// of degree 3, a ring and a matching: LPA 93 -> 42 ms, local moving 138 -> 70;
+// degree 2: 58 -> 30 and 62 -> 41; as much from 3e6 vertices on).
 constexpr int64_t MAX_ISOLATED = (int64_t)1 << 23;
 constexpr int TRACE_COLS = 8;             // examined, arcs, moved, deferred, candidates, arcs of moved, -, -
 constexpr int HEAD = 8;                   // int64 words before the trace: rounds, moves, status
@@ -526,7 +529,9 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
   __shared__ int occ_n[PNW];
   __shared__ int bincnt[2][8];  // by parity of the step: vertices per bin, then [7]: next task
   __shared__ int n_mv;
-  __shared__ uint32_t sums[5];  // a CTA has at most 2^31 / 152 vertices of at most 1,024 arcs
+  // A CTA's counters of a round, then the high words of those that count arcs: 456 CTAs (the fewest that fill the GPU;
+  // smaller grids have few arcs) of 2^31 vertices of up to 1,024 arcs may have 4.8e9 each. A thread's stay below 2^32.
+  __shared__ uint32_t sums[5], sums_hi[5];
   __shared__ int hub_moves, s_last;
   __shared__ int start[PNW][8];
   __shared__ typename S::K red_k[PNW];
@@ -555,19 +560,20 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
   // the CTA's counters of a round, added to the round's trace row; returns moved + deferred
   auto account = [&](const Tally& t, int more_moves) -> unsigned {
     if (__any_sync(FULL, t.act | t.cand)) {
-      const uint32_t c[5] = {t.act, t.arcs, t.cand, t.def, t.marcs};  // a warp's arcs of a round stay below 2^32
+      const uint32_t c[5] = {t.act, t.arcs, t.cand, t.def, t.marcs};
 #pragma unroll
       for (int q = 0; q < 5; ++q) {
-        const uint32_t x = __reduce_add_sync(FULL, c[q]);
-        if (lane == 0 && x) atomicAdd(&sums[q], x);
+        unsigned long long x = __reduce_add_sync(FULL, q == 0 || q == 3 ? c[q] : c[q] & 0xffffu);
+        if (q != 0 && q != 3) x += (unsigned long long)__reduce_add_sync(FULL, c[q] >> 16) << 16;
+        if (lane == 0 && x) add_words(&sums[q], &sums_hi[q], x);
       }
     }
     __syncthreads();
     const int nm = more_moves ? hub_moves : n_mv;
     const unsigned changed = (unsigned)nm + sums[3];
     if (tid < 6) {
-      const unsigned long long x = tid == 0 ? sums[0] : tid == 1 ? sums[1] : tid == 2 ? (unsigned long long)nm
-                                 : tid == 3 ? sums[3] : tid == 4 ? sums[2] : sums[4];
+      const int q = tid < 2 ? tid : tid == 3 ? 3 : tid == 4 ? 2 : 4;
+      const unsigned long long x = tid == 2 ? (unsigned long long)nm : ((unsigned long long)sums_hi[q] << 32) | sums[q];
       if (x) atomicAdd(&L.head[HEAD + (int64_t)round * TRACE_COLS + tid], x);
     }
     return changed;
@@ -577,7 +583,7 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
     uint32_t* nxt_map = round & 1 ? L.flag0 : L.flag1;
     const bool frontier = s.mark != 0;
     if (tid == 0) n_mv = hub_moves = 0;
-    if (tid < 5) sums[tid] = 0;
+    if (tid < 5) sums[tid] = sums_hi[tid] = 0;
     const S sc{s, L, round, round == 0 && L.first_rows, frontier ? nxt_map : nullptr, mv, mv_stride, &n_mv};
     Tally t;
     bool hubs_here = false;
@@ -636,7 +642,7 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
     if (!grid_meet(L.bar + 3 * (int64_t)round, changed, hubs_here, total, hubs, s.status)) return;
     if (hubs) {  // the same in every CTA: read the hubs' tables
       const ResidentHubs& r = L.rh;
-      if (tid < 5) sums[tid] = 0;
+      if (tid < 5) sums[tid] = sums_hi[tid] = 0;
       __syncthreads();
       Tally th;
       const int n_slices = r.slice[r.nh];

@@ -169,8 +169,6 @@ __device__ __forceinline__ void warp_rows_sum(const int64_t row[4], const unsign
 // addition. Atomics on one address run one after another: 1e5 vertices in about
 // a hundred communities took 44.6 us with an atomic per vertex. A key that finds
 // no slot within four probes is added to the global array at once.
-// The 64-bit sums are two words with a carry: a 64-bit shared atomic takes 425
-// cycles (3,200 when a warp's lanes meet on one), a 32-bit one 16 (64).
 struct CtaSums {
   static constexpr int SLOTS = 512;
   uint32_t lo[SLOTS], hi[SLOTS];
@@ -188,9 +186,7 @@ struct CtaSums {
       int32_t c = *(volatile int32_t*)&key[h];
       if (c == EMPTY) c = atomicCAS(&key[h], EMPTY, k);
       if (c == EMPTY || c == k) {
-        const uint32_t xl = (uint32_t)x, old = atomicAdd(&lo[h], xl);
-        const uint32_t up = (uint32_t)(x >> 32) + (old + xl < old ? 1u : 0u);
-        if (up) atomicAdd(&hi[h], up);
+        add_words(&lo[h], &hi[h], x);
         return (int)h;
       }
       h = (h + 1) & (SLOTS - 1);

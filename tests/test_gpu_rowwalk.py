@@ -116,3 +116,24 @@ def test_noalloc_reports_a_bad_column_before_a_bad_weight(arc):
         with pytest.raises(cd.CDError) as e:
             cd.cd_modularity_noalloc(off, cols.cuda(), w.cuda(), lab)
         assert e.value.status == status
+
+
+@pytest.mark.parametrize("n", [40, 3000, 20000])
+def test_community_sums_past_32_bits(n):
+    # every CTA's sum of one community takes carries out of its low word
+    import paper_2507_06471_gb300 as cd
+    rng = np.random.default_rng(n)
+    edges = sorted({(int(a), int(b)) for a, b in np.sort(rng.integers(0, n, (4 * n, 2)), axis=1) if a != b})
+    g = synth.from_edge_list(n, edges, rng.integers(2**30, 2**31 - 1, len(edges)).tolist())
+    off, cols, w = g.numpy()
+    G = cd.Graph(g.off.cuda(), g.cols.cuda(), g.w.cuda())
+    for lab in (np.zeros(n), np.arange(n) % 3, np.arange(n)):
+        lab = lab.astype(np.int32)
+        q = oracle.modularity(off, cols, w, lab)[0]
+        dl = torch.from_numpy(lab).cuda()
+        for got in (G.modularity(dl), cd.cd_modularity_noalloc(g.off.cuda(), g.cols.cuda(), g.w.cuda(), dl)):
+            assert abs(got - q) <= 1e-12 * max(1.0, abs(q))
+        olab, omoves, otr = oracle.local_move(off, cols, w, labels_in=lab, max_iter=3)
+        moved, moves, rounds = G.local_move(labels=dl, max_iter=3)
+        assert np.array_equal(moved.cpu().numpy(), olab) and (moves, rounds) == (omoves, otr.rounds)
+    G.close()
