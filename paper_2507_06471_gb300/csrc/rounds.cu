@@ -69,7 +69,7 @@ constexpr int64_t SHARED_LOOP_ARCS = (int64_t)1 << 22;
 constexpr int64_t MAX_ISOLATED = (int64_t)1 << 23;
 constexpr int TRACE_COLS = 8;             // examined, arcs, moved, deferred, candidates, arcs of moved, -, -
 constexpr int HEAD = 8;                   // int64 words before the trace: rounds, moves, status
-constexpr int64_t WAIT_LIMIT = (int64_t)1 << 24;  // polls of one barrier (seconds), then CD_ETIMEOUT
+constexpr int64_t WAIT_LIMIT = (int64_t)1 << 24;  // polls of one barrier at most (seconds), then CD_ETIMEOUT
 
 struct LoopCtx {
   int64_t n, nwords, n32;  // vertices, flag words, vertices rounded up to whole words
@@ -79,6 +79,7 @@ struct LoopCtx {
   uint32_t* flag1;
   int32_t max_iter, first_rows, t_warp, t_hub, per_graph;
   int64_t threshold;
+  int64_t polls;              // of a barrier at most
   int32_t* last_change;       // per_graph: 1 + the last round in which a vertex of the graph wanted to move
   unsigned long long* bar;    // three words per round, zero
   unsigned long long* head;   // HEAD words, then TRACE_COLS per round, zero
@@ -89,7 +90,7 @@ struct LoopCtx {
 // Every CTA arrives once; `add` (changed vertices, < 2^32 in all) and `hubs`
 // are summed over the CTAs (at most 2^15). False: a wait ran out.
 __device__ __forceinline__ bool grid_meet(unsigned long long* word, unsigned add, unsigned hubs, unsigned& sum,
-                                          unsigned& hub_sum, int32_t* status) {
+                                          unsigned& hub_sum, int64_t limit, int32_t* status) {
   __shared__ unsigned long long got;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -99,7 +100,7 @@ __device__ __forceinline__ bool grid_meet(unsigned long long* word, unsigned add
     int64_t polls = 0;
     for (;;) {
       asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(word) : "memory");
-      if ((x >> 48) >= gridDim.x || ++polls >= WAIT_LIMIT) break;
+      if ((x >> 48) >= gridDim.x || ++polls >= limit) break;
       __nanosleep(40);  // arrivals go to the same word
     }
     if ((x >> 48) < gridDim.x) {
@@ -639,7 +640,7 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
     const unsigned changed = account(t, 0);
     const int nm = n_mv;
     unsigned total, hubs, none;
-    if (!grid_meet(L.bar + 3 * (int64_t)round, changed, hubs_here, total, hubs, s.status)) return;
+    if (!grid_meet(L.bar + 3 * (int64_t)round, changed, hubs_here, total, hubs, L.polls, s.status)) return;
     if (hubs) {  // the same in every CTA: read the hubs' tables
       const ResidentHubs& r = L.rh;
       if (tid < 5) sums[tid] = sums_hi[tid] = 0;
@@ -765,7 +766,7 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
       }
       const unsigned more = account(th, 1);
       unsigned hub_total;
-      if (!grid_meet(L.bar + 3 * (int64_t)round + 1, more, 0, hub_total, none, s.status)) return;
+      if (!grid_meet(L.bar + 3 * (int64_t)round + 1, more, 0, hub_total, none, L.polls, s.status)) return;
       total += hub_total;
       // the neighbours of the moved hubs
       if (frontier) {
@@ -797,7 +798,7 @@ __global__ void __launch_bounds__(PNT, sizeof(V) == 4 ? 4 : 3) k_rounds(const __
       for (int64_t w = b * PNT + tid; w < L.nwords; w += G * PNT) cur_map[w] = 0;
     ++round;
     if (LOUV ? total == 0 : (int64_t)total <= L.threshold) break;
-    if (round < L.max_iter && !grid_meet(L.bar + 3 * (int64_t)round - 1, 0, 0, total, none, s.status)) return;
+    if (round < L.max_iter && !grid_meet(L.bar + 3 * (int64_t)round - 1, 0, 0, total, none, L.polls, s.status)) return;
   }
   if (b == 0 && tid == 0) L.head[0] = (unsigned long long)round;
 }
@@ -927,6 +928,7 @@ int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, i
   L.flag0 = g->flag[0];
   L.flag1 = g->flag[1];
   L.max_iter = o.max_iter;
+  L.polls = g->loop_polls ? g->loop_polls : WAIT_LIMIT;
   L.first_rows = singletons && g->cols_distinct;
   L.t_warp = g->t_warp;
   L.t_hub = g->t_hub;
@@ -1008,3 +1010,10 @@ int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, i
 }
 
 }  // namespace cd
+
+// For tests: the polls after which a barrier of g's resident loops gives up (0: as always).
+extern "C" int cd_test_resident_loop(cd_graph* g, int64_t polls) {
+  if (!g || polls < 0) return CD_EINVAL;
+  g->loop_polls = polls;
+  return CD_OK;
+}

@@ -92,3 +92,32 @@ def test_other_values_of_device_loop_are_the_default(loop):
     G.close()
     assert np.array_equal(got[0][0], want[0]) and list(got[0][1]) == list(want[1]) and got[1] == trace
     assert got[2] == launches != host[2]
+
+
+def set_loop(G, polls):
+    import ctypes
+    import paper_2507_06471_gb300 as cd
+    f = cd.lib().cd_test_resident_loop
+    f.argtypes = [ctypes.c_void_p, ctypes.c_int64]
+    assert f(G.h, polls) == cd.CD_OK
+
+
+@pytest.mark.parametrize("hubs", [False, True])
+@pytest.mark.parametrize("call", ["lpa", "local_move"])
+def test_wait_that_runs_out(hubs, call):
+    # a barrier that gives up at its first look ends the run with CD_ETIMEOUT; the handle's next run is right, hub tables
+    # cut short included
+    import paper_2507_06471_gb300 as cd
+    g = hub_graph(5, 0) if hubs else synth.sbm(20_000, 100, "0.08", "0.0005", seed=4, wmax=5)
+    assert len(g.cols) > 100 * 512  # a hundred CTAs or more, which do not all arrive at once
+    G = upload(g)
+    want = run(G, 0, call)
+    for _ in range(2):
+        set_loop(G, 1)
+        with pytest.raises(cd.CDError) as e:
+            run(G, 1, call)
+        assert e.value.status == cd.CD_ETIMEOUT
+        set_loop(G, 0)
+        got = run(G, 1, call)
+        assert got[1] == want[1] and all(np.array_equal(a, b) for a, b in zip(got[0], want[0]))
+    G.close()
