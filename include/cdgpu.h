@@ -80,7 +80,11 @@ typedef struct cd_params {
                                round) in batched runs (cd_batch_*), and in others if at least 2^22 arcs and
                                max_iter > 16 make the graph worth its making; the rest keeps the host loop.
                                The round number, the stop tests and the trace stay on the device, so a
-                               level costs one launch and no per-round host synchronisation. 2: the
+                               level costs one launch and no per-round host synchronisation. The resident
+                               kernel starts when the GPU has room for all its CTAs (on larger graphs all
+                               there is): it waits for kernels of other streams to end, and a caller whose
+                               own kernel runs until it sees this call's result has to choose 0 or 2. Where
+                               the runtime refuses such a launch the per-round kernels run. 2: the
                                captured graph in every run, also where 1 is resident. 0: the host loop
                                everywhere (one read-back per round). Results are identical in every mode;
                                timing != 0 (per-round events) and the asynchronous mode are never

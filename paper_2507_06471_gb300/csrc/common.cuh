@@ -191,7 +191,9 @@ struct cd_graph {
   // they save), and a resident loop takes 1 / workers of the GPU at most, so that the workers' loops run side by side:
   // loops that fill the GPU run one after another, and most of a loop's time is latency. Coarse graphs inherit it.
   int workers = 0;
-  int64_t loop_polls = 0;  // what a test sets for the resident loop (0: nothing): polls of a barrier
+  // What a test sets for the resident loop (0: nothing): polls of a barrier, CTAs.
+  int64_t loop_polls = 0;
+  int64_t loop_ctas = 0;
   bool bins_set = false;           // thresholds chosen by cd_graph_set_bins / cd_autotune (kept by coarse graphs)
 
   // run state (one allocation, made on first use; the pointers below are parts of it)
@@ -350,7 +352,10 @@ constexpr int64_t GRAPH_LOOP_ARCS = (int64_t)1 << 22;
 constexpr int32_t GRAPH_LOOP_ROUNDS = 16;
 
 // rounds.cu: the whole round loop as one resident kernel (graphs without hubs or
-// with few of them).
+// with few of them). LOOP_REFUSED: the runtime did not take the launch (more CTAs
+// than this context may have at once); nothing ran and the per-round kernels
+// take the run.
+constexpr int LOOP_REFUSED = 1;
 bool resident_rounds_apply(const cd_graph* g, const RunOpts& o, bool per_graph_stop);
 int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, int64_t* moves_out, int32_t* rounds_out,
                     std::vector<int32_t>* graph_rounds);

@@ -853,14 +853,21 @@ int launch_loop(cd_graph* g, const ScanCtx& s, LoopCtx L) {
     resident.set(r);
   }
   const int64_t useful = std::max(g->nnz / ARCS_PER_CTA, L.n / CH_VERTS);
-  const int64_t grid = std::max<int64_t>(1, std::min(std::min<int64_t>(std::max(1, r / std::max(1, g->workers)), L.n), useful));
+  const int64_t fit = std::max(1, r / std::max(1, g->workers));
+  const int64_t grid = g->loop_ctas ? g->loop_ctas : std::max<int64_t>(1, std::min(std::min(fit, L.n), useful));
   // the largest units that still give every CTA four
   L.lgu = 5;
   while (L.lgu > 0 && (L.n >> L.lgu) < 4 * grid) --L.lgu;
   L.nunits = (L.n + ((int64_t)1 << L.lgu) - 1) >> L.lgu;
   void* args[] = {(void*)&s, (void*)&L};
+  const cudaError_t e =
+      cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)grid), dim3(PNT), args, sm, g->stream);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+    cudaGetLastError();
+    return LOOP_REFUSED;
+  }
+  CD_CHECK(e);
   note_launch();
-  CD_CHECK(cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)grid), dim3(PNT), args, sm, g->stream));
   return CD_OK;
 }
 
@@ -980,6 +987,7 @@ int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, i
   };
   rc = run();
   scratch.free(st);
+  if (rc == LOOP_REFUSED) return rc;
   if (rc) {  // the hubs' tables may hold entries of the round that was cut short
     drop_resident_hubs(g);
     if (status) cudaMemsetAsync(g->status, 0, sizeof(int32_t), st);
@@ -1011,9 +1019,11 @@ int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, i
 
 }  // namespace cd
 
-// For tests: the polls after which a barrier of g's resident loops gives up (0: as always).
-extern "C" int cd_test_resident_loop(cd_graph* g, int64_t polls) {
-  if (!g || polls < 0) return CD_EINVAL;
+// For tests: the polls after which a barrier of g's resident loops gives up, and
+// the CTAs they are launched with (0: as always).
+extern "C" int cd_test_resident_loop(cd_graph* g, int64_t polls, int64_t ctas) {
+  if (!g || polls < 0 || ctas < 0) return CD_EINVAL;
   g->loop_polls = polls;
+  g->loop_ctas = ctas;
   return CD_OK;
 }

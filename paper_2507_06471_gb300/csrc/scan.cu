@@ -2216,8 +2216,9 @@ namespace {
 int run_lpa_any(cd_graph* g, const RunOpts& o, int32_t* rounds_out, std::vector<int32_t>* rounds) {
   int rc = ensure_run_state(g);
   if (rc) return rc;
-  if (resident_rounds_apply(g, o, rounds != nullptr))
-    return resident_rounds(g, o, false, true, nullptr, rounds_out, rounds);
+  if (resident_rounds_apply(g, o, rounds != nullptr) &&
+      (rc = resident_rounds(g, o, false, true, nullptr, rounds_out, rounds)) != LOOP_REFUSED)
+    return rc;
   if (g->n > 0)
     CD_LAUNCH(k_init_singletons<<<grid_cap((g->n + NT - 1) / NT), NT, 0, g->stream>>>(g->C, g->sigma, g->csize,
                                                                             g->degw, g->n, 0));
@@ -2243,21 +2244,21 @@ int run_local_move(cd_graph* g, const RunOpts& o, int init_given, int64_t* moves
   int rc = ensure_run_state(g);
   if (rc) return rc;
   cudaStream_t st = g->stream;
-  const bool resident = resident_rounds_apply(g, o, false);
-  if (g->n > 0) {
-    if (init_given) {
-      CD_CHECK(cudaMemsetAsync(g->sigma, 0, g->n * sizeof(int64_t), st));
-      CD_CHECK(cudaMemsetAsync(g->csize, 0, g->n * sizeof(int32_t), st));
-      // four vertices a thread, so that a CTA has something to sum
-      CD_LAUNCH(k_init_given<<<grid_cap((g->n + 4 * NT - 1) / (4 * NT), 152 * 8), NT, 0, st>>>(g->C, g->sigma, g->csize,
-                                                                                     g->degw, g->n));
-    } else if (!resident) {
-      CD_LAUNCH(k_init_singletons<<<grid_cap((g->n + NT - 1) / NT), NT, 0, st>>>(g->C, g->sigma, g->csize,
-                                                                       g->degw, g->n, 1));
-    }
+  if (g->n > 0 && init_given) {
+    CD_CHECK(cudaMemsetAsync(g->sigma, 0, g->n * sizeof(int64_t), st));
+    CD_CHECK(cudaMemsetAsync(g->csize, 0, g->n * sizeof(int32_t), st));
+    // four vertices a thread, so that a CTA has something to sum
+    CD_LAUNCH(k_init_given<<<grid_cap((g->n + 4 * NT - 1) / (4 * NT), 152 * 8), NT, 0, st>>>(g->C, g->sigma, g->csize,
+                                                                                   g->degw, g->n));
   }
   CD_CHECK(cudaGetLastError());
-  if (resident) return resident_rounds(g, o, true, !init_given, moves_out, rounds_out, nullptr);
+  if (resident_rounds_apply(g, o, false) &&
+      (rc = resident_rounds(g, o, true, !init_given, moves_out, rounds_out, nullptr)) != LOOP_REFUSED)
+    return rc;
+  if (g->n > 0 && !init_given)
+    CD_LAUNCH(k_init_singletons<<<grid_cap((g->n + NT - 1) / NT), NT, 0, st>>>(g->C, g->sigma, g->csize,
+                                                                     g->degw, g->n, 1));
+  CD_CHECK(cudaGetLastError());
   RunOpts os = o;
   os.singleton_start = !init_given;
   return run_rounds(g, os, true, moves_out, rounds_out);

@@ -94,12 +94,12 @@ def test_other_values_of_device_loop_are_the_default(loop):
     assert got[2] == launches != host[2]
 
 
-def set_loop(G, polls):
+def set_loop(G, polls, ctas):
     import ctypes
     import paper_2507_06471_gb300 as cd
     f = cd.lib().cd_test_resident_loop
-    f.argtypes = [ctypes.c_void_p, ctypes.c_int64]
-    assert f(G.h, polls) == cd.CD_OK
+    f.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int64]
+    assert f(G.h, polls, ctas) == cd.CD_OK
 
 
 @pytest.mark.parametrize("hubs", [False, True])
@@ -113,11 +113,40 @@ def test_wait_that_runs_out(hubs, call):
     G = upload(g)
     want = run(G, 0, call)
     for _ in range(2):
-        set_loop(G, 1)
+        set_loop(G, 1, 0)
         with pytest.raises(cd.CDError) as e:
             run(G, 1, call)
         assert e.value.status == cd.CD_ETIMEOUT
-        set_loop(G, 0)
+        set_loop(G, 0, 0)
         got = run(G, 1, call)
         assert got[1] == want[1] and all(np.array_equal(a, b) for a, b in zip(got[0], want[0]))
     G.close()
+
+
+@pytest.mark.parametrize("hubs", [False, True])
+def test_launch_that_is_refused(hubs):
+    # more CTAs than fit at once: the runtime refuses the launch and the per-round kernels take the run
+    import paper_2507_06471_gb300 as cd
+    g = hub_graph(5, 3) if hubs else synth.sbm(5000, 20, "0.05", "0.0005", seed=4, wmax=5)
+    G = upload(g)
+    start = torch.arange(g.n, dtype=torch.int32, device="cuda") // 3
+    calls = [("lpa", {}), ("local_move", {}), ("local_move", {"labels": start}), ("louvain", {})]
+    want = [run(G, 0, call, **kw) for call, kw in calls]
+    set_loop(G, 0, 32_000)
+    got = [run(G, 1, call, **kw) for call, kw in calls]
+    G.close()
+    for a, b in zip(got, want):
+        assert a[1] == b[1] and all(np.array_equal(x, y) for x, y in zip(a[0], b[0]))
+    assert all(a[2] > 20 for a in got)  # a kernel or more a round
+    # a batched run, whose graphs stop by themselves
+    graphs = [synth.sbm(n, 5, "0.2", "0.002", seed=n, wmax=3) for n in (300, 900, 80)]
+    packed, vstart = synth.pack_batch(graphs)
+    B = cd.Graph(packed.off.cuda(), packed.cols.cuda(), packed.w.cuda())
+    B.set_batches(vstart)
+    for call in ("batch_lpa", "batch_louvain"):
+        want = run(B, 0, call)
+        set_loop(B, 0, 32_000)
+        got = run(B, 1, call)
+        set_loop(B, 0, 0)
+        assert got[1] == want[1] and all(np.array_equal(x, y) for x, y in zip(got[0], want[0]))
+    B.close()
