@@ -2351,9 +2351,11 @@ int cd_autotune(cd_graph* g, const cd_params* p, int32_t rounds, int32_t* t_warp
   for (int i = 0; i < 3 && !rc; ++i)
     for (int j = 0; j < 4 && !rc; ++j) {
       if (th[j] < tw[i]) continue;
-      if ((rc = rebin(g, tw[i], th[j])) || (rc = ensure_bins(g))) break;
       RunOpts o = opts_from(p, 0);
       o.max_iter = rounds;
+      // laid out before the clock starts, as on a handle that is kept: what the runs will use
+      if ((rc = rebin(g, tw[i], th[j]))) break;
+      if ((rc = !resident_rounds_apply(g, o, false) ? ensure_bins(g) : g->nhubs > 0 ? ensure_resident_hubs(g) : CD_OK)) break;
       cudaEventRecord(a, g->stream);
       rc = run_lpa(g, o, nullptr);
       if (!rc) rc = run_local_move(g, o, 0, nullptr, nullptr);

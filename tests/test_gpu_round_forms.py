@@ -150,3 +150,28 @@ def test_launch_that_is_refused(hubs):
         set_loop(B, 0, 0)
         assert got[1] == want[1] and all(np.array_equal(x, y) for x, y in zip(got[0], want[0]))
     B.close()
+
+
+@pytest.mark.parametrize("hubs", [False, True])
+def test_autotune_prepares_what_its_runs_use(hubs):
+    # the kernels launched are those of the same runs by hand: nothing is laid out that no run uses
+    import paper_2507_06471_gb300 as cd
+    g = hub_graph(5, 3) if hubs else synth.sbm(5000, 20, "0.05", "0.0005", seed=4, wmax=5)
+    A, B = upload(g), upload(g)
+    before = cd.cd_launch_count()
+    best = cd.cd_autotune(A.h, cd.cd_params_default(), 2)
+    tuned = cd.cd_launch_count() - before
+    before = cd.cd_launch_count()
+    for t_warp in (64, 128, 256):
+        for t_hub in (512, 1024, 2048, 4096):
+            cd.cd_graph_set_bins(B.h, t_warp, t_hub)
+            B.lpa(max_iter=2)
+            B.local_move(max_iter=2)
+    cd.cd_graph_set_bins(B.h, *best)
+    by_hand = cd.cd_launch_count() - before
+    lab, rounds = A.lpa()
+    olab, otr = oracle.lpa(*g.numpy())
+    A.close()
+    B.close()
+    assert tuned == by_hand
+    assert rounds == otr.rounds and np.array_equal(lab.cpu().numpy(), olab)
