@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(NT, 6) k_scan_tile(ScanCtx s, const int32_t* _
 
 // GROUP threads per vertex (a warp, or a named-barrier group of 128 or 512
 // threads), each group with its own CAP-slot shared-memory table.
-template <bool LOUV, class W, class V, int GROUP, int NTB, int CAP, int BIN, bool PF, bool NK>
+template <bool LOUV, class W, class V, int GROUP, int NTB, int CAP, int BIN, bool NK>
 __global__ void __launch_bounds__(NTB, GROUP == 32 ? ((LOUV || !W::unit) ? 4 : 5) : 2)
     k_scan_group(ScanCtx s, const int32_t* __restrict__ list, const unsigned long long* __restrict__ count_p) {
   typedef typename KeyOf<LOUV, NK>::T K;
@@ -156,31 +156,10 @@ __global__ void __launch_bounds__(NTB, GROUP == 32 ? ((LOUV || !W::unit) ? 4 : 5
   if (gl == 0) occ_n[gid] = 0;
   group_sync<GROUP, NTB>(gid);
   int64_t n_act = 0, n_arcs = 0, n_cand = 0, n_def = 0, n_marcs = 0;
-  // Software pipeline over the group's vertices: while vertex i is processed,
-  // the header of vertex i + stride (activity, row bounds, label, deg_w) and
-  // the list entry of vertex i + 2 stride are already in flight.
   const int64_t stride = (int64_t)gridDim.x * GPB;
-  int64_t i = (int64_t)blockIdx.x * GPB + gid;
-  int32_t v_nx = 0, v_nn = 0;
-  VHdr h_nx{};
-  if constexpr (PF) {
-    v_nx = i < count ? list[i] : 0;
-    h_nx = load_hdr<LOUV>(s, v_nx, i < count);
-    v_nn = i + stride < count ? list[i + stride] : 0;
-  }
-  for (; i < count; i += stride) {
-    int32_t v;
-    VHdr h;
-    if constexpr (PF) {
-      v = v_nx;
-      h = h_nx;
-      v_nx = v_nn;
-      h_nx = load_hdr<LOUV>(s, v_nx, i + stride < count);
-      v_nn = i + 2 * stride < count ? list[i + 2 * stride] : 0;
-    } else {
-      v = list[i];
-      h = load_hdr<LOUV>(s, v, true);
-    }
+  for (int64_t i = (int64_t)blockIdx.x * GPB + gid; i < count; i += stride) {
+    const int32_t v = list[i];
+    const VHdr h = load_hdr<LOUV>(s, v, true);
     if (!h.act) continue;  // uniform within the group
     const int64_t beg = h.beg, end = h.end;
     const int64_t d = end - beg;
@@ -1489,9 +1468,9 @@ int set_smem_attrs() {
   if (done.get()) return CD_OK;
   CD_CHECK(cudaFuncSetAttribute(k_scan_warp<LOUV, W, V, NK>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)warp_smem<V>()));
-  CD_CHECK(cudaFuncSetAttribute(k_scan_group<LOUV, W, V, 512, 512, BLK4_CAP_SLOTS, B_BLK4, false, NK>,
+  CD_CHECK(cudaFuncSetAttribute(k_scan_group<LOUV, W, V, 512, 512, BLK4_CAP_SLOTS, B_BLK4, NK>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)blk4_smem<V>()));
-  CD_CHECK(cudaFuncSetAttribute(k_scan_group<LOUV, W, V, 128, 512, BLK1_CAP_SLOTS, B_BLK1, false, NK>,
+  CD_CHECK(cudaFuncSetAttribute(k_scan_group<LOUV, W, V, 128, 512, BLK1_CAP_SLOTS, B_BLK1, NK>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)blk1_smem<V>()));
   CD_CHECK(cudaFuncSetAttribute(k_hub_prepare, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HUB_PREP_SMEM));
   CD_CHECK(cudaFuncSetAttribute(k_hub_build_cl<W, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hub_cl_smem<0>()));
@@ -1641,7 +1620,7 @@ int launch_round(cd_graph* g, ScanCtx& s, const int32_t* lists, const unsigned l
   if (cnt(B_BLK4) > 0) {
     {
       KTimer t(g, K_SCAN_BLK512, 0.0, bs.s[2]);
-      auto kern = k_scan_group<LOUV, W, V, 512, 512, BLK4_CAP_SLOTS, B_BLK4, false, NK>;
+      auto kern = k_scan_group<LOUV, W, V, 512, 512, BLK4_CAP_SLOTS, B_BLK4, NK>;
       CD_LAUNCH((kern<<<wave_grid(kern, 512, blk4_smem<V>(), cnt(B_BLK4)), 512, blk4_smem<V>(), bs.s[2]>>>(
           s, lst(B_BLK4), dcnt(B_BLK4))));
     }
@@ -1650,7 +1629,7 @@ int launch_round(cd_graph* g, ScanCtx& s, const int32_t* lists, const unsigned l
   if (cnt(B_BLK1) > 0) {
     {
       KTimer t(g, K_SCAN_BLK128, 0.0, bs.s[2]);
-      auto kern = k_scan_group<LOUV, W, V, 128, 512, BLK1_CAP_SLOTS, B_BLK1, false, NK>;
+      auto kern = k_scan_group<LOUV, W, V, 128, 512, BLK1_CAP_SLOTS, B_BLK1, NK>;
       CD_LAUNCH((kern<<<wave_grid(kern, 512, blk1_smem<V>(), (cnt(B_BLK1) + 3) / 4), 512, blk1_smem<V>(), bs.s[2]>>>(
           s, lst(B_BLK1), dcnt(B_BLK1))));
     }
