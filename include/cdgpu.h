@@ -108,8 +108,9 @@ typedef struct cd_round_trace {
 /* Per-kernel totals of the last run (cd_profile_get; timing = 1). One entry per
  * launch group: ingest, scan_tile4/8/16/32, scan_warp, scan_blk128, scan_blk512
  * (the degree bins' scans; round 0 of a run is counted under its bin),
- * hub_prepare (hub-table compactions, clears and routing), hub_build (hub-table
- * builds), hub_eval, hub_mark (flags and logged hub-histogram updates of
+ * hub_prepare (hub-table compactions, clears and the sorting of flagged hubs),
+ * hub_build (hub-table builds, repeated ones included, and the routing of the
+ * evaluations), hub_eval, hub_mark (flags and logged hub-histogram updates of
  * committed moves), apply_moves, frontier, renumber, agg_emit, radix_sort,
  * agg_reduce, modularity. */
 typedef struct cd_kernel_profile {

@@ -154,7 +154,7 @@ struct cd_graph {
   uint32_t* hub_pref = nullptr;        // per 32-vertex word: hubs with smaller vertex ids (hub number = rank)
   uint32_t* hub_bits = nullptr;            // (n+31)/32: bit v set iff v is a hub
   int64_t* hub_tab = nullptr;              // nhubs+1
-  int64_t* hub_cc = nullptr;               // nhubs: slots in use, [0, hub_cc) of the allocation
+  int64_t* hub_cc = nullptr;               // nhubs: slots in use, [0, hub_cc) of the allocation (past them: stale)
   int32_t* hub_live = nullptr;             // nhubs: live entries counted by the evaluate items of a round
   unsigned long long* hub_slot = nullptr;  // hub_slots words (x2 when wide)
   int32_t* hub_item_hub = nullptr;         // per build/mark item (HUB_CHUNK arcs): hub

@@ -218,7 +218,6 @@ __global__ void k_offsets_check(const OffT* in, int64_t n, int64_t nnz, int64_t*
 // the columns' latency and the row marks: R-MAT 24 (5.2e8 arcs) 3.8 -> 1.5 ms
 // against rows by a lane, a warp or a CTA each with 64-bit shared counters;
 // 613 vertices 21.5 -> 5.9 us, upload of R-MAT 2^20 796 -> 326 us.
-constexpr int64_t HUB_LOG_DIV = 4;  // budget of logged hub updates per round: hub arcs / 4
 constexpr int ST_UNSORTED = 4 + NBINS;
 
 template <class W>
@@ -565,7 +564,7 @@ void take_bins(cd_graph* g, const unsigned long long* cnt) {
 }
 
 // Scalars, bins and hub structures of a graph whose CSR, weights and deg_w
-// are in place; stats from k_ingest.
+// are in place; stats from the ingest kernels.
 int finish_graph(cd_graph* g, const unsigned long long* stats, const unsigned long long* bins) {
   g->cols_distinct = stats[ST_UNSORTED] == 0;  // strictly increasing rows; aggregation sets it for coarse rows
   g->vol = (int64_t)stats[0];
@@ -595,6 +594,7 @@ int build_bins(cd_graph* g) {
 }
 
 // The bin lists, and the hub histograms' layout.
+constexpr int64_t HUB_LOG_DIV = 4;  // budget of logged hub updates per round: hub arcs / 4
 int fill_bins(cd_graph* g) {
   cudaStream_t s = g->stream;
   const int64_t listed = g->bin_start[NBINS], nh = g->nhubs, words = (g->n + 31) / 32;

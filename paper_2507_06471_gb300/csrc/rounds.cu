@@ -881,7 +881,7 @@ int dispatch_loop(cd_graph* g, const ScanCtx& s, const LoopCtx& L) {
   return v32 ? launch_loop<LOUV, WI64, uint32_t, NK>(g, s, L) : launch_loop<LOUV, WI64, unsigned long long, NK>(g, s, L);
 }
 
-// The parts of the context the resident kernel uses (no hubs, no counters).
+// The parts of the context the resident kernel uses (its hubs and counters are in LoopCtx).
 ScanCtx loop_ctx(cd_graph* g, const RunOpts& o, bool louv, bool nk) {
   ScanCtx s{};
   s.off = g->off;

@@ -10,7 +10,8 @@
 //   Louvain: the c != A = C[v] of largest g(c) = vol(V) k_{v,c} - deg_w(v)
 //            Sigma_tot[c] (smallest c on ties) and moves iff
 //            G = g(c) - vol(V) k_{v,A} + deg_w(v) (Sigma_tot[A] - deg_w(v)) > 0,
-//            where G = dQ_{v->c} vol(V)^2 / 2 (Eq. deltaQ, exact in 128 bits).
+//            where G = dQ_{v->c} vol(V)^2 / 2 (Eq. deltaQ, exact: in 64 bits
+//            when vol(V) < 2^31, else in 128).
 // A vertex whose decision differs from its label commits only if the pinned
 // SplitMix64 coin says so; otherwise it defers and stays active.
 //
@@ -2097,7 +2098,7 @@ int run_rounds(cd_graph* g, const RunOpts& o, bool louv, int64_t* moves_out, int
         bytes = (double)fa * (8 + 4 + 1) + (double)farcs * (4 + wbytes) + (louv ? (double)fa * 24 + (double)fc * 8 : 0.0);
       } else if (b == -1)  // hub table builds: the arcs they read, the slots they wrote
         bytes = (double)h[C_HUB_BARCS] * (4 + 4 + wbytes) + (double)h[C_HUB_BSLOTS] * 8;
-      else if (b == -2)  // hub preparation: slots cleared, or read and written by compactions; the route
+      else if (b == -2)  // hub preparation: slots cleared, or read and written by compactions; the hubs sorted
         bytes = (double)h[C_HUB_PSLOTS] * 8 + (double)g->nhubs * 8;
       else if (b == B_HUB)  // hub evaluate: the candidates of every active hub
         bytes = (double)cb * (12 + 12 + (louv ? 8 : 0)) + (double)ab * (8 + 4);

@@ -107,7 +107,7 @@ struct ScanCtx {
   const uint32_t* hub_pref;
   const uint32_t* hub_bits;
   const int64_t* hub_tab;
-  int64_t* hub_cc;                   // per hub: slots in use, [0, hub_cc) of its allocation (the rest empty)
+  int64_t* hub_cc;                   // per hub: slots in use, [0, hub_cc) of its allocation (what lies past them is stale)
   int32_t* hub_live;                 // per hub: live entries counted by this round's evaluate items
   unsigned long long* hub_slot;
   int hub_wide;
