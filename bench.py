@@ -302,7 +302,7 @@ KERNEL_BYTES = {
     "hub_build": "hub-table builds: (column 4 + label 4 + weight) per arc of a rebuilt hub + 8 per table slot "
                  "written (the implementation's data structure, not a per-round figure of the method; the "
                  "method's per-round bytes are under 'rounds')",
-    "hub_prepare": "8 per hub-table slot cleared, or read and written by a compaction, + 8 per hub (routing)",
+    "hub_prepare": "8 per hub-table slot cleared, or read and written by a compaction, + 8 per hub (sorting)",
     "hub_eval": "per live histogram entry 24 (+ 8 Sigma_tot for Louvain) + 12 per examined hub",
     "hub_mark": "5 per arc of a moved hub (column, flag) + 64 per logged hub-histogram update",
     "scan_warp": "per examined vertex 13 (+ 24 Louvain) + per scanned arc (column 4 + label 4 + weight) "
@@ -315,8 +315,10 @@ KERNEL_BYTES = {
 def sources_digest() -> str:
     """Digest of the kernel sources a committed ncu figure was taken on."""
     h = hashlib.sha256()
-    for name in ("scan.cu", "graph.cu", "common.cuh"):
-        h.update(open(os.path.join(ROOT, "paper_2507_06471_gb300", "csrc", name), "rb").read())
+    for name in ("scan.cu", "scan.cuh", "graph.cu", "common.cuh"):  # scan.cuh: device code of the scan kernels
+        path = os.path.join(ROOT, "paper_2507_06471_gb300", "csrc", name)
+        if os.path.exists(path):
+            h.update(open(path, "rb").read())
     return h.hexdigest()[:16]
 
 
@@ -345,9 +347,9 @@ def kernel_group(name: str) -> str:
     base = m.group(1)
     rest = name[m.end():]
     targs = rest[1:rest.find(">")].split(",") if rest.startswith("<") else []
-    if base in ("k_hub_sort", "k_hub_prepare", "k_hub_retry", "k_hub_route"):
+    if base in ("k_hub_sort", "k_hub_prepare", "k_hub_route"):
         return "hub_prepare"
-    if base in ("k_hub_build_cl", "k_hub_build"):
+    if base in ("k_hub_build_cl", "k_hub_retry", "k_hub_build"):
         return "hub_build"
     if base in ("k_hub_eval_small", "k_hub_eval"):
         return "hub_eval"

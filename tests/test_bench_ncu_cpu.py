@@ -124,3 +124,20 @@ def test_summary_wide_layout_and_traffic(tmp_path, capsys, monkeypatch):
     assert bench.ncu_traffic("hub_build", 1.0e9) == (None, None)  # no capture covers it
     (csrc / "scan.cu").write_text("// changed kernel source\n")
     assert bench.ncu_traffic("scan_warp", 2.0e9) == (None, None)  # stale once the sources change
+
+
+@pytest.mark.parametrize("name", ["scan.cu", "scan.cuh", "graph.cu", "common.cuh"])
+def test_traffic_is_stale_once_any_source_of_the_scan_kernels_changes(name, tmp_path, monkeypatch):
+    csrc = tmp_path / "paper_2507_06471_gb300" / "csrc"
+    csrc.mkdir(parents=True)
+    for n in os.listdir(os.path.join(ROOT, "paper_2507_06471_gb300", "csrc")):
+        (csrc / n).write_bytes(open(os.path.join(ROOT, "paper_2507_06471_gb300", "csrc", n), "rb").read())
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    before = bench.sources_digest()
+    (csrc / name).write_text((csrc / name).read_text() + "// changed\n")
+    assert bench.sources_digest() != before
+
+
+def test_retried_rebuilds_are_builds():
+    assert bench.kernel_group("cd::<unnamed>::k_hub_retry(cd::<unnamed>::ScanCtx)") == "hub_build"
+    assert bench.kernel_group("cd::<unnamed>::k_hub_sort(cd::<unnamed>::ScanCtx)") == "hub_prepare"
