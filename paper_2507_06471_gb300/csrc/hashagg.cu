@@ -473,6 +473,22 @@ __global__ void k_ag_tables_own(const int32_t* __restrict__ ll, int64_t nl, cons
 // weights: a slot is one word (key << 32 | weight), claimed with its weight or
 // added to with one atomic; the sums stay below 2^31, so the weight never
 // carries into the key. 64-bit weights: key and weight in two arrays.
+//
+// The rows of the coarse graph come out in the order of these tables, so their
+// hash must have nothing in common with that of the shared-memory tables that
+// read such rows in chunks (smem_insert: the golden ratio's multiplier). With the
+// golden ratio here too, 4,096 columns in a row had a few hundred homes at most
+// among 8,192 slots, and an insert walked past hundreds. The hub builds of the
+// first round with labels on R-MAT 26's coarse graph: 260 ms so, 152 with the rows
+// extracted 32 slots at a time by whichever warp comes, 64 with SplitMix64's
+// output function. (Another multiplier alone is as fast, but keys that are
+// neighbours under one multiplier differ by few values, which crowd as well.)
+__device__ __forceinline__ uint64_t merge_home(int32_t key, unsigned lg) {
+  uint64_t z = (uint32_t)key;
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+  return (z ^ (z >> 31)) >> (64 - lg);
+}
 template <class V>
 __global__ void __launch_bounds__(NT) k_ag_merge(const int64_t* __restrict__ sstart, const int32_t* __restrict__ ch_seg,
                                                  const int64_t* __restrict__ ch_off, const int32_t* __restrict__ dch,
@@ -490,7 +506,7 @@ __global__ void __launch_bounds__(NT) k_ag_merge(const int64_t* __restrict__ sst
     for (int j = threadIdx.x; j < d; j += NT) {
       const int32_t key = ab[p + j];
       const V w = aw[p + j];
-      uint64_t h = ((uint64_t)(uint32_t)key * 0x9E3779B97F4A7C15ull) >> (64 - lg);
+      uint64_t h = merge_home(key, lg);
       for (uint64_t probe = 0; probe <= mask; ++probe) {
         if constexpr (sizeof(V) == 4) {
           const unsigned long long mine = ((unsigned long long)(uint32_t)key << 32) | w;

@@ -59,3 +59,32 @@ def test_segment_edges(sizes, wmax, loops):
     assert coarse.vol == G.vol
     coarse.close()
     G.close()
+
+
+@pytest.mark.parametrize("wmax", [1, 2_000_000_000])
+@pytest.mark.parametrize("leaves", [20_000, 200_000])
+def test_long_rows_spread_over_the_tables_that_read_them(leaves, wmax):
+    # the columns of a long coarse row come in the order of the table they were merged in; read in chunks of 4,096 and
+    # 1,024, they must spread over shared-memory tables of twice that many slots as any labels do (4,096 random ones have
+    # 3,223 homes among 8,192 slots, 1,024 have 806 among 2,048), not crowd into a few
+    import paper_2507_06471_gb300 as cd
+    rng = np.random.default_rng(leaves)
+    n = leaves + 1
+    off = np.concatenate([[0], leaves + np.arange(leaves + 1)]).astype(np.int64)
+    cols = np.concatenate([1 + np.arange(leaves), np.zeros(leaves)]).astype(np.int32)
+    w = None
+    if wmax > 1:
+        ws = rng.integers(wmax // 2, wmax, leaves).astype(np.int32)
+        w = torch.from_numpy(np.concatenate([ws, ws])).cuda()
+    G = cd.Graph(torch.from_numpy(off).cuda(), torch.from_numpy(cols).cuda(), w)
+    assert (G.vol < 2**31) == (wmax == 1)  # both widths of the segments
+    coarse, k = G.aggregate(torch.arange(n, dtype=torch.int32, device="cuda"))
+    coff, ccols, _ = coarse.download()
+    coarse.close()
+    G.close()
+    assert k == n and coff[1] == leaves and np.array_equal(np.sort(ccols[:leaves]), np.arange(1, n))
+    hashes = (ccols[:leaves].astype(np.uint64) * np.uint64(2654435761)) & np.uint64(0xFFFFFFFF)
+    for chunk, lg, least in ((4096, 13, 2500), (1024, 11, 600)):
+        homes = hashes >> np.uint64(32 - lg)
+        for at in range(0, leaves - chunk, chunk):
+            assert len(np.unique(homes[at:at + chunk])) >= least, at
