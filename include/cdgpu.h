@@ -73,12 +73,14 @@ typedef struct cd_params {
                                labels in lockstep); results vary from run to run. 0 (default):
                                synchronous rounds, reproducible */
   int32_t device_loop;      /* Where the round loop runs. 1 (default): on the device where that pays. All
-                               rounds of a run or Louvain level run as one resident kernel on graphs
-                               without hubs (vertices of more than t_hub arcs) and on graphs of at most
-                               2^24 arcs with at most 4,095 of them; otherwise the rounds after the first
-                               run as one captured CUDA graph (a conditional WHILE node whose body is one
-                               round) in batched runs (cd_batch_*), and in others if at least 2^22 arcs and
-                               max_iter > 16 make the graph worth its making; the rest keeps the host loop.
+                               rounds of a run or Louvain level run as one resident kernel on graphs of up
+                               to 2^23 arcs with hubs (vertices of more than t_hub arcs; 4,095 at most) and
+                               2^25 without, half that for local moving and half again without a frontier
+                               (any number at low mean degrees, and in batched runs with a frontier and no
+                               hubs; batched runs: 2^24 otherwise); else the rounds after the first run as
+                               one captured CUDA graph (a conditional WHILE node whose body is one round) in
+                               batched runs (cd_batch_*), and in others if at least 2^22 arcs and max_iter >
+                               16 make the graph worth its making; the rest keeps the host loop.
                                The round number, the stop tests and the trace stay on the device, so a
                                level costs one launch and no per-round host synchronisation. The resident
                                kernel starts when the GPU has room for all its CTAs (on larger graphs all

@@ -356,7 +356,7 @@ constexpr int32_t GRAPH_LOOP_ROUNDS = 16;
 // than this context may have at once); nothing ran and the per-round kernels
 // take the run.
 constexpr int LOOP_REFUSED = 1;
-bool resident_rounds_apply(const cd_graph* g, const RunOpts& o, bool per_graph_stop);
+bool resident_rounds_apply(const cd_graph* g, const RunOpts& o, bool louv, bool per_graph_stop);
 int resident_rounds(cd_graph* g, const RunOpts& o, bool louv, bool singletons, int64_t* moves_out, int32_t* rounds_out,
                     std::vector<int32_t>* graph_rounds);
 int begin_run(cd_graph* g, const cd_params* p);  // validates params, resets trace/profile

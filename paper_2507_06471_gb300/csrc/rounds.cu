@@ -64,9 +64,41 @@ constexpr int64_t SHARED_LOOP_ARCS = (int64_t)1 << 22;
 // LPA with 1e6 arcs among 1e5 vertices: 2.85 -> 1.76 ms with 1e7 vertices in all,
 // 3.08 -> 5.58 ms with 5e7. Graphs of few isolated vertices need no such line: the
 // lists then hold every vertex and are gone through every round too (1e8 vertices
-// of degree 3, a ring and a matching: LPA 93 -> 42 ms, local moving 138 -> 70;
-// degree 2: 58 -> 30 and 62 -> 41; as much from 3e6 vertices on).
+// of degree 3, a ring and a matching: LPA 93 -> 42 ms, local moving 138 -> 70; degree
+// 2: 58 -> 30 and 62 -> 41). What limits those is their arcs, see resident_arcs.
 constexpr int64_t MAX_ISOLATED = (int64_t)1 << 23;
+// Arcs of a run at most. The resident loop saves what a round costs beside its
+// work; the per-round kernels do the work itself faster (more warps per SM, rows dealt
+// out as they are flagged and not by vertex, hub histograms kept from round to round),
+// all the more without a frontier, where every round is a full one, and for local
+// moving, whose rounds hold more work. Resident time over that of the per-round
+// kernels (captured, below 2^22 arcs the host loop), at both sides of the lines:
+//   hubs (R-MAT, edge factors 4 to 32)   LPA         1.5e6..8.2e6 0.40..0.93   1.5e7 1.22..1.43
+//                                        local move  1.6e6..4.1e6 0.45..1.09   7e6..8.2e6 1.05..1.67
+//     without a frontier                 LPA         1.6e6..4.1e6 0.46..0.82   7e6..8.2e6 0.94..1.39
+//                                        local move  1.6e6..2.0e6 0.54..1.25   3.4e6..4.1e6 0.70..1.79
+//   no hubs, mean degree 32 to 128       LPA         3e6..3.2e7 0.50..0.92     3.8e7..1.9e8 0.99..1.19
+//                                        local move  3e6..1.3e7 0.44..0.91     1.9e7..1.9e8 1.06..1.45
+//     8 to 20 (LFR-style 12)             LPA         to 1.6e8 0.30..0.99
+//                                        local move  to 2.4e7 0.34..1.02       3.6e7..1.6e8 0.90..1.62
+//     2 to 4                             both        to 3e8 0.27..1.00
+//     without a frontier, any degree     LPA         to 1.6e7 0.35..1.06       1.9e7..1.6e8 0.91..1.29
+//                                        local move  to 8e6 0.42..0.95         9.6e6..1.9e8 0.95..1.75
+//   (4,000 stars of 400 arcs over a sparse graph, 4e6 arcs: local move 1.16, 1.29 without a frontier)
+// Batched runs are held to 2^24 without a frontier only (Louvain: 1.1e7 0.89, 4.7e7
+// and 5.7e7 1.09..1.15; with one 0.45..0.83 to 5.7e7): most of their graphs stop early.
+constexpr int64_t MEAN_LOW = 4, MEAN_MID = 24;  // mean degrees of vertices that have arcs
+inline int64_t resident_arcs(const cd_graph* g, const RunOpts& o, bool louv) {
+  if (o.batched) return o.use_frontier ? INT64_MAX : (int64_t)1 << 24;
+  int64_t most = (int64_t)1 << (g->nhubs ? 23 : 25);
+  if (g->nhubs == 0 && o.use_frontier) {
+    const int64_t linked = g->n - g->n_isolated;
+    if (g->nnz <= (louv ? MEAN_LOW : MEAN_MID) * linked) return INT64_MAX;
+    if (g->nnz <= MEAN_MID * linked) return most;
+  }
+  if (louv) most /= 2;
+  return o.use_frontier ? most : most / 2;
+}
 constexpr int TRACE_COLS = 8;             // examined, arcs, moved, deferred, candidates, arcs of moved, -, -
 constexpr int HEAD = 8;                   // int64 words before the trace: rounds, moves, status
 constexpr int64_t WAIT_LIMIT = (int64_t)1 << 24;  // polls of one barrier at most (seconds), then CD_ETIMEOUT
@@ -912,11 +944,12 @@ ScanCtx loop_ctx(cd_graph* g, const RunOpts& o, bool louv, bool nk) {
 
 }  // namespace
 
-bool resident_rounds_apply(const cd_graph* g, const RunOpts& o, bool per_graph_stop) {
+bool resident_rounds_apply(const cd_graph* g, const RunOpts& o, bool louv, bool per_graph_stop) {
   return o.device_loop && !o.device_loop_all && !g->timing && !o.async_mode && o.max_iter > 0 && g->n > 0 &&
          g->n_isolated <= std::max(g->n - g->n_isolated, MAX_ISOLATED) &&
          (g->workers <= 1 || g->nnz <= SHARED_LOOP_ARCS) &&
          (g->nhubs == 0 || (g->nhubs <= RH_MAX_HUBS && g->nnz <= RH_MAX_ARCS)) &&
+         g->nnz <= resident_arcs(g, o, louv) &&
          g->bin_start[B_BLK4 + 1] == g->bin_start[B_BLK4] && (!per_graph_stop || (o.threshold == 0 && o.use_frontier));
 }
 

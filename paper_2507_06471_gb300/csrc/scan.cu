@@ -2196,7 +2196,7 @@ namespace {
 int run_lpa_any(cd_graph* g, const RunOpts& o, int32_t* rounds_out, std::vector<int32_t>* rounds) {
   int rc = ensure_run_state(g);
   if (rc) return rc;
-  if (resident_rounds_apply(g, o, rounds != nullptr) &&
+  if (resident_rounds_apply(g, o, false, rounds != nullptr) &&
       (rc = resident_rounds(g, o, false, true, nullptr, rounds_out, rounds)) != LOOP_REFUSED)
     return rc;
   if (g->n > 0)
@@ -2232,7 +2232,7 @@ int run_local_move(cd_graph* g, const RunOpts& o, int init_given, int64_t* moves
                                                                                    g->degw, g->n));
   }
   CD_CHECK(cudaGetLastError());
-  if (resident_rounds_apply(g, o, false) &&
+  if (resident_rounds_apply(g, o, true, false) &&
       (rc = resident_rounds(g, o, true, !init_given, moves_out, rounds_out, nullptr)) != LOOP_REFUSED)
     return rc;
   if (g->n > 0 && !init_given)
@@ -2335,7 +2335,9 @@ int cd_autotune(cd_graph* g, const cd_params* p, int32_t rounds, int32_t* t_warp
       o.max_iter = rounds;
       // laid out before the clock starts, as on a handle that is kept: what the runs will use
       if ((rc = rebin(g, tw[i], th[j]))) break;
-      if ((rc = !resident_rounds_apply(g, o, false) ? ensure_bins(g) : g->nhubs > 0 ? ensure_resident_hubs(g) : CD_OK)) break;
+      for (int louv = 0; louv < 2 && !rc; ++louv)
+        rc = !resident_rounds_apply(g, o, louv, false) ? ensure_bins(g) : g->nhubs > 0 ? ensure_resident_hubs(g) : CD_OK;
+      if (rc) break;
       cudaEventRecord(a, g->stream);
       rc = run_lpa(g, o, nullptr);
       if (!rc) rc = run_local_move(g, o, 0, nullptr, nullptr);

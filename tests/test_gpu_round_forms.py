@@ -175,3 +175,58 @@ def test_autotune_prepares_what_its_runs_use(hubs):
     B.close()
     assert tuned == by_hand
     assert rounds == otr.rounds and np.array_equal(lab.cpu().numpy(), olab)
+
+
+def graph_of(arcs, mean, hub):
+    """A random graph of exactly `arcs` arcs, of mean degree `mean` or so, with a hub of 1,500 arcs or without."""
+    n = arcs // mean
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(arcs % 1000 + mean)
+    u, v = torch.randint(1, n, (2, int(arcs * 0.53)), generator=gen, device="cuda")
+    keys = synth.canonical_keys(u[u != v], v[u != v])
+    star = torch.arange(1, 1501 if hub else 1, device="cuda")  # 0 is in no pair: keys (0, leaf)
+    m = arcs // 2 - len(star)
+    assert len(keys) >= m
+    keys = torch.sort(torch.cat([keys[torch.randperm(len(keys), generator=gen, device="cuda")[:m]], star])).values
+    return synth.csr_from_edge_keys(keys, n, None)
+
+
+# (arcs the resident loop takes at most, mean degree, hub, call, use_frontier)
+LINES = [(1 << 23, 40, True, "lpa", 1), (1 << 22, 40, True, "local_move", 1), (1 << 22, 40, True, "lpa", 0),
+         (1 << 21, 40, True, "local_move", 0), (1 << 24, 40, False, "local_move", 1), (1 << 24, 40, False, "lpa", 0),
+         (1 << 23, 40, False, "local_move", 0), (1 << 23, 12, False, "local_move", 0), (1 << 25, 40, False, "lpa", 1)]
+
+
+@pytest.mark.parametrize("most,mean,hub,call,frontier", LINES)
+def test_resident_loop_up_to_so_many_arcs(most, mean, hub, call, frontier):
+    for arcs in (most, most + 2):
+        g = graph_of(arcs, mean, hub)
+        G = upload(g)
+        assert G.nnz == arcs
+        getattr(G, call)(use_frontier=frontier, max_iter=3)  # lays the structures out
+        a, b = (run(G, loop, call, use_frontier=frontier, max_iter=3) for loop in (1, 0))
+        G.close()
+        assert a[1] == b[1] and all(np.array_equal(x, y) for x, y in zip(a[0], b[0]))
+        assert (a[2] == 2) == (arcs <= most) and (a[2] == b[2]) == (arcs > most)
+
+
+@pytest.mark.parametrize("mean,call", [(3, "lpa"), (3, "local_move"), (20, "lpa")])
+def test_resident_loop_of_low_degrees_has_no_such_line(mean, call):
+    G = upload(graph_of((1 << 25) + 1000, mean, False))
+    a, b = (run(G, loop, call, max_iter=3) for loop in (1, 0))
+    G.close()
+    assert a[2] == 2 and a[1] == b[1] and all(np.array_equal(x, y) for x, y in zip(a[0], b[0]))
+
+
+@pytest.mark.parametrize("frontier", [0, 1])
+def test_resident_loop_of_batches_up_to_so_many_arcs(frontier):
+    for arcs in (1 << 24, (1 << 24) + 2):
+        g = graph_of(arcs, 40, False)
+        G = upload(g)
+        G.set_batches(np.array([0, g.n]))
+        kw = dict(use_frontier=frontier, max_iter=3, max_levels=1)
+        G.batch_louvain(**kw)
+        a, b, c = (run(G, loop, "batch_louvain", **kw) for loop in (1, 0, 2))
+        G.close()
+        assert a[1] == b[1] and all(np.array_equal(x, y) for x, y in zip(a[0], b[0]))
+        assert (a[2] == c[2]) == (frontier == 0 and arcs > 1 << 24)
