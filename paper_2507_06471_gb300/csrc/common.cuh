@@ -343,7 +343,7 @@ void release_batches(cd_graph* g);
 int run_local_move(cd_graph* g, const RunOpts& o, int init_given, int64_t* moves_out,
                    int32_t* rounds_out);
 RunOpts opts_from(const cd_params* p, int32_t level);
-// A solo run on a graph with hubs of at least GRAPH_LOOP_ARCS arcs and with at
+// A solo run that is not resident on a graph of at least GRAPH_LOOP_ARCS arcs and with at
 // least GRAPH_LOOP_ROUNDS rounds to go takes the captured graph too: its launches
 // follow one another without the host's gaps and read-backs (LPA 19.7 -> 18.7 ms
 // and Louvain 135 -> 129 ms on R-MAT 22, 8.6 -> 7.5 and 65.5 -> 61.7 ms on R-MAT

@@ -1,5 +1,5 @@
 // The round loop of a run or Louvain level as one resident kernel, for graphs
-// without hubs or with few of them: every round of Label Propagation
+// without hubs or with few of them up to the sizes of resident_arcs: every round of Label Propagation
 // (Algorithm 1) or local moving (Algorithm 2), synchronous, with the decisions,
 // coins, counters and stop tests of the per-round kernels in scan.cu (the
 // results are the same).
