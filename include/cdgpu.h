@@ -84,8 +84,8 @@ typedef struct cd_params {
                                The round number, the stop tests and the trace stay on the device, so a
                                level costs one launch and no per-round host synchronisation. The resident
                                kernel starts when the GPU has room for all its CTAs (on larger graphs all
-                               there is): it waits for kernels of other streams to end, and a caller whose
-                               own kernel runs until it sees this call's result has to choose 0 or 2. Where
+                               there is): it waits for kernels of other streams to end, the loops of other
+                               host threads among them, and a caller whose own kernel runs until it sees this call's result has to choose 0 or 2. Where
                                the runtime refuses such a launch the per-round kernels run. 2: the
                                captured graph in every run, also where 1 is resident. 0: the host loop
                                everywhere (one read-back per round). Results are identical in every mode;

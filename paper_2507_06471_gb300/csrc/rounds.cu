@@ -1,8 +1,8 @@
 // The round loop of a run or Louvain level as one resident kernel, for graphs
-// without hubs or with few of them up to the sizes of resident_arcs: every round of Label Propagation
-// (Algorithm 1) or local moving (Algorithm 2), synchronous, with the decisions,
-// coins, counters and stop tests of the per-round kernels in scan.cu (the
-// results are the same).
+// without hubs or with few of them up to the sizes of resident_arcs: every round
+// of Label Propagation (Algorithm 1) or local moving (Algorithm 2), synchronous,
+// with the decisions, coins, counters and stop tests of the per-round kernels in
+// scan.cu (the results are the same).
 //
 // Why: a round of a small graph, or a late round of a large one, examines few
 // vertices, and its time is latency: a dozen launches of 3 to 8 us each, a
