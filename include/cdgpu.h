@@ -87,8 +87,9 @@ typedef struct cd_params {
                                there is): it waits for kernels of other streams to end, the loops of other
                                host threads among them, and a caller whose own kernel runs until it sees
                                this call's result has to choose 0 or 2. Where the runtime refuses such a
-                               launch the per-round kernels run. 2: the captured graph in every run, also where 1 is resident. 0: the host loop
-                               everywhere (one read-back per round). Results are identical in every mode;
+                               launch the per-round kernels run. 2: the captured graph in every run, also
+                               where 1 is resident. 0: the host loop everywhere (one read-back per round).
+                               Results are identical in every mode;
                                timing != 0 (per-round events) and the asynchronous mode are never
                                resident, and timing != 0 always uses the host loop */
 } cd_params;
